@@ -3,6 +3,7 @@
 // decoded populations (FP64), and the deterministic FP64 reduction of the
 // scalar diagnostics.
 #include "aa.cuh"
+#include "expansion.cuh"
 
 namespace flame {
 namespace {
@@ -200,28 +201,186 @@ struct SiteReal<float> {
   using type = double;
 };
 
+// What a moments launch writes: the density and velocity need the fluid
+// populations, the current needs everything (CUR implies FLUID); B comes from
+// the magnetic ones alone.  The shell spectra ask for u and B, the band loss
+// for B only, and the unused part is neither loaded nor computed.
 // O: the element type of the outputs (FP64 for flame_moments, FP32 for
 // flame_moments_f32).
-template <class T, bool ODD, class O>
-__global__ void moments_kernel(const T* __restrict__ pop, Grid g, StepConsts k, O* __restrict__ rho,
-                               O* __restrict__ u, O* __restrict__ B, O* __restrict__ J, long long os) {
+template <class O>
+struct MomentsOut {
+  O *rho, *u, *B, *J;
+  long long os;  // stride between the components of u, B and J
+  template <class M>
+  __device__ __forceinline__ void store(const M& m, const StepConsts& k, long long o) const {
+    if (rho) rho[o] = (O)m.rho(k);
+    for (int a = 0; a < 3; ++a) {
+      if (u) u[a * os + o] = (O)m.U[a];
+      if (B) B[a * os + o] = (O)m.B(k, a);
+      if (J) J[a * os + o] = (O)m.J[a];
+    }
+  }
+};
+
+// 16-bit storage: FP32 per site.
+template <class T, bool ODD, class O, bool FLUID, bool CUR>
+__global__ void moments_kernel(const T* __restrict__ pop, Grid g, StepConsts k, MomentsOut<O> out) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z + g.z0;
   if (x >= g.nx || y >= g.ny) return;
   const int site = (z * g.ny + y) * g.nx + x;
   const Nbr nb = make_nbr(x, y, z, g);
-  using R = typename SiteReal<T>::type;
-  R sf[kQ], sg[3][kM];
+  float sf[kQ], sg[3][kM];
   load_site<T, ODD>(pop, site, nb, g.n3, sf, sg);
-  const SiteMoments<R> m = site_moments(sf, sg, k);
-  const long long o = site - (long long)g.z0 * g.nx * g.ny;  // index among the updated sites
-  if (rho) rho[o] = (O)m.rho(k);
-  for (int a = 0; a < 3; ++a) {
-    if (u) u[a * os + o] = (O)m.U[a];
-    if (B) B[a * os + o] = (O)m.B(k, a);
-    if (J) J[a * os + o] = (O)m.J[a];
+  const SiteMoments<float> m = site_moments(sf, sg, k);
+  MomentsOut<O> o = out;
+  if (!FLUID) o.rho = o.u = nullptr;
+  if (!CUR) o.J = nullptr;
+  o.store(m, k, site - (long long)g.z0 * g.nx * g.ny);  // index among the updated sites
+}
+
+// FP32 storage: FP64 moments.  Bound by the FP64 pipe, which has 1/64 of the
+// FP32 rate: the 48 conversions and ~220 operations per site of summing,
+// dividing and solving in FP64 took 1012 us at 128^3 (8.0 ms at 256^3).  The
+// sums over the populations are linear, so they are taken as three-term FP32
+// expansions (72 bits, more than FP64 holds) in the order of the step
+// kernel's 1-D passes and turned into FP64 by their bits; the quotients by
+// rho and the current's solve stay in FP64: 18 operations per site without
+// the current, 65 with it.  128^3: 389 us for all moments, 155 us for u and
+// B (84 us of HBM traffic).
+struct SiteMoments64 {
+  double drho, U[3], dB[3], J[3];
+  __device__ __forceinline__ double rho(const StepConsts& k) const { return (double)k.rho0 + drho; }
+  __device__ __forceinline__ double B(const StepConsts& k, int a) const { return (double)k.Bref[a] + dB[a]; }
+};
+
+// 216 sum_i w_i s_i and 216 sum_i w_i c_ia s_i from the populations in
+// velocity-cube order.
+__device__ __forceinline__ void fluid_sums(const float (&s)[kQ], F3& r216, F3 (&j216)[3]) {
+  F3 M00[3], M10[3], M01[3];
+#pragma unroll
+  for (int pz = 0; pz < 3; ++pz) {
+    F3 m0[3];
+    F2 m1[3];
+#pragma unroll
+    for (int py = 0; py < 3; ++py) {
+      const int q = 3 * (py + 3 * pz);
+      m0[py] = add3(two_sum(s[q + 2], s[q]), 4.f * s[q + 1]);
+      m1[py] = two_diff(s[q + 2], s[q]);
+    }
+    M00[pz] = add3(add3(m0[2], m0[0]), scaled(4.f, m0[1]));
+    M01[pz] = add3(m0[2], -m0[0]);
+    M10[pz] = add3(add3(m1[2], m1[0]), scaled(4.f, m1[1]));
   }
+  r216 = add3(add3(M00[2], M00[0]), scaled(4.f, M00[1]));
+  j216[0] = add3(add3(M10[2], M10[0]), scaled(4.f, M10[1]));
+  j216[1] = add3(add3(M01[2], M01[0]), scaled(4.f, M01[1]));
+  j216[2] = add3(M00[2], -M00[0]);
+}
+
+// a / b given r = 1 / b: the remainder of the first quotient corrects it.
+__device__ __forceinline__ double quotient(double a, double b, double r) {
+  const double q = a * r;
+  return fma(fma(-q, b, a), r, q);
+}
+
+// A site whose sums overflow FP32 or are not finite.
+template <bool ODD>
+__device__ __noinline__ void general_moments(const float* pop, int site, Nbr nb, long long n3, StepConsts k,
+                                             SiteMoments64* m) {
+  double sf[kQ], sg[3][kM];
+  load_site<float, ODD, double>(pop, site, nb, n3, sf, sg);
+  const SiteMoments<double> d = site_moments(sf, sg, k);
+  m->drho = d.drho;
+  for (int a = 0; a < 3; ++a) {
+    m->U[a] = d.U[a];
+    m->dB[a] = d.dB[a];
+    m->J[a] = d.J[a];
+  }
+}
+
+template <bool ODD, class O, bool FLUID, bool CUR>
+__global__ void __launch_bounds__(128)
+    moments64_kernel(const float* __restrict__ pop, Grid g, StepConsts k, MomentsOut<O> out) {
+  static_assert(FLUID || !CUR, "the current needs the velocity");
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z + g.z0;
+  if (x >= g.nx || y >= g.ny) return;
+  const int site = (z * g.ny + y) * g.nx + x;
+  const Nbr nb = make_nbr(x, y, z, g);
+  const long long n3 = g.n3;
+  float s[kQ], sg[3][kM];
+  if constexpr (FLUID) {
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) s[q] = pop[src27<ODD>(idx27(q % 3, (q / 3) % 3, q / 9), site, nb, n3)];
+  }
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+#pragma unroll
+    for (int i = 0; i < kM; ++i) sg[b][i] = pop[src7<ODD>(b, i, site, nb, n3)];
+
+  SiteMoments64 m;
+  float chk = 0.f;  // the last terms carry a NaN from any overflow or non-finite value
+  F3 r216, j216[3], sB[3], A8[3];
+  if constexpr (FLUID) {
+    fluid_sums(s, r216, j216);
+    chk = (r216.l + j216[0].l) + (j216[1].l + j216[2].l);
+  }
+  F2 d[3][3];  // 8 Lambda_ab
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    F2 f[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      f[a] = two_sum(sg[b][2 * a + 1], sg[b][2 * a + 2]);
+      d[a][b] = two_diff(sg[b][2 * a + 1], sg[b][2 * a + 2]);
+    }
+    sB[b] = add3(add3(add3(f[0], f[1]), f[2]), 2.f * sg[b][0]);  // 8 dB
+    chk += sB[b].l;
+  }
+  if constexpr (CUR) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      A8[a] = add3(d[(a + 1) % 3][(a + 2) % 3], -d[(a + 2) % 3][(a + 1) % 3]);
+      chk += A8[a].l;
+    }
+  }
+  if (isfinite(chk)) {
+#pragma unroll
+    for (int b = 0; b < 3; ++b) m.dB[b] = to_double(scaled(0.125f, sB[b]));
+    if constexpr (FLUID) {
+      const double r = to_double(r216), rho216 = fma(216.0, (double)k.rho0, r), ir = 1.0 / rho216;
+      m.drho = r * (1.0 / 216.0);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) m.U[a] = quotient(to_double(j216[a]), rho216, ir);
+    }
+    if constexpr (CUR) {
+      const double gq = 4.0 * (double)k.omegaB, sH = 2.0 * (double)k.alphaH * gq;
+      const double B[3] = {m.B(k, 0), m.B(k, 1), m.B(k, 2)};
+      double y[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int b = (a + 1) % 3, c = (a + 2) % 3;
+        y[a] = fma(2.0 * gq, m.U[b] * B[c] - m.U[c] * B[b], -gq * to_double(scaled(0.125f, A8[a])));
+      }
+      const double b2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
+      const double t = sH * sH * (y[0] * B[0] + y[1] * B[1] + y[2] * B[2]);
+      const double den = fma(sH * sH, b2, 1.0), iden = 1.0 / den;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int b = (a + 1) % 3, c = (a + 2) % 3;
+        m.J[a] = quotient(fma(t, B[a], fma(-sH, y[b] * B[c] - y[c] * B[b], y[a])), den, iden);
+      }
+    }
+  } else {
+    general_moments<ODD>(pop, site, nb, n3, k, &m);
+  }
+  MomentsOut<O> o = out;
+  if (!FLUID) o.rho = o.u = nullptr;
+  if (!CUR) o.J = nullptr;
+  o.store(m, k, site - (long long)g.z0 * g.nx * g.ny);  // index among the updated sites
 }
 
 template <class T, bool ODD>
@@ -362,14 +521,26 @@ __global__ void reduce_final_kernel(const double* __restrict__ partials, int nbl
 // Block of `threads` threads: x-rows of up to `threads` sites, several
 // rows per block when nx is small.
 
+template <class T, class O, bool FLUID, bool CUR>
+void moments_go(int odd, const void* pop, Grid g, const StepConsts& k, const MomentsOut<O>& out, cudaStream_t s) {
+  const dim3 b = site_block(g), gr = site_grid(g, b);
+  const T* p = static_cast<const T*>(pop);
+  if constexpr (sizeof(T) == 4) {
+    if (odd) moments64_kernel<true, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);
+    else moments64_kernel<false, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);
+  } else {
+    if (odd) moments_kernel<T, true, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);
+    else moments_kernel<T, false, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);
+  }
+}
+
 template <class T, class O>
 cudaError_t moments_t(int odd, const void* pop, Grid g, const StepConsts& k, O* rho, O* u, O* B, O* J,
                       long long os, cudaStream_t s) {
-  const dim3 b = site_block(g), gr = site_grid(g, b);
-  if (odd)
-    moments_kernel<T, true, O><<<gr, b, 0, s>>>(static_cast<const T*>(pop), g, k, rho, u, B, J, os);
-  else
-    moments_kernel<T, false, O><<<gr, b, 0, s>>>(static_cast<const T*>(pop), g, k, rho, u, B, J, os);
+  const MomentsOut<O> out{rho, u, B, J, os};
+  if (J) moments_go<T, O, true, true>(odd, pop, g, k, out, s);
+  else if (rho || u) moments_go<T, O, true, false>(odd, pop, g, k, out, s);
+  else moments_go<T, O, false, false>(odd, pop, g, k, out, s);
   return cudaGetLastError();
 }
 

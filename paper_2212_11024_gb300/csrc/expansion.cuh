@@ -1,0 +1,87 @@
+// expansion.cuh -- sums of FP32 values carried as unevaluated sums of two or
+// three FP32 numbers (error-free transformations: Knuth's TwoSum, Dekker's
+// FastTwoSum and the FMA product; Shewchuk 1997, Ogita, Rump and Oishi 2005).
+//
+// Why: GB300 does 128 FP32 operations per clock and SM but only two FP64
+// operations, and a conversion between the two types costs as much as an
+// FP64 operation (measured: add, multiply, fma 1.7, F2F 2.0, division 0.22
+// per clock and SM).  A sum of FP32 values that an FP64 add would take costs
+// 64 FP32 issue slots; the same sum as a three-term expansion costs 13 and
+// is more exact (72 bits carried against 53).
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace flame {
+
+struct F2 {  // h + l
+  float h, l;
+};
+struct F3 {  // h + m + l
+  float h, m, l;
+};
+
+// a + b = h + l exactly.
+__device__ __forceinline__ F2 two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  const float t = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ F2 two_diff(float a, float b) { return two_sum(a, -b); }
+// The same for |a| >= |b| (or a = 0).
+__device__ __forceinline__ F2 fast_two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+
+__device__ __forceinline__ F2 operator-(F2 a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ F3 operator-(F3 a) { return {-a.h, -a.m, -a.l}; }
+
+// Three-term sums; the terms are left unnormalised (each level holds the
+// rounding errors of the one above).
+__device__ __forceinline__ F3 add3(F2 a, F2 b) {
+  const F2 s = two_sum(a.h, b.h), t = two_sum(a.l, b.l), v = two_sum(s.l, t.h);
+  return {s.h, v.h, __fadd_rn(t.l, v.l)};
+}
+__device__ __forceinline__ F3 add3(F3 a, F2 b) {
+  const F2 s = two_sum(a.h, b.h), t = two_sum(a.m, b.l), v = two_sum(s.l, t.h);
+  return {s.h, v.h, __fadd_rn(a.l, __fadd_rn(t.l, v.l))};
+}
+__device__ __forceinline__ F3 add3(F3 a, F3 b) {
+  const F2 s = two_sum(a.h, b.h), t = two_sum(a.m, b.m), v = two_sum(s.l, t.h);
+  return {s.h, v.h, __fadd_rn(__fadd_rn(a.l, b.l), __fadd_rn(t.l, v.l))};
+}
+__device__ __forceinline__ F3 add3(F2 a, float b) {
+  const F2 s = two_sum(a.h, b), t = two_sum(a.l, s.l);
+  return {s.h, t.h, t.l};
+}
+__device__ __forceinline__ F3 add3(F3 a, float b) {
+  const F2 s = two_sum(a.h, b), t = two_sum(a.m, s.l);
+  return {s.h, t.h, __fadd_rn(a.l, t.l)};
+}
+// c a power of two
+__device__ __forceinline__ F2 scaled(float c, F2 a) { return {c * a.h, c * a.l}; }
+__device__ __forceinline__ F3 scaled(float c, F3 a) { return {c * a.h, c * a.m, c * a.l}; }
+
+// h + l as FP64, |l| <= ulp(h) / 2, rounded to nearest: the 53-bit result is
+// assembled from h's bits and l as an integer in units of its last place, so
+// that no FP64 instruction is issued.  Values of h outside [2^-75, 2^127]
+// take FP64 instructions.
+__device__ __forceinline__ double to_double(F2 a) {
+  const unsigned hb = __float_as_uint(a.h), mag = hb & 0x7fffffffu, e = mag >> 23;
+  if (mag == 0u) return (double)a.l;
+  if (e < 52u || e > 253u) return (double)a.h + (double)a.l;
+  // l in units of 2^(exponent(h) - 52), signed like h
+  const float unit = __uint_as_float((306u - e) << 23);
+  int n = __float2int_rn(__uint_as_float(__float_as_uint(a.l) ^ (hb & 0x80000000u)) * unit);
+  // below a power of two the last place is half as large
+  if ((mag & 0x007fffffu) == 0u && n < 0) n *= 2;
+  const long long bits = ((long long)mag << 29) + (896ll << 52) + n;
+  return __longlong_as_double(bits | ((long long)(hb >> 31) << 63));
+}
+__device__ __forceinline__ double to_double(F3 a) {
+  const F2 t = two_sum(a.h, a.m);
+  return to_double(two_sum(t.h, __fadd_rn(t.l, a.l)));
+}
+
+}  // namespace flame

@@ -1,0 +1,118 @@
+"""FP64 diagnostics of FP32 storage (moments and reductions), whose sums run
+in FP32 expansions, against extended-precision sums of the same stored
+values, at the edges of a warp and a block, for zero, tiny, ordinary and
+overflowing values and for both AA parities."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+EPS = 2.0 ** -53
+C27, W27, XI7, W7 = (np.asarray(v) for v in O.lattice())
+
+
+def _slots():
+    """(storage slot, velocity, weight, opposite's storage slot) per natural slot (flame.h)."""
+    fl = [int((c[0] + 1) + 3 * (c[1] + 1) + 9 * (c[2] + 1)) for c in C27]
+    out = [(fl[q], C27[q], W27[q], 26 - fl[q]) for q in range(27)]
+    opp = [0, 2, 1, 4, 3, 6, 5]
+    return out + [(27 + 3 * i + b, XI7[i], W7[i], 27 + 3 * opp[i] + b) for b in range(3) for i in range(7)]
+
+
+def _blob(shape, scale, seed):
+    g = np.random.default_rng(seed).standard_normal((48,) + shape)
+    return (scale * g).astype(np.float32)
+
+
+def _pre_collision(blob, parity):
+    s = np.empty(blob.shape, dtype=np.longdouble)
+    for q, (slot, c, _, opp) in enumerate(_slots()):
+        src = blob[slot] if parity == 0 else np.roll(blob[opp], (int(c[2]), int(c[1]), int(c[0])), (0, 1, 2))
+        s[q] = src
+    return s
+
+
+def _reference(s, omB, aH, Bref):
+    """(moments, their rounding scales) in extended precision."""
+    w = np.array([v[2] for v in _slots()], dtype=np.longdouble)[:, None, None, None]
+    t = w * s
+    a = np.abs(t)
+    drho = t[:27].sum(0)
+    rho = 1 + drho
+    j = np.stack([(C27[:, k, None, None, None] * t[:27]).sum(0) for k in range(3)])
+    U = j / rho
+    sU = a[:27].sum(0) / np.abs(rho) * (1 + np.abs(U) * a[:27].sum(0))
+    g = t[27:].reshape(3, 7, *s.shape[1:])
+    dB, sB = g.sum(1), np.abs(g).sum(1)
+    B = dB + np.asarray(Bref)[:, None, None, None]
+    lam = np.stack([np.stack([g[b, 2 * k + 1] - g[b, 2 * k + 2] for b in range(3)]) for k in range(3)])
+    A = np.stack([lam[1, 2] - lam[2, 1], lam[2, 0] - lam[0, 2], lam[0, 1] - lam[1, 0]])
+    gq = 4 * omB
+    sH = 2 * aH * gq
+    y = -gq * (A - 2 * np.cross(U, B, axis=0))
+    den = 1 + sH ** 2 * (B * B).sum(0)
+    J = (y - sH * np.cross(y, B, axis=0) + sH ** 2 * (y * B).sum(0) * B) / den
+    mB, mU = np.abs(B).max(0) + sB.max(0), np.abs(U).max(0) + sU
+    sy = gq * (np.abs(g).sum((0, 1)) + 4 * mU * mB)
+    sJ = sy * (1 + 2 * sH * mB + 3 * (sH * mB) ** 2) / den
+    return (dict(rho=rho, u=U, B=B, J=J),
+            dict(rho=1 + a[:27].sum(0), u=sU, B=sB + np.abs(B), J=sJ * (1 + (sH * mB) ** 2 / den)))
+
+
+@pytest.mark.parametrize("shape", [(2, 3, 5), (1, 2, 32), (3, 2, 129)])
+@pytest.mark.parametrize("scale", [0.0, 1e-28, 0.05])
+@pytest.mark.parametrize("parity", [0, 1])
+def test_moments_of_fp32_storage_are_fp64(shape, scale, parity):
+    """Each moment within 64 units of FP64 rounding of its terms' magnitude
+    (the sums have at most 27 terms, the current's solve about 40 operations)."""
+    from paper_2212_11024_gb300 import Flame
+    nz, ny, nx = shape
+    Bref = (0.0, 0.03, 0.1)
+    sim = Flame(nx, ny, nz, 0.625, 0.625, 1.5, storage="fp32", B_ref=Bref)
+    blob = _blob(shape, scale, 5)
+    sim.set_state(torch.from_numpy(blob.reshape(-1).view(np.uint8).copy()).cuda(), parity, parity)
+    m = {k: v.cpu().numpy() for k, v in sim.moments().items()}
+    only = torch.empty((3,) + shape, dtype=torch.float64, device="cuda")
+    sim.moments(dict(B=only))
+    uB = {k: torch.empty((3,) + shape, dtype=torch.float64, device="cuda") for k in ("u", "B")}
+    sim.moments(uB)
+    f32 = {k: v.cpu().numpy() for k, v in sim.moments(dtype=torch.float32).items()}
+    sim.close()
+    f = np.float32
+    ref, tol = _reference(_pre_collision(blob, parity), float(f(1 / 0.625)), 1.5, [float(f(b)) for b in Bref])
+    for k in ref:
+        err = np.abs(m[k] - ref[k])
+        assert (err <= 64 * EPS * tol[k]).all(), (k, float((err / (EPS * tol[k] + 1e-300)).max()))
+        assert np.array_equal(f32[k], m[k].astype(np.float32))
+    assert np.array_equal(only.cpu().numpy(), m["B"])
+    assert all(np.array_equal(uB[k].cpu().numpy(), m[k]) for k in uB)
+    if scale == 0.0:
+        assert not m["u"].any() and not m["J"].any() and (m["rho"] == 1.0).all()
+
+
+def test_moments_of_overflowing_and_nonfinite_sites():
+    """Sites whose sums leave FP32's range keep their FP64 moments, and a
+    non-finite population makes its own site non-finite only."""
+    from paper_2212_11024_gb300 import Flame
+    shape = (2, 2, 33)
+    blob = _blob(shape, 0.05, 6)
+    blob[:27, 0, 1, 7] = 3e37
+    blob[5, 1, 0, 32] = np.inf
+    blob[30, 1, 1, 0] = np.nan
+    sim = Flame(33, 2, 2, 0.625, 0.625, 1.5, storage="fp32")
+    sim.set_state(torch.from_numpy(blob.reshape(-1).view(np.uint8).copy()).cuda(), 0, 0)
+    m = {k: v.cpu().numpy() for k, v in sim.moments().items()}
+    sim.close()
+    with np.errstate(all="ignore"):
+        ref, tol = _reference(_pre_collision(blob, 0), float(np.float32(1 / 0.625)), 1.5, (0, 0, 0))
+        off = {k: np.abs(m[k] - ref[k]) for k in ref}
+    bad = np.zeros(shape, bool)
+    bad[1, 0, 32] = bad[1, 1, 0] = True
+    for k in ref:
+        ok = np.broadcast_to(~bad, ref[k].shape)
+        assert (off[k][ok] <= 64 * EPS * np.broadcast_to(tol[k], ref[k].shape)[ok]).all(), k
+    assert not np.isfinite(m["rho"][1, 0, 32]) and not np.isfinite(m["B"][:, 1, 1, 0]).all()
+    assert np.isfinite(m["u"][:, 1, 1, 0]).all()
