@@ -453,7 +453,8 @@ flame_status flame_init_adjoint(flame_ctx *ctx, const double *d_u, const double 
  * memory d_scalars (caller-owned), asynchronously on the context's stream;
  * the non-finite count is in d_scalars[FLAME_S_NONFINITE], not in the
  * status.  nblocks: reduction blocks, 1..FLAME_STATIC_REDUCE_BLOCKS_MAX, or
- * 0 for 4 per SM; larger values fail with FLAME_ERR_PARAM.
+ * 0 for the resident ones (two or three per SM by storage); larger values
+ * fail with FLAME_ERR_PARAM.
  * The partial sums live in a fixed device array that each device holds from
  * library load until exit.  The first call on a device looks up that
  * array's device address (cudaGetSymbolAddress, with the device made

@@ -121,15 +121,6 @@ flame_status sync_and_check(flame_ctx* c) {
   return c->sticky;
 }
 
-int reduce_blocks(const flame_ctx* c) {
-  long long want = (long long)c->nsm * 4;
-  const long long per = (c->g.n3i + 255) / 256;
-  if (want > per) want = per;
-  if (want < 1) want = 1;
-  if (want > flame::kRedBlocksMax) want = flame::kRedBlocksMax;
-  return (int)want;
-}
-
 // FP64 power of a D2Z half spectrum binned into integer shells.
 __global__ void shell_bin_kernel(const cufftDoubleComplex* __restrict__ F, flame::Grid g, int nshell,
                                  int zero_mean, double* __restrict__ shells) {
@@ -473,7 +464,7 @@ static flame_status reduce_raw(flame_ctx* c, double* r) {
       return cuda_fail(c, e);
     }
   }
-  const int nb = reduce_blocks(c);
+  const int nb = flame::reduce_block_count(c->p.storage, c->nsm, c->g.n3i, flame::kRedBlocksMax);
   double* out = c->d_red + (size_t)flame::kRedBlocksMax * flame::kRedVals;
   e = flame::launch_reduce(c->p.storage, c->parity, c->state, c->g, c->k, nb, c->d_red, out, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e);

@@ -63,6 +63,44 @@ __device__ __forceinline__ F3 add3(F3 a, float b) {
 __device__ __forceinline__ F2 scaled(float c, F2 a) { return {c * a.h, c * a.l}; }
 __device__ __forceinline__ F3 scaled(float c, F3 a) { return {c * a.h, c * a.m, c * a.l}; }
 
+// Two-term arithmetic (double-float: 48 bits or more), each result
+// normalised to |l| <= ulp(h) / 2 where it is passed on to another sum.
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  const F2 s = two_sum(a.h, b.h);
+  return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ F2 add2(F2 a, float b) {
+  const F2 s = two_sum(a.h, b);
+  return fast_two_sum(s.h, __fadd_rn(s.l, a.l));
+}
+// ... without the normalisation, for a few terms in a row
+__device__ __forceinline__ F2 add2u(F2 a, F2 b) {
+  const F2 s = two_sum(a.h, b.h);
+  return {s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ F2 add2u(F2 a, float b) {
+  const F2 s = two_sum(a.h, b);
+  return {s.h, __fadd_rn(s.l, a.l)};
+}
+__device__ __forceinline__ F2 mul2(float a, float b) {
+  const float h = __fmul_rn(a, b);
+  return {h, __fmaf_rn(a, b, -h)};
+}
+__device__ __forceinline__ F2 mul2(float a, F2 b) {
+  const float h = __fmul_rn(a, b.h);
+  return {h, __fmaf_rn(a, b.l, __fmaf_rn(a, b.h, -h))};
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  const float h = __fmul_rn(a.h, b.h);
+  return {h, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -h)))};
+}
+// a / b given r = 1 / b.h
+__device__ __forceinline__ F2 div2(F2 a, F2 b, float r) {
+  const float q = __fmul_rn(a.h, r);
+  const float e = __fadd_rn(__fmaf_rn(-q, b.l, __fmaf_rn(-q, b.h, a.h)), a.l);
+  return fast_two_sum(q, __fmul_rn(e, r));
+}
+
 // h + l as FP64, |l| <= ulp(h) / 2, rounded to nearest: the 53-bit result is
 // assembled from h's bits and l as an integer in units of its last place, so
 // that no FP64 instruction is issued.  Values of h outside [2^-75, 2^127]

@@ -121,6 +121,16 @@ constexpr int kRedVals = 17;
 // Upper bound on the reduction's block count (its partials fill
 // kRedBlocksMax * kRedVals doubles of scratch).
 constexpr int kRedBlocksMax = 1024;
+// The reduction's block count over n sites on nsm SMs, `most` at most: as
+// many blocks as are resident (two per SM for FP32 storage, three for
+// 16-bit), so that one wave takes all sites.
+inline int reduce_block_count(int storage, int nsm, long long n, int most) {
+  long long want = (long long)nsm * (storage == 1 ? 2 : 3);
+  const long long per = (n + 255) / 256;
+  if (want > per) want = per;
+  if (want > most) want = most;
+  return want < 1 ? 1 : (int)want;
+}
 
 // Moments of the listed sites: out[10 j + (rho, u[3], B[3], J[3])].
 cudaError_t launch_probe(int storage, int odd, const void* pop, Grid g, const StepConsts& k, int n,

@@ -22,6 +22,7 @@
 
 #include "flame.h"
 #include "flame_internal.h"
+#include "reduce_final.cuh"
 
 namespace {
 
@@ -59,17 +60,11 @@ cudaError_t scratch_address(int device, double** out) {
 __global__ void finalize_kernel(const double* __restrict__ partials, int nblocks, double n3, double br0, double br1,
                                 double br2, double* __restrict__ out) {
   __shared__ double r[flame::kRedVals];
-  const int v = threadIdx.x;
-  if (v < flame::kRedVals) {
-    double a = partials[v];
-    for (int b = 1; b < nblocks; ++b) {
-      const double t = partials[(long long)b * flame::kRedVals + v];
-      a = (v == 14) ? fmax(a, t) : a + t;
-    }
-    r[v] = a;
-  }
+  const int v = threadIdx.x >> 5;  // a warp per quantity
+  const double a = flame::reduce_partials_warp(partials, nblocks, v);
+  if ((threadIdx.x & 31) == 0) r[v] = a;
   __syncthreads();
-  if (v != 0) return;
+  if (threadIdx.x != 0) return;
   const double br[3] = {br0, br1, br2};
   double bm[3], dbm2 = 0.0, hc_corr = 0.0;
   out[FLAME_S_MASS] = r[0];
@@ -98,20 +93,15 @@ extern "C" flame_status flame_reduce_static(flame_ctx* ctx, int nblocks, double*
   if (v.status != FLAME_OK && v.status != FLAME_ERR_NONFINITE) return static_cast<flame_status>(v.status);
   if (!v.initialized) return FLAME_ERR_STATE;
   if (nblocks < 0 || nblocks > FLAME_STATIC_REDUCE_BLOCKS_MAX) return FLAME_ERR_PARAM;
-  if (nblocks == 0) {
-    long long want = (long long)v.nsm * 4;
-    const long long per = (v.g.n3i + 255) / 256;
-    if (want > per) want = per;
-    if (want > FLAME_STATIC_REDUCE_BLOCKS_MAX) want = FLAME_STATIC_REDUCE_BLOCKS_MAX;
-    nblocks = want < 1 ? 1 : (int)want;
-  }
+  if (nblocks == 0)
+    nblocks = flame::reduce_block_count(v.storage, v.nsm, v.g.n3i, FLAME_STATIC_REDUCE_BLOCKS_MAX);
   // failures are recorded in the context's sticky status, as in flame_reduce
   double* scratch = nullptr;
   cudaError_t e = scratch_address(v.device, &scratch);
   if (e != cudaSuccess) return static_cast<flame_status>(flame_ctx_cuda_fail(ctx, e));
   e = flame::launch_reduce_partials(v.storage, v.parity, v.state, v.g, v.k, nblocks, scratch, v.stream);
   if (e != cudaSuccess) return static_cast<flame_status>(flame_ctx_cuda_fail(ctx, e));
-  finalize_kernel<<<1, 32, 0, v.stream>>>(scratch, nblocks, (double)v.g.n3i, v.Bref[0], v.Bref[1], v.Bref[2],
+  finalize_kernel<<<1, 32 * flame::kRedVals, 0, v.stream>>>(scratch, nblocks, (double)v.g.n3i, v.Bref[0], v.Bref[1], v.Bref[2],
                                           d_scalars);
   return static_cast<flame_status>(flame_ctx_cuda_fail(ctx, cudaGetLastError()));
 }

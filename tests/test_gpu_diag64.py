@@ -116,3 +116,98 @@ def test_moments_of_overflowing_and_nonfinite_sites():
         assert (off[k][ok] <= 64 * EPS * np.broadcast_to(tol[k], ref[k].shape)[ok]).all(), k
     assert not np.isfinite(m["rho"][1, 0, 32]) and not np.isfinite(m["B"][:, 1, 1, 0]).all()
     assert np.isfinite(m["u"][:, 1, 1, 0]).all()
+
+
+def _sums(s, omB, aH, Bref):
+    """(flame_reduce_sums, the magnitudes of their terms) in extended precision."""
+    m, tol = _reference(s, omB, aH, Bref)
+    w = np.array([v[2] for v in _slots()], dtype=np.longdouble)[:, None, None, None]
+    t = w * s
+    lam = sum(t[27 + 7 * a + 2 * a + 1] - t[27 + 7 * a + 2 * a + 2] for a in range(3))
+    slam = sum(np.abs(t[27 + 7 * a + 2 * a + 1]) + np.abs(t[27 + 7 * a + 2 * a + 2]) for a in range(3))
+    b = m["B"] - np.asarray(Bref)[:, None, None, None]
+    sb, su, sJ = tol["B"], tol["u"] + np.abs(m["u"]), tol["J"] + np.abs(m["J"])
+    u, J, rho = m["u"], m["J"], m["rho"]
+    dv, sd = 4 * omB * lam, 4 * omB * slam
+    out = [rho.sum()] + [(rho * u[a]).sum() for a in range(3)] + [m["B"][a].sum() for a in range(3)]
+    out += [(u * u).sum(), (b * b).sum(), (u * b).sum()] + [u[a].sum() for a in range(3)]
+    out += [(J * J).sum(), np.sqrt((u * u).sum(0).max()), (dv * dv).sum(), 0.0, rho.size]
+    mag = [tol["rho"].sum()] + [(np.abs(rho) * su[a]).sum() for a in range(3)] + [sb[a].sum() for a in range(3)]
+    mag += [(su * su).sum(), (sb * sb).sum(), (su * sb).sum()] + [su[a].sum() for a in range(3)]
+    mag += [(sJ * sJ).sum(), su.max() * 2, (sd * sd).sum(), 0.0, 0.0]
+    return np.array(out, dtype=np.longdouble), np.array(mag, dtype=np.longdouble)
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 5), (1, 2, 128), (3, 5, 129), (41, 32, 64)])
+@pytest.mark.parametrize("scale", [0.0, 1e-20, 0.05, 1e20])
+def test_sums_of_fp32_storage(shape, scale):
+    """flame_reduce_sums within 2^-43 of the magnitude of the terms (two-term
+    arithmetic of about 40 operations a site), the maximum speed to FP64
+    rounding; 1e20 leaves the expansions' range, so blocks sum in FP64."""
+    from paper_2212_11024_gb300 import Flame
+    nz, ny, nx = shape
+    Bref = (0.0, 0.03, 0.1)
+    sim = Flame(nx, ny, nz, 0.625, 0.625, 1.5, storage="fp32", B_ref=Bref)
+    blob = _blob(shape, scale, 8)
+    sim.set_state(torch.from_numpy(blob.reshape(-1).view(np.uint8).copy()).cuda(), 1, 1)
+    got = sim.reduce_sums()
+    stat = sim.reduce_static().cpu().numpy()
+    red = sim.reduce()
+    sim.close()
+    f = np.float32
+    ref, mag = _sums(_pre_collision(blob, 1), float(f(1 / 0.625)), 1.5, [float(f(b)) for b in Bref])
+    assert (np.abs(got - ref) <= 2.0 ** -43 * mag).all(), ((np.abs(got - ref) / (mag + 1e-300)).tolist())
+    assert abs(got[14] - ref[14]) <= 64 * EPS * mag[14]
+    assert np.allclose(stat, [red[k] for k in list(red)[:14]], rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("storage", ["fp16", "bf16"])
+def test_sums_of_16_bit_storage(storage):
+    """The sums against FP64 sums of flame_moments' fields: the per-site
+    arithmetic is the same FP32 arithmetic, the sums are exact to 2^-43 of
+    their terms' magnitude (2^-22 for the squares, which flame_moments'
+    caller forms from the rounded fields)."""
+    from paper_2212_11024_gb300 import Flame
+    shape = (5, 7, 129)
+    sim = Flame(129, 7, 5, 0.6, 0.7, 1.5, storage=storage, B_ref=(0.0, 0.03, 0.1))
+    gen = torch.Generator().manual_seed(3)
+    vals = 0.05 * torch.randn(48 * 5 * 7 * 129, generator=gen)
+    dt = torch.float16 if storage == "fp16" else torch.bfloat16
+    sim.set_state(vals.to(dt).view(torch.uint8).cuda(), 0, 0)
+    got = sim.reduce_sums()
+    m = {k: v.cpu().numpy() for k, v in sim.moments().items()}
+    sim.close()
+    f = np.float32
+    b = m["B"] - np.array([0.0, f(0.03), f(0.1)], dtype=np.float64)[:, None, None, None]
+    u, J = m["u"], m["J"]
+    exact = 2.0 ** -43
+    for v, t, tol in [(0, m["rho"], exact)] + [(1 + a, m["rho"] * u[a], exact) for a in range(3)] + \
+            [(4 + a, m["B"][a], exact) for a in range(3)] + [(10 + a, u[a], exact) for a in range(3)] + \
+            [(7, u * u, 2.0 ** -22), (8, b * b, 2.0 ** -22), (9, u * b, 2.0 ** -22), (13, J * J, 2.0 ** -22)]:
+        assert abs(got[v] - t.sum()) <= tol * np.abs(t).sum(), v
+    assert abs(got[14] - np.sqrt((u * u).sum(0).max())) <= 2.0 ** -22 * got[14]
+    assert got[16] == 0 and got[17] == 5 * 7 * 129
+
+
+def test_sums_with_nonfinite_sites():
+    """Non-finite sites are counted and left out; the other blocks' and the
+    same block's finite sites are still summed."""
+    from paper_2212_11024_gb300 import Flame, flame
+    shape = (2, 20, 64)
+    for dt, storage in ((torch.float32, "fp32"), (torch.float16, "fp16")):
+        vals = (0.05 * torch.randn((48,) + shape, generator=torch.Generator().manual_seed(4))).to(dt)
+        clean = vals.clone()
+        clean[:, 0, 3, 5] = 0
+        clean[:, 1, 19, 63] = 0
+        vals[3, 0, 3, 5] = float("nan")
+        vals[9, 1, 19, 63] = float("inf")
+        sums = []
+        for v in (vals, clean):
+            sim = Flame(64, 20, 2, 0.6, 0.7, 1.5, storage=storage)
+            sim.set_state(v.reshape(-1).view(torch.uint8).cuda(), 0, 0)
+            sums.append(sim.reduce_sums())
+            sim.close()
+        bad, ok = sums
+        assert bad[16] == 2 and ok[16] == 0
+        # the cleared sites are at rest: rho = 1, everything else zero
+        assert abs(bad[0] + 2 - ok[0]) < 1e-9 and np.allclose(bad[1:16], ok[1:16], rtol=1e-6, atol=1e-9)
