@@ -10,10 +10,10 @@ namespace flame {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Initialisation (once per run).  The arithmetic type R is FP64 for FP32
-// storage and FP32 for 16-bit storage, whose encoding rounds to 2^-11 (FP16)
-// or 2^-8 (BF16) relative, far above FP32's 2^-24; the gradients too are
-// taken in R.
+// Initialisation (once per run).  The arithmetic type R is FP32 for 16-bit
+// storage, whose encoding rounds to 2^-11 (FP16) or 2^-8 (BF16) relative, far
+// above FP32's 2^-24; the gradients too are taken in R.  FP32 storage takes
+// two-term FP32 arithmetic (init_site2), and FP64 where that does not reach.
 
 // Periodic central difference of field f along axis a at (x, y, z), in the
 // per-site arithmetic type R (GB300's FP64 pipe is 1/64 of its FP32 rate, so
@@ -35,91 +35,248 @@ __device__ __forceinline__ R cdiff(const F* f, int a, int x, int y, int z, const
 }
 
 // F: the element type of the caller's fields (FP64 for flame_init, FP32 for
-// flame_init_f32).
+// flame_init_f32).  Writes the site's populations and returns its speed
+// max(|B|/sqrt(rho), |u|).
 template <class T, class R, class F>
-__global__ void init_kernel(T* __restrict__ pop, Grid g, StepConsts k, int noneq, const F* __restrict__ rho_f,
-                            const F* __restrict__ u, const F* __restrict__ Bf, const F* __restrict__ gu,
-                            const F* __restrict__ gB, unsigned* __restrict__ speed_bits) {
+__device__ __forceinline__ float init_site(T* __restrict__ pop, const Grid& g, const StepConsts& k, int noneq,
+                                           const F* __restrict__ rho_f, const F* __restrict__ u,
+                                           const F* __restrict__ Bf, const F* __restrict__ gu,
+                                           const F* __restrict__ gB, int x, int y, int z) {
+      const long long n3 = g.n3;
+      const long long site = ((long long)z * g.ny + y) * g.nx + x;
+      const R rho = rho_f ? (R)rho_f[site] : (R)1;
+      const R U[3] = {(R)u[site], (R)u[n3 + site], (R)u[2 * n3 + site]};
+      const R B[3] = {(R)Bf[site], (R)Bf[n3 + site], (R)Bf[2 * n3 + site]};
+      R du[9], dB[9];
+  #pragma unroll
+      for (int a = 0; a < 3; ++a)
+  #pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          du[3 * a + b] = gu ? (R)gu[(3 * a + b) * n3 + site] : cdiff<R>(u + b * n3, a, x, y, z, g);
+          dB[3 * a + b] = gB ? (R)gB[(3 * a + b) * n3 + site] : cdiff<R>(Bf + b * n3, a, x, y, z, g);
+        }
+      const R J0[3] = {dB[5] - dB[7], dB[6] - dB[2], dB[1] - dB[3]};  // curl B
+      const R omega = (R)k.omega, omegaB = (R)k.omegaB, aH = (R)k.alphaH;
+      const R Br[3] = {(R)k.Bref[0], (R)k.Bref[1], (R)k.Bref[2]};
+      const R b[3] = {B[0] - Br[0], B[1] - Br[1], B[2] - Br[2]};
+      R N[3][3];
+  #pragma unroll
+      for (int a = 0; a < 3; ++a)
+  #pragma unroll
+        for (int c = 0; c < 3; ++c) N[a][c] = Br[a] * b[c] + b[a] * Br[c] + b[a] * b[c];
+      const R miso = Br[0] * b[0] + Br[1] * b[1] + Br[2] * b[2] + (R)0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
+      const R trN3 = (N[0][0] + N[1][1] + N[2][2]) / (R)3;
+      R Pn[3][3];  // first-order non-equilibrium stress -(rho cs^2/omega)(du + du^T)
+  #pragma unroll
+      for (int a = 0; a < 3; ++a)
+  #pragma unroll
+        for (int c = 0; c < 3; ++c) Pn[a][c] = noneq ? -(rho / ((R)3 * omega)) * (du[3 * a + c] + du[3 * c + a]) : (R)0;
+      const R trPn3 = (Pn[0][0] + Pn[1][1] + Pn[2][2]) / (R)3;
+      const R drho = rho - (R)k.rho0;
+  #pragma unroll
+      for (int i = 0; i < kQ; ++i) {
+        const int c[3] = {cx27(i), cy27(i), cz27(i)};
+        R E = 0;  // prod(psi/w1) - 1, accumulated stably
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const R uu = U[a] * U[a];
+          const R ea = c[a] == 0 ? (R)-1.5 * uu : (R)3 * uu + (R)(3 * c[a]) * U[a];
+          E = E + ea + E * ea;
+        }
+        R cNc = 0, cPc = 0;
+  #pragma unroll
+        for (int a = 0; a < 3; ++a)
+  #pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            if (c[a] * c[d] == 0) continue;
+            cNc += (R)(c[a] * c[d]) * N[a][d];
+            cPc += (R)(c[a] * c[d]) * Pn[a][d];
+          }
+        const R c2 = (R)(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
+        const R L = (R)4.5 * (miso * (c2 - (R)1) - cNc + trN3);
+        const R ne = (R)4.5 * (cPc - trPn3);
+        pop[(long long)phys(i) * n3 + site] = Codec<T>::enc((float)(drho + rho * E + L + ne));
+      }
+      const R V[3] = {U[0] - aH * J0[0], U[1] - aH * J0[1], U[2] - aH * J0[2]};
+  #pragma unroll
+      for (int bb = 0; bb < 3; ++bb)
+  #pragma unroll
+        for (int i = 0; i < kM; ++i) {
+          const int xi[3] = {mx7(i), my7(i), mz7(i)};
+          R l0 = 0, ne = 0;
+  #pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            if (xi[a] == 0) continue;
+            l0 += (R)xi[a] * (V[a] * B[bb] - B[a] * V[bb]);
+            ne += (R)xi[a] * dB[3 * a + bb];
+          }
+          const R v = b[bb] + (R)4 * l0 - (noneq ? ne / omegaB : (R)0);
+          pop[(long long)phys(mslot(bb, i)) * n3 + site] = Codec<T>::enc((float)v);
+        }
+      const R va = sqrt((B[0] * B[0] + B[1] * B[1] + B[2] * B[2]) / rho);
+      const R um = sqrt(U[0] * U[0] + U[1] * U[1] + U[2] * U[2]);
+      return (float)fmax(va, um);
+}
+
+// FP32 storage: the populations are FP64 values rounded to FP32.  Their ~770
+// FP64 operations a site (and conversions, which cost as much) were all this
+// kernel did: 2932 us at 128^3 (23.4 ms at 256^3), where the bytes take 74;
+// now 520 us (4.2 ms), bound by FP32 issue.  They are computed
+// in two-term FP32 arithmetic (48 bits: the rounded results are FP64's but
+// for one in 2^20 or so) and in the columns of the step's collision: for each
+// (c_x, c_y) the three values along c_z are Z0 + Z1 c_z + Z2 c_z^2, the
+// Lorentz term's N and the non-equilibrium stress P entering as K = N - P.
+// FP64 fields are split by integer operations.  Sites with values outside
+// [2^-40, 2^40] (density) or 2^40 (fields) take the FP64 path.
+struct InitConsts {
+  F2 p;    // -1 / (3 omega), or 0 without the non-equilibrium parts
+  F2 iwB;  // 1 / omega_B, or 0
+};
+
+__device__ __forceinline__ F2 field2(const double* f, long long i) { return from_double(f[i]); }
+__device__ __forceinline__ F2 field2(const float* f, long long i) { return {f[i], 0.f}; }
+__device__ __forceinline__ float rounded(F2 a) { return __fadd_rn(a.h, a.l); }
+
+template <class F>
+__device__ __noinline__ float init_site_fp64(float* pop, Grid g, StepConsts k, int noneq, const F* rho_f, const F* u,
+                                             const F* Bf, const F* gu, const F* gB, int x, int y, int z) {
+  return init_site<float, double, F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+}
+
+template <class F>
+__device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid& g, const StepConsts& k,
+                                            const InitConsts& ic, int noneq, const F* __restrict__ rho_f,
+                                            const F* __restrict__ u, const F* __restrict__ Bf,
+                                            const F* __restrict__ gu, const F* __restrict__ gB, int x, int y, int z) {
+  const long long n3 = g.n3;
+  const int site = (z * g.ny + y) * g.nx + x;
+  const Nbr nb = make_nbr(x, y, z, g);
+  const int fwd[3] = {nb.xp, nb.yp, nb.zp}, back[3] = {nb.xm, nb.ym, nb.zm};
+  // d_a F_b
+  auto grad = [&](const F* f, const F* gf, int a, int b) -> F2 {
+    if (gf) return field2(gf + (3 * a + b) * n3, site);
+    return scaled(0.5f, add2(field2(f + b * n3, site + fwd[a]), -field2(f + b * n3, site + back[a])));
+  };
+  const F2 rho = rho_f ? field2(rho_f, site) : F2{1.f, 0.f};
+  F2 U[3], B[3], b[3], dB[9], S[6];
+  float top = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    U[a] = field2(u + a * n3, site);
+    B[a] = field2(Bf + a * n3, site);
+    top = fmaxf(top, fmaxf(fabsf(U[a].h), fabsf(B[a].h)));
+    if (isnan(U[a].h) || isnan(B[a].h)) top = __uint_as_float(0x7f800000u);
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    dB[i] = grad(Bf, gB, i / 3, i % 3);
+    top = isnan(dB[i].h) ? __uint_as_float(0x7f800000u) : fmaxf(top, fabsf(dB[i].h));
+  }
+  constexpr int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};  // xx yy zz xy xz yz
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {  // d_a u_b + d_b u_a
+    S[i] = i < 3 ? scaled(2.f, grad(u, gu, i, i)) : add2(grad(u, gu, ia[i], ib[i]), grad(u, gu, ib[i], ia[i]));
+    top = isnan(S[i].h) ? __uint_as_float(0x7f800000u) : fmaxf(top, fabsf(S[i].h));
+  }
+  if (!(top < 0x1p40f && rho.h < 0x1p40f && rho.h > 0x1p-40f))
+    return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+  float* out = pop + site;
+  auto put = [&](int slot, F2 v) { out[(long long)slot * n3] = rounded(v); };
+#pragma unroll
+  for (int a = 0; a < 3; ++a) b[a] = add2(B[a], -k.Bref[a]);
+
+  // magnetic: b_b + sign (4 (V_a B_b - B_a V_b) - d_a B_b / omega_B), V = U - d_i curl B
+  {
+    F2 V[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int p = (a + 1) % 3, q = (a + 2) % 3;
+      V[a] = add2(U[a], mul2(-k.alphaH, add2(dB[3 * p + q], -dB[3 * q + p])));
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      put(kQ + c, b[c]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const F2 ne = -mul2(ic.iwB, dB[3 * a + c]);
+        const F2 t = a == c ? ne : add2u(scaled(4.f, add2(mul2(V[a], B[c]), -mul2(B[a], V[c]))), ne);
+        put(kQ + 3 * (2 * a + 1) + c, add2u(b[c], t));
+        put(kQ + 3 * (2 * a + 2) + c, add2u(b[c], -t));
+      }
+    }
+  }
+
+  // fluid
+  F2 K[6], miso{0.f, 0.f};
+  const F2 rp = mul2(rho, ic.p);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int a = ia[i], c = ib[i];
+    const F2 N = add2u(mul2(b[c], B[a]), mul2(k.Bref[c], b[a]));
+    K[i] = add2(N, -mul2(rp, S[i]));
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) miso = add2u(miso, scaled(0.5f, mul2(b[a], add2(B[a], k.Bref[a]))));
+  const F2 drho = add2(rho, -k.rho0);
+  const F2 base0 = add2(drho, add2(mul2(1.5f, add2(add2u(K[0], K[1]), K[2])), mul2(-4.5f, miso)));
+  const F2 LA = mul2(4.5f, add2(miso, -K[0])), LB = mul2(4.5f, add2(miso, -K[1])), LZ = mul2(4.5f, add2(miso, -K[2]));
+  const F2 LC = mul2(9.f, K[3]), NX = mul2(-9.f, K[4]), NY = mul2(-9.f, K[5]);
+  F2 ex[3], ey[3];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    F2* e = h ? ey : ex;
+    const F2 uu = mul2(U[h], U[h]), u3 = mul2(3.f, U[h]), q = mul2(3.f, uu);
+    e[0] = add2(q, -u3);
+    e[1] = mul2(-1.5f, uu);
+    e[2] = add2(q, u3);
+  }
+  const F2 uzz = mul2(U[2], U[2]);
+  const F2 e0z = mul2(-1.5f, uzz), e1z = mul2(3.f, U[2]), e2z = mul2(4.5f, uzz);
+#pragma unroll
+  for (int py = 0; py < 3; ++py)
+#pragma unroll
+    for (int px = 0; px < 3; ++px) {
+      const int cx = px - 1, cy = py - 1;
+      const F2 rexy = mul2(rho, add2(mul2(ex[px], ey[py]), add2(ex[px], ey[py])));
+      const F2 gg = add2(rexy, rho);
+      F2 L = base0;
+      if (cx) L = add2u(L, LA);
+      if (cy) L = add2u(L, LB);
+      if (cx * cy) L = add2u(L, cx * cy > 0 ? -LC : LC);
+      const F2 Z0 = add2u(add2u(mul2(gg, e0z), rexy), L);
+      F2 Z1 = mul2(gg, e1z);
+      if (cx) Z1 = add2u(Z1, cx > 0 ? NX : -NX);
+      if (cy) Z1 = add2u(Z1, cy > 0 ? NY : -NY);
+      const F2 tz = add2u(Z0, add2u(mul2(gg, e2z), LZ));
+      put(px + 3 * py, add2u(tz, -Z1));
+      put(px + 3 * py + 9, Z0);
+      put(px + 3 * py + 18, add2u(tz, Z1));
+    }
+
+  // max(|B|^2 / rho, |u|^2), then its root: a Newton step on the FP32 one
+  const F2 b2 = add2(add2u(mul2(B[0], B[0]), mul2(B[1], B[1])), mul2(B[2], B[2]));
+  const F2 u2 = add2(add2u(mul2(U[0], U[0]), mul2(U[1], U[1])), mul2(U[2], U[2]));
+  const F2 va = div2(b2, rho, 1.f / rho.h);
+  const F2 s2 = va.h > u2.h || (va.h == u2.h && va.l > u2.l) ? va : u2;
+  const float r = sqrtf(s2.h);
+  return r > 0x1p-40f ? r + __fadd_rn(__fmaf_rn(-r, r, s2.h), s2.l) / (2.f * r) : r;
+}
+
+template <class T, class R, class F>
+__global__ void __launch_bounds__(128)
+    init_kernel(T* __restrict__ pop, Grid g, StepConsts k, InitConsts ic, int noneq, const F* __restrict__ rho_f,
+                const F* __restrict__ u, const F* __restrict__ Bf, const F* __restrict__ gu,
+                const F* __restrict__ gB, unsigned* __restrict__ speed_bits) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z + g.z0;
   const bool in = x < g.nx && y < g.ny;
   float sp = 0.f;
   if (in) {
-    const long long n3 = g.n3;
-    const long long site = ((long long)z * g.ny + y) * g.nx + x;
-    const R rho = rho_f ? (R)rho_f[site] : (R)1;
-    const R U[3] = {(R)u[site], (R)u[n3 + site], (R)u[2 * n3 + site]};
-    const R B[3] = {(R)Bf[site], (R)Bf[n3 + site], (R)Bf[2 * n3 + site]};
-    R du[9], dB[9];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        du[3 * a + b] = gu ? (R)gu[(3 * a + b) * n3 + site] : cdiff<R>(u + b * n3, a, x, y, z, g);
-        dB[3 * a + b] = gB ? (R)gB[(3 * a + b) * n3 + site] : cdiff<R>(Bf + b * n3, a, x, y, z, g);
-      }
-    const R J0[3] = {dB[5] - dB[7], dB[6] - dB[2], dB[1] - dB[3]};  // curl B
-    const R omega = (R)k.omega, omegaB = (R)k.omegaB, aH = (R)k.alphaH;
-    const R Br[3] = {(R)k.Bref[0], (R)k.Bref[1], (R)k.Bref[2]};
-    const R b[3] = {B[0] - Br[0], B[1] - Br[1], B[2] - Br[2]};
-    R N[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) N[a][c] = Br[a] * b[c] + b[a] * Br[c] + b[a] * b[c];
-    const R miso = Br[0] * b[0] + Br[1] * b[1] + Br[2] * b[2] + (R)0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
-    const R trN3 = (N[0][0] + N[1][1] + N[2][2]) / (R)3;
-    R Pn[3][3];  // first-order non-equilibrium stress -(rho cs^2/omega)(du + du^T)
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) Pn[a][c] = noneq ? -(rho / ((R)3 * omega)) * (du[3 * a + c] + du[3 * c + a]) : (R)0;
-    const R trPn3 = (Pn[0][0] + Pn[1][1] + Pn[2][2]) / (R)3;
-    const R drho = rho - (R)k.rho0;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-      const int c[3] = {cx27(i), cy27(i), cz27(i)};
-      R E = 0;  // prod(psi/w1) - 1, accumulated stably
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const R uu = U[a] * U[a];
-        const R ea = c[a] == 0 ? (R)-1.5 * uu : (R)3 * uu + (R)(3 * c[a]) * U[a];
-        E = E + ea + E * ea;
-      }
-      R cNc = 0, cPc = 0;
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          if (c[a] * c[d] == 0) continue;
-          cNc += (R)(c[a] * c[d]) * N[a][d];
-          cPc += (R)(c[a] * c[d]) * Pn[a][d];
-        }
-      const R c2 = (R)(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
-      const R L = (R)4.5 * (miso * (c2 - (R)1) - cNc + trN3);
-      const R ne = (R)4.5 * (cPc - trPn3);
-      pop[(long long)phys(i) * n3 + site] = Codec<T>::enc((float)(drho + rho * E + L + ne));
-    }
-    const R V[3] = {U[0] - aH * J0[0], U[1] - aH * J0[1], U[2] - aH * J0[2]};
-#pragma unroll
-    for (int bb = 0; bb < 3; ++bb)
-#pragma unroll
-      for (int i = 0; i < kM; ++i) {
-        const int xi[3] = {mx7(i), my7(i), mz7(i)};
-        R l0 = 0, ne = 0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          if (xi[a] == 0) continue;
-          l0 += (R)xi[a] * (V[a] * B[bb] - B[a] * V[bb]);
-          ne += (R)xi[a] * dB[3 * a + bb];
-        }
-        const R v = b[bb] + (R)4 * l0 - (noneq ? ne / omegaB : (R)0);
-        pop[(long long)phys(mslot(bb, i)) * n3 + site] = Codec<T>::enc((float)v);
-      }
-    const R va = sqrt((B[0] * B[0] + B[1] * B[1] + B[2] * B[2]) / rho);
-    const R um = sqrt(U[0] * U[0] + U[1] * U[1] + U[2] * U[2]);
-    sp = (float)fmax(va, um);
+    if constexpr (sizeof(T) == 4)
+      sp = init_site2<F>(pop, g, k, ic, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+    else
+      sp = init_site<T, R, F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
     if (!isfinite(sp)) sp = __uint_as_float(0x7f800000u);
   }
   // max speed: one atomic per warp (non-negative floats order like their bits)
@@ -772,22 +929,29 @@ cudaError_t moments_t(int odd, const void* pop, Grid g, const StepConsts& k, O* 
   return cudaGetLastError();
 }
 
+F2 split(double v) {
+  const float h = (float)v;
+  return {h, (float)(v - (double)h)};
+}
+
 template <class F>
 cudaError_t init_t(int storage, void* pop, Grid g, const StepConsts& k, int noneq, const F* rho, const F* u,
                    const F* B, const F* gu, const F* gB, unsigned* speed_bits, cudaStream_t s) {
   const dim3 b = site_block(g), gr = site_grid(g, b);
+  const InitConsts ic{noneq ? split(-1.0 / (3.0 * (double)k.omega)) : F2{0.f, 0.f},
+                      noneq ? split(1.0 / (double)k.omegaB) : F2{0.f, 0.f}};
   switch (storage) {
     case 1:
-      init_kernel<float, double, F><<<gr, b, 0, s>>>(static_cast<float*>(pop), g, k, noneq, rho, u, B, gu, gB,
+      init_kernel<float, double, F><<<gr, b, 0, s>>>(static_cast<float*>(pop), g, k, ic, noneq, rho, u, B, gu, gB,
                                                       speed_bits);
       break;
     case 2:
-      init_kernel<__half, float, F><<<gr, b, 0, s>>>(static_cast<__half*>(pop), g, k, noneq, rho, u, B, gu, gB,
+      init_kernel<__half, float, F><<<gr, b, 0, s>>>(static_cast<__half*>(pop), g, k, ic, noneq, rho, u, B, gu, gB,
                                                       speed_bits);
       break;
     case 3:
-      init_kernel<__nv_bfloat16, float, F><<<gr, b, 0, s>>>(static_cast<__nv_bfloat16*>(pop), g, k, noneq, rho, u,
-                                                             B, gu, gB, speed_bits);
+      init_kernel<__nv_bfloat16, float, F><<<gr, b, 0, s>>>(static_cast<__nv_bfloat16*>(pop), g, k, ic, noneq, rho,
+                                                             u, B, gu, gB, speed_bits);
       break;
     default:
       return cudaErrorInvalidValue;

@@ -101,6 +101,22 @@ __device__ __forceinline__ F2 div2(F2 a, F2 b, float r) {
   return fast_two_sum(q, __fmul_rn(e, r));
 }
 
+// An FP64 value as h + l (48 bits or more): h takes the top 24 bits of the
+// significand, l the 29 below.  Magnitudes in [2^-74, 2^126) and zero by
+// integer operations, others by FP64 instructions.
+__device__ __forceinline__ F2 from_double(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), sign = hi & 0x80000000u;
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e < 949u || e > 1148u) {
+    if (x == 0.0) return {0.f, 0.f};
+    const float h = (float)x;
+    return {h, (float)(x - (double)h)};
+  }
+  const unsigned h = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
+  const float l = __int2float_rn((int)(lo & 0x1fffffffu)) * __uint_as_float((e - 948u) << 23);
+  return {__uint_as_float(h | sign), __uint_as_float(__float_as_uint(l) | sign)};
+}
+
 // h + l as FP64, |l| <= ulp(h) / 2, rounded to nearest: the 53-bit result is
 // assembled from h's bits and l as an integer in units of its last place, so
 // that no FP64 instruction is issued.  Values of h outside [2^-75, 2^127]

@@ -211,3 +211,71 @@ def test_sums_with_nonfinite_sites():
         assert bad[16] == 2 and ok[16] == 0
         # the cleared sites are at rest: rho = 1, everything else zero
         assert abs(bad[0] + 2 - ok[0]) < 1e-9 and np.allclose(bad[1:16], ok[1:16], rtol=1e-6, atol=1e-9)
+
+
+def _stored(f, Bref):
+    """Deviations from rest over the weight of oracle populations f [48, ...]."""
+    s = np.empty(f.shape)
+    feq = O.feq_hermite(1.0, np.zeros(3)) + O.lorentz(np.array(Bref, dtype=float))
+    geq = O.geq_hall(np.array(Bref, dtype=float), np.zeros(3), np.zeros(3), 0.0).reshape(21)
+    rest = np.concatenate([feq, geq])
+    for q, (slot, _, w, _) in enumerate(_slots()):
+        s[slot] = (f[q] - rest[q]) / w
+    return s
+
+
+@pytest.mark.parametrize("shape", [(3, 4, 5), (2, 3, 129), (9, 8, 32)])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("given", ["u B", "rho", "gradients", "no noneq"])
+def test_initial_populations_of_fp32_storage(shape, dtype, given):
+    """Every stored value is the oracle's FP64 value rounded to FP32: within
+    0.501 units of its last place (half a unit of rounding and the two-term
+    arithmetic's 2^-44) and 1e-12 (the oracle's FP64 rounding of populations
+    of order one, divided by weights down to 1/216)."""
+    from paper_2212_11024_gb300 import Flame
+    nz, ny, nx = shape
+    r = np.random.default_rng(11)
+    u, B = (0.05 * r.standard_normal((3,) + shape)).astype(dtype), (0.05 * r.standard_normal((3,) + shape)).astype(dtype)
+    u[:, 0, 0, 1] = 0.0
+    B[:, 0, 1, 2] = 0.0
+    u[:, 1, 1, 0] = 1e-30
+    rho = (1 + 0.01 * r.standard_normal(shape)).astype(dtype) if given == "rho" else None
+    gu, gB = ((0.01 * r.standard_normal((9,) + shape)).astype(dtype) if given == "gradients" else None for _ in range(2))
+    Bref, tau, d_i = (0.0, 0.03125, 0.125), 0.625, 1.5
+    noneq = given != "no noneq"
+    sim = Flame(nx, ny, nz, tau, tau, d_i, storage="fp32", B_ref=Bref, init_noneq=noneq)
+    sim.init(rho, u, B, gu, gB)
+    got = sim.state.view(torch.float32).cpu().numpy().reshape((48,) + shape)
+    speed = sim.info()["max_speed"]
+    sim.close()
+    f64 = [None if a is None else a.astype(np.float64) for a in (rho, u, B, gu, gB)]
+    stored_tau = 1.0 / float(np.float32(1.0 / tau))  # the library holds the rates 1 / tau in FP32
+    p = O.Params(nx, ny, nz, stored_tau, stored_tau, d_i)
+    ref = _stored(O.init(p, *f64, noneq), Bref)
+    tol = 0.501 * np.spacing(np.abs(ref).astype(np.float32)).astype(np.float64) + 1e-12
+    assert (np.abs(got - ref) <= tol).all(), float((np.abs(got - ref) / tol).max())
+    rr = 1.0 if rho is None else f64[0]
+    top = max(np.sqrt((f64[2] ** 2).sum(0) / rr).max(), np.sqrt((f64[1] ** 2).sum(0)).max())
+    assert abs(speed - top) <= 0.51 * np.spacing(np.float32(top))
+
+
+def test_initial_populations_beyond_two_term_range():
+    """Fields of 1e13 take the FP64 path: rounded FP64 values there too, and
+    a non-finite field is reported."""
+    from paper_2212_11024_gb300 import Flame, flame
+    shape = (3, 4, 33)
+    r = np.random.default_rng(12)
+    u, B = 0.05 * r.standard_normal((3,) + shape), 0.05 * r.standard_normal((3,) + shape)
+    B[:, 1, 2, 20] = 1e13
+    sim = Flame(33, 4, 3, 0.625, 0.625, 0.0, storage="fp32")
+    sim.init(None, u, B)
+    got = sim.state.view(torch.float32).cpu().numpy().reshape((48,) + shape)
+    ref = _stored(O.init(O.Params(33, 4, 3, 0.625, 0.625, 0.0), None, u, B), (0, 0, 0))
+    mag = np.abs(ref).max(0)
+    assert (np.abs(got - ref) <= 1e-6 * mag + 1e-9).all()
+    u[0, 0, 0, 0] = np.nan
+    B[0, 0, 0, 0] = np.inf
+    with pytest.raises(flame.FlameError) as e:
+        sim.init(None, u, B)
+    assert e.value.status == flame.FLAME_ERR_NONFINITE
+    sim.close()
