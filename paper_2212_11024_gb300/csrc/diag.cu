@@ -121,12 +121,14 @@ __device__ __forceinline__ float init_site(T* __restrict__ pop, const Grid& g, c
 // FP32 storage: the populations are FP64 values rounded to FP32.  Their ~770
 // FP64 operations a site (and conversions, which cost as much) were all this
 // kernel did: 2932 us at 128^3 (23.4 ms at 256^3), where the bytes take 74;
-// now 520 us (4.2 ms), bound by FP32 issue.  They are computed
+// now 385 us (3.0 ms), bound by FP32 issue.  They are computed
 // in two-term FP32 arithmetic (48 bits: the rounded results are FP64's but
 // for one in 2^20 or so) and in the columns of the step's collision: for each
 // (c_x, c_y) the three values along c_z are Z0 + Z1 c_z + Z2 c_z^2, the
 // Lorentz term's N and the non-equilibrium stress P entering as K = N - P.
-// FP64 fields are split by integer operations.  Sites with values outside
+// FP64 fields are split by integer operations.  Blocks of 128 threads by
+// registers: 168 (three per SM) 551 us, 128 (four) 462, 96 (five) 411, 80
+// (six, some of the field values reloaded) 385.  Sites with values outside
 // [2^-40, 2^40] (density) or 2^40 (fields) take the FP64 path.
 struct InitConsts {
   F2 p;    // -1 / (3 omega), or 0 without the non-equilibrium parts
@@ -263,7 +265,7 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
 }
 
 template <class T, class R, class F>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 1)
     init_kernel(T* __restrict__ pop, Grid g, StepConsts k, InitConsts ic, int noneq, const F* __restrict__ rho_f,
                 const F* __restrict__ u, const F* __restrict__ Bf, const F* __restrict__ gu,
                 const F* __restrict__ gB, unsigned* __restrict__ speed_bits) {
@@ -406,7 +408,8 @@ __global__ void moments_kernel(const T* __restrict__ pop, Grid g, StepConsts k, 
 // kernel's 1-D passes and turned into FP64 by their bits; the quotients by
 // rho and the current's solve stay in FP64: 18 operations per site without
 // the current, 65 with it.  128^3: 389 us for all moments, 155 us for u and
-// B (84 us of HBM traffic).
+// B (84 us of HBM traffic).  64 registers, eight blocks per SM: B alone, bound
+// by HBM, 50 us against 58 with six blocks; the others do not change.
 struct SiteMoments64 {
   double drho, U[3], dB[3], J[3];
   __device__ __forceinline__ double rho(const StepConsts& k) const { return (double)k.rho0 + drho; }
@@ -513,7 +516,7 @@ __device__ __noinline__ void general_moments(const float* pop, int site, Nbr nb,
 }
 
 template <bool ODD, class O, bool FLUID, bool CUR>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 8)
     moments64_kernel(const float* __restrict__ pop, Grid g, StepConsts k, MomentsOut<O> out) {
   static_assert(FLUID || !CUR, "the current needs the velocity");
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
