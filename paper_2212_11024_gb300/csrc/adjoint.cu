@@ -29,6 +29,7 @@
 #include <type_traits>
 
 #include "aa.cuh"
+#include "expansion.cuh"
 
 namespace flame {
 namespace {
@@ -558,7 +559,85 @@ __global__ void __launch_bounds__(kAdjThreads<T>, kAdjMinBlocks<T>)
 // Initialisation adjoint (FP64), local part: per site the contributions to
 // u_bar and B_bar that do not go through a gradient, and the adjoints of the
 // central-difference gradients (d_a u_b, d_a B_b at [3a+b]).
-__global__ void init_adjoint_local_kernel(Grid g, StepConsts k, const double* __restrict__ u,
+//
+// Bound by the FP64 pipe (1/64 of the FP32 rate, conversions included):
+// per-velocity sums with every product written out took ~1430 operations a
+// site, 675 us at 64^3.  Now the sums that do not depend on the fields run
+// as three-term FP32 expansions of the FP32 lambda, lambda is widened by its
+// bits, and the equilibrium's U derivatives are separable 1-D passes that
+// share their partial sums, in FP64 (90 operations of ~175): 100 us.
+
+// The power of two that keeps sums of n values within FP32's range (1 but
+// for values near its end).
+template <int N>
+__device__ __forceinline__ float sum_scale(const float (&l)[N]) {
+  float m = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) m = fmaxf(m, fabsf(l[i]));
+  return m < 0x1p100f ? 1.f : 0x1p-20f;
+}
+
+// 216 sum_i w_i l_i times 1, c_a c_b of l in velocity-cube order: r, and
+// R = xx, yy, zz, xy, xz, yz.
+__device__ __forceinline__ void second_sums(const float (&lam)[kQ], double& r, double (&R)[6]) {
+  const float sc = sum_scale(lam);
+  float l[kQ];
+#pragma unroll
+  for (int q = 0; q < kQ; ++q) l[q] = sc * lam[q];
+  F3 Y00[3], Y02[3], Y10[3], Y20[3], Y01[3], Y11[3];  // [x function][y function] per pz
+#pragma unroll
+  for (int pz = 0; pz < 3; ++pz) {
+    F3 a0[3];
+    F2 a1[3], a2[3];
+#pragma unroll
+    for (int py = 0; py < 3; ++py) {
+      const int q = 3 * (py + 3 * pz);
+      a2[py] = two_sum(l[q + 2], l[q]);
+      a1[py] = two_diff(l[q + 2], l[q]);
+      a0[py] = add3(a2[py], 4.f * l[q + 1]);
+    }
+    Y02[pz] = add3(a0[2], a0[0]);
+    Y00[pz] = add3(Y02[pz], scaled(4.f, a0[1]));
+    Y01[pz] = add3(a0[2], -a0[0]);
+    Y10[pz] = add3(add3(a1[2], a1[0]), scaled(4.f, a1[1]));
+    Y11[pz] = add3(a1[2], -a1[0]);
+    Y20[pz] = add3(add3(a2[2], a2[0]), scaled(4.f, a2[1]));
+  }
+  auto w = [](const F3 (&y)[3]) { return to_double(add3(add3(y[2], y[0]), scaled(4.f, y[1]))); };
+  auto c = [](const F3 (&y)[3]) { return to_double(add3(y[2], -y[0])); };
+  r = w(Y00);
+  R[0] = w(Y20);
+  R[1] = w(Y02);
+  R[2] = to_double(add3(Y00[2], Y00[0]));
+  R[3] = w(Y11);
+  R[4] = c(Y10);
+  R[5] = c(Y01);
+  if (sc != 1.f) {
+    r *= 0x1p20;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) R[i] *= 0x1p20;
+  }
+}
+
+// psi(u) and its derivative at c = -1, 0, 1 (the undivided 1-D equilibrium).
+struct Axis64 {
+  double psi[3], dpsi[3];
+  __device__ __forceinline__ explicit Axis64(double u) {
+    const double h = fma(0.5 * u, u, 1.0 / 6.0), g = 0.5 * u;
+    psi[0] = h - g;
+    psi[1] = fma(-u, u, 2.0 / 3.0);
+    psi[2] = h + g;
+    dpsi[0] = u - 0.5;
+    dpsi[1] = -2.0 * u;
+    dpsi[2] = u + 0.5;
+  }
+};
+__device__ __forceinline__ double dot3(const double (&f)[3], double a, double b, double c) {
+  return fma(f[2], c, fma(f[1], b, f[0] * a));
+}
+
+__global__ void __launch_bounds__(128, 4)
+    init_adjoint_local_kernel(Grid g, StepConsts k, const double* __restrict__ u,
                                           const double* __restrict__ Bf, const float* __restrict__ lam,
                                           double* __restrict__ ubl, double* __restrict__ Bbl,
                                           double* __restrict__ dub, double* __restrict__ dBb,
@@ -570,88 +649,111 @@ __global__ void init_adjoint_local_kernel(Grid g, StepConsts k, const double* __
   if (x < g.nx && y < g.ny) {
     const long long n3 = g.n3;
     const long long site = ((long long)z * g.ny + y) * g.nx + x;
+    float l[kQ];
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) l[q] = lam[(long long)idx27(q % 3, (q / 3) % 3, q / 9) * n3 + site];
     const double U[3] = {u[site], u[n3 + site], u[2 * n3 + site]};
+
+    // equilibrium part of u_bar: sum_i l_i d(psi psi psi)/du_a
+    double Ub[3];
+    {
+      const Axis64 ax(U[0]), ay(U[1]), az(U[2]);
+      double P[3], Px[3], Py[3];  // per pz: psi psi, dpsi psi, psi dpsi
+#pragma unroll
+      for (int pz = 0; pz < 3; ++pz) {
+        double X[3], D[3];
+#pragma unroll
+        for (int py = 0; py < 3; ++py) {
+          const int q = 3 * (py + 3 * pz);
+          const double a = widened(l[q]), b = widened(l[q + 1]), c = widened(l[q + 2]);
+          X[py] = dot3(ax.psi, a, b, c);
+          D[py] = dot3(ax.dpsi, a, b, c);
+        }
+        P[pz] = dot3(ay.psi, X[0], X[1], X[2]);
+        Py[pz] = dot3(ay.dpsi, X[0], X[1], X[2]);
+        Px[pz] = dot3(ay.psi, D[0], D[1], D[2]);
+      }
+      Ub[0] = dot3(az.psi, Px[0], Px[1], Px[2]);
+      Ub[1] = dot3(az.psi, Py[0], Py[1], Py[2]);
+      Ub[2] = dot3(az.dpsi, P[0], P[1], P[2]);
+    }
+    // H = sum_i l_i w_i H2_i; Lorentz part of B_bar; the gradients of u
     const double B[3] = {Bf[site], Bf[n3 + site], Bf[2 * n3 + site]};
-    // central-difference gradient of B for J0 = curl B
-    const int xp = x + 1 == g.nx ? 0 : x + 1, xm = x == 0 ? g.nx - 1 : x - 1;
-    const int yp = y + 1 == g.ny ? 0 : y + 1, ym = y == 0 ? g.ny - 1 : y - 1;
-    const int zp = z + 1 == g.nz ? 0 : z + 1, zm = z == 0 ? g.nz - 1 : z - 1;
-    auto at = [&](int xx, int yy, int zz) { return ((long long)zz * g.ny + yy) * g.nx + xx; };
-    double dB[3][3];
-    for (int b = 0; b < 3; ++b) {
-      const double* F = Bf + b * n3;
-      dB[0][b] = 0.5 * (F[at(xp, y, z)] - F[at(xm, y, z)]);
-      dB[1][b] = 0.5 * (F[at(x, yp, z)] - F[at(x, ym, z)]);
-      dB[2][b] = 0.5 * (F[at(x, y, zp)] - F[at(x, y, zm)]);
-    }
-    const double al = (double)k.alphaH, omB = (double)k.omegaB, om = (double)k.omega;
-    const double J0[3] = {dB[1][2] - dB[2][1], dB[2][0] - dB[0][2], dB[0][1] - dB[1][0]};
-    const double V[3] = {U[0] - al * J0[0], U[1] - al * J0[1], U[2] - al * J0[2]};
-    double lf[kQ], lg[3][kM];
-    for (int i = 0; i < kQ; ++i) lf[i] = (double)lam[(long long)i * n3 + site];
-    for (int b = 0; b < 3; ++b)
-      for (int i = 0; i < kM; ++i) lg[b][i] = (double)lam[(long long)mslot(b, i) * n3 + site];
-    // H = sum_i lf w H2; Lorentz part of B_bar; equilibrium part of u_bar
-    double r0 = 0.0, R[3][3] = {{0.0}}, Ub[3] = {0.0, 0.0, 0.0};
-    for (int i = 0; i < kQ; ++i) {
-      const int c[3] = {cx27(i), cy27(i), cz27(i)};
-      const double wt = w27d(i) * lf[i];
-      r0 += wt;
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) R[a][b] += wt * c[a] * c[b];
-      double ps[3], dps[3];
-      for (int a = 0; a < 3; ++a) {
-        const double uu = U[a] * U[a];
-        ps[a] = c[a] == 0 ? 2.0 / 3.0 - uu : 0.5 * (1.0 / 3.0 + uu + c[a] * U[a]);
-        dps[a] = c[a] == 0 ? -2.0 * U[a] : U[a] + 0.5 * c[a];
-      }
-      Ub[0] += lf[i] * dps[0] * ps[1] * ps[2];
-      Ub[1] += lf[i] * ps[0] * dps[1] * ps[2];
-      Ub[2] += lf[i] * ps[0] * ps[1] * dps[2];
-    }
-    double H[3][3];
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) H[a][b] = R[a][b] - (a == b ? r0 / 3.0 : 0.0);
-    const double trH = H[0][0] + H[1][1] + H[2][2];
     double Bb[3];
-    for (int a = 0; a < 3; ++a) Bb[a] = 4.5 * (trH * B[a] - 2.0 * (H[a][0] * B[0] + H[a][1] * B[1] + H[a][2] * B[2]));
+    {
+      double r0, R[6];
+      second_sums(l, r0, R);
+      const double k216 = 1.0 / 216.0, t3 = r0 * (1.0 / 648.0);
+      const double Hd[3] = {fma(R[0], k216, -t3), fma(R[1], k216, -t3), fma(R[2], k216, -t3)};
+      const double Hxy = R[3] * k216, Hxz = R[4] * k216, Hyz = R[5] * k216;
+      const double trH = Hd[0] + Hd[1] + Hd[2];
+      Bb[0] = 4.5 * (trH * B[0] - 2.0 * dot3(B, Hd[0], Hxy, Hxz));
+      Bb[1] = 4.5 * (trH * B[1] - 2.0 * dot3(B, Hxy, Hd[1], Hyz));
+      Bb[2] = 4.5 * (trH * B[2] - 2.0 * dot3(B, Hxz, Hyz, Hd[2]));
+      const double cu = -3.0 / (double)k.omega;  // rho = 1 initial density
+      const double off[3] = {cu * Hxy, cu * Hxz, cu * Hyz};
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) dub[(3 * a + b) * n3 + site] = a == b ? cu * Hd[a] : off[a + b - 1];
+    }
     // Hall equilibrium: mu = W lg, m0, Q[a][b] = sum_i mu_bi xi_ia
-    double Q[3][3], Vb[3];
+    double Q[3][3];
+#pragma unroll
     for (int b = 0; b < 3; ++b) {
-      double m0 = 0.25 * lg[b][0];
-      for (int i = 1; i < kM; ++i) m0 += 0.125 * lg[b][i];
-      Bb[b] += m0;
-      for (int a = 0; a < 3; ++a) Q[a][b] = 0.125 * (lg[b][2 * a + 1] - lg[b][2 * a + 2]);
-    }
-    for (int c = 0; c < 3; ++c) {
-      double qtv = 0.0, qv = 0.0, qb = 0.0, qtb = 0.0;
-      for (int a = 0; a < 3; ++a) {
-        qtv += Q[a][c] * V[a];
-        qv += Q[c][a] * V[a];
-        qb += Q[c][a] * B[a];
-        qtb += Q[a][c] * B[a];
+      float lg[kM];
+#pragma unroll
+      for (int i = 0; i < kM; ++i) lg[i] = lam[(long long)mslot(b, i) * n3 + site];
+      const float sc = sum_scale(lg);
+#pragma unroll
+      for (int i = 0; i < kM; ++i) lg[i] *= sc;
+      const F3 m0 = add3(add3(add3(two_sum(lg[1], lg[2]), two_sum(lg[3], lg[4])), two_sum(lg[5], lg[6])), 2.f * lg[0]);
+      double m = to_double(scaled(0.125f, m0));
+#pragma unroll
+      for (int a = 0; a < 3; ++a) Q[a][b] = to_double(scaled(0.125f, two_diff(lg[2 * a + 1], lg[2 * a + 2])));
+      if (sc != 1.f) {
+        m *= 0x1p20;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) Q[a][b] *= 0x1p20;
       }
-      Bb[c] += 4.0 * (qtv - qv);
-      Vb[c] = 4.0 * (qb - qtb);
+      Bb[b] += m;
     }
-    for (int a = 0; a < 3; ++a) Ub[a] += Vb[a];
-    const double J0b[3] = {-al * Vb[0], -al * Vb[1], -al * Vb[2]};
+    // central-difference J0 = curl B, V = u - d_i J0
+    const double al = (double)k.alphaH;
+    double J0[3], V[3];
+    {
+      const int xp = x + 1 == g.nx ? 0 : x + 1, xm = x == 0 ? g.nx - 1 : x - 1;
+      const int yp = y + 1 == g.ny ? 0 : y + 1, ym = y == 0 ? g.ny - 1 : y - 1;
+      const int zp = z + 1 == g.nz ? 0 : z + 1, zm = z == 0 ? g.nz - 1 : z - 1;
+      auto at = [&](int b, int xx, int yy, int zz) { return Bf[b * n3 + ((long long)zz * g.ny + yy) * g.nx + xx]; };
+      auto dx = [&](int b) { return at(b, xp, y, z) - at(b, xm, y, z); };
+      auto dy = [&](int b) { return at(b, x, yp, z) - at(b, x, ym, z); };
+      auto dz = [&](int b) { return at(b, x, y, zp) - at(b, x, y, zm); };
+      J0[0] = 0.5 * (dy(2) - dz(1));
+      J0[1] = 0.5 * (dz(0) - dx(2));
+      J0[2] = 0.5 * (dx(1) - dy(0));
+#pragma unroll
+      for (int a = 0; a < 3; ++a) V[a] = fma(-al, J0[a], U[a]);
+    }
+    // Bbar += 4 (Q^T V - Q V), Vbar = 4 (Q B - Q^T B): by the antisymmetric part of Q
+    const double X01 = 4.0 * (Q[0][1] - Q[1][0]), X02 = 4.0 * (Q[0][2] - Q[2][0]), X12 = 4.0 * (Q[1][2] - Q[2][1]);
+    Bb[0] -= fma(X01, V[1], X02 * V[2]);
+    Bb[1] += fma(X01, V[0], -X12 * V[2]);
+    Bb[2] += fma(X02, V[0], X12 * V[1]);
+    const double Vb[3] = {fma(X01, B[1], X02 * B[2]), fma(-X01, B[0], X12 * B[2]), -fma(X02, B[0], X12 * B[1])};
     abar = -(Vb[0] * J0[0] + Vb[1] * J0[1] + Vb[2] * J0[2]);
-    double db[3][3];
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) db[a][b] = -Q[a][b] / omB;
-    db[1][2] += J0b[0];
-    db[2][1] -= J0b[0];
-    db[2][0] += J0b[1];
-    db[0][2] -= J0b[1];
-    db[0][1] += J0b[2];
-    db[1][0] -= J0b[2];
+    const double iwB = 1.0 / (double)k.omegaB;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-      ubl[a * n3 + site] = Ub[a];
+      ubl[a * n3 + site] = Ub[a] + Vb[a];
       Bbl[a * n3 + site] = Bb[a];
+#pragma unroll
       for (int b = 0; b < 3; ++b) {
-        dBb[(3 * a + b) * n3 + site] = db[a][b];
-        dub[(3 * a + b) * n3 + site] = -(3.0 / om) * H[a][b];  // rho = 1 initial density
+        // -Q / omega_B, and through J0 = curl B the adjoint -d_i Vbar
+        double d = -iwB * Q[a][b];
+        if (b == (a + 1) % 3) d = fma(-al, Vb[(a + 2) % 3], d);
+        if (b == (a + 2) % 3) d = fma(al, Vb[(a + 1) % 3], d);
+        dBb[(3 * a + b) * n3 + site] = d;
       }
     }
   }

@@ -101,6 +101,14 @@ __device__ __forceinline__ F2 div2(F2 a, F2 b, float r) {
   return fast_two_sum(q, __fmul_rn(e, r));
 }
 
+// An FP32 value as FP64 by its bits (a conversion instruction costs as much
+// as an FP64 operation).
+__device__ __forceinline__ double widened(float x) {
+  const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u >= 0x7f000000u) return (double)x;  // zero, subnormal or not finite
+  return __hiloint2double((int)((mag >> 3) + (896u << 20) | (b & 0x80000000u)), (int)(b << 29));
+}
+
 // An FP64 value as h + l (48 bits or more): h takes the top 24 bits of the
 // significand, l the 29 below.  Magnitudes in [2^-74, 2^126) and zero by
 // integer operations, others by FP64 instructions.

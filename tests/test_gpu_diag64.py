@@ -279,3 +279,35 @@ def test_initial_populations_beyond_two_term_range():
         sim.init(None, u, B)
     assert e.value.status == flame.FLAME_ERR_NONFINITE
     sim.close()
+
+
+@pytest.mark.parametrize("shape", [(5, 6, 4), (3, 4, 33), (2, 3, 129)])
+@pytest.mark.parametrize("scale", [1.0, 1e36])
+def test_init_adjoint_is_fp64(shape, scale):
+    """flame_init_adjoint against FP64 autograd with rates that FP32 holds
+    exactly (tau = 0.8): 2^-44 of the largest component (sums of up to 48
+    terms and ~200 operations in FP64), also where sums of lambda leave
+    FP32's range."""
+    import ctypes
+
+    from oracle import torch_ref as R
+    from paper_2212_11024_gb300 import Flame
+    from paper_2212_11024_gb300.flame import library
+    nz, ny, nx = shape
+    r = np.random.default_rng(13)
+    u, B = 0.05 * r.standard_normal((3,) + shape), 0.05 * r.standard_normal((3,) + shape)
+    lam = (scale * r.standard_normal((48,) + shape)).astype(np.float32)
+    sim = Flame(nx, ny, nz, 0.8, 0.8, 1.5)
+    ud, Bd, l0 = torch.tensor(u, device="cuda"), torch.tensor(B, device="cuda"), torch.tensor(lam, device="cuda")
+    ub, Bb = torch.empty_like(ud), torch.empty_like(Bd)
+    ddi = torch.zeros(1, dtype=torch.float64, device="cuda")
+    rc = library().flame_init_adjoint(sim._ctx, *(ctypes.c_void_p(t.data_ptr()) for t in (ud, Bd, l0, ub, Bb, ddi)))
+    assert rc == 0
+    torch.cuda.synchronize()
+    sim.close()
+    ut, Bt = torch.tensor(u, requires_grad=True), torch.tensor(B, requires_grad=True)
+    d = torch.tensor(1.5, dtype=torch.float64, requires_grad=True)
+    g = torch.autograd.grad((R.init(ut, Bt, 0.8, 0.8, d) * torch.tensor(lam.astype(np.float64))).sum(), [ut, Bt, d])
+    for got, ref in ((ub.cpu().numpy(), g[0].numpy()), (Bb.cpu().numpy(), g[1].numpy())):
+        assert np.abs(got - ref).max() <= 2.0 ** -44 * np.abs(ref).max()
+    assert abs(float(ddi[0]) - float(g[2])) <= 2.0 ** -40 * np.abs(g[1].numpy()).sum()
