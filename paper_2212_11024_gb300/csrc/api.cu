@@ -121,32 +121,64 @@ flame_status sync_and_check(flame_ctx* c) {
   return c->sticky;
 }
 
-// FP64 power of a D2Z half spectrum binned into integer shells.
-__global__ void shell_bin_kernel(const cufftDoubleComplex* __restrict__ F, flame::Grid g, int nshell,
-                                 int zero_mean, double* __restrict__ shells) {
+// round(sqrt(m2)): for m2 below 2^24 from the FP32 root, corrected by the
+// integers n^2 - n < m2 <= n^2 + n that round to n.
+__device__ __forceinline__ int shell_of(long long m2) {
+  if (m2 >= 1 << 24) return __double2int_rn(sqrt((double)m2));
+  const int m = (int)m2;
+  int n = __float2int_rn(sqrtf((float)m));
+  if (m > n * n + n) ++n;
+  if (n > 0 && m <= n * n - n) --n;
+  return n;
+}
+
+// FP64 power of a D2Z half spectrum binned into integer shells.  A shared
+// FP64 atomicAdd is a compare-and-swap loop: 21 clocks for a warp on distinct
+// addresses, 618 on one (measured), and neighbouring modes of a row mostly
+// share a shell; with FP64 square roots that made 46 us a field at 128^3.
+// So each warp first sums its runs of equal shells (lanes hold consecutive
+// modes) by shuffles, as many levels as its longest run needs, and only the
+// last lane of a run adds to the histogram: the addresses of a warp's adds
+// differ.
+__global__ void __launch_bounds__(256)
+    shell_bin_kernel(const cufftDoubleComplex* __restrict__ F, flame::Grid g, int nshell, int zero_mean,
+                     double* __restrict__ shells) {
   extern __shared__ double hist[];
   for (int i = threadIdx.x; i < nshell; i += blockDim.x) hist[i] = 0.0;
   __syncthreads();
-  const int hx = g.nx / 2 + 1;
-  const long long total = (long long)g.nz * g.ny * hx;
-  const double inv = 1.0 / ((double)g.n3 * (double)g.n3);
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-    const int kx = (int)(t % hx);
-    const int ky = (int)((t / hx) % g.ny);
-    const int kz = (int)(t / ((long long)hx * g.ny));
-    const int my = ky <= g.ny / 2 ? ky : ky - g.ny;
-    const int mz = kz <= g.nz / 2 ? kz : kz - g.nz;
-    if (zero_mean && kx == 0 && my == 0 && mz == 0) continue;
-    const long long m2 = (long long)kx * kx + (long long)my * my + (long long)mz * mz;
-    const int n = __double2int_rn(sqrt((double)m2));
-    if (n >= nshell) continue;
-    const double w = (kx == 0 || (g.nx % 2 == 0 && kx == g.nx / 2)) ? 1.0 : 2.0;
-    const cufftDoubleComplex v = F[t];
-    atomicAdd(&hist[n], w * (v.x * v.x + v.y * v.y) * inv);
+  const unsigned hx = g.nx / 2 + 1, total = (unsigned)g.nz * (unsigned)g.ny * hx;  // below 2^32: N3 < 2^31
+  const int lane = threadIdx.x & 31;
+  for (unsigned long long t0 = blockIdx.x * blockDim.x; t0 < total; t0 += (unsigned long long)gridDim.x * blockDim.x) {
+    const unsigned long long t = t0 + threadIdx.x;
+    int n = -1;  // no shell: past the end, dropped, or the mean
+    double p = 0.0;
+    if (t < total) {
+      const unsigned row = (unsigned)t / hx;
+      const int kx = (int)((unsigned)t - row * hx), kz = (int)(row / (unsigned)g.ny), ky = (int)(row - (unsigned)kz * g.ny);
+      const int my = ky <= g.ny / 2 ? ky : ky - g.ny;
+      const int mz = kz <= g.nz / 2 ? kz : kz - g.nz;
+      const long long m2 = (long long)kx * kx + (long long)my * my + (long long)mz * mz;
+      n = shell_of(m2);
+      if (n >= nshell || (zero_mean && m2 == 0)) n = -1;
+      const cufftDoubleComplex v = F[t];
+      p = v.x * v.x + v.y * v.y;
+      if (kx != 0 && 2 * kx != g.nx) p += p;  // the conjugate mode is not stored
+    }
+    const int before = __shfl_up_sync(0xffffffffu, n, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || before != n);
+    const int dist = lane - (31 - __clz(heads & (0xffffffffu >> (31 - lane))));
+    const int longest = __reduce_max_sync(0xffffffffu, dist);
+    for (int o = 1; o <= longest; o <<= 1) {
+      const double q = __shfl_up_sync(0xffffffffu, p, o);
+      if (dist >= o) p += q;
+    }
+    const bool last = lane == 31 || (heads >> (lane + 1)) & 1u;
+    if (last && n >= 0) atomicAdd(&hist[n], p);
   }
   __syncthreads();
+  const double inv = 1.0 / ((double)g.n3 * (double)g.n3);
   for (int i = threadIdx.x; i < nshell; i += blockDim.x)
-    if (hist[i] != 0.0) atomicAdd(&shells[i], hist[i]);
+    if (hist[i] != 0.0) atomicAdd(&shells[i], hist[i] * inv);
 }
 
 }  // namespace
@@ -156,7 +188,7 @@ cudaError_t launch_shell_bin(const void* spec, Grid g, int nshell, int zero_mean
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  shell_bin_kernel<<<nsm * 2, 256, (size_t)nshell * sizeof(double), s>>>(
+  shell_bin_kernel<<<nsm * 4, 256, (size_t)nshell * sizeof(double), s>>>(
       static_cast<const cufftDoubleComplex*>(spec), g, nshell, zero_mean, shells);
   return cudaGetLastError();
 }
