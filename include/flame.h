@@ -107,8 +107,10 @@ typedef struct {
                          pairs), in the tiling timed fastest for the row length: x rows
                          staged in shared memory by TMA, a whole row per block tile
                          (most lengths that are multiples of 8 from 64 to 1024) or half a
-                         row (608, 624, 640), or unstaged pairs loaded and stored
-                         straight from HBM (every other even length); odd nx and FP32
+                         row (608, 624, 640), or site pairs of rows of any even length
+                         (every other even length): staged as the windows around the
+                         rows where that fills a block's lanes (from 176), else loaded
+                         and stored straight from HBM; odd nx and FP32
                          storage use the one-site kernel; 1: always the one-site kernel;
                          2: staged whole rows (nx a multiple of 8 in 64..1024), 3: staged
                          half rows (nx > 256 a multiple of 16), 4: unstaged pairs (nx
@@ -304,7 +306,8 @@ int flame_reduce_combine(const flame_params *p, const double *h_sums, double *h_
  * allocated as flame_create requires): FLAME_KERNEL_SITE (one site per
  * thread), FLAME_KERNEL_ROWS (x rows staged in shared memory, two sites per
  * thread), FLAME_KERNEL_HALF_ROWS (half rows staged) or FLAME_KERNEL_PAIRS
- * (site pairs unstaged); the choice flame_params.kernel leaves to the
+ * (site pairs of rows of any even length: unstaged, or, by the library's
+ * choice only, staged as the aligned windows around the rows); the choice flame_params.kernel leaves to the
  * library, or the one it forces where it applies.  Host only, no GPU
  * needed.  Returns 0 for invalid parameters. */
 enum { FLAME_KERNEL_SITE = 1, FLAME_KERNEL_ROWS = 2, FLAME_KERNEL_HALF_ROWS = 3, FLAME_KERNEL_PAIRS = 4 };
@@ -474,8 +477,8 @@ flame_status flame_reduce_static(flame_ctx *ctx, int nblocks, double *d_scalars)
  * `tries` polls per wait, synchronises, and returns FLAME_ERR_TIMEOUT
  * (sticky, like any failure); the state and the step count are left as they
  * were.  Errors: FLAME_ERR_PARAM (tries == 0, or the context does not run
- * the row kernel: FP16/BF16 storage (any variant), kernel = 0, nx as listed
- * at flame_params.kernel), FLAME_ERR_STATE (before flame_init). */
+ * the row kernel on staged rows: FP16/BF16 storage (any variant), nx as
+ * listed at flame_params.kernel), FLAME_ERR_STATE (before flame_init). */
 flame_status flame_debug_stall_next_step(flame_ctx *ctx, unsigned tries);
 
 /* Release the context and its internal workspace (not the caller's state). */

@@ -54,7 +54,10 @@ cudaError_t launch_step(int storage, int odd, void* pop, Grid g, const StepConst
 // non-finite moment; bit 2: a staged copy did not complete within the wait
 // limit.
 bool step_row_supported(Grid g, int storage, int variant, const void* pop, int kernel = 0);
-// The segments per tile launch_step_row uses (0: the pair kernel, no staging).
+// The segments per tile launch_step_row uses (1: whole rows, 2: half rows, 0:
+// the pair kernel, no staging; kWindows: whole rows of any even length, staged
+// as the aligned windows around them).
+constexpr int kWindows = 3;
 int row_segments(int nx, int kernel);
 // step_row_supported with staged rows (the kernels whose copies have waits).
 bool step_row_staged(Grid g, int storage, int variant, const void* pop, int kernel = 0);

@@ -58,8 +58,26 @@ cudaError_t step_row_flame(const RowCall& c) { return row_call<kVarFlame>(c); }
 // fits once per SM (520-648: 20.0-24.9, half rows 22.5-26.7, ahead of the
 // pair kernel from 608 where a half row is whole 16-byte units) and at
 // 776-792 (24.4-25.0).  Ties (within 0.3) keep whole rows.  Odd row lengths
-// take the one-site kernel.
+// take the one-site kernel.  Even lengths that are no multiple of 8 are staged
+// as windows where enough of a resident block's lanes hold a pair
+// (window_pays), else they take the pair kernel.
+//
+// Windows run a block of whole warps per row at 128 registers, 512 threads'
+// worth per SM, so what counts is the pairs those hold.  GLUPS windows / pair
+// kernel (pairs per SM): 126 25.1 / 24.9 (504), 158 22.3 / 24.8 (395), 190 26.5
+// / 25.0 (475), 198 22.8 / 25.1 (396), 222 27.2 / 25.0 (444), 250 28.1 / 25.0
+// (500), 258 23.6 / 25.3 (387), 286 26.0 / 25.2 (429), 300 26.7 / 25.2 (450), 318
+// 28.0 / 24.8 (477), 340 24.4 / 24.9 (340), 382 26.9 / 25.3 (382), 446 28.3 / 25.3
+// (446), 510 28.0 / 25.2 (510), 700 25.4 / 24.9 (350), 766 26.4 / 25.0 (383), 892
+// 26.8 / 25.2 (446), 1022 28.7 / 25.1 (511).
+static bool window_pays(int nx) {
+  if (nx % 2 != 0 || nx % 8 == 0 || nx < 176 || nx > 1024) return false;
+  const int threads = (nx / 2 + 31) / 32 * 32, pairs = 512 / threads * (nx / 2);
+  return pairs >= (threads <= 160 ? 425 : 380);
+}
+
 int row_auto_segments(int nx) {
+  if (window_pays(nx)) return kWindows;
   if (nx % 8 != 0 || nx < 64 || nx > 1024) return 0;
   if ((nx > 64 && nx < 104) || (nx > 128 && nx < 160) || (nx >= 776 && nx <= 792)) return 0;
   if (nx > 512 && nx <= 648) return nx >= 608 && nx % 16 == 0 ? 2 : 0;
@@ -93,8 +111,12 @@ bool step_row_supported(Grid g, int storage, int variant, const void* pop, int k
     case 4: return pair_ok(g, storage, variant, pop);
   }
   // automatic: the pair kernel or a staged tiling for every even row length
-  return pair_ok(g, storage, variant, pop) &&
-         (row_auto_segments(g.nx) == 0 || staged_ok(g, storage, variant, pop));
+  if (!pair_ok(g, storage, variant, pop)) return false;
+  switch (row_auto_segments(g.nx)) {
+    case 0: return true;
+    case kWindows: return (reinterpret_cast<uintptr_t>(pop) & 15u) == 0;
+  }
+  return staged_ok(g, storage, variant, pop);
 }
 
 int row_segments(int nx, int kernel) {

@@ -39,10 +39,11 @@
 // run at a 128-byte aligned place in shared memory (run_stride); longer rows
 // by one bulk copy per storage slot.  Warp 0, which issues the copies, is always
 // whole (nx / 2 >= 32 threads); the last warp of a block may be partial.
-// The same packed collision also runs unstaged (step_pair_kernel: loads and
-// stores straight from HBM, any even row length).  flame_step picks among
-// whole rows, half rows and the pair kernel by row length
-// (row_auto_segments).
+// Rows of other even lengths are staged by the windows around them
+// (step_window_kernel), and the same packed collision also runs unstaged
+// (step_pair_kernel: loads and stores straight from HBM, any even row
+// length).  flame_step picks among whole rows, half rows, windows and the
+// pair kernel by row length (row_auto_segments).
 #pragma once
 
 #include <cuda.h>
@@ -75,7 +76,7 @@ struct RowWait {
 struct RowCall {
   int storage, odd;
   int segments;  // 1: a tile is a whole row; 2: half a row (rows of more than 256 sites);
-                 // 0: no staging (the pair kernel)
+                 // 0: no staging (the pair kernel); kWindows: a whole row of any even length
   void* pop;
   Grid g;
   StepConsts k;
@@ -431,6 +432,31 @@ __device__ __forceinline__ void prefetch_curl(const T* Bfd, long long n3, long l
   prefetch_l1(Bx + rzm + gx0);
   prefetch_l1(Bx + ryp + gx0);
   prefetch_l1(Bx + rym + gx0);
+}
+// J = periodic central-difference curl of the pre-collision field at the
+// pair (gx0, gx0 + 1) of row (y, z); the face neighbours in y and z are
+// whole-pair loads.
+template <class T>
+__device__ __forceinline__ void pair_curl(const T* __restrict__ Bfd, const Grid& g, int y, int z, int gx0, int gxm0,
+                                          int gxp1, f2 (&J)[3]) {
+  const int nx = g.nx, ny = g.ny, nz = g.nz;
+  auto wr = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };
+  const long long r0 = ((long long)z * ny + y) * nx;
+  const long long ryp = ((long long)z * ny + wr(y + 1, ny)) * nx;
+  const long long rym = ((long long)z * ny + wr(y - 1, ny)) * nx;
+  const long long rzp = ((long long)wr(z + 1, nz) * ny + y) * nx;
+  const long long rzm = ((long long)wr(z - 1, nz) * ny + y) * nx;
+  const T *Bx = Bfd, *By = Bfd + g.n3, *Bz = Bfd + 2 * g.n3;
+  // the pair (x0, x1) of a row as one 32-bit load, a single value as one 16-bit load
+  auto at = [&](const T* b, long long r) { return f2{dec2(b + r + gx0)}; };
+  auto one = [&](const T* b, long long i) { return Codec<T>::dec(b[i]); };
+  const f2 by0 = at(By, r0), bz0 = at(Bz, r0);
+  // B(x + 1) - B(x - 1) at x = x0, x1
+  const f2 dxBy = pack(by0.v.y, one(By, r0 + gxp1)) - pack(one(By, r0 + gxm0), by0.v.x);
+  const f2 dxBz = pack(bz0.v.y, one(Bz, r0 + gxp1)) - pack(one(Bz, r0 + gxm0), bz0.v.x);
+  J[0] = 0.5f * ((at(Bz, ryp) - at(Bz, rym)) - (at(By, rzp) - at(By, rzm)));
+  J[1] = 0.5f * ((at(Bx, rzp) - at(Bx, rzm)) - dxBz);
+  J[2] = 0.5f * (dxBy - (at(Bx, ryp) - at(Bx, rym)));
 }
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -821,26 +847,8 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
         if constexpr (kDirect) G.st(kQ + 3 * (ODD ? i : opp7(i)) + c, mx7(i), v);
         else A.st(kQ + 3 * (ODD ? i : opp7(i)) + c, mx7(i), v);
       };
-      // J = periodic central-difference curl of the pre-collision field at
-      // the pair (the face neighbours in y and z are whole-pair loads).
       auto curl_b = [&](f2 (&J)[3]) {
-        const int y = (tile / H) % ny, z = (tile / H) / ny + g.z0;
-        const long long r0 = ((long long)z * ny + y) * nx;
-        const long long ryp = ((long long)z * ny + wrap(y + 1, ny)) * nx;
-        const long long rym = ((long long)z * ny + wrap(y - 1, ny)) * nx;
-        const long long rzp = ((long long)wrap(z + 1, nz) * ny + y) * nx;
-        const long long rzm = ((long long)wrap(z - 1, nz) * ny + y) * nx;
-        const T *Bx = Bfd, *By = Bfd + g.n3, *Bz = Bfd + 2 * g.n3;
-        // the pair (x0, x1) of a row as one 32-bit load, a single value as one 16-bit load
-        auto at = [&](const T* b, long long r) { return f2{dec2(b + r + gx0)}; };
-        auto one = [&](const T* b, long long i) { return Codec<T>::dec(b[i]); };
-        const f2 by0 = at(By, r0), bz0 = at(Bz, r0);
-        // B(x + 1) - B(x - 1) at x = x0, x1
-        const f2 dxBy = pack(by0.v.y, one(By, r0 + gxp1)) - pack(one(By, r0 + gxm0), by0.v.x);
-        const f2 dxBz = pack(bz0.v.y, one(Bz, r0 + gxp1)) - pack(one(Bz, r0 + gxm0), bz0.v.x);
-        J[0] = 0.5f * ((at(Bz, ryp) - at(Bz, rym)) - (at(By, rzp) - at(By, rzm)));
-        J[1] = 0.5f * ((at(Bx, rzp) - at(Bx, rzm)) - dxBz);
-        J[2] = 0.5f * (dxBy - (at(Bx, ryp) - at(Bx, rym)));
+        pair_curl(Bfd, g, (tile / H) % ny, (tile / H) / ny + g.z0, gx0, gxm0, gxp1, J);
       };
       auto mid = [&]() {
         if constexpr (kMidRefill) {
@@ -890,6 +898,162 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
   if (warp == 0) bulk_wait_done();
 }
 
+// ------------------------------------------- rows of any even length, staged
+// The row kernel's tensor maps and bulk copies want rows of whole 16-byte
+// units.  For other even lengths a tile (a whole row again) is staged by one
+// bulk copy per storage slot of the aligned window around the row: up to 14
+// bytes of the neighbouring rows on either side come along and are never
+// looked at (they belong to other tiles, which may be writing them).  The
+// state starts on a 256-byte boundary and is a multiple of 16 bytes long
+// (96 N3), so that every window lies inside it.
+//
+// With R the position of the row's first site in its slot-plane, slot s's
+// window starts (s N3 + R) mod 8 values before the row.  The staged copies lie
+// `pitch` values apart with pitch = N3 (mod 8), so that with m = R mod 8 the
+// value at x is at s pitch + m + x: m depends on the source row only (nine
+// rows on odd steps) and is even, so that unshifted pairs stay 32-bit
+// accesses.  Results go straight to HBM, as for the long rows of the row
+// kernel, and a stage is refilled when its tile's collision ends.
+//
+// PITCH > 0 (rows of up to 256 sites, N3 a multiple of 8) fixes the pitch at
+// compile time, and every warp issues its share of the copies; PITCH = 0
+// reads it from the grid, and warp 0 issues them (FP16, ~4M-site lattices,
+// GLUPS: 250 sites 28.1 against 26.7, 222 27.2 against 25.4; longer rows 28.0
+// by warp 0 against 27.3 shared out at 510).  The unstaged pair kernel runs
+// at 24.7-25.3 at all of these.  Tried at 250 sites and not kept: the results
+// in place and stored by 48 bulk copies and 32-bit stores of the rows' ends
+// (22.2), the windows by tensor-map boxes of [48][N3] (27.9).
+//
+// (two rows' windows overrun their nx values by up to 7 on either side, and
+// their m differ by up to 7)
+__host__ __device__ constexpr int window_pitch(int nx, long long n3) { return (nx + 21 + 7) / 8 * 8 + (int)(n3 & 7); }
+// the compile-time pitches: rows of up to pitch - 24 sites
+constexpr int window_bound_threads(int pitch) { return pitch ? (pitch - 24) / 2 : kRowMaxThreads; }
+
+// Stages the windows of tile (y, z) in stage st: slot s by warp s mod nw, with
+// one arrival of each warp that calls on the stage's barrier.
+template <class T, bool ODD>
+struct WindowIO {
+  const T* state;
+  T* rows;  // [stage][48][pitch]
+  unsigned long long* bars;
+  long long n3;
+  int nx, ny, nz, z0, pitch, lane, warp, nw;
+  bool stall;
+
+  __device__ __forceinline__ void issue(int tile, int st) const {
+    const int y = tile % ny, z = tile / ny + z0;
+    const unsigned bar = smem_addr(&bars[st]);
+    T* dst = rows + (size_t)st * kPop * pitch;
+    const T* src[2];
+    unsigned at[2], bytes[2] = {0u, 0u};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int s = warp + nw * (lane + 32 * h);
+      if (s >= kPop) continue;
+      const int r = s / 3;
+      const int ys = ODD ? wrap(y + run_dy(r), ny) : y, zs = ODD ? wrap(z + run_dz(r), nz) : z;
+      const int row = (zs * ny + ys) * nx;  // N3 < 2^31
+      const long long first = (long long)s * n3 + row;
+      const int mis = (int)(first & 7);
+      src[h] = state + (first - mis);
+      at[h] = smem_addr(dst + ((s * pitch + (row & 7)) & ~7));
+      bytes[h] = (unsigned)((mis + nx + 7) & ~7) * sizeof(T);
+    }
+    const unsigned total = __reduce_add_sync(0xffffffffu, bytes[0] + bytes[1]);
+    if (lane == 0) mbar_expect_tx(bar, total);
+    __syncwarp();
+    if (stall) return;
+    if (bytes[0]) bulk_load(at[0], src[0], bytes[0], bar);
+    if (bytes[1]) bulk_load(at[1], src[1], bytes[1], bar);
+  }
+};
+
+template <class T, bool ODD, int VAR, int PITCH>
+__global__ void __launch_bounds__(window_bound_threads(PITCH), 512 / window_bound_threads(PITCH))
+    step_window_kernel(const T* __restrict__ state, Grid g, StepConsts k, unsigned* __restrict__ flag,
+                       const T* __restrict__ Bfd, const __grid_constant__ SlotBases<T> bases, RowWait wt) {
+  constexpr bool kSpread = PITCH > 0;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = PITCH ? PITCH : window_pitch(nx, g.n3);
+  T* rows = reinterpret_cast<T*>(smem);
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(smem + (size_t)2 * kPop * pitch * sizeof(T));
+  const int ntiles = ny * g.nzi;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kSpread ? (int)(blockDim.x >> 5) : 1;
+  const bool issues = kSpread || warp == 0;
+  if (threadIdx.x == 0) {
+    mbar_init(smem_addr(&bars[0]), nw);
+    mbar_init(smem_addr(&bars[1]), nw);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const WindowIO<T, ODD> io{state, rows, bars, g.n3, nx, ny, nz, g.z0, pitch, lane, kSpread ? warp : 0, nw,
+                            wt.stall != 0};
+  const int first = blockIdx.x, stride = gridDim.x;
+  if (issues)
+    for (int st = 0; st < 2; ++st)
+      if (first + st * stride < ntiles) io.issue(first + st * stride, st);
+
+  const int gx0 = 2 * threadIdx.x, gx1 = gx0 + 1;
+  const int gxm0 = gx0 == 0 ? nx - 1 : gx0 - 1, gxp1 = gx1 == nx - 1 ? 0 : gx1 + 1;
+  int it = 0;
+  for (int tile = first; tile < ntiles; tile += stride, ++it) {
+    const int st = it & 1;
+    const bool ok = mbar_wait(smem_addr(&bars[st]), (it >> 1) & 1, wt.tries);
+    if (ok && gx0 < nx) {  // the last warp may hold fewer pairs
+      const int y = tile % ny, z = tile / ny + g.z0;
+      const T* R = rows + (size_t)st * kPop * pitch;
+      PairGlobal<T, ODD> G;
+      G.base = &bases;
+      G.dm = gxm0 - gx0;
+      G.dp = gxp1 - gx1;
+      int m[3][3];
+#pragma unroll
+      for (int dz = 0; dz < 3; ++dz)
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+          const int row = (ODD || (dz == 1 && dy == 1)) ? (wrap(z + dz - 1, nz) * ny + wrap(y + dy - 1, ny)) * nx : 0;
+          G.off[dz][dy] = row + gx0;
+          m[dz][dy] = row & 7;
+        }
+      // staged storage slot s of this pair moved by d sites (as PairAccess::ld)
+      auto ld = [&](int s, int d) -> f2 {
+        const int r = s / 3;
+        const T* p = R + s * pitch + (ODD ? m[run_dz(r) + 1][run_dy(r) + 1] : m[1][1]);
+        if (!ODD || d == 0) return Codec2<T>::dec(p + gx0);
+        if (d < 0) return pack(Codec<T>::dec(p[gxm0]), Codec<T>::dec(p[gx0]));
+        return pack(Codec<T>::dec(p[gx1]), Codec<T>::dec(p[gxp1]));
+      };
+      auto ldf = [&](int px, int py, int pz) {
+        const int q = px + 3 * py + 9 * pz;
+        return ld(ODD ? 26 - q : q, 1 - px);
+      };
+      auto ldg = [&](int c, int i) { return ld(kQ + 3 * (ODD ? opp7(i) : i) + c, -mx7(i)); };
+      auto stf = [&](int px, int py, int pz, f2 v) {
+        const int q = px + 3 * py + 9 * pz;
+        G.st(ODD ? q : 26 - q, px - 1, v);
+      };
+      auto stg = [&](int c, int i, f2 v) { G.st(kQ + 3 * (ODD ? i : opp7(i)) + c, mx7(i), v); };
+      auto curl_b = [&](f2 (&J)[3]) { pair_curl(Bfd, g, y, z, gx0, gxm0, gxp1, J); };
+      auto mid = [] {};
+      if constexpr (VAR == kVarFdCurrent)
+        prefetch_curl(Bfd, g.n3, ((long long)z * ny + y) * nx, ((long long)z * ny + wrap(y + 1, ny)) * nx,
+                      ((long long)z * ny + wrap(y - 1, ny)) * nx, ((long long)wrap(z + 1, nz) * ny + y) * nx,
+                      ((long long)wrap(z - 1, nz) * ny + y) * nx, gx0, gxm0, gxp1);
+      collide_pair<VAR>(ldf, ldg, stf, stg, curl_b, mid, k, flag);
+    }
+    // Every thread is done with this stage before it is refilled.
+    if (__syncthreads_or(!ok)) {
+      // as in the row kernel: report, let the copies in flight finish (bounded), stop
+      if (threadIdx.x == 0) atomicOr(flag, 2u);
+      for (int j = it; j < it + 2; ++j)
+        if (first + j * stride < ntiles) (void)mbar_wait(smem_addr(&bars[j & 1]), (j >> 1) & 1, wt.tries);
+      return;
+    }
+    if (issues && tile + 2 * stride < ntiles) io.issue(tile + 2 * stride, st);
+  }
+}
+
 // The pair kernel: the row kernel's packed collision of the site pair
 // (x0, x0 + 1) with its populations loaded from and stored to HBM directly,
 // no staging -- any even row length.  Under the AA pattern a pair writes
@@ -929,22 +1093,7 @@ __global__ void __launch_bounds__(kPairThreads, 4)
     G.st(ODD ? q : 26 - q, px - 1, v);
   };
   auto stg = [&](int c, int i, f2 v) { G.st(kQ + 3 * (ODD ? i : opp7(i)) + c, mx7(i), v); };
-  auto curl_b = [&](f2 (&J)[3]) {
-    const long long r0 = ((long long)z * ny + y) * nx;
-    const long long ryp = ((long long)z * ny + wrap(y + 1, ny)) * nx;
-    const long long rym = ((long long)z * ny + wrap(y - 1, ny)) * nx;
-    const long long rzp = ((long long)wrap(z + 1, nz) * ny + y) * nx;
-    const long long rzm = ((long long)wrap(z - 1, nz) * ny + y) * nx;
-    const T *Bx = Bfd, *By = Bfd + g.n3, *Bz = Bfd + 2 * g.n3;
-    auto at = [&](const T* b, long long r) { return f2{dec2(b + r + gx0)}; };
-    auto one = [&](const T* b, long long i) { return Codec<T>::dec(b[i]); };
-    const f2 by0 = at(By, r0), bz0 = at(Bz, r0);
-    const f2 dxBy = pack(by0.v.y, one(By, r0 + gxp1)) - pack(one(By, r0 + gxm0), by0.v.x);
-    const f2 dxBz = pack(bz0.v.y, one(Bz, r0 + gxp1)) - pack(one(Bz, r0 + gxm0), bz0.v.x);
-    J[0] = 0.5f * ((at(Bz, ryp) - at(Bz, rym)) - (at(By, rzp) - at(By, rzm)));
-    J[1] = 0.5f * ((at(Bx, rzp) - at(Bx, rzm)) - dxBz);
-    J[2] = 0.5f * (dxBy - (at(Bx, ryp) - at(Bx, rym)));
-  };
+  auto curl_b = [&](f2 (&J)[3]) { pair_curl(Bfd, g, y, z, gx0, gxm0, gxp1, J); };
   auto mid = [] {};
   if constexpr (VAR == kVarFdCurrent)
     prefetch_curl(Bfd, g.n3, ((long long)z * ny + y) * nx, ((long long)z * ny + wrap(y + 1, ny)) * nx,
@@ -983,19 +1132,16 @@ size_t row_smem_bytes(int nx, size_t elem, int stages, int H = 1) {
 // 224 26.5 / 28.8, 248 28.8 / 28.6; 192: 29.4 with three).
 constexpr int row_stages(int nx) { return nx > 128 && nx < 200 ? 3 : 2; }
 
-// Launch configuration of one instantiation, cached per device (the
-// shared-memory opt-in and the resident blocks per SM depend on the device
-// and on nx only); a mutex makes concurrent host threads safe.
+// Grid of one persistent instantiation, cached per device (the shared-memory
+// opt-in and the resident blocks per SM depend on the device, the block and
+// its shared memory only); a mutex makes concurrent host threads safe.
 constexpr int kMaxDevices = 64;
 
-template <class T, bool ODD, int NX, int S, int VAR, int H>
-cudaError_t row_config(const Grid& g, int* grid, size_t* smem_out) {
-  auto kern = step_row_kernel<T, ODD, NX, S, VAR, H>;
-  const int threads = g.nx / (2 * H);
-  const size_t smem = row_smem_bytes(g.nx, sizeof(T), S, H);
+template <auto Kern>
+cudaError_t persistent_grid(int threads, size_t smem, long long ntiles, int* grid) {
   struct Cache {
     size_t attr_smem, occ_smem;
-    int occ, nsm;
+    int occ_threads, occ, nsm;
   };
   static Cache cache[kMaxDevices];
   static std::mutex mu;
@@ -1006,28 +1152,29 @@ cudaError_t row_config(const Grid& g, int* grid, size_t* smem_out) {
   std::lock_guard<std::mutex> lock(mu);
   Cache& c = cache[dev];
   if (smem > c.attr_smem) {
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
     c.attr_smem = smem;
   }
-  if (smem != c.occ_smem) {
+  if (smem != c.occ_smem || threads != c.occ_threads) {
     int per = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, Kern, threads, smem)) != cudaSuccess) return e;
     if (per < 1) return cudaErrorInvalidConfiguration;
     c.occ = per;
     c.occ_smem = smem;
+    c.occ_threads = threads;
   }
   if (c.nsm == 0 && (e = cudaDeviceGetAttribute(&c.nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const long long ntiles = (long long)g.ny * g.nzi * H, slots = (long long)c.occ * c.nsm;
+  const long long slots = (long long)c.occ * c.nsm;
   *grid = (int)(ntiles < slots ? ntiles : slots);
-  *smem_out = smem;
   return cudaSuccess;
 }
 
 template <class T, bool ODD, int NX, int S, int VAR, int H = 1>
 cudaError_t row_launch(const RowCall& c) {
   int grid = 0;
-  size_t smem = 0;
-  cudaError_t e = row_config<T, ODD, NX, S, VAR, H>(c.g, &grid, &smem);
+  const size_t smem = row_smem_bytes(c.g.nx, sizeof(T), S, H);
+  cudaError_t e = persistent_grid<&step_row_kernel<T, ODD, NX, S, VAR, H>>(c.g.nx / (2 * H), smem,
+                                                                         (long long)c.g.ny * c.g.nzi * H, &grid);
   RowMaps maps{};
   if (e == cudaSuccess && H == 1 && c.g.nx <= kBoxMaxX) e = row_maps(c.pop, c.g, &maps);
   if (e != cudaSuccess || !c.launch) return e;
@@ -1039,9 +1186,35 @@ cudaError_t row_launch(const RowCall& c) {
   return cudaGetLastError();
 }
 
+// Blocks of whole warps covering a row's pairs.
+template <class T, bool ODD, int VAR, int PITCH>
+cudaError_t window_go(const RowCall& c) {
+  const int threads = (c.g.nx / 2 + 31) / 32 * 32, pitch = PITCH ? PITCH : window_pitch(c.g.nx, c.g.n3);
+  const size_t smem = 2 * (kPop * (size_t)pitch * sizeof(T) + sizeof(unsigned long long));
+  int grid = 0;
+  const cudaError_t e = persistent_grid<&step_window_kernel<T, ODD, VAR, PITCH>>(
+      threads, smem, (long long)c.g.ny * c.g.nzi, &grid);
+  if (e != cudaSuccess || !c.launch) return e;
+  SlotBases<T> bases;
+  for (int sl = 0; sl < kPop; ++sl) bases.p[sl] = static_cast<T*>(c.pop) + (size_t)sl * (size_t)c.g.n3;
+  step_window_kernel<T, ODD, VAR, PITCH><<<grid, threads, smem, c.s>>>(
+      static_cast<const T*>(c.pop), c.g, c.k, c.flag, static_cast<const T*>(c.Bfd), bases, c.wt);
+  return cudaGetLastError();
+}
+
+template <class T, bool ODD, int VAR>
+cudaError_t window_launch(const RowCall& c) {
+  const int nx = c.g.nx;
+  if (nx % 2 != 0 || nx < 64 || nx > 2 * kRowMaxThreads) return cudaErrorInvalidValue;
+  if (c.g.n3 % 8 == 0 && nx > 128 && nx <= 256)
+    return nx > 192 ? window_go<T, ODD, VAR, 280>(c) : window_go<T, ODD, VAR, 216>(c);
+  return window_go<T, ODD, VAR, 0>(c);
+}
+
 template <class T, bool ODD, int VAR>
 cudaError_t row_nx(const RowCall& c) {
   if (c.segments == 0) return pair_launch<T, ODD, VAR>(c);
+  if (c.segments == kWindows) return window_launch<T, ODD, VAR>(c);
   // the alignment the staging copies need (see the requirements above)
   if (c.g.nx % 8 != 0) return cudaErrorInvalidValue;
   if (c.segments == 2) {
