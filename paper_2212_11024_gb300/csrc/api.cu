@@ -37,7 +37,8 @@ struct flame_ctx {
   flame_status sticky;
   double cfl, max_speed;
   int nonfinite;
-  unsigned* d_flags;  // [0] non-finite flag, [1] max speed (float bits)
+  unsigned* d_flags;  // [0] non-finite flag, [1] max speed (float bits), [2..3] the several-step launches' barrier
+  bool multi;         // flame_step may take several steps in one launch (small lattices)
   // internal workspace (lazily allocated)
   double* d_red;      // kRedBlocksMax * kRedVals partials + kRedVals result
   double* d_fields;   // 6 * fft_stride(N3) doubles: u, B for spectra; FP32 fields of the host-buffer calls
@@ -227,6 +228,12 @@ size_t flame_state_bytes(const flame_params* p) {
          elem_bytes(p->storage);
 }
 
+// n steps of the context in one launch (flame::launch_steps).
+static flame::MultiCall multi_call(flame_ctx* c, int n) {
+  return flame::MultiCall{c->p.storage, c->parity, c->state, c->g, c->k, c->d_flags, c->d_flags + 2,
+                          c->p.variant, c->p.kernel, n, c->stream};
+}
+
 // flame_create and flame_create_fields (d_state null: no population state).
 static flame_status create_ctx(flame_ctx** out, const flame_params* p, void* d_state, void* stream) {
   flame_ctx* c = new (std::nothrow) flame_ctx;
@@ -241,8 +248,8 @@ static flame_status create_ctx(flame_ctx** out, const flame_params* p, void* d_s
     delete c;
     return FLAME_ERR_CUDA;
   }
-  if (cudaMalloc(&c->d_flags, 2 * sizeof(unsigned)) != cudaSuccess ||
-      cudaMemsetAsync(c->d_flags, 0, 2 * sizeof(unsigned), c->stream) != cudaSuccess) {
+  if (cudaMalloc(&c->d_flags, 4 * sizeof(unsigned)) != cudaSuccess ||
+      cudaMemsetAsync(c->d_flags, 0, 4 * sizeof(unsigned), c->stream) != cudaSuccess) {
     cudaFree(c->d_flags);
     delete c;
     return FLAME_ERR_CUDA;
@@ -265,6 +272,10 @@ static flame_status create_ctx(flame_ctx** out, const flame_params* p, void* d_s
   c->g.z0 = p->halo_z;
   c->g.nzi = p->nz;
   c->g.n3i = (long long)p->nx * p->ny * p->nz;
+  if (d_state && flame::launch_steps(multi_call(c, 0), &c->multi) != cudaSuccess) {
+    flame_destroy(c);
+    return FLAME_ERR_CUDA;
+  }
   // The graph of the first G steps after flame_init (parity 0) is captured
   // here, with the context, so that the first flame_step does not pay for
   // the capture; the parity-1 graph is captured on its first use.
@@ -359,6 +370,10 @@ flame_status flame_init_f32(flame_ctx* c, const float* d_rho, const float* d_u, 
   return init_from<float>(c, d_rho, d_u, d_B, d_gradu, d_gradB);
 }
 
+// Steps of one several-step launch at most (about a millisecond of a lattice
+// that takes them).
+constexpr int kMultiMost = 256;
+
 // Capture graph_steps step launches starting at `parity` into c->graph[parity].
 static cudaError_t capture_graph(flame_ctx* c, int parity) {
   cudaStream_t cs;
@@ -415,12 +430,35 @@ flame_status flame_step(flame_ctx* c, int n) {
       if (st != FLAME_OK) return st;
     }
   }
-  for (int i = 0; i < n; ++i) {
-    cudaError_t e = flame::launch_step(c->p.storage, c->parity, c->state, c->g, c->k, c->d_flags, c->stream,
-                                       c->p.variant, c->d_bfield, c->p.kernel);
+  // a stream under capture gets plain launches
+  bool multi = c->multi && n > 1;
+  if (multi) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    multi = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  }
+  while (n > 0) {
+    int m = 1;
+    if (multi && n > 1) {
+      // as many as up to the next check
+      m = n < kMultiMost ? n : kMultiMost;
+      if (c->p.check_every > 0) {
+        const long long left = c->p.check_every - c->step % c->p.check_every;
+        if (m > left) m = (int)left;
+      }
+    }
+    cudaError_t e;
+    if (m > 1) {
+      bool taken = false;
+      e = flame::launch_steps(multi_call(c, m), &taken);
+      if (e == cudaSuccess && !taken) e = cudaErrorInvalidConfiguration;
+    } else {
+      e = flame::launch_step(c->p.storage, c->parity, c->state, c->g, c->k, c->d_flags, c->stream, c->p.variant,
+                             c->d_bfield, c->p.kernel);
+    }
     if (e != cudaSuccess) return cuda_fail(c, e);
-    c->parity ^= 1;
-    ++c->step;
+    c->parity ^= m & 1;
+    c->step += m;
+    n -= m;
     if (c->p.check_every > 0 && c->step % c->p.check_every == 0) {
       st = sync_and_check(c);
       if (st != FLAME_OK) return st;

@@ -45,6 +45,24 @@ constexpr int kVarFdCurrent = 3;  // J from the central-difference curl of B
 cudaError_t launch_step(int storage, int odd, void* pop, Grid g, const StepConsts& k, unsigned* flag,
                         cudaStream_t s, int variant = kVarFlame, void* Bfd = nullptr, int kernel = 0);
 
+// Several steps in one launch (step_multi.cu), for a lattice whose sites (or
+// pairs, where the packed kernels apply) are at most the threads resident at
+// once; the same populations as n launches of launch_step.  sync: two zeroed
+// words that the launch leaves zeroed.  *taken: whether the lattice is small
+// enough (n = 0 only asks); not for kVarFdCurrent.
+struct MultiCall {
+  int storage, odd;
+  void* pop;
+  Grid g;
+  StepConsts k;
+  unsigned* flag;
+  unsigned* sync;
+  int variant, kernel;
+  int n;
+  cudaStream_t s;
+};
+cudaError_t launch_steps(const MultiCall& c, bool* taken);
+
 // The step for 16-bit storage, two sites per thread in packed FP32 pairs
 // (step_row.cuh): as a persistent kernel over x rows staged in shared memory
 // (64 <= nx <= 1024 with nx a multiple of 8, a 16-byte aligned state; half

@@ -593,8 +593,21 @@ struct SlotBases {
 // z + dz) (periodic) plus the pair's first site x0, so that a store is one
 // address computation on the slot's base; dm = xm0 - x0 and dp = xp1 - x1
 // are the shifted sites' offsets (the wrap at the row's ends).
-template <class T, bool ODD>
+// L2: loads past L1, for a kernel that takes several steps.
+template <class T, bool ODD, bool L2 = false>
 struct PairGlobal {
+  static __device__ __forceinline__ float one(const T* p) {
+    if constexpr (L2) return Codec<T>::dec(__ldcg(p));
+    else return Codec<T>::dec(*p);
+  }
+  static __device__ __forceinline__ f2 two(const T* p) {
+    if constexpr (L2) {
+      const unsigned w = __ldcg(reinterpret_cast<const unsigned*>(p));
+      return Codec2<T>::dec(reinterpret_cast<const T*>(&w));
+    } else {
+      return Codec2<T>::dec(p);
+    }
+  }
   const SlotBases<T>* base;
   int off[3][3];
   int dm, dp;
@@ -602,9 +615,9 @@ struct PairGlobal {
     const int r = s / 3;
     const int dy = ODD ? run_dy(r) : 0, dz = ODD ? run_dz(r) : 0;
     const T* row = base->p[s] + off[dz + 1][dy + 1];
-    if (!ODD || d == 0) return Codec2<T>::dec(row);
-    if (d < 0) return pack(Codec<T>::dec(row[dm]), Codec<T>::dec(row[0]));
-    return pack(Codec<T>::dec(row[1]), Codec<T>::dec(row[1 + dp]));
+    if (!ODD || d == 0) return two(row);
+    if (d < 0) return pack(one(row + dm), one(row));
+    return pack(one(row + 1), one(row + 1 + dp));
   }
   __device__ __forceinline__ void st(int s, int d, f2 v) const {
     const int r = s / 3;
@@ -1061,19 +1074,16 @@ __global__ void __launch_bounds__(window_bound_threads(PITCH), 512 / window_boun
 // its inputs before it writes (as in the staged rows, which it updates in
 // place), so pairs need no synchronisation.  One pair per thread.
 constexpr int kPairThreads = 128;
-template <class T, bool ODD, int VAR>
-__global__ void __launch_bounds__(kPairThreads, 4)
-    step_pair_kernel(Grid g, StepConsts k, unsigned* __restrict__ flag, const T* __restrict__ Bfd,
-                     const __grid_constant__ SlotBases<T> bases) {
+template <class T, bool ODD, int VAR, bool L2>
+__device__ __forceinline__ void step_pair(const Grid& g, const StepConsts& k, unsigned* __restrict__ flag,
+                                          const T* __restrict__ Bfd, const SlotBases<T>& bases, long long p) {
   const int nx = g.nx, ny = g.ny, nz = g.nz, pairs = nx / 2;
-  const long long p = (long long)blockIdx.x * kPairThreads + threadIdx.x;
-  if (p >= (long long)pairs * ny * g.nzi) return;
   const int xp = (int)(p % pairs);
   const long long rowi = p / pairs;
   const int y = (int)(rowi % ny), z = (int)(rowi / ny) + g.z0;
   const int gx0 = 2 * xp, gx1 = gx0 + 1;
   const int gxm0 = gx0 == 0 ? nx - 1 : gx0 - 1, gxp1 = gx1 == nx - 1 ? 0 : gx1 + 1;
-  PairGlobal<T, ODD> G;
+  PairGlobal<T, ODD, L2> G;
   G.base = &bases;
   G.dm = gxm0 - gx0;
   G.dp = gxp1 - gx1;
@@ -1100,6 +1110,15 @@ __global__ void __launch_bounds__(kPairThreads, 4)
                   ((long long)z * ny + wrap(y - 1, ny)) * nx, ((long long)wrap(z + 1, nz) * ny + y) * nx,
                   ((long long)wrap(z - 1, nz) * ny + y) * nx, gx0, gxm0, gxp1);
   collide_pair<VAR>(ldf, ldg, stf, stg, curl_b, mid, k, flag);
+}
+
+template <class T, bool ODD, int VAR>
+__global__ void __launch_bounds__(kPairThreads, 4)
+    step_pair_kernel(Grid g, StepConsts k, unsigned* __restrict__ flag, const T* __restrict__ Bfd,
+                     const __grid_constant__ SlotBases<T> bases) {
+  const long long p = (long long)blockIdx.x * kPairThreads + threadIdx.x;
+  if (p >= (long long)(g.nx / 2) * g.ny * g.nzi) return;
+  step_pair<T, ODD, VAR, false>(g, k, flag, Bfd, bases, p);
 }
 
 template <class T, bool ODD, int VAR>
