@@ -406,14 +406,31 @@ __global__ void moments_kernel(const T* __restrict__ pop, Grid g, StepConsts k, 
 // sums over the populations are linear, so they are taken as three-term FP32
 // expansions (72 bits, more than FP64 holds) in the order of the step
 // kernel's 1-D passes and turned into FP64 by their bits; the quotients by
-// rho and the current's solve stay in FP64: 18 operations per site without
-// the current, 65 with it.  128^3: 389 us for all moments, 155 us for u and
-// B (84 us of HBM traffic).  64 registers, eight blocks per SM: B alone, bound
-// by HBM, 50 us against 58 with six blocks; the others do not change.
+// rho and the current's solve stay in FP64: about 20 operations per site
+// without the current, 55 with it.  128^3: 298 us for all moments (393 with
+// divisions and the constants widened by every thread), 132 us for u and B
+// (84 us of HBM traffic).  64 registers, eight blocks per SM: B alone, bound by
+// HBM, 46 us against 58 with six blocks; the others do not change.
+// The step's FP32 constants widened once on the host (a conversion per thread
+// costs as much as an FP64 operation): gq = 4 omega_B, s = 2 d_i gq.
+struct Consts64 {
+  double rho0, rho0x216, Bref[3], gq2, gq8, s, ss;
+  explicit Consts64(const StepConsts& k) {
+    rho0 = (double)k.rho0;
+    rho0x216 = 216.0 * rho0;
+    for (int a = 0; a < 3; ++a) Bref[a] = (double)k.Bref[a];
+    const double gq = 4.0 * (double)k.omegaB;
+    gq2 = 2.0 * gq;
+    gq8 = -0.125 * gq;
+    s = 2.0 * (double)k.alphaH * gq;
+    ss = s * s;
+  }
+};
+
 struct SiteMoments64 {
-  double drho, U[3], dB[3], J[3];
-  __device__ __forceinline__ double rho(const StepConsts& k) const { return (double)k.rho0 + drho; }
-  __device__ __forceinline__ double B(const StepConsts& k, int a) const { return (double)k.Bref[a] + dB[a]; }
+  double rho_, U[3], B_[3], J[3];
+  __device__ __forceinline__ double rho(const StepConsts&) const { return rho_; }
+  __device__ __forceinline__ double B(const StepConsts&, int a) const { return B_[a]; }
 };
 
 // The sums of an expansion type: F3 for FP64 results, F2 (unnormalised, 48
@@ -507,17 +524,17 @@ __device__ __noinline__ void general_moments(const float* pop, int site, Nbr nb,
   double sf[kQ], sg[3][kM];
   load_site<float, ODD, double>(pop, site, nb, n3, sf, sg);
   const SiteMoments<double> d = site_moments(sf, sg, k);
-  m->drho = d.drho;
+  m->rho_ = d.rho(k);
   for (int a = 0; a < 3; ++a) {
     m->U[a] = d.U[a];
-    m->dB[a] = d.dB[a];
+    m->B_[a] = d.B(k, a);
     m->J[a] = d.J[a];
   }
 }
 
 template <bool ODD, class O, bool FLUID, bool CUR>
 __global__ void __launch_bounds__(128, 8)
-    moments64_kernel(const float* __restrict__ pop, Grid g, StepConsts k, MomentsOut<O> out) {
+    moments64_kernel(const float* __restrict__ pop, Grid g, StepConsts k, Consts64 d, MomentsOut<O> out) {
   static_assert(FLUID || !CUR, "the current needs the velocity");
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -537,41 +554,40 @@ __global__ void __launch_bounds__(128, 8)
     fluid_sums(s, r216, j216);
     chk = (r216.l + j216[0].l) + (j216[1].l + j216[2].l);
   }
-  F2 d[3][3];
-  magnetic_sums(sg, sB, d);
+  F2 lam8[3][3];
+  magnetic_sums(sg, sB, lam8);
   chk += (sB[0].l + sB[1].l) + sB[2].l;
   if constexpr (CUR) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      A8[a] = add3(d[(a + 1) % 3][(a + 2) % 3], -d[(a + 2) % 3][(a + 1) % 3]);
+      A8[a] = add3(lam8[(a + 1) % 3][(a + 2) % 3], -lam8[(a + 2) % 3][(a + 1) % 3]);
       chk += A8[a].l;
     }
   }
   if (isfinite(chk)) {
 #pragma unroll
-    for (int b = 0; b < 3; ++b) m.dB[b] = to_double(scaled(0.125f, sB[b]));
+    for (int b = 0; b < 3; ++b) m.B_[b] = d.Bref[b] + to_double(scaled(0.125f, sB[b]));
     if constexpr (FLUID) {
-      const double r = to_double(r216), rho216 = fma(216.0, (double)k.rho0, r), ir = 1.0 / rho216;
-      m.drho = r * (1.0 / 216.0);
+      const double r = to_double(r216), rho216 = d.rho0x216 + r, ir = reciprocal(rho216);
+      m.rho_ = fma(r, 1.0 / 216.0, d.rho0);
 #pragma unroll
       for (int a = 0; a < 3; ++a) m.U[a] = quotient(to_double(j216[a]), rho216, ir);
     }
     if constexpr (CUR) {
-      const double gq = 4.0 * (double)k.omegaB, sH = 2.0 * (double)k.alphaH * gq;
-      const double B[3] = {m.B(k, 0), m.B(k, 1), m.B(k, 2)};
+      const double* B = m.B_;
       double y[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const int b = (a + 1) % 3, c = (a + 2) % 3;
-        y[a] = fma(2.0 * gq, m.U[b] * B[c] - m.U[c] * B[b], -gq * to_double(scaled(0.125f, A8[a])));
+        y[a] = fma(d.gq2, m.U[b] * B[c] - m.U[c] * B[b], d.gq8 * to_double(A8[a]));
       }
       const double b2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
-      const double t = sH * sH * (y[0] * B[0] + y[1] * B[1] + y[2] * B[2]);
-      const double den = fma(sH * sH, b2, 1.0), iden = 1.0 / den;
+      const double t = d.ss * (y[0] * B[0] + y[1] * B[1] + y[2] * B[2]);
+      const double iden = reciprocal(fma(d.ss, b2, 1.0));
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const int b = (a + 1) % 3, c = (a + 2) % 3;
-        m.J[a] = quotient(fma(t, B[a], fma(-sH, y[b] * B[c] - y[c] * B[b], y[a])), den, iden);
+        m.J[a] = fma(t, B[a], fma(-d.s, y[b] * B[c] - y[c] * B[b], y[a])) * iden;
       }
     }
   } else {
@@ -914,8 +930,9 @@ void moments_go(int odd, const void* pop, Grid g, const StepConsts& k, const Mom
   const dim3 b = site_block(g), gr = site_grid(g, b);
   const T* p = static_cast<const T*>(pop);
   if constexpr (sizeof(T) == 4) {
-    if (odd) moments64_kernel<true, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);
-    else moments64_kernel<false, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);
+    const Consts64 d(k);
+    if (odd) moments64_kernel<true, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, d, out);
+    else moments64_kernel<false, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, d, out);
   } else {
     if (odd) moments_kernel<T, true, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);
     else moments_kernel<T, false, O, FLUID, CUR><<<gr, b, 0, s>>>(p, g, k, out);

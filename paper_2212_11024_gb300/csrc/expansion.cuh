@@ -109,6 +109,20 @@ __device__ __forceinline__ double widened(float x) {
   return __hiloint2double((int)((mag >> 3) + (896u << 20) | (b & 0x80000000u)), (int)(b << 29));
 }
 
+// 1 / d to an FP64 unit or so: two Newton-Raphson steps r += r (1 - d r) on
+// the FP32 reciprocal of d's top 24 bits, each doubling its bits (24, 47, 94):
+// four FP64 operations, where a division takes about eight times the issue
+// slots of one (measured 0.22 a clock and SM against 1.7).  Magnitudes outside
+// [2^-100, 2^100] are divided.
+__device__ __forceinline__ double reciprocal(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), e = (hi >> 20) & 0x7ffu;
+  if (e < 923u || e > 1123u) return 1.0 / d;
+  const unsigned top = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | ((unsigned)__double2loint(d) >> 29);
+  const double r0 = widened(1.f / __uint_as_float(top | (hi & 0x80000000u)));
+  const double r1 = fma(r0, fma(-d, r0, 1.0), r0);
+  return fma(r1, fma(-d, r1, 1.0), r1);
+}
+
 // An FP64 value as h + l (48 bits or more): h takes the top 24 bits of the
 // significand, l the 29 below.  Magnitudes in [2^-74, 2^126) and zero by
 // integer operations, others by FP64 instructions.
