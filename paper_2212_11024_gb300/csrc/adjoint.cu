@@ -34,102 +34,45 @@
 namespace flame {
 namespace {
 
-// 96 registers without spills: 64-thread blocks, ten per SM, for FP32
-// storage; 128-thread blocks, five per SM, for 16-bit storage.  The lambda gather
-// goes into shared memory by asynchronous copies (cp.async) that are in
-// flight during the forward recompute, and lambda is read from there where
-// it is used rather than held in registers; for 16-bit storage the state
-// loads are issued before the copies, for FP32 after them; both carry a
-// 256-byte L2 prefetch hint.  The d_i
-// contributions are summed per warp in FP64 (no block barrier) and the
-// partials added in a fixed order by two small kernels.  Timed at
-// 256^3 (GLUPS FP32 / FP16 storage): one 256-thread block of 185 registers
-// per SM with per-velocity sums 5.6 / 5.3; 1-D passes, 128 x 3 (168
-// registers) 8.30 / 8.53; lambda gathered into registers after the
-// recompute, 128 x 4, 9.37 / 10.1; gathered by cp.async 9.71 / 10.1; lambda
-// read from shared memory where used, 128 x 5, 9.71 / 10.39 (128 x 6, 80
-// registers with spills: 9.26 / 9.85); the partials summed by one block had
-// cost ~5 %: 10.23 / 10.91 with the two-level sum, 10.27 / 11.0 with the
-// per-storage load order and 64 x 10, 10.51 / 11.16 with read-only state
-// loads and 256-byte L2 prefetch hints on them and on the lambda copies
-// (10.46 / 11.06 for the state loads alone; f32x2 pairs inside the 1-D
-// passes: 10.35 / 11.04, not kept); with the hints, 128 x 5 10.52 / 11.31
-// against 64 x 10 10.57 / 11.23, hence the block per storage (128-byte
-// state prefetch: 10.51 / 11.18).  (Per-warp sums in FP32 gained 0.7 %
+// One site per thread: its 48 state values and the 48 lambda values of x + c_q
+// are loaded at once into registers (read-only, with a 256-byte L2 prefetch
+// hint), and the whole reverse sweep runs on them.  Bound by memory: with
+// the collision left out, these loads and stores alone take 1267 us at 256^3
+// FP16 (6.3 TB/s) and 1383 us FP32 (6.9).  What matters is bytes in flight, so
+// warps are traded for registers: 64-thread blocks, seven per SM (six for FP32
+// storage at odd parity).  us at 256^3, even / odd parity:
+//   lambda gathered by 4-byte cp.async into shared memory (bound by those
+//   copies: 1483 with the collision left out)       FP32 1572 / 1566, FP16 1512 / 1486
+//   lambda loaded after the forward recompute, 128 x 5   1526 / 1706,      1433 / 1724
+//   all loads first, 128 threads x 4                     1416 / 1500,      1395 / 1388
+//   ... 128 x 3                                          1427 / 1469,      1454 / 1642
+//   ... 64 x 7                                           1416 / 1514,      1393 / 1363
+//   rows of state and lambda staged by 16-byte cp.async  1661 / 2205,      1540 / 1853
+// The d_i contributions are summed per warp in FP64 and the partials added in
+// a fixed order by one small kernel.  (Per-warp sums in FP32 gained 0.7 %
 // but, where the sites' terms cancel -- a random lambda: sum |a| / |sum a|
 // ~ 5000 -- they added ~5x the rounding of the per-site arithmetic to d_i.)
-template <class T>
-constexpr int kAdjThreads = sizeof(T) == 2 ? 128 : 64;
-template <class T>
-constexpr int kAdjMinBlocks = sizeof(T) == 2 ? 5 : 10;
+constexpr int kAdjThreads = 64;
+template <class T, bool ODD>
+constexpr int kAdjMinBlocks = sizeof(T) == 4 && ODD ? 6 : 7;
 
-// 1-D functions of the undivided equilibrium and inverse-moment maps, and
-// their derivatives in u, at velocity component c (index p = c + 1).
-// (The u derivative of F0 equals F1.)
-struct Axis {
-  float psi[3], dpsi[3], F0[3], F1[3];
-  __device__ __forceinline__ explicit Axis(float u) {
-    const float uu = u * u;
-    psi[1] = 2.f / 3.f - uu;
-    dpsi[1] = -2.f * u;
-    F0[1] = 1.f - uu;
-    F1[1] = -2.f * u;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const float c = h == 0 ? -1.f : 1.f;
-      const int p = h == 0 ? 0 : 2;
-      psi[p] = 0.5f * (1.f / 3.f + uu + c * u);
-      dpsi[p] = u + 0.5f * c;
-      F0[p] = 0.5f * (uu + c * u);
-      F1[p] = u + 0.5f * c;
-    }
-  }
+// The fluid part contracts lambda over the velocity cube with products of 1-D
+// functions of the velocity and U: psi (the equilibrium), F0, F1, F2 (the
+// inverse-moment maps) and their U derivatives.  On a line (a-, a0, a+) of the
+// cube, with h = (a+ - a-)/2 and e = (a- + a+)/2 - a0,
+//     F2 = e,  F1 = h + 2 u e,  F0 = a0 + u h + u^2 e,  psi = F0 + e/3,
+//     dF0/du = dpsi/du = F1,  dF1/du = 2 e,  and with the 1-D weights
+//     w = a0 + e/3,  w c = h/3,  w c^2 = (a0 + e)/3.
+// So lambda is first taken into this basis along the three axes (108
+// operations, no U), and every contraction is a short polynomial in it.
+struct Line {
+  float v[3];  // a0, h, e
 };
-
-// Separable sums over the velocity cube, sum_p t[pz][py][px] fx(px) fy(py)
-// fz(pz), as three 1-D passes (x, then y, then z), so that the partial sums
-// are shared between the many products the adjoint needs.  A 1-D function
-// of p = c + 1 is a table of values (Fv: the U-dependent factors) or one of
-// the constant tables (Fc) written out, so that their zero entries cost
-// nothing: F2 = (1/2, -1, 1/2) (the second-order inverse map), dF1 =
-// (1, -2, 1) (u derivative of F1), the 1-D weights w = (1/6, 2/3, 1/6), w c,
-// w c^2, and (1, 4, 1), c, c^2 (moments of the 216-scaled weights).
-enum : int { kFnF2, kFnDF1, kFnW, kFnWC, kFnWC2, kFnM0, kFnM1, kFnM2 };
-template <int K>
-struct Fc {};
-struct Fv {
-  const float* f;
-};
-__device__ __forceinline__ float app(Fv F, float a0, float a1, float a2) {
-  return fmaf(a2, F.f[2], fmaf(a1, F.f[1], a0 * F.f[0]));
+__device__ __forceinline__ Line line(float am, float a0, float ap) {
+  return {{a0, 0.5f * (ap - am), fmaf(0.5f, am + ap, -a0)}};
 }
-template <int K>
-__device__ __forceinline__ float app(Fc<K>, float a0, float a1, float a2) {
-  if constexpr (K == kFnF2) return fmaf(0.5f, a0 + a2, -a1);
-  else if constexpr (K == kFnDF1) return fmaf(-2.f, a1, a0 + a2);
-  else if constexpr (K == kFnW) return fmaf(2.f / 3.f, a1, (1.f / 6.f) * (a0 + a2));
-  else if constexpr (K == kFnWC) return (1.f / 6.f) * (a2 - a0);
-  else if constexpr (K == kFnWC2) return (1.f / 6.f) * (a0 + a2);
-  else if constexpr (K == kFnM0) return fmaf(4.f, a1, a0 + a2);
-  else if constexpr (K == kFnM1) return a2 - a0;
-  else return a0 + a2;
-}
-template <class F>
-__device__ __forceinline__ void xpass(const float (&t)[3][3][3], F f, float (&o)[3][3]) {
-#pragma unroll
-  for (int pz = 0; pz < 3; ++pz)
-#pragma unroll
-    for (int py = 0; py < 3; ++py) o[pz][py] = app(f, t[pz][py][0], t[pz][py][1], t[pz][py][2]);
-}
-template <class F>
-__device__ __forceinline__ void ypass(const float (&x)[3][3], F f, float (&o)[3]) {
-#pragma unroll
-  for (int pz = 0; pz < 3; ++pz) o[pz] = app(f, x[pz][0], x[pz][1], x[pz][2]);
-}
-template <class F>
-__device__ __forceinline__ float zpass(const float (&y)[3], F f) {
-  return app(f, y[0], y[1], y[2]);
-}
+__device__ __forceinline__ float f0(float u, float uu, float a, float h, float e) { return fmaf(uu, e, fmaf(u, h, a)); }
+__device__ __forceinline__ float f1(float u2, float h, float e) { return fmaf(u2, e, h); }
 
 // Per-warp partial sums (no block barrier at the end of the step kernel);
 // blocks are whole warps (site_block rounds x to 32).
@@ -152,20 +95,8 @@ __device__ __forceinline__ void block_sum_to(double v, double* out) {
   }
 }
 
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ float lds(const float* p) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"((unsigned)__cvta_generic_to_shared(p)));
-  return v;
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Read-only state loads with an L2 prefetch-size hint (the neighbouring
-// warps' segments of the same rows arrive with the first request).
+// Read-only loads with an L2 prefetch-size hint (the neighbouring warps'
+// segments of the same rows arrive with the first request).
 template <class T>
 __device__ __forceinline__ float ld_state(const T* p) {
   if constexpr (sizeof(T) == 4) {
@@ -188,367 +119,360 @@ struct LamSlots {
   float* out[kPop];
 };
 
+// The collision's transpose at one site.  sf, sg: the stored pre-collision
+// values (deviations over weights); lam: lambda_{t+1} at the site's streamed
+// destinations x + c_q, natural slots; out(q, v) takes lambda_t.  Returns the
+// site's term of dL/d(d_i).
+template <class Out>
+__device__ __forceinline__ float adjoint_site(const StepConsts& k, const float (&sf)[kQ], const float (&sg)[3][kM],
+                                              const float (&lam)[kPop], const Out& out) {
+      // sums of 216 w_i f_i times 1, c_a and c_a c_b, by 1-D passes with (1, 4, 1)
+      float drho, jv[3], pv[3][3];
+      {
+        float m0[9], m1[9], m2[9];
+  #pragma unroll
+        for (int q = 0; q < 9; ++q) {
+          const float am = sf[idx27(0, q % 3, q / 3)], a0 = sf[idx27(1, q % 3, q / 3)], ap = sf[idx27(2, q % 3, q / 3)];
+          m2[q] = am + ap;
+          m0[q] = fmaf(4.f, a0, m2[q]);
+          m1[q] = ap - am;
+        }
+        float M00[3], M01[3], M02[3], M10[3], M11[3], M20[3];
+  #pragma unroll
+        for (int pz = 0; pz < 3; ++pz) {
+          const int q = 3 * pz;
+          M02[pz] = m0[q] + m0[q + 2];
+          M00[pz] = fmaf(4.f, m0[q + 1], M02[pz]);
+          M01[pz] = m0[q + 2] - m0[q];
+          M10[pz] = fmaf(4.f, m1[q + 1], m1[q] + m1[q + 2]);
+          M11[pz] = m1[q + 2] - m1[q];
+          M20[pz] = fmaf(4.f, m2[q + 1], m2[q] + m2[q + 2]);
+        }
+        pv[2][2] = M00[0] + M00[2];
+        drho = fmaf(4.f, M00[1], pv[2][2]) / 216.f;
+        jv[2] = M00[2] - M00[0];
+        jv[1] = fmaf(4.f, M01[1], M01[0] + M01[2]);
+        pv[1][2] = M01[2] - M01[0];
+        pv[1][1] = fmaf(4.f, M02[1], M02[0] + M02[2]);
+        jv[0] = fmaf(4.f, M10[1], M10[0] + M10[2]);
+        pv[0][2] = M10[2] - M10[0];
+        pv[0][1] = fmaf(4.f, M11[1], M11[0] + M11[2]);
+        pv[0][0] = fmaf(4.f, M20[1], M20[0] + M20[2]);
+      }
+      const float rho = k.rho0 + drho;
+      const float U[3] = {jv[0] / (216.f * rho), jv[1] / (216.f * rho), jv[2] / (216.f * rho)};
+      float dB[3], Lm[3][3];
+  #pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        dB[b] = 0.25f * sg[b][0] + 0.125f * (sg[b][1] + sg[b][2] + sg[b][3] + sg[b][4] + sg[b][5] + sg[b][6]);
+        Lm[0][b] = 0.125f * (sg[b][1] - sg[b][2]);
+        Lm[1][b] = 0.125f * (sg[b][3] - sg[b][4]);
+        Lm[2][b] = 0.125f * (sg[b][5] - sg[b][6]);
+      }
+      const float B[3] = {k.Bref[0] + dB[0], k.Bref[1] + dB[1], k.Bref[2] + dB[2]};
+      const float gam = 4.f * k.omegaB, al = k.alphaH;
+      const float Av[3] = {Lm[1][2] - Lm[2][1], Lm[2][0] - Lm[0][2], Lm[0][1] - Lm[1][0]};
+      float yv[3];
+      {
+        const float uxb[3] = {U[1] * B[2] - U[2] * B[1], U[2] * B[0] - U[0] * B[2], U[0] * B[1] - U[1] * B[0]};
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) yv[a] = -gam * (Av[a] - 2.f * uxb[a]);
+      }
+      const float s = 2.f * gam * al;
+      const float b2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
+      const float iden = 1.f / (1.f + s * s * b2);
+      float J[3], V[3];
+      {
+        const float yxb[3] = {yv[1] * B[2] - yv[2] * B[1], yv[2] * B[0] - yv[0] * B[2], yv[0] * B[1] - yv[1] * B[0]};
+        const float yb = yv[0] * B[0] + yv[1] * B[1] + yv[2] * B[2];
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          J[a] = (yv[a] - s * yxb[a] + s * s * yb * B[a]) * iden;
+          V[a] = U[a] - al * J[a];
+        }
+      }
+      // D = (1 - w) dev(Pi - rho U U - M(B)); in deviations dev(Pi~ - rho U U + N)
+      float D[3][3];
+      {
+        const float Br[3] = {k.Bref[0], k.Bref[1], k.Bref[2]};
+        float S[3][3];
+  #pragma unroll
+        for (int a = 0; a < 3; ++a)
+  #pragma unroll
+          for (int b = a; b < 3; ++b) {
+            const float N = Br[a] * dB[b] + dB[a] * Br[b] + dB[a] * dB[b];
+            S[a][b] = pv[a][b] / 216.f - rho * U[a] * U[b] + N;
+          }
+        const float r = 1.f - k.omega;
+        const float tr3 = (S[0][0] + S[1][1] + S[2][2]) / 3.f;
+  #pragma unroll
+        for (int a = 0; a < 3; ++a)
+  #pragma unroll
+          for (int b = a; b < 3; ++b) D[a][b] = r * (a == b ? S[a][b] - tr3 : S[a][b]);
+      }
+
+          // ---- magnetic collision
+      const float omB = k.omegaB;
+      float Bb[3], Vb[3], Q[3][3];  // Q[a][b] = sum_i mu_bi xi_ia
+  #pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        float l[kM];
+  #pragma unroll
+        for (int i = 0; i < kM; ++i) l[i] = lam[kQ + kM * b + i];
+        float m0 = 0.25f * l[0];
+  #pragma unroll
+        for (int i = 1; i < kM; ++i) m0 += 0.125f * l[i];
+        Bb[b] = omB * m0;
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) Q[a][b] = omB * 0.125f * (l[2 * a + 1] - l[2 * a + 2]);
+      }
+  #pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float qtv = 0.f, qv = 0.f, qb = 0.f, qtb = 0.f;
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          qtv += Q[a][c] * V[a];
+          qv += Q[c][a] * V[a];
+          qb += Q[c][a] * B[a];
+          qtb += Q[a][c] * B[a];
+        }
+        Bb[c] += 4.f * (qtv - qv);
+        Vb[c] = 4.f * (qb - qtb);
+      }
+      float Ub[3] = {Vb[0], Vb[1], Vb[2]};
+      float Jb[3] = {-al * Vb[0], -al * Vb[1], -al * Vb[2]};
+      float abar = -(Vb[0] * J[0] + Vb[1] * J[1] + Vb[2] * J[2]);
+      // J = M^-1 y
+      float lJ[3];
+      {
+        const float jxb[3] = {Jb[1] * B[2] - Jb[2] * B[1], Jb[2] * B[0] - Jb[0] * B[2], Jb[0] * B[1] - Jb[1] * B[0]};
+        const float jb = Jb[0] * B[0] + Jb[1] * B[1] + Jb[2] * B[2];
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) lJ[a] = (Jb[a] + s * jxb[a] + s * s * jb * B[a]) * iden;
+      }
+      {
+        const float JxB[3] = {J[1] * B[2] - J[2] * B[1], J[2] * B[0] - J[0] * B[2], J[0] * B[1] - J[1] * B[0]};
+        const float sbar = -(lJ[0] * JxB[0] + lJ[1] * JxB[1] + lJ[2] * JxB[2]);
+        abar += 2.f * gam * sbar;
+        const float lxj[3] = {lJ[1] * J[2] - lJ[2] * J[1], lJ[2] * J[0] - lJ[0] * J[2], lJ[0] * J[1] - lJ[1] * J[0]};
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) Bb[a] -= s * lxj[a];
+      }
+      // y = -gamma (A - 2 U x B)
+      float Lb[3][3];
+      {
+        const float* yb = lJ;
+        const float bxy[3] = {B[1] * yb[2] - B[2] * yb[1], B[2] * yb[0] - B[0] * yb[2], B[0] * yb[1] - B[1] * yb[0]};
+        const float yxu[3] = {yb[1] * U[2] - yb[2] * U[1], yb[2] * U[0] - yb[0] * U[2], yb[0] * U[1] - yb[1] * U[0]};
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          Ub[a] += 2.f * gam * bxy[a];
+          Bb[a] += 2.f * gam * yxu[a];
+        }
+        const float Ab[3] = {-gam * yb[0], -gam * yb[1], -gam * yb[2]};
+        Lb[0][0] = Lb[1][1] = Lb[2][2] = 0.f;
+        Lb[1][2] = Ab[0];
+        Lb[2][1] = -Ab[0];
+        Lb[2][0] = Ab[1];
+        Lb[0][2] = -Ab[1];
+        Lb[0][1] = Ab[2];
+        Lb[1][0] = -Ab[2];
+      }
+
+      // ---- fluid collision: contractions of fbar* with products of 1-D functions
+      const float Dxx = D[0][0], Dyy = D[1][1], Dzz = D[2][2], Dxy = D[0][1], Dxz = D[0][2], Dyz = D[1][2];
+      float rb, Ueq[3], UP[3];
+      float Dbxx, Dbyy, Dbzz, Dbxy, Dbxz, Dbyz;
+      {
+        constexpr float third = 1.f / 3.f;
+        float M[3][3][3];  // [z][y][x basis]
+  #pragma unroll
+        for (int pz = 0; pz < 3; ++pz)
+  #pragma unroll
+          for (int py = 0; py < 3; ++py) {
+            const Line l = line(lam[idx27(0, py, pz)], lam[idx27(1, py, pz)],
+                                lam[idx27(2, py, pz)]);
+  #pragma unroll
+            for (int a = 0; a < 3; ++a) M[pz][py][a] = l.v[a];
+          }
+  #pragma unroll
+        for (int pz = 0; pz < 3; ++pz)
+  #pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const Line l = line(M[pz][0][a], M[pz][1][a], M[pz][2][a]);
+  #pragma unroll
+            for (int b = 0; b < 3; ++b) M[pz][b][a] = l.v[b];
+          }
+  #pragma unroll
+        for (int b = 0; b < 3; ++b)
+  #pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const Line l = line(M[0][b][a], M[1][b][a], M[2][b][a]);
+  #pragma unroll
+            for (int c = 0; c < 3; ++c) M[c][b][a] = l.v[c];
+          }
+        // Lorentz: H = sum_i w_i fbar_i H2_i, by w c^2 - w/3 = (2/9) e
+        {
+          auto w2 = [&](float v0, float v1, float v2, float v3) { return fmaf(third, fmaf(third, v3, v1 + v2), v0); };
+          const float Hxx = (2.f / 9.f) * w2(M[0][0][2], M[0][2][2], M[2][0][2], M[2][2][2]);
+          const float Hyy = (2.f / 9.f) * w2(M[0][2][0], M[0][2][2], M[2][2][0], M[2][2][2]);
+          const float Hzz = (2.f / 9.f) * w2(M[2][0][0], M[2][0][2], M[2][2][0], M[2][2][2]);
+          const float Hxy = (1.f / 9.f) * fmaf(third, M[2][1][1], M[0][1][1]);
+          const float Hxz = (1.f / 9.f) * fmaf(third, M[1][2][1], M[1][0][1]);
+          const float Hyz = (1.f / 9.f) * fmaf(third, M[1][1][2], M[1][1][0]);
+          const float trH = Hxx + Hyy + Hzz;
+          Bb[0] += 4.5f * (trH * B[0] - 2.f * (Hxx * B[0] + Hxy * B[1] + Hxz * B[2]));
+          Bb[1] += 4.5f * (trH * B[1] - 2.f * (Hxy * B[0] + Hyy * B[1] + Hyz * B[2]));
+          Bb[2] += 4.5f * (trH * B[2] - 2.f * (Hxz * B[0] + Hyz * B[1] + Hzz * B[2]));
+        }
+        const float ux = U[0], uy = U[1], uz = U[2], ux2 = 2.f * ux, uy2 = 2.f * uy, uz2 = 2.f * uz;
+        const float uxx = ux * ux, uyy = uy * uy, uzz = uz * uz;
+        // F0x, F1x and F2x (e), then along y: Bpq[z basis] with x function p and y function q
+        float B00[3], B01[3], B02[3], B10[3], B11[3], B12[3], B20[3], B21[3], B22[3];
+  #pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float A0[3], A1[3], A2[3];
+  #pragma unroll
+          for (int b = 0; b < 3; ++b) {
+            A0[b] = f0(ux, uxx, M[c][b][0], M[c][b][1], M[c][b][2]);
+            A1[b] = f1(ux2, M[c][b][1], M[c][b][2]);
+            A2[b] = M[c][b][2];
+          }
+          B00[c] = f0(uy, uyy, A0[0], A0[1], A0[2]);
+          B01[c] = f1(uy2, A0[1], A0[2]);
+          B02[c] = A0[2];
+          B10[c] = f0(uy, uyy, A1[0], A1[1], A1[2]);
+          B11[c] = f1(uy2, A1[1], A1[2]);
+          B12[c] = A1[2];
+          B20[c] = f0(uy, uyy, A2[0], A2[1], A2[2]);
+          B21[c] = f1(uy2, A2[1], A2[2]);
+          B22[c] = A2[2];
+        }
+        auto F0z = [&](const float (&v)[3]) { return f0(uz, uzz, v[0], v[1], v[2]); };
+        auto F1z = [&](const float (&v)[3]) { return f1(uz2, v[1], v[2]); };
+        auto Pz = [&](const float (&v)[3]) { return fmaf(third, v[2], F0z(v)); };
+        // equilibrium: rho prod psi and its U derivatives
+        {
+          float pp[3], dp[3], pd[3];
+  #pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            pp[c] = fmaf(third, fmaf(third, B22[c], B02[c] + B20[c]), B00[c]);
+            dp[c] = fmaf(third, B12[c], B10[c]);
+            pd[c] = fmaf(third, B21[c], B01[c]);
+          }
+          rb = Pz(pp);
+          Ueq[0] = Pz(dp);
+          Ueq[1] = Pz(pd);
+          Ueq[2] = F1z(pp);
+        }
+        // P(D, U): Dbar and the U derivatives
+        const float g111 = F1z(B11), g021 = F1z(B02), g120 = F0z(B12), g210 = F0z(B21), g201 = F1z(B20);
+        Dbxx = F0z(B20);
+        Dbyy = F0z(B02);
+        Dbzz = B00[2];
+        Dbxy = F0z(B11);
+        Dbxz = F1z(B10);
+        Dbyz = F1z(B01);
+        UP[0] = fmaf(Dyz, g111, fmaf(Dzz, B10[2], fmaf(Dyy, g120, 2.f * fmaf(Dxy, g210, Dxz * g201))));
+        UP[1] = fmaf(Dxz, g111, fmaf(Dzz, B01[2], fmaf(Dxx, g210, 2.f * fmaf(Dxy, g120, Dyz * g021))));
+        UP[2] = fmaf(Dxy, g111, fmaf(Dyy, g021, fmaf(Dxx, g201, 2.f * fmaf(Dxz, B10[2], Dyz * B01[2]))));
+      }
+  #pragma unroll
+      for (int a = 0; a < 3; ++a) Ub[a] += rho * Ueq[a] + UP[a];
+      // D -> S -> (Pi, rho, U, B)
+      const float r = 1.f - k.omega;
+      const float trD3 = (Dbxx + Dbyy + Dbzz) / 3.f;
+      const float Sb[3][3] = {{r * (Dbxx - trD3), r * Dbxy, r * Dbxz},
+                              {r * Dbxy, r * (Dbyy - trD3), r * Dbyz},
+                              {r * Dbxz, r * Dbyz, r * (Dbzz - trD3)}};
+      {
+        const float trS = Sb[0][0] + Sb[1][1] + Sb[2][2];
+  #pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          rb -= Sb[a][a] * U[a] * U[a];
+          Ub[a] -= 2.f * rho * Sb[a][a] * U[a];
+          Bb[a] += -trS * B[a] + 2.f * Sb[a][a] * B[a];
+        }
+        const int pa[3] = {0, 0, 1}, pb[3] = {1, 2, 2};
+  #pragma unroll
+        for (int p = 0; p < 3; ++p) {
+          const int a = pa[p], b = pb[p];
+          rb -= Sb[a][b] * U[a] * U[b];
+          Ub[a] -= rho * Sb[a][b] * U[b];
+          Ub[b] -= rho * Sb[a][b] * U[a];
+          Bb[a] += Sb[a][b] * B[b];
+          Bb[b] += Sb[a][b] * B[a];
+        }
+      }
+      // U = j / rho
+      const float jb[3] = {Ub[0] / rho, Ub[1] / rho, Ub[2] / rho};
+      rb -= (Ub[0] * U[0] + Ub[1] * U[1] + Ub[2] * U[2]) / rho;
+
+      // ---- moments -> populations: fbar_i = rhobar + jbar.c_i + Pibar : c_i c_i,
+      // per (c_x, c_y) column as base + lin c_z + Pibar_zz c_z^2
+  #pragma unroll
+      for (int py = 0; py < 3; ++py)
+  #pragma unroll
+        for (int px = 0; px < 3; ++px) {
+          const int cx = px - 1, cy = py - 1;
+          float base = rb, lin = jb[2];
+          if (cx != 0) {
+            base += (cx > 0 ? jb[0] : -jb[0]) + Sb[0][0];
+            lin += cx > 0 ? Sb[0][2] : -Sb[0][2];
+          }
+          if (cy != 0) {
+            base += (cy > 0 ? jb[1] : -jb[1]) + Sb[1][1];
+            lin += cy > 0 ? Sb[1][2] : -Sb[1][2];
+          }
+          if (cx * cy != 0) base += cx * cy > 0 ? Sb[0][1] : -Sb[0][1];
+          const float side = base + Sb[2][2];
+          out(idx27(px, py, 0), side - lin);
+          out(idx27(px, py, 1), base);
+          out(idx27(px, py, 2), side + lin);
+        }
+  #pragma unroll
+      for (int b = 0; b < 3; ++b)
+  #pragma unroll
+        for (int i = 0; i < kM; ++i) {
+          float v = (1.f - omB) * lam[kQ + kM * b + i] + Bb[b];
+          if (i > 0) {
+            const int a = (i - 1) >> 1;
+            v += (i & 1) ? Lb[a][b] : -Lb[a][b];
+          }
+          out(mslot(b, i), v);
+        }
+  return abar;
+}
+
 template <class T, bool ODD>
-__global__ void __launch_bounds__(kAdjThreads<T>, kAdjMinBlocks<T>)
+__global__ void __launch_bounds__(kAdjThreads, (kAdjMinBlocks<T, ODD>))
     adjoint_step_kernel(Slots<T> P, Grid g, StepConsts k, const __grid_constant__ LamSlots L,
                         double* __restrict__ partials) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z + g.z0;
-  const bool live = x < g.nx && y < g.ny;
-  __shared__ float lsm[kPop][kAdjThreads<T>];
   double abar_site = 0.0;
-  if (live) {
+  if (x < g.nx && y < g.ny) {
     const int site = (z * g.ny + y) * g.nx + x;
     const Nbr nb = make_nbr(x, y, z, g);
-
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    auto lgv = [&](int b, int i) { return lds(&lsm[kQ + kM * b + i][tid]); };
-    auto issue_gather = [&]() {
-      // ---- gather dL/df* (streaming transpose: from x + c_q) as asynchronous
-      // copies into shared memory, in flight during the forward recompute
+    float sf[kQ], sg[3][kM], lam[kPop];
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) cp_async4(&lsm[i][tid], L.in[i] + site + nb(cx27(i), cy27(i), cz27(i)));
-#pragma unroll
-      for (int b = 0; b < 3; ++b)
-#pragma unroll
-        for (int i = 0; i < kM; ++i)
-          cp_async4(&lsm[kQ + kM * b + i][tid], L.in[mslot(b, i)] + site + nb(mx7(i), my7(i), mz7(i)));
-      cp_async_commit();
-    };
-    // 16-bit storage: the state loads first; FP32: the lambda copies first
-    // (each measured faster)
-    constexpr bool kStateFirst = sizeof(T) == 2;
-    if (!kStateFirst) issue_gather();
-
-    // ---- forward recompute (deviation variables, as in the step kernel)
-    float sf[kQ];
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-      const int slot = ODD ? opp27(i) : i;
-      sf[i] = ld_state<T>(P.p[slot] + site + src_off<ODD>(nb, cx27(i), cy27(i), cz27(i)));
-    }
-    float sg[3][kM];
+    for (int i = 0; i < kQ; ++i)
+      sf[i] = ld_state<T>(P.p[ODD ? opp27(i) : i] + site + src_off<ODD>(nb, cx27(i), cy27(i), cz27(i)));
 #pragma unroll
     for (int b = 0; b < 3; ++b)
 #pragma unroll
       for (int i = 0; i < kM; ++i)
         sg[b][i] = ld_state<T>(P.p[mslot(b, ODD ? opp7(i) : i)] + site + src_off<ODD>(nb, mx7(i), my7(i), mz7(i)));
-    if (kStateFirst) issue_gather();
-    // sums of 216 w_i f_i times 1, c_a and c_a c_b, by 1-D passes with (1, 4, 1)
-    float drho, jv[3], pv[3][3];
-    {
-      float tc[3][3][3];
+    // dL/df* by the streaming transpose: lambda_{t+1} at x + c_q
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) tc[cz27(i) + 1][cy27(i) + 1][cx27(i) + 1] = sf[i];
-      const Fc<kFnM0> m0;
-      const Fc<kFnM1> m1;
-      const Fc<kFnM2> m2;
-      float X0[3][3], X1[3][3], X2[3][3], Y[3];
-      xpass(tc, m0, X0);
-      xpass(tc, m1, X1);
-      xpass(tc, m2, X2);
-      ypass(X0, m0, Y);
-      drho = zpass(Y, m0) / 216.f;
-      jv[2] = zpass(Y, m1);
-      pv[2][2] = zpass(Y, m2);
-      ypass(X0, m1, Y);
-      jv[1] = zpass(Y, m0);
-      pv[1][2] = zpass(Y, m1);
-      ypass(X0, m2, Y);
-      pv[1][1] = zpass(Y, m0);
-      ypass(X1, m0, Y);
-      jv[0] = zpass(Y, m0);
-      pv[0][2] = zpass(Y, m1);
-      ypass(X1, m1, Y);
-      pv[0][1] = zpass(Y, m0);
-      ypass(X2, m0, Y);
-      pv[0][0] = zpass(Y, m0);
-    }
-    const float rho = k.rho0 + drho;
-    const float U[3] = {jv[0] / (216.f * rho), jv[1] / (216.f * rho), jv[2] / (216.f * rho)};
-    float dB[3], lam[3][3];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      dB[b] = 0.25f * sg[b][0] + 0.125f * (sg[b][1] + sg[b][2] + sg[b][3] + sg[b][4] + sg[b][5] + sg[b][6]);
-      lam[0][b] = 0.125f * (sg[b][1] - sg[b][2]);
-      lam[1][b] = 0.125f * (sg[b][3] - sg[b][4]);
-      lam[2][b] = 0.125f * (sg[b][5] - sg[b][6]);
-    }
-    const float B[3] = {k.Bref[0] + dB[0], k.Bref[1] + dB[1], k.Bref[2] + dB[2]};
-    const float gam = 4.f * k.omegaB, al = k.alphaH;
-    const float Av[3] = {lam[1][2] - lam[2][1], lam[2][0] - lam[0][2], lam[0][1] - lam[1][0]};
-    float yv[3];
-    {
-      const float uxb[3] = {U[1] * B[2] - U[2] * B[1], U[2] * B[0] - U[0] * B[2], U[0] * B[1] - U[1] * B[0]};
-#pragma unroll
-      for (int a = 0; a < 3; ++a) yv[a] = -gam * (Av[a] - 2.f * uxb[a]);
-    }
-    const float s = 2.f * gam * al;
-    const float b2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
-    const float iden = 1.f / (1.f + s * s * b2);
-    float J[3], V[3];
-    {
-      const float yxb[3] = {yv[1] * B[2] - yv[2] * B[1], yv[2] * B[0] - yv[0] * B[2], yv[0] * B[1] - yv[1] * B[0]};
-      const float yb = yv[0] * B[0] + yv[1] * B[1] + yv[2] * B[2];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        J[a] = (yv[a] - s * yxb[a] + s * s * yb * B[a]) * iden;
-        V[a] = U[a] - al * J[a];
-      }
-    }
-    // D = (1 - w) dev(Pi - rho U U - M(B)); in deviations dev(Pi~ - rho U U + N)
-    float D[3][3];
-    {
-      const float Br[3] = {k.Bref[0], k.Bref[1], k.Bref[2]};
-      float S[3][3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = a; b < 3; ++b) {
-          const float N = Br[a] * dB[b] + dB[a] * Br[b] + dB[a] * dB[b];
-          S[a][b] = pv[a][b] / 216.f - rho * U[a] * U[b] + N;
-        }
-      const float r = 1.f - k.omega;
-      const float tr3 = (S[0][0] + S[1][1] + S[2][2]) / 3.f;
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = a; b < 3; ++b) D[a][b] = r * (a == b ? S[a][b] - tr3 : S[a][b]);
-    }
-
-    cp_async_wait_all();
-
-    // ---- magnetic collision
-    const float omB = k.omegaB;
-    float Bb[3], Vb[3], Q[3][3];  // Q[a][b] = sum_i mu_bi xi_ia
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      float l[kM];
-#pragma unroll
-      for (int i = 0; i < kM; ++i) l[i] = lgv(b, i);
-      float m0 = 0.25f * l[0];
-#pragma unroll
-      for (int i = 1; i < kM; ++i) m0 += 0.125f * l[i];
-      Bb[b] = omB * m0;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) Q[a][b] = omB * 0.125f * (l[2 * a + 1] - l[2 * a + 2]);
+    for (int q = kQ; q < kPop; ++q) {
+      const int i = (q - kQ) % kM;
+      lam[q] = ld_state<float>(L.in[q] + site + nb(mx7(i), my7(i), mz7(i)));
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      float qtv = 0.f, qv = 0.f, qb = 0.f, qtb = 0.f;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        qtv += Q[a][c] * V[a];
-        qv += Q[c][a] * V[a];
-        qb += Q[c][a] * B[a];
-        qtb += Q[a][c] * B[a];
-      }
-      Bb[c] += 4.f * (qtv - qv);
-      Vb[c] = 4.f * (qb - qtb);
-    }
-    float Ub[3] = {Vb[0], Vb[1], Vb[2]};
-    float Jb[3] = {-al * Vb[0], -al * Vb[1], -al * Vb[2]};
-    float abar = -(Vb[0] * J[0] + Vb[1] * J[1] + Vb[2] * J[2]);
-    // J = M^-1 y
-    float lJ[3];
-    {
-      const float jxb[3] = {Jb[1] * B[2] - Jb[2] * B[1], Jb[2] * B[0] - Jb[0] * B[2], Jb[0] * B[1] - Jb[1] * B[0]};
-      const float jb = Jb[0] * B[0] + Jb[1] * B[1] + Jb[2] * B[2];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) lJ[a] = (Jb[a] + s * jxb[a] + s * s * jb * B[a]) * iden;
-    }
-    {
-      const float JxB[3] = {J[1] * B[2] - J[2] * B[1], J[2] * B[0] - J[0] * B[2], J[0] * B[1] - J[1] * B[0]};
-      const float sbar = -(lJ[0] * JxB[0] + lJ[1] * JxB[1] + lJ[2] * JxB[2]);
-      abar += 2.f * gam * sbar;
-      const float lxj[3] = {lJ[1] * J[2] - lJ[2] * J[1], lJ[2] * J[0] - lJ[0] * J[2], lJ[0] * J[1] - lJ[1] * J[0]};
-#pragma unroll
-      for (int a = 0; a < 3; ++a) Bb[a] -= s * lxj[a];
-    }
-    // y = -gamma (A - 2 U x B)
-    float Lb[3][3];
-    {
-      const float* yb = lJ;
-      const float bxy[3] = {B[1] * yb[2] - B[2] * yb[1], B[2] * yb[0] - B[0] * yb[2], B[0] * yb[1] - B[1] * yb[0]};
-      const float yxu[3] = {yb[1] * U[2] - yb[2] * U[1], yb[2] * U[0] - yb[0] * U[2], yb[0] * U[1] - yb[1] * U[0]};
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        Ub[a] += 2.f * gam * bxy[a];
-        Bb[a] += 2.f * gam * yxu[a];
-      }
-      const float Ab[3] = {-gam * yb[0], -gam * yb[1], -gam * yb[2]};
-      Lb[0][0] = Lb[1][1] = Lb[2][2] = 0.f;
-      Lb[1][2] = Ab[0];
-      Lb[2][1] = -Ab[0];
-      Lb[2][0] = Ab[1];
-      Lb[0][2] = -Ab[1];
-      Lb[0][1] = Ab[2];
-      Lb[1][0] = -Ab[2];
-    }
-
-    // ---- fluid collision: contractions of fbar* = lf with products of 1-D
-    // functions (grouped by the x function, 1-D passes)
-    const Axis ax(U[0]), ay(U[1]), az(U[2]);
-    const float Dxx = D[0][0], Dyy = D[1][1], Dzz = D[2][2], Dxy = D[0][1], Dxz = D[0][2], Dyz = D[1][2];
-    float rb, Ueq[3], UP[3] = {0.f, 0.f, 0.f};
-    float Dbxx, Dbyy, Dbzz, Dbxy, Dbxz, Dbyz;
-    float r0, R[3][3];
-    {
-      float tl[3][3][3];
-#pragma unroll
-      for (int i = 0; i < kQ; ++i) tl[cz27(i) + 1][cy27(i) + 1][cx27(i) + 1] = lds(&lsm[i][tid]);
-      const Fv Px{ax.psi}, Py{ay.psi}, Pz{az.psi}, DPx{ax.dpsi}, DPy{ay.dpsi}, DPz{az.dpsi};
-      const Fv F0x{ax.F0}, F0y{ay.F0}, F0z{az.F0}, F1x{ax.F1}, F1y{ay.F1}, F1z{az.F1};
-      const Fc<kFnF2> F2c;
-      const Fc<kFnDF1> dF1c;
-      const Fc<kFnW> Wc;
-      const Fc<kFnWC> WCc;
-      const Fc<kFnWC2> WC2c;
-      float X[3][3], Y[3];
-      // equilibrium: rho prod psi and its U derivatives
-      xpass(tl, Px, X);
-      ypass(X, Py, Y);
-      rb = zpass(Y, Pz);
-      Ueq[2] = zpass(Y, DPz);
-      ypass(X, DPy, Y);
-      Ueq[1] = zpass(Y, Pz);
-      xpass(tl, DPx, X);
-      ypass(X, Py, Y);
-      Ueq[0] = zpass(Y, Pz);
-      // P(D, U): Dbar and the U derivatives (dF0 = F1)
-      xpass(tl, F0x, X);
-      ypass(X, F2c, Y);
-      Dbyy = zpass(Y, F0z);
-      UP[2] = fmaf(Dyy, zpass(Y, F1z), UP[2]);
-      ypass(X, F0y, Y);
-      Dbzz = zpass(Y, F2c);
-      ypass(X, F1y, Y);
-      Dbyz = zpass(Y, F1z);
-      UP[1] = fmaf(Dzz, zpass(Y, F2c), UP[1]);
-      UP[2] = fmaf(Dyz, zpass(Y, dF1c), UP[2]);
-      ypass(X, dF1c, Y);
-      UP[1] = fmaf(Dyz, zpass(Y, F1z), UP[1]);
-      xpass(tl, F1x, X);
-      ypass(X, F1y, Y);
-      Dbxy = zpass(Y, F0z);
-      {
-        const float t111 = zpass(Y, F1z);
-        UP[0] = fmaf(Dyz, t111, UP[0]);
-        UP[1] = fmaf(Dxz, t111, UP[1]);
-        UP[2] = fmaf(Dxy, t111, UP[2]);
-      }
-      ypass(X, F0y, Y);
-      Dbxz = zpass(Y, F1z);
-      UP[0] = fmaf(Dzz, zpass(Y, F2c), UP[0]);
-      UP[2] = fmaf(Dxz, zpass(Y, dF1c), UP[2]);
-      ypass(X, F2c, Y);
-      UP[0] = fmaf(Dyy, zpass(Y, F0z), UP[0]);
-      ypass(X, dF1c, Y);
-      UP[1] = fmaf(Dxy, zpass(Y, F0z), UP[1]);
-      xpass(tl, F2c, X);
-      ypass(X, F0y, Y);
-      Dbxx = zpass(Y, F0z);
-      UP[2] = fmaf(Dxx, zpass(Y, F1z), UP[2]);
-      ypass(X, F1y, Y);
-      UP[1] = fmaf(Dxx, zpass(Y, F0z), UP[1]);
-      xpass(tl, dF1c, X);
-      ypass(X, F1y, Y);
-      UP[0] = fmaf(Dxy, zpass(Y, F0z), UP[0]);
-      ypass(X, F0y, Y);
-      UP[0] = fmaf(Dxz, zpass(Y, F1z), UP[0]);
-      // Lorentz term: r0 = sum w_i fbar_i, R_ab = sum w_i fbar_i c_a c_b
-      xpass(tl, Wc, X);
-      ypass(X, Wc, Y);
-      r0 = zpass(Y, Wc);
-      R[2][2] = zpass(Y, WC2c);
-      ypass(X, WC2c, Y);
-      R[1][1] = zpass(Y, Wc);
-      ypass(X, WCc, Y);
-      R[1][2] = zpass(Y, WCc);
-      xpass(tl, WC2c, X);
-      ypass(X, Wc, Y);
-      R[0][0] = zpass(Y, Wc);
-      xpass(tl, WCc, X);
-      ypass(X, WCc, Y);
-      R[0][1] = zpass(Y, Wc);
-      ypass(X, Wc, Y);
-      R[0][2] = zpass(Y, WCc);
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Ub[a] += rho * Ueq[a] + UP[a];
-    // Lorentz: H = R - r0 I / 3
-    {
-      const float H[3][3] = {{R[0][0] - r0 / 3.f, R[0][1], R[0][2]},
-                             {R[0][1], R[1][1] - r0 / 3.f, R[1][2]},
-                             {R[0][2], R[1][2], R[2][2] - r0 / 3.f}};
-      const float trH = H[0][0] + H[1][1] + H[2][2];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) Bb[a] += 4.5f * (trH * B[a] - 2.f * (H[a][0] * B[0] + H[a][1] * B[1] + H[a][2] * B[2]));
-    }
-    // D -> S -> (Pi, rho, U, B)
-    const float r = 1.f - k.omega;
-    const float trD3 = (Dbxx + Dbyy + Dbzz) / 3.f;
-    const float Sb[3][3] = {{r * (Dbxx - trD3), r * Dbxy, r * Dbxz},
-                            {r * Dbxy, r * (Dbyy - trD3), r * Dbyz},
-                            {r * Dbxz, r * Dbyz, r * (Dbzz - trD3)}};
-    {
-      const float trS = Sb[0][0] + Sb[1][1] + Sb[2][2];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        rb -= Sb[a][a] * U[a] * U[a];
-        Ub[a] -= 2.f * rho * Sb[a][a] * U[a];
-        Bb[a] += -trS * B[a] + 2.f * Sb[a][a] * B[a];
-      }
-      const int pa[3] = {0, 0, 1}, pb[3] = {1, 2, 2};
-#pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        const int a = pa[p], b = pb[p];
-        rb -= Sb[a][b] * U[a] * U[b];
-        Ub[a] -= rho * Sb[a][b] * U[b];
-        Ub[b] -= rho * Sb[a][b] * U[a];
-        Bb[a] += Sb[a][b] * B[b];
-        Bb[b] += Sb[a][b] * B[a];
-      }
-    }
-    // U = j / rho
-    const float jb[3] = {Ub[0] / rho, Ub[1] / rho, Ub[2] / rho};
-    rb -= (Ub[0] * U[0] + Ub[1] * U[1] + Ub[2] * U[2]) / rho;
-
-    // ---- moments -> populations: fbar_i = rhobar + jbar.c_i + Pibar : c_i c_i,
-    // per (c_x, c_y) column as base + lin c_z + Pibar_zz c_z^2
-#pragma unroll
-    for (int py = 0; py < 3; ++py)
-#pragma unroll
-      for (int px = 0; px < 3; ++px) {
-        const int cx = px - 1, cy = py - 1;
-        float base = rb, lin = jb[2];
-        if (cx != 0) {
-          base += (cx > 0 ? jb[0] : -jb[0]) + Sb[0][0];
-          lin += cx > 0 ? Sb[0][2] : -Sb[0][2];
-        }
-        if (cy != 0) {
-          base += (cy > 0 ? jb[1] : -jb[1]) + Sb[1][1];
-          lin += cy > 0 ? Sb[1][2] : -Sb[1][2];
-        }
-        if (cx * cy != 0) base += cx * cy > 0 ? Sb[0][1] : -Sb[0][1];
-        const float side = base + Sb[2][2];
-        L.out[idx27(px, py, 0)][site] = side - lin;
-        L.out[idx27(px, py, 1)][site] = base;
-        L.out[idx27(px, py, 2)][site] = side + lin;
-      }
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int i = 0; i < kM; ++i) {
-        float v = (1.f - omB) * lgv(b, i) + Bb[b];
-        if (i > 0) {
-          const int a = (i - 1) >> 1;
-          v += (i & 1) ? Lb[a][b] : -Lb[a][b];
-        }
-        L.out[mslot(b, i)][site] = v;
-      }
-    abar_site = (double)abar;
+    for (int q = 0; q < kQ; ++q) lam[q] = ld_state<float>(L.in[q] + site + nb(cx27(q), cy27(q), cz27(q)));
+    abar_site = (double)adjoint_site(k, sf, sg, lam, [&](int q, float v) { L.out[q][site] = v; });
   }
   const long long blk = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
   const int warp = (threadIdx.x + blockDim.x * threadIdx.y) >> 5;
@@ -791,45 +715,67 @@ __global__ void init_adjoint_stencil_kernel(Grid g, const double* __restrict__ u
   }
 }
 
-// Deterministic two-level sum of n partials: kSumBlocks blocks sum fixed
-// chunks into stage[], then one block sums the stage.
-constexpr int kSumBlocks = 256;
-__global__ void sum_chunks_kernel(const double* __restrict__ partials, long long n, double* __restrict__ stage) {
-  __shared__ double sh[256];
+// Deterministic sum of n partials: up to kSumBlocks blocks sum fixed chunks into
+// stage[], and the last of them to finish adds the stage in a fixed order and
+// leaves the ticket at zero.  (Two kernels had taken 8 us a step.)
+constexpr int kSumBlocks = 64;
+constexpr int kSumThreads = 256;
+__device__ __forceinline__ double sum_of_block(double a) {
+  __shared__ double sh[kSumThreads / 32];
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
+  __syncthreads();
+  a = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < kSumThreads / 32; ++w) a += sh[w];
+  return a;
+}
+__global__ void __launch_bounds__(kSumThreads)
+    sum_partials_kernel(const double* __restrict__ partials, long long n, double* stage, unsigned* ticket,
+                        double* __restrict__ out) {
+  __shared__ bool last;
   const long long per = (n + gridDim.x - 1) / gridDim.x;
   const long long lo = per * blockIdx.x, hi = lo + per < n ? lo + per : n;
   double a = 0.0;
-  for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) a += partials[i];
-  sh[threadIdx.x] = a;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
+  for (long long i = lo + threadIdx.x; i < hi; i += kSumThreads) a += partials[i];
+  a = sum_of_block(a);
+  if (threadIdx.x == 0) {
+    __stcg(stage + blockIdx.x, a);
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __threadfence();
   }
-  if (threadIdx.x == 0) stage[blockIdx.x] = sh[0];
-}
-__global__ void sum_partials_kernel(const double* __restrict__ partials, long long n, double* __restrict__ out) {
-  __shared__ double sh[256];
-  double a = 0.0;
-  for (long long i = threadIdx.x; i < n; i += blockDim.x) a += partials[i];
-  sh[threadIdx.x] = a;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
+  if (!last) return;
+  double t = threadIdx.x < gridDim.x ? __ldcg(stage + threadIdx.x) : 0.0;
+  t = sum_of_block(t);
+  if (threadIdx.x == 0) {
+    *out = t;
+    *ticket = 0u;
   }
-  if (threadIdx.x == 0) *out = sh[0];
 }
-// Sum of n partials (the buffer holds n + kSumBlocks doubles) into *out.
-inline void sum_partials(double* partials, long long n, double* out, cudaStream_t s) {
-  sum_chunks_kernel<<<kSumBlocks, 256, 0, s>>>(partials, n, partials + n);
-  sum_partials_kernel<<<1, 256, 0, s>>>(partials + n, kSumBlocks, out);
+// Sum of n partials into *out; the buffer holds n partials, kSumBlocks doubles
+// and the ticket (zeroed when it was allocated).
+inline void sum_partials(double* partials, long long cap, long long n, double* out, cudaStream_t s) {
+  const long long want = (n + 4 * kSumThreads - 1) / (4 * kSumThreads);
+  double* stage = partials + cap;
+  sum_partials_kernel<<<(unsigned)(want < kSumBlocks ? want : kSumBlocks), kSumThreads, 0, s>>>(
+      partials, n, stage, reinterpret_cast<unsigned*>(stage + kSumBlocks), out);
+}
+
+// The partials of either adjoint: one per warp of the step kernel, one per
+// block of the initialisation's.
+inline long long partials_cap(const Grid& g) {
+  const dim3 b = site_block(g, kAdjThreads), gr = site_grid(g, b);
+  const dim3 bi = site_block(g, 128), gi = site_grid(g, bi);
+  const long long a = (long long)gr.x * gr.y * gr.z * ((b.x * b.y) >> 5), c = (long long)gi.x * gi.y * gi.z;
+  return a > c ? a : c;
 }
 
 template <class T>
 cudaError_t adjoint_t(int odd, const void* pop, Grid g, const StepConsts& k, const float* lin, float* lout,
                       double* partials, double* ddi, cudaStream_t s) {
-  const dim3 b = site_block(g, kAdjThreads<T>), gr = site_grid(g, b);
+  const dim3 b = site_block(g, kAdjThreads), gr = site_grid(g, b);
   const long long nblk = (long long)gr.x * gr.y * gr.z;
   const Slots<T> P = make_slots<T>(pop, g);
   LamSlots L;
@@ -841,25 +787,13 @@ cudaError_t adjoint_t(int odd, const void* pop, Grid g, const StepConsts& k, con
     adjoint_step_kernel<T, true><<<gr, b, 0, s>>>(P, g, k, L, partials);
   else
     adjoint_step_kernel<T, false><<<gr, b, 0, s>>>(P, g, k, L, partials);
-  sum_partials(partials, nblk * ((b.x * b.y) >> 5), ddi, s);
+  sum_partials(partials, partials_cap(g), nblk * ((b.x * b.y) >> 5), ddi, s);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-long long adjoint_partials_needed(Grid g) {
-  // per warp of the step kernel (either block shape), per block of the
-  // initialisation adjoint
-  long long need = 0;
-  for (int threads : {kAdjThreads<float>, kAdjThreads<__half>}) {
-    const dim3 b = site_block(g, threads), gr = site_grid(g, b);
-    const long long a = (long long)gr.x * gr.y * gr.z * ((b.x * b.y) >> 5);
-    if (a > need) need = a;
-  }
-  const dim3 bi = site_block(g, 128), gi = site_grid(g, bi);
-  const long long c = (long long)gi.x * gi.y * gi.z;
-  return (need > c ? need : c) + kSumBlocks;
-}
+long long adjoint_partials_needed(Grid g) { return partials_cap(g) + kSumBlocks + 1; }
 
 cudaError_t launch_step_adjoint(int storage, int odd, const void* pop, Grid g, const StepConsts& k, const float* lin,
                                 float* lout, double* partials, double* ddi, cudaStream_t s) {
@@ -882,7 +816,7 @@ cudaError_t launch_init_adjoint(Grid g, const StepConsts& k, const double* u, co
   double* dBb = ws + 15 * n3;
   init_adjoint_local_kernel<<<gr, b, 0, s>>>(g, k, u, B, lam, ubl, Bbl, dub, dBb, partials);
   init_adjoint_stencil_kernel<<<gr, b, 0, s>>>(g, ubl, Bbl, dub, dBb, ubar, Bbar);
-  sum_partials(partials, (long long)gr.x * gr.y * gr.z, ddi, s);
+  sum_partials(partials, partials_cap(g), (long long)gr.x * gr.y * gr.z, ddi, s);
   return cudaGetLastError();
 }
 

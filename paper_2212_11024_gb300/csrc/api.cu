@@ -918,6 +918,18 @@ flame_status flame_set_state(flame_ctx* c, const void* d_src, long long step, in
   return FLAME_OK;
 }
 
+// The adjoints' partial sums and their ticket, zeroed (on the context's stream).
+static cudaError_t adj_partials(flame_ctx* c) {
+  if (c->d_adj_partials) return cudaSuccess;
+  const size_t bytes = sizeof(double) * (size_t)flame::adjoint_partials_needed(c->g);
+  cudaError_t e = cudaMalloc(&c->d_adj_partials, bytes);
+  if (e != cudaSuccess) {
+    c->d_adj_partials = nullptr;
+    return e;
+  }
+  return cudaMemsetAsync(c->d_adj_partials, 0, bytes, c->stream);
+}
+
 flame_status flame_step_adjoint(flame_ctx* c, const void* d_state, int parity, const float* d_adj_in,
                                 float* d_adj_out, double* d_ddi) {
   const Range range("flame_step_adjoint");
@@ -927,13 +939,8 @@ flame_status flame_step_adjoint(flame_ctx* c, const void* d_state, int parity, c
   if (parity != 0 && parity != 1) return FLAME_ERR_STATE;
   if (d_adj_in == d_adj_out) return FLAME_ERR_PARAM;
   cudaError_t e;
-  if (!c->d_adj_partials) {
-    e = cudaMalloc(&c->d_adj_partials, sizeof(double) * (size_t)flame::adjoint_partials_needed(c->g));
-    if (e != cudaSuccess) {
-      c->d_adj_partials = nullptr;
-      return cuda_fail(c, e);
-    }
-  }
+  e = adj_partials(c);
+  if (e != cudaSuccess) return cuda_fail(c, e);
   return cuda_fail(c, flame::launch_step_adjoint(c->p.storage, parity, d_state, c->g, c->k, d_adj_in, d_adj_out,
                                                  c->d_adj_partials, d_ddi, c->stream));
 }
@@ -945,13 +952,8 @@ flame_status flame_init_adjoint(flame_ctx* c, const double* d_u, const double* d
   if (c->p.variant != FLAME_SCHEME || c->p.halo_z) return FLAME_ERR_PARAM;
   if (c->sticky == FLAME_ERR_CUDA) return c->sticky;
   cudaError_t e;
-  if (!c->d_adj_partials) {
-    e = cudaMalloc(&c->d_adj_partials, sizeof(double) * (size_t)flame::adjoint_partials_needed(c->g));
-    if (e != cudaSuccess) {
-      c->d_adj_partials = nullptr;
-      return cuda_fail(c, e);
-    }
-  }
+  e = adj_partials(c);
+  if (e != cudaSuccess) return cuda_fail(c, e);
   if (!c->d_adj_ws) {
     e = cudaMalloc(&c->d_adj_ws, sizeof(double) * 24 * (size_t)c->g.n3);
     if (e != cudaSuccess) {
