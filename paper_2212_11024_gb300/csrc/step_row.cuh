@@ -753,8 +753,8 @@ struct RowIO {
   }
 };
 
-// Launch bounds per instantiation: 128 registers per thread (512 threads'
-// worth per SM); a block has nx / (2 H) threads.
+// Launch bounds per instantiation: 512 threads' worth per SM (128 registers
+// per thread, 168 at 384-site rows); a block has nx / (2 H) threads.
 constexpr int row_bound_threads(int nx, int H = 1) { return nx ? nx / (2 * H) : kRowMaxThreads; }
 constexpr int row_bound_blocks(int nx, int H = 1) { return 512 / row_bound_threads(nx, H); }
 
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
   // +4 %; at 256-site rows the extra address arithmetic made it slower).  No
   // location is read or written by more than one tile, so the order of these
   // stores and of other tiles' loads does not matter.
-  constexpr bool kDirect = kRowStages == 2 && (NX == 512 || NX == 0 || H > 1);
+  constexpr bool kDirect = kRowStages == 2 && (NX > 256 || NX == 0 || H > 1);
   if (warp == 0)
     for (int s = 0; s < kAhead; ++s)
       if (first + s * stride < ntiles) io.issue(first + s * stride, s);
@@ -1148,8 +1148,10 @@ size_t row_smem_bytes(int nx, size_t elem, int stages, int H = 1) {
 // 30.1).  The general instantiation: three stages with TMA stores from 129
 // to 199 sites, two with direct stores from 200 (~4M-site lattices, GLUPS
 // three / two stages: 136 21.2 / 20.7, 160 25.2 / 24.2, 200 23.9 / 26.5,
-// 224 26.5 / 28.8, 248 28.8 / 28.6; 192: 29.4 with three).
-constexpr int row_stages(int nx) { return nx > 128 && nx < 200 ? 3 : 2; }
+// 224 26.5 / 28.8, 248 28.8 / 28.6).  Compile-time row lengths: 192 with two
+// stages 31.7 against 29.8 for the general one's three (finite-difference
+// current 23.1 / 22.0), 384 with direct stores 30.4 against 29.2.
+constexpr int row_stages(int nx) { return nx > 128 && nx < 200 && nx != 192 ? 3 : 2; }
 
 // Grid of one persistent instantiation, cached per device (the shared-memory
 // opt-in and the resident blocks per SM depend on the device, the block and
@@ -1243,7 +1245,9 @@ cudaError_t row_nx(const RowCall& c) {
   switch (c.g.nx) {
     case 64: return row_launch<T, ODD, 64, row_stages(64), VAR>(c);
     case 128: return row_launch<T, ODD, 128, row_stages(128), VAR>(c);
+    case 192: return row_launch<T, ODD, 192, row_stages(192), VAR>(c);
     case 256: return row_launch<T, ODD, 256, row_stages(256), VAR>(c);
+    case 384: return row_launch<T, ODD, 384, row_stages(384), VAR>(c);
     case 512: return row_launch<T, ODD, 512, row_stages(512), VAR>(c);
     default:
       return row_stages(c.g.nx) == 3 ? row_launch<T, ODD, 0, 3, VAR>(c) : row_launch<T, ODD, 0, 2, VAR>(c);

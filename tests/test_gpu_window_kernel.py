@@ -8,10 +8,11 @@ from gpu_helpers import turbulence
 from paper_2212_11024_gb300 import flame as F
 
 B0 = np.array([0.0, 0.02, 0.05])
-# (nz, ny, nx): N3 a multiple of 8 and not, compile-time and run-time pitches,
+# (nz, ny, nx): two compile-time row lengths (staged by the same rule), then windows:
+# N3 a multiple of 8 and not, compile-time and run-time pitches,
 # single rows (windows at both ends of the state), partly filled last warps
-SHAPES = [(1, 4, 182), (3, 1, 182), (4, 1, 190), (2, 3, 222), (2, 4, 250), (1, 1, 250), (3, 2, 254), (1, 2, 318),
-          (3, 1, 446), (2, 1, 1022)]
+SHAPES = [(2, 3, 192), (1, 2, 384), (1, 4, 182), (3, 1, 182), (4, 1, 190), (2, 3, 222), (2, 4, 250), (1, 1, 250),
+          (3, 2, 254), (1, 2, 318), (3, 1, 446), (2, 1, 1022)]
 
 
 def _run(shape, storage, variant, kernel, n, graph=0):
