@@ -52,33 +52,33 @@ class _Run:
         dev = sim.device
         lam = seed.clone()
         other = torch.empty_like(lam)
-        ddi = torch.zeros(1, dtype=torch.float64, device=dev)
-        ddi_total = torch.zeros(1, dtype=torch.float64, device=dev)
+        # dL/d(d_i) of every step, and of the initialisation in the last place
+        ddi = torch.zeros(self.nsteps + 1, dtype=torch.float64, device=dev)
         starts = sorted(self.ckpt.keys())
         for s0 in reversed(starts):
             s1 = min(s0 + self.k, self.nsteps)
             blob, step, par = self.ckpt[s0]
-            sim.set_state(blob, step, par)
-            seg = []
-            for _ in range(s0, s1):
-                seg.append(sim.get_state())
+            seg = [(blob, par)]  # the states s0 .. s1 - 1: the checkpoint and the replayed ones
+            if s1 - s0 > 1:
+                sim.set_state(blob, step, par)
+            for _ in range(s0 + 1, s1):
                 sim.step(1)
-            for blob_t, _, par_t in reversed(seg):
+                blob_t, _, par_t = sim.get_state()
+                seg.append((blob_t, par_t))
+            for t, (blob_t, par_t) in zip(range(s1 - 1, s0 - 1, -1), reversed(seg)):
                 _check(lib.flame_step_adjoint(sim._ctx, ctypes.c_void_p(blob_t.data_ptr()), int(par_t),
                                               ctypes.c_void_p(lam.data_ptr()), ctypes.c_void_p(other.data_ptr()),
-                                              ctypes.c_void_p(ddi.data_ptr())), "flame_step_adjoint")
+                                              ctypes.c_void_p(ddi.data_ptr() + 8 * t)), "flame_step_adjoint")
                 lam, other = other, lam
-                ddi_total += ddi
             del seg
         ubar = torch.empty((3,) + self.shape, dtype=torch.float64, device=dev)
         Bbar = torch.empty((3,) + self.shape, dtype=torch.float64, device=dev)
         _check(lib.flame_init_adjoint(sim._ctx, ctypes.c_void_p(u0.data_ptr()), ctypes.c_void_p(B0.data_ptr()),
                                       ctypes.c_void_p(lam.data_ptr()), ctypes.c_void_p(ubar.data_ptr()),
-                                      ctypes.c_void_p(Bbar.data_ptr()), ctypes.c_void_p(ddi.data_ptr())),
+                                      ctypes.c_void_p(Bbar.data_ptr()), ctypes.c_void_p(ddi.data_ptr() + 8 * self.nsteps)),
                "flame_init_adjoint")
-        ddi_total += ddi
         sim.sync()
-        return ubar, Bbar, ddi_total[0]
+        return ubar, Bbar, ddi.sum()
 
     def close(self):
         self.sim.close()

@@ -12,6 +12,7 @@
 #include "flame.h"
 #include "flame_internal.h"
 #include "lattice.cuh"
+#include "plans.h"
 
 namespace {
 // An NVTX range over one entry point: the host-side span of each call shows on
@@ -45,8 +46,7 @@ struct flame_ctx {
   void* d_spec;       // nz * ny * (nx/2+1) cufftDoubleComplex
   double* d_shells;   // 2 * nshell_cap doubles
   int nshell_cap;
-  cufftHandle plan;
-  bool has_plan;
+  flame::FftPlan plan;  // of the shell spectra
   void* d_bfield;            // [3][N3] values of the storage type, FLAME_FD_CURRENT only
   cudaGraphExec_t graph[2];  // graph_steps launches starting at parity 0 / 1
   bool has_graph[2];
@@ -837,11 +837,9 @@ static flame_status spectra_of(flame_ctx* c, int nshell, const double* d_u, cons
     }
     c->nshell_cap = nshell;
   }
-  if (!c->has_plan) {
-    if (cufftPlan3d(&c->plan, c->g.nz, c->g.ny, c->g.nx, CUFFT_D2Z) != CUFFT_SUCCESS) return cuda_fail(c, cudaErrorUnknown);
-    c->has_plan = true;
-  }
-  if (cufftSetStream(c->plan, c->stream) != CUFFT_SUCCESS) return cuda_fail(c, cudaErrorUnknown);
+  if (!c->plan.live && flame::plan_take(c->g, CUFFT_D2Z, &c->plan) != CUFFT_SUCCESS)
+    return cuda_fail(c, cudaErrorUnknown);
+  if (cufftSetStream(c->plan.handle, c->stream) != CUFFT_SUCCESS) return cuda_fail(c, cudaErrorUnknown);
   double* u = c->d_fields;
   double* B = c->d_fields + 3 * n3;
   if (!d_u) {
@@ -858,7 +856,7 @@ static flame_status spectra_of(flame_ctx* c, int nshell, const double* d_u, cons
   if (e != cudaSuccess) return cuda_fail(c, e);
   for (int f = 0; f < 6; ++f) {
     double* src = c->d_fields + (size_t)f * n3;
-    if (cufftExecD2Z(c->plan, src, static_cast<cufftDoubleComplex*>(c->d_spec)) != CUFFT_SUCCESS)
+    if (cufftExecD2Z(c->plan.handle, src, static_cast<cufftDoubleComplex*>(c->d_spec)) != CUFFT_SUCCESS)
       return cuda_fail(c, cudaErrorUnknown);
     e = flame::launch_shell_bin(c->d_spec, c->g, nshell, f >= 3, c->d_shells + (f >= 3 ? nshell : 0), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e);
@@ -1045,7 +1043,7 @@ flame_status flame_debug_stall_next_step(flame_ctx* c, unsigned tries) {
 void flame_destroy(flame_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  if (c->has_plan) cufftDestroy(c->plan);
+  flame::plan_give(c->g, &c->plan);
   for (int p = 0; p < 2; ++p)
     if (c->has_graph[p]) cudaGraphExecDestroy(c->graph[p]);
   cudaFree(c->d_flags);

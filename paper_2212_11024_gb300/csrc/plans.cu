@@ -1,0 +1,117 @@
+// plans.cu -- cuFFT plans that outlive a context.
+//
+// Making a 64^3 FP64 plan takes the host 350-500 us and destroying one 60, so
+// a run that makes a context for one gradient (two plans) spent 0.9 ms of its
+// 5.6 on them.  A context takes its plans from a pool and gives them back when
+// it is destroyed; between the two they are its own, and the stream is set
+// before each use.  The pool is bounded: it keeps at most kMostPlans idle plans
+// without a work area of more than kMostWork bytes and destroys the oldest
+// beyond that.  A plan belongs to one driver context of one device (a device
+// that was reset gets a new one) and is given out in that context only.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+#include <cufft.h>
+
+#include <mutex>
+
+#include "plans.h"
+
+namespace flame {
+namespace {
+
+constexpr int kMostPlans = 8;
+constexpr size_t kMostWork = 8u << 20;
+
+struct Key {
+  unsigned long long ctx;
+  int device, type, nx, ny, nz;
+  bool operator==(const Key& k) const {
+    return ctx == k.ctx && device == k.device && type == k.type && nx == k.nx && ny == k.ny && nz == k.nz;
+  }
+};
+
+// The current driver context's id, unique for the life of the process; false
+// where it cannot be had (then plans are not pooled).
+bool context_id(unsigned long long* id) {
+  using Fn = CUresult(CUDAAPI*)(CUcontext, unsigned long long*);
+  static const Fn get = [] {
+    cudaDriverEntryPointQueryResult q;
+    void* fn = nullptr;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Fn>(fn) : nullptr;
+  }();
+  return get && get(nullptr, id) == CUDA_SUCCESS;
+}
+
+struct Pool {
+  std::mutex mu;
+  Key key[kMostPlans];
+  cufftHandle plan[kMostPlans];
+  int n = 0;
+};
+// never destroyed: contexts may be released during the process's exit, after
+// static objects are gone
+Pool& pool() {
+  static Pool* p = new Pool;
+  return *p;
+}
+
+Key key_of(const FftPlan& f, const Grid& g) { return Key{f.ctx, f.device, (int)f.type, g.nx, g.ny, g.nz}; }
+
+}  // namespace
+
+cufftResult plan_take(const Grid& g, cufftType type, FftPlan* f) {
+  f->type = type;
+  f->pooled = cudaGetDevice(&f->device) == cudaSuccess && context_id(&f->ctx);
+  cufftResult r = CUFFT_SUCCESS;
+  if (f->pooled) {
+    const Key k = key_of(*f, g);
+    Pool& p = pool();
+    std::lock_guard<std::mutex> lock(p.mu);
+    for (int i = p.n - 1; i >= 0; --i)
+      if (p.key[i] == k) {
+        f->handle = p.plan[i];
+        f->live = true;
+        --p.n;
+        for (int j = i; j < p.n; ++j) {
+          p.key[j] = p.key[j + 1];
+          p.plan[j] = p.plan[j + 1];
+        }
+        return r;
+      }
+  }
+  r = cufftPlan3d(&f->handle, g.nz, g.ny, g.nx, type);
+  f->live = r == CUFFT_SUCCESS;
+  return r;
+}
+
+void plan_give(const Grid& g, FftPlan* f) {
+  if (!f->live) return;
+  f->live = false;
+  size_t work = 0;
+  if (!f->pooled || cufftGetSize(f->handle, &work) != CUFFT_SUCCESS || work > kMostWork) {
+    cufftDestroy(f->handle);
+    return;
+  }
+  Pool& p = pool();
+  cufftHandle old = 0;
+  bool drop = false;
+  {
+    std::lock_guard<std::mutex> lock(p.mu);
+    if (p.n == kMostPlans) {
+      // the oldest; one of a driver context that is gone went with it
+      drop = p.key[0].ctx == f->ctx;
+      old = p.plan[0];
+      --p.n;
+      for (int j = 0; j < p.n; ++j) {
+        p.key[j] = p.key[j + 1];
+        p.plan[j] = p.plan[j + 1];
+      }
+    }
+    p.key[p.n] = key_of(*f, g);
+    p.plan[p.n++] = f->handle;
+  }
+  if (drop) cufftDestroy(old);
+}
+
+}  // namespace flame

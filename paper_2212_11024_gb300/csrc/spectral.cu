@@ -17,6 +17,7 @@
 
 #include "flame.h"
 #include "flame_internal.h"
+#include "plans.h"
 
 namespace flame {
 
@@ -24,8 +25,7 @@ namespace flame {
 // H = nz * ny * (nx/2 + 1) complex values, grown on demand.
 struct SpectralWs {
   Grid g;
-  cufftHandle d2z, z2d;
-  bool has_d2z, has_z2d;
+  FftPlan d2z, z2d;
   double* real;
   int nreal;
   cufftDoubleComplex* cplx;
@@ -36,8 +36,8 @@ struct SpectralWs {
 void spectral_ws_free(void* p) {
   SpectralWs* w = static_cast<SpectralWs*>(p);
   if (!w) return;
-  if (w->has_d2z) cufftDestroy(w->d2z);
-  if (w->has_z2d) cufftDestroy(w->z2d);
+  plan_give(w->g, &w->d2z);
+  plan_give(w->g, &w->z2d);
   cudaFree(w->real);
   cudaFree(w->cplx);
   cudaFree(w->hist);
@@ -285,15 +285,9 @@ cudaError_t ensure_ws(flame_ctx* ctx, const CtxView& v, int nreal, int ncplx, Sp
     w->ncplx = ncplx;
   }
   if (!w->hist && (e = cudaMalloc(&w->hist, (3 * kMaxShell + 1) * sizeof(double))) != cudaSuccess) return e;
-  if (!w->has_d2z) {
-    if (cufftPlan3d(&w->d2z, v.g.nz, v.g.ny, v.g.nx, CUFFT_D2Z) != CUFFT_SUCCESS) return cudaErrorUnknown;
-    w->has_d2z = true;
-  }
-  if (!w->has_z2d) {
-    if (cufftPlan3d(&w->z2d, v.g.nz, v.g.ny, v.g.nx, CUFFT_Z2D) != CUFFT_SUCCESS) return cudaErrorUnknown;
-    w->has_z2d = true;
-  }
-  if (cufftSetStream(w->d2z, v.stream) != CUFFT_SUCCESS || cufftSetStream(w->z2d, v.stream) != CUFFT_SUCCESS)
+  if (!w->d2z.live && plan_take(v.g, CUFFT_D2Z, &w->d2z) != CUFFT_SUCCESS) return cudaErrorUnknown;
+  if (!w->z2d.live && plan_take(v.g, CUFFT_Z2D, &w->z2d) != CUFFT_SUCCESS) return cudaErrorUnknown;
+  if (cufftSetStream(w->d2z.handle, v.stream) != CUFFT_SUCCESS || cufftSetStream(w->z2d.handle, v.stream) != CUFFT_SUCCESS)
     return cudaErrorUnknown;
   *out = w;
   return cudaSuccess;
@@ -301,11 +295,11 @@ cudaError_t ensure_ws(flame_ctx* ctx, const CtxView& v, int nreal, int ncplx, Sp
 
 cudaError_t d2z(SpectralWs* w, const double* src, cufftDoubleComplex* dst) {
   // the real input of an out-of-place D2Z transform is left unchanged
-  return cufftExecD2Z(w->d2z, const_cast<double*>(src), dst) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown;
+  return cufftExecD2Z(w->d2z.handle, const_cast<double*>(src), dst) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown;
 }
 cudaError_t z2d(SpectralWs* w, cufftDoubleComplex* src, double* dst) {
   // overwrites src
-  return cufftExecZ2D(w->z2d, src, dst) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown;
+  return cufftExecZ2D(w->z2d.handle, src, dst) == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown;
 }
 
 flame_status fail(flame_ctx* ctx, cudaError_t e) { return static_cast<flame_status>(flame_ctx_cuda_fail(ctx, e)); }
