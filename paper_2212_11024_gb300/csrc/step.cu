@@ -4,6 +4,7 @@
 // (the same algebra and variants, two sites per thread) does not apply.
 // launch_step chooses between the two; the finite-difference current's B
 // pre-pass (bfield_kernel) serves both.
+#include "pdl.cuh"
 #include "step_site.cuh"
 
 namespace flame {
@@ -25,6 +26,10 @@ constexpr int kStepMinBlocks = 3;
 template <class T, bool ODD, int VAR, bool FLAT = false>
 __global__ void __launch_bounds__(kStepThreads, kStepMinBlocks)
     step_kernel(Slots<T> P, Grid g, StepConsts k, unsigned* __restrict__ flag, const T* __restrict__ Bfd) {
+  if constexpr (kChained<VAR>) {
+    next_kernel_may_come();
+    after_previous_kernel();
+  }
   int x, y, z;
   if constexpr (FLAT) {
     // consecutive sites of the updated planes (N3 < 2^31)
@@ -130,18 +135,15 @@ cudaError_t bfield_t(int odd, const void* pop, Grid g, void* Bfd_, cudaStream_t 
 }
 
 template <class T, int VAR>
-void step_launch(int odd, const Slots<T>& P, Grid g, const StepConsts& k, unsigned* flag, const T* Bfd, dim3 gr,
+cudaError_t step_launch(int odd, const Slots<T>& P, Grid g, const StepConsts& k, unsigned* flag, const T* Bfd, dim3 gr,
                  dim3 b, bool flat, cudaStream_t s) {
-  if (flat) {
-    if (odd)
-      step_kernel<T, true, VAR, true><<<gr, b, 0, s>>>(P, g, k, flag, Bfd);
-    else
-      step_kernel<T, false, VAR, true><<<gr, b, 0, s>>>(P, g, k, flag, Bfd);
-  } else if (odd) {
-    step_kernel<T, true, VAR><<<gr, b, 0, s>>>(P, g, k, flag, Bfd);
-  } else {
-    step_kernel<T, false, VAR><<<gr, b, 0, s>>>(P, g, k, flag, Bfd);
-  }
+  auto go = [&](auto kern) {
+    if constexpr (kChained<VAR>) return launch_chained(kern, gr, b, 0, s, P, g, k, flag, Bfd);
+    kern<<<gr, b, 0, s>>>(P, g, k, flag, Bfd);
+    return cudaGetLastError();
+  };
+  if (flat) return odd ? go(step_kernel<T, true, VAR, true>) : go(step_kernel<T, false, VAR, true>);
+  return odd ? go(step_kernel<T, true, VAR>) : go(step_kernel<T, false, VAR>);
 }
 
 template <class T>
@@ -157,19 +159,17 @@ cudaError_t step_t(int odd, void* pop, Grid g, const StepConsts& k, unsigned* fl
   }
   const Slots<T> P = make_slots<T>(pop, g);
   switch (variant) {
-    case kVarFlame: step_launch<T, kVarFlame>(odd, P, g, k, flag, nullptr, gr, b, flat, s); break;
-    case kVarBgkFluid: step_launch<T, kVarBgkFluid>(odd, P, g, k, flag, nullptr, gr, b, flat, s); break;
-    case kVarEmhd: step_launch<T, kVarEmhd>(odd, P, g, k, flag, nullptr, gr, b, flat, s); break;
+    case kVarFlame: return step_launch<T, kVarFlame>(odd, P, g, k, flag, nullptr, gr, b, flat, s);
+    case kVarBgkFluid: return step_launch<T, kVarBgkFluid>(odd, P, g, k, flag, nullptr, gr, b, flat, s);
+    case kVarEmhd: return step_launch<T, kVarEmhd>(odd, P, g, k, flag, nullptr, gr, b, flat, s);
     case kVarFdCurrent: {
       if (!Bfd) return cudaErrorInvalidValue;
       const cudaError_t e = bfield_t<T>(odd, pop, g, Bfd, s);
       if (e != cudaSuccess) return e;
-      step_launch<T, kVarFdCurrent>(odd, P, g, k, flag, static_cast<const T*>(Bfd), gr, b, flat, s);
-      break;
+      return step_launch<T, kVarFdCurrent>(odd, P, g, k, flag, static_cast<const T*>(Bfd), gr, b, flat, s);
     }
-    default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 

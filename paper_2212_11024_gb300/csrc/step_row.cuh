@@ -53,6 +53,7 @@
 #include <mutex>
 
 #include "aa.cuh"
+#include "pdl.cuh"
 
 namespace flame {
 
@@ -806,6 +807,7 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
   // location is read or written by more than one tile, so the order of these
   // stores and of other tiles' loads does not matter.
   constexpr bool kDirect = kRowStages == 2 && (NX > 256 || NX == 0 || H > 1);
+  if constexpr (kChained<VAR>) after_previous_kernel();
   if (warp == 0)
     for (int s = 0; s < kAhead; ++s)
       if (first + s * stride < ntiles) io.issue(first + s * stride, s);
@@ -908,6 +910,12 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
       }
     }
   }
+  // Here and not at the start: several blocks share an SM, and the next
+  // kernel's waiting blocks beside working ones cost more than they save (FP16
+  // us per step plain, from the start, here: 128^3 69.6, 70.6, 67.2; 192^3
+  // 226.0, 227.0, 224.4; 512 x 256 x 256 1059.6, 1060.8, 1057.3; 256^3 alone
+  // gained more from the start: 514.0, 508.5, 510.9).
+  if constexpr (kChained<VAR>) next_kernel_may_come();
   if (warp == 0) bulk_wait_done();
 }
 
@@ -1003,6 +1011,10 @@ __global__ void __launch_bounds__(window_bound_threads(PITCH), 512 / window_boun
   const WindowIO<T, ODD> io{state, rows, bars, g.n3, nx, ny, nz, g.z0, pitch, lane, kSpread ? warp : 0, nw,
                             wt.stall != 0};
   const int first = blockIdx.x, stride = gridDim.x;
+  if constexpr (kChained<VAR>) {
+    next_kernel_may_come();
+    after_previous_kernel();
+  }
   if (issues)
     for (int st = 0; st < 2; ++st)
       if (first + st * stride < ntiles) io.issue(first + st * stride, st);
@@ -1116,6 +1128,10 @@ template <class T, bool ODD, int VAR>
 __global__ void __launch_bounds__(kPairThreads, 4)
     step_pair_kernel(Grid g, StepConsts k, unsigned* __restrict__ flag, const T* __restrict__ Bfd,
                      const __grid_constant__ SlotBases<T> bases) {
+  if constexpr (kChained<VAR>) {
+    next_kernel_may_come();
+    after_previous_kernel();
+  }
   const long long p = (long long)blockIdx.x * kPairThreads + threadIdx.x;
   if (p >= (long long)(g.nx / 2) * g.ny * g.nzi) return;
   step_pair<T, ODD, VAR, false>(g, k, flag, Bfd, bases, p);
@@ -1130,6 +1146,9 @@ cudaError_t pair_launch(const RowCall& c) {
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   SlotBases<T> bases;
   for (int sl = 0; sl < kPop; ++sl) bases.p[sl] = static_cast<T*>(c.pop) + (size_t)sl * (size_t)c.g.n3;
+  if constexpr (kChained<VAR>)
+    return launch_chained(step_pair_kernel<T, ODD, VAR>, dim3((unsigned)blocks), dim3(kPairThreads), 0, c.s, c.g, c.k,
+                          c.flag, static_cast<const T*>(c.Bfd), bases);
   step_pair_kernel<T, ODD, VAR><<<(unsigned)blocks, kPairThreads, 0, c.s>>>(c.g, c.k, c.flag,
                                                                          static_cast<const T*>(c.Bfd), bases);
   return cudaGetLastError();
@@ -1201,6 +1220,9 @@ cudaError_t row_launch(const RowCall& c) {
   if (e != cudaSuccess || !c.launch) return e;
   SlotBases<T> bases;
   for (int sl = 0; sl < kPop; ++sl) bases.p[sl] = static_cast<T*>(c.pop) + (size_t)sl * (size_t)c.g.n3;
+  if constexpr (kChained<VAR>)
+    return launch_chained(step_row_kernel<T, ODD, NX, S, VAR, H>, dim3(grid), dim3(c.g.nx / (2 * H)), smem, c.s,
+                          static_cast<T*>(c.pop), c.g, c.k, c.flag, static_cast<const T*>(c.Bfd), maps, bases, c.wt);
   step_row_kernel<T, ODD, NX, S, VAR, H>
       <<<grid, c.g.nx / (2 * H), smem, c.s>>>(static_cast<T*>(c.pop), c.g, c.k, c.flag,
                                               static_cast<const T*>(c.Bfd), maps, bases, c.wt);
@@ -1218,6 +1240,9 @@ cudaError_t window_go(const RowCall& c) {
   if (e != cudaSuccess || !c.launch) return e;
   SlotBases<T> bases;
   for (int sl = 0; sl < kPop; ++sl) bases.p[sl] = static_cast<T*>(c.pop) + (size_t)sl * (size_t)c.g.n3;
+  if constexpr (kChained<VAR>)
+    return launch_chained(step_window_kernel<T, ODD, VAR, PITCH>, dim3(grid), dim3(threads), smem, c.s,
+                          static_cast<const T*>(c.pop), c.g, c.k, c.flag, static_cast<const T*>(c.Bfd), bases, c.wt);
   step_window_kernel<T, ODD, VAR, PITCH><<<grid, threads, smem, c.s>>>(
       static_cast<const T*>(c.pop), c.g, c.k, c.flag, static_cast<const T*>(c.Bfd), bases, c.wt);
   return cudaGetLastError();
