@@ -415,6 +415,17 @@ flame_status flame_get_state(flame_ctx *ctx, void *d_dst, long long *step, int *
  * Errors: FLAME_ERR_STATE (parity not 0/1, step < 0).  Asynchronous. */
 flame_status flame_set_state(flame_ctx *ctx, const void *d_src, long long step, int parity);
 
+/* One flame_step from the state blob d_from to d_to (both flame_state_bytes,
+ * 256-byte aligned, not overlapping), for a run that keeps its states: d_from
+ * holds the populations at the context's step count and parity, which advance
+ * by one.  Either may be the context's own state; where d_to is not, that one
+ * is left as it was and the caller goes on from d_to, by this call or by
+ * flame_set_state.  The same bits as flame_step.  Whole lattices of the
+ * FLAME_SCHEME variant only; no check_every.  Errors: FLAME_ERR_PARAM,
+ * FLAME_ERR_STATE (no state yet), FLAME_ERR_CUDA, sticky errors.
+ * Asynchronous. */
+flame_status flame_step_between(flame_ctx *ctx, const void *d_from, void *d_to);
+
 /* Adjoint (vector-Jacobian product) of one flame_step, for gradients of a
  * loss of a later state (the hand-written reverse of Sec. 3's collision and
  * streaming; the paper has no adjoint, its equations define the forward map).

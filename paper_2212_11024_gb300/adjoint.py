@@ -44,10 +44,19 @@ class _Run:
         if nsteps * sim.state.numel() <= KEEP_ALL * torch.cuda.mem_get_info(sim.device)[0]:
             self.k = 1
         self.ckpt = {}
-        for t in range(nsteps):
-            if t % self.k == 0:
-                self.ckpt[t] = sim.get_state()
-            sim.step(1)
+        if self.k == 1 and nsteps > 0:
+            # every state is kept: each step writes the next one's buffer
+            blob, step, par = sim.get_state()
+            for t in range(nsteps):
+                self.ckpt[t] = blob, step + t, par ^ (t & 1)
+                after = torch.empty_like(blob) if t + 1 < nsteps else sim.state
+                sim.step_between(blob, after)
+                blob = after
+        else:
+            for t in range(nsteps):
+                if t % self.k == 0:
+                    self.ckpt[t] = sim.get_state()
+                sim.step(1)
         sim.sync()
         self.nsteps = nsteps
         # the loss of the last state and the adjoint seed dL/df (flame_band_energy)

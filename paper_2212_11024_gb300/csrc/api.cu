@@ -916,6 +916,24 @@ flame_status flame_set_state(flame_ctx* c, const void* d_src, long long step, in
   return FLAME_OK;
 }
 
+flame_status flame_step_between(flame_ctx* c, const void* d_from, void* d_to) {
+  const Range range("flame_step_between");
+  const flame_status st = usable(c);
+  if (st != FLAME_OK) return st;
+  if (!d_from || !d_to || c->p.variant != FLAME_SCHEME || c->p.halo_z) return FLAME_ERR_PARAM;
+  if (((uintptr_t)d_from | (uintptr_t)d_to) % 256) return FLAME_ERR_PARAM;
+  const size_t bytes = flame_state_bytes(&c->p);
+  const uintptr_t a = (uintptr_t)d_from, b = (uintptr_t)d_to;
+  if (a < b + bytes && b < a + bytes) return FLAME_ERR_PARAM;
+  if (!c->initialized || !c->state) return FLAME_ERR_STATE;
+  const cudaError_t e = flame::launch_step_between(c->p.storage, c->parity, d_from, d_to, c->g, c->k, c->d_flags,
+                                                   c->stream, c->p.kernel);
+  if (e != cudaSuccess) return cuda_fail(c, e);
+  c->parity ^= 1;
+  c->step += 1;
+  return FLAME_OK;
+}
+
 // The adjoints' partial sums and their ticket, zeroed (on the context's stream).
 static cudaError_t adj_partials(flame_ctx* c) {
   if (c->d_adj_partials) return cudaSuccess;

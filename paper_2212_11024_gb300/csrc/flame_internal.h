@@ -45,6 +45,12 @@ constexpr int kVarFdCurrent = 3;  // J from the central-difference curl of B
 cudaError_t launch_step(int storage, int odd, void* pop, Grid g, const StepConsts& k, unsigned* flag,
                         cudaStream_t s, int variant = kVarFlame, void* Bfd = nullptr, int kernel = 0);
 
+// The step of the kVarFlame scheme on a whole lattice from the state `from` to
+// another one, `to` (not overlapping): the one-site kernel writes there, the
+// packed kernels, whose tiles go back where they came from, step a copy.
+cudaError_t launch_step_between(int storage, int odd, const void* from, void* to, Grid g, const StepConsts& k,
+                                unsigned* flag, cudaStream_t s, int kernel);
+
 // Several steps in one launch (step_multi.cu), for a lattice whose sites (or
 // pairs, where the packed kernels apply) are at most the threads resident at
 // once; the same populations as n launches of launch_step.  sync: two zeroed

@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(kSiteThreads, 2)
   };
   steps(
       odd, n, flag, sync,
-      [&] { each([&](int x, int y, int z) { step_site<T, false, VAR, true>(P, g, k, flag, nullptr, x, y, z); }); },
-      [&] { each([&](int x, int y, int z) { step_site<T, true, VAR, true>(P, g, k, flag, nullptr, x, y, z); }); });
+      [&] { each([&](int x, int y, int z) { step_site<T, false, VAR, true>(P, P, g, k, flag, nullptr, x, y, z); }); },
+      [&] { each([&](int x, int y, int z) { step_site<T, true, VAR, true>(P, P, g, k, flag, nullptr, x, y, z); }); });
 }
 
 template <class T, int VAR>

@@ -43,8 +43,10 @@ __device__ __forceinline__ T load_pop(const T* p) {
   else return *p;
 }
 
+// Reads the populations of P and writes those of O: the state itself, or another
+// one (every location is written by the site that read it).
 template <class T, bool ODD, int VAR, bool L2>
-__device__ __forceinline__ void step_site(const Slots<T>& P, const Grid& g, const StepConsts& k,
+__device__ __forceinline__ void step_site(const Slots<T>& P, const Slots<T>& O, const Grid& g, const StepConsts& k,
                                           unsigned* __restrict__ flag, const T* __restrict__ Bfd, int x, int y, int z) {
   const int site = (z * g.ny + y) * g.nx + x;
   const Nbr nb = make_nbr(x, y, z, g);
@@ -165,7 +167,7 @@ __device__ __forceinline__ void step_site(const Slots<T>& P, const Grid& g, cons
     const float om = k.omegaB, cm = 1.f - k.omegaB;
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      P.p[mslot(b, ODD ? 0 : opp7(0))][site] = Codec<T>::enc(cm * sg[b][0] + om * dB[b]);
+      O.p[mslot(b, ODD ? 0 : opp7(0))][site] = Codec<T>::enc(cm * sg[b][0] + om * dB[b]);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const float l0 = (a == b) ? 0.f : 4.f * (V[a] * B[b] - B[a] * V[b]);
@@ -173,7 +175,7 @@ __device__ __forceinline__ void step_site(const Slots<T>& P, const Grid& g, cons
         for (int h = 1; h <= 2; ++h) {
           const int i = 2 * a + h;
           const float v = cm * sg[b][i] + om * (h == 1 ? dB[b] + l0 : dB[b] - l0);
-          P.p[mslot(b, ODD ? i : opp7(i))][site + dst_off<ODD>(nb, mx7(i), my7(i), mz7(i))] = Codec<T>::enc(v);
+          O.p[mslot(b, ODD ? i : opp7(i))][site + dst_off<ODD>(nb, mx7(i), my7(i), mz7(i))] = Codec<T>::enc(v);
         }
       }
     }
@@ -261,7 +263,7 @@ __device__ __forceinline__ void step_site(const Slots<T>& P, const Grid& g, cons
       for (int pz = 0; pz < 3; ++pz) {
         const int i = idx27(px, py, pz);
         const int slot = ODD ? i : opp27(i);
-        P.p[slot][site + dst_off<ODD>(nb, cx, cy, pz - 1)] = Codec<T>::enc(vz[pz]);
+        O.p[slot][site + dst_off<ODD>(nb, cx, cy, pz - 1)] = Codec<T>::enc(vz[pz]);
       }
     }
 }

@@ -101,6 +101,7 @@ def _lib():
             "flame_lattice": (i, [P(i), P(i)]),
             "flame_reduce_static": (i, [vp, i, vp]),
             "flame_probe": (i, [vp, i, vp, vp]),
+            "flame_step_between": (i, [vp, vp, vp]),
             "flame_step_adjoint": (i, [vp, vp, i, vp, vp, vp]),
             "flame_init_adjoint": (i, [vp, vp, vp, vp, vp, vp, vp]),
             "flame_debug_stall_next_step": (i, [vp, ctypes.c_uint]),
@@ -540,6 +541,19 @@ class Flame:
         self._after(cur, dst)
         _check(rc, "flame_get_state")
         return dst, int(step.value), int(par.value)
+
+    def step_between(self, src, dst):
+        """flame_step_between: one step from the state blob `src`, at this
+        run's step and parity, to the blob `dst` (either may be self.state)."""
+        if self.state is None:
+            raise FlameError(FLAME_ERR_STATE, "flame_step_between (a context without state)")
+        for b in (src, dst):
+            if b.numel() != self.state.numel() or b.dtype != self.state.dtype or not b.is_contiguous():
+                raise ValueError("state blob does not match these parameters")
+        cur = self._before()
+        rc = self._lib.flame_step_between(self._ctx_or_raise(), self._ptr(src), self._ptr(dst))
+        self._after(cur, src, dst)
+        _check(rc, "flame_step_between")
 
     def set_state(self, src, step, parity):
         if self.state is None:
