@@ -30,6 +30,7 @@
 
 #include "aa.cuh"
 #include "expansion.cuh"
+#include "pdl.cuh"
 
 namespace flame {
 namespace {
@@ -95,17 +96,18 @@ __device__ __forceinline__ void block_sum_to(double v, double* out) {
   }
 }
 
-// Read-only loads with an L2 prefetch-size hint (the neighbouring warps'
-// segments of the same rows arrive with the first request).
+// Loads with an L2 prefetch-size hint (the neighbouring warps' segments of the
+// same rows arrive with the first request).  Not read-only ones: the kernel may
+// have started before the one that writes these buffers ended.
 template <class T>
 __device__ __forceinline__ float ld_state(const T* p) {
   if constexpr (sizeof(T) == 4) {
     float v;
-    asm volatile("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
   } else {
     unsigned short h;
-    asm volatile("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(h) : "l"(p));
+    asm volatile("ld.global.L2::256B.b16 %0, [%1];" : "=h"(h) : "l"(p));
     if constexpr (std::is_same_v<T, __half>) return __half2float(__ushort_as_half(h));
     else return __bfloat162float(__ushort_as_bfloat16(h));
   }
@@ -448,6 +450,8 @@ template <class T, bool ODD>
 __global__ void __launch_bounds__(kAdjThreads, (kAdjMinBlocks<T, ODD>))
     adjoint_step_kernel(Slots<T> P, Grid g, StepConsts k, const __grid_constant__ LamSlots L,
                         double* __restrict__ partials) {
+  next_kernel_may_come();
+  after_previous_kernel();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z + g.z0;
@@ -731,13 +735,15 @@ __device__ __forceinline__ double sum_of_block(double a) {
   return a;
 }
 __global__ void __launch_bounds__(kSumThreads)
-    sum_partials_kernel(const double* __restrict__ partials, long long n, double* stage, unsigned* ticket,
+    sum_partials_kernel(const double* partials, long long n, double* stage, unsigned* ticket,
                         double* __restrict__ out) {
   __shared__ bool last;
+  next_kernel_may_come();
+  after_previous_kernel();
   const long long per = (n + gridDim.x - 1) / gridDim.x;
   const long long lo = per * blockIdx.x, hi = lo + per < n ? lo + per : n;
   double a = 0.0;
-  for (long long i = lo + threadIdx.x; i < hi; i += kSumThreads) a += partials[i];
+  for (long long i = lo + threadIdx.x; i < hi; i += kSumThreads) a += __ldcg(partials + i);
   a = sum_of_block(a);
   if (threadIdx.x == 0) {
     __stcg(stage + blockIdx.x, a);
@@ -756,11 +762,12 @@ __global__ void __launch_bounds__(kSumThreads)
 }
 // Sum of n partials into *out; the buffer holds n partials, kSumBlocks doubles
 // and the ticket (zeroed when it was allocated).
-inline void sum_partials(double* partials, long long cap, long long n, double* out, cudaStream_t s) {
+inline cudaError_t sum_partials(double* partials, long long cap, long long n, double* out, cudaStream_t s) {
   const long long want = (n + 4 * kSumThreads - 1) / (4 * kSumThreads);
   double* stage = partials + cap;
-  sum_partials_kernel<<<(unsigned)(want < kSumBlocks ? want : kSumBlocks), kSumThreads, 0, s>>>(
-      partials, n, stage, reinterpret_cast<unsigned*>(stage + kSumBlocks), out);
+  return launch_chained(sum_partials_kernel, dim3((unsigned)(want < kSumBlocks ? want : kSumBlocks)), dim3(kSumThreads), 0,
+                        s, static_cast<const double*>(partials), n, stage,
+                        reinterpret_cast<unsigned*>(stage + kSumBlocks), out);
 }
 
 // The partials of either adjoint: one per warp of the step kernel, one per
@@ -783,12 +790,10 @@ cudaError_t adjoint_t(int odd, const void* pop, Grid g, const StepConsts& k, con
     L.in[q] = lin + (size_t)q * (size_t)g.n3;
     L.out[q] = lout + (size_t)q * (size_t)g.n3;
   }
-  if (odd)
-    adjoint_step_kernel<T, true><<<gr, b, 0, s>>>(P, g, k, L, partials);
-  else
-    adjoint_step_kernel<T, false><<<gr, b, 0, s>>>(P, g, k, L, partials);
-  sum_partials(partials, partials_cap(g), nblk * ((b.x * b.y) >> 5), ddi, s);
-  return cudaGetLastError();
+  auto go = [&](auto kern) { return launch_chained(kern, gr, b, 0, s, P, g, k, L, partials); };
+  const cudaError_t e = odd ? go(adjoint_step_kernel<T, true>) : go(adjoint_step_kernel<T, false>);
+  if (e != cudaSuccess) return e;
+  return sum_partials(partials, partials_cap(g), nblk * ((b.x * b.y) >> 5), ddi, s);
 }
 
 }  // namespace
@@ -816,7 +821,8 @@ cudaError_t launch_init_adjoint(Grid g, const StepConsts& k, const double* u, co
   double* dBb = ws + 15 * n3;
   init_adjoint_local_kernel<<<gr, b, 0, s>>>(g, k, u, B, lam, ubl, Bbl, dub, dBb, partials);
   init_adjoint_stencil_kernel<<<gr, b, 0, s>>>(g, ubl, Bbl, dub, dBb, ubar, Bbar);
-  sum_partials(partials, partials_cap(g), (long long)gr.x * gr.y * gr.z, ddi, s);
+  const cudaError_t e = sum_partials(partials, partials_cap(g), (long long)gr.x * gr.y * gr.z, ddi, s);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
