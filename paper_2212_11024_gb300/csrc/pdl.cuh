@@ -39,7 +39,9 @@ __device__ __forceinline__ void after_previous_kernel() { asm volatile("griddepc
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool plain = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  const bool asked = cudaStreamIsCapturing(s, &cap) == cudaSuccess;
+  if (!asked) (void)cudaGetLastError();  // the launch below reports what is wrong
+  const bool plain = !asked || cap != cudaStreamCaptureStatusNone;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
