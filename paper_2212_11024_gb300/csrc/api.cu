@@ -570,7 +570,7 @@ int flame_step_kernel(const flame_params* p) {
   // looked at
   const void* aligned = reinterpret_cast<const void*>(static_cast<uintptr_t>(256));
   if (!flame::step_row_supported(g, p->storage, p->variant, aligned, p->kernel)) return FLAME_KERNEL_SITE;
-  switch (flame::row_segments(g.nx, p->kernel)) {
+  switch (flame::row_segments(g, p->kernel, p->variant)) {
     case 0:
     case flame::kWindows: return FLAME_KERNEL_PAIRS;
     case 2: return FLAME_KERNEL_HALF_ROWS;

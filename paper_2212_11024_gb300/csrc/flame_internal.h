@@ -28,6 +28,19 @@ struct Grid {
   long long n3i;   // nx * ny * nzi: the sites updated, and the size of per-site outputs
 };
 
+// floor(2^32 / d) of nx and ny (2^32 - 1 for d = 1), for the quotients of kernels
+// that number sites or rows through the lattice (quotient in aa.cuh).  The last
+// argument of those kernels and no part of Grid: 8 bytes more there moved the
+// arguments after it, and rows of run-time lengths, whose code does not use it,
+// took 1-2 % longer, windows 2-5 %.
+struct Reciprocals {
+  unsigned x, y;
+};
+inline Reciprocals reciprocals(const Grid& g) {
+  auto of = [](int d) { return d == 1 ? 0xffffffffu : (unsigned)(0x100000000ull / (unsigned)d); };
+  return {of(g.nx), of(g.ny)};
+}
+
 // Scheme variants (flame_variant).
 constexpr int kVarFlame = 0;      // the paper's scheme
 constexpr int kVarBgkFluid = 1;   // BGK fluid collision
@@ -82,7 +95,7 @@ bool step_row_supported(Grid g, int storage, int variant, const void* pop, int k
 // the pair kernel, no staging; kWindows: whole rows of any even length, staged
 // as the aligned windows around them).
 constexpr int kWindows = 3;
-int row_segments(int nx, int kernel);
+int row_segments(const Grid& g, int kernel, int variant);
 // step_row_supported with staged rows (the kernels whose copies have waits).
 bool step_row_staged(Grid g, int storage, int variant, const void* pop, int kernel = 0);
 // Settles the launch configuration of the kernel launch_step would use

@@ -24,15 +24,16 @@ constexpr int kStepThreads = 256;
 constexpr int kStepMinBlocks = 3;
 
 // The site of this thread; false where it has none.
-template <bool FLAT>
-__device__ __forceinline__ bool site_of(const Grid& g, int& x, int& y, int& z) {
+template <class T, bool FLAT>
+__device__ __forceinline__ bool site_of(const Grid& g, const Reciprocals& rc, int& x, int& y, int& z) {
   if constexpr (FLAT) {
     // consecutive sites of the updated planes (N3 < 2^31)
     const int p = blockIdx.x * kStepThreads + threadIdx.x;
     if (p >= (int)g.n3i) return false;
-    const int r = p / g.nx;
+    // (FP32 storage waits for HBM either way: 0.5 % slower by quotient)
+    const int r = sizeof(T) == 2 ? quotient(p, g.nx, rc.x) : p / g.nx;
     x = p - r * g.nx;
-    const int zz = r / g.ny;
+    const int zz = sizeof(T) == 2 ? quotient(r, g.ny, rc.y) : r / g.ny;
     y = r - zz * g.ny;
     z = zz + g.z0;
   } else {
@@ -46,13 +47,14 @@ __device__ __forceinline__ bool site_of(const Grid& g, int& x, int& y, int& z) {
 
 template <class T, bool ODD, int VAR, bool FLAT = false>
 __global__ void __launch_bounds__(kStepThreads, kStepMinBlocks)
-    step_kernel(Slots<T> P, Grid g, StepConsts k, unsigned* __restrict__ flag, const T* __restrict__ Bfd) {
+    step_kernel(Slots<T> P, Grid g, StepConsts k, unsigned* __restrict__ flag, const T* __restrict__ Bfd,
+                Reciprocals rc) {
   if constexpr (kChained<VAR>) {
     next_kernel_may_come();
     after_previous_kernel();
   }
   int x, y, z;
-  if (!site_of<FLAT>(g, x, y, z)) return;
+  if (!site_of<T, FLAT>(g, rc, x, y, z)) return;
   step_site<T, ODD, VAR, false>(P, P, g, k, flag, Bfd, x, y, z);
 }
 
@@ -64,11 +66,11 @@ __global__ void __launch_bounds__(kStepThreads, kStepMinBlocks)
 template <class T, bool ODD, bool FLAT>
 __global__ void __launch_bounds__(kStepThreads, kStepMinBlocks)
     step_between_kernel(const __grid_constant__ Slots<T> P, const __grid_constant__ Slots<T> O, Grid g, StepConsts k,
-                        unsigned* __restrict__ flag) {
+                        unsigned* __restrict__ flag, Reciprocals rc) {
   next_kernel_may_come();
   after_previous_kernel();
   int x, y, z;
-  if (!site_of<FLAT>(g, x, y, z)) return;
+  if (!site_of<T, FLAT>(g, rc, x, y, z)) return;
   step_site<T, ODD, kVarFlame, false>(P, O, g, k, flag, nullptr, x, y, z);
 }
 
@@ -159,8 +161,8 @@ template <class T, int VAR>
 cudaError_t step_launch(int odd, const Slots<T>& P, Grid g, const StepConsts& k, unsigned* flag, const T* Bfd, dim3 gr,
                  dim3 b, bool flat, cudaStream_t s) {
   auto go = [&](auto kern) {
-    if constexpr (kChained<VAR>) return launch_chained(kern, gr, b, 0, s, P, g, k, flag, Bfd);
-    kern<<<gr, b, 0, s>>>(P, g, k, flag, Bfd);
+    if constexpr (kChained<VAR>) return launch_chained(kern, gr, b, 0, s, P, g, k, flag, Bfd, reciprocals(g));
+    kern<<<gr, b, 0, s>>>(P, g, k, flag, Bfd, reciprocals(g));
     return cudaGetLastError();
   };
   if (flat) return odd ? go(step_kernel<T, true, VAR, true>) : go(step_kernel<T, false, VAR, true>);
@@ -182,7 +184,7 @@ cudaError_t between_t(int odd, const void* from, void* to, Grid g, const StepCon
   dim3 b, gr;
   const bool flat = step_shape(g, &b, &gr);
   const Slots<T> P = make_slots<T>(from, g), O = make_slots<T>(to, g);
-  auto go = [&](auto kern) { return launch_chained(kern, gr, b, 0, s, P, O, g, k, flag); };
+  auto go = [&](auto kern) { return launch_chained(kern, gr, b, 0, s, P, O, g, k, flag, reciprocals(g)); };
   if (flat) return odd ? go(step_between_kernel<T, true, true>) : go(step_between_kernel<T, false, true>);
   return odd ? go(step_between_kernel<T, true, false>) : go(step_between_kernel<T, false, false>);
 }

@@ -74,10 +74,11 @@ __device__ __forceinline__ void steps(int odd, int n, unsigned* flag, unsigned* 
 
 template <class T, int VAR>
 __global__ void __launch_bounds__(kSiteThreads, 2)
-    step_sites_kernel(Slots<T> P, Grid g, StepConsts k, unsigned* flag, unsigned* sync, int odd, int n) {
+    step_sites_kernel(Slots<T> P, Grid g, StepConsts k, unsigned* flag, unsigned* sync, int odd, int n,
+                      Reciprocals rc) {
   auto each = [&](auto&& f) {
     for (int p = blockIdx.x * kSiteThreads + threadIdx.x; p < (int)g.n3i; p += gridDim.x * kSiteThreads) {
-      const int r = p / g.nx, zz = r / g.ny;
+      const int r = quotient(p, g.nx, rc.x), zz = quotient(r, g.ny, rc.y);
       f(p - r * g.nx, r - zz * g.ny, zz + g.z0);
     }
   };
@@ -90,16 +91,16 @@ __global__ void __launch_bounds__(kSiteThreads, 2)
 template <class T, int VAR>
 __global__ void __launch_bounds__(kMultiPairThreads, 4)
     step_pairs_kernel(Grid g, StepConsts k, unsigned* flag, const __grid_constant__ SlotBases<T> bases, unsigned* sync,
-                      int odd, int n) {
-  const long long total = (long long)(g.nx / 2) * g.ny * g.nzi, stride = (long long)gridDim.x * kMultiPairThreads;
-  const long long first = (long long)blockIdx.x * kMultiPairThreads + threadIdx.x;
+                      int odd, int n, Reciprocals rc) {
+  const int total = (g.nx / 2) * g.ny * g.nzi, stride = gridDim.x * kMultiPairThreads;
+  const int first = blockIdx.x * kMultiPairThreads + threadIdx.x;
   steps(
       odd, n, flag, sync,
       [&] {
-        for (long long p = first; p < total; p += stride) step_pair<T, false, VAR, true>(g, k, flag, nullptr, bases, p);
+        for (int p = first; p < total; p += stride) step_pair<T, false, VAR, true>(g, k, flag, nullptr, bases, rc, p);
       },
       [&] {
-        for (long long p = first; p < total; p += stride) step_pair<T, true, VAR, true>(g, k, flag, nullptr, bases, p);
+        for (int p = first; p < total; p += stride) step_pair<T, true, VAR, true>(g, k, flag, nullptr, bases, rc, p);
       });
 }
 
@@ -125,7 +126,8 @@ cudaError_t sites_go(const MultiCall& c, bool* taken) {
   StepConsts k = c.k;
   unsigned *flag = c.flag, *sync = c.sync;
   int odd = c.odd, n = c.n;
-  void* args[] = {&P, &g, &k, &flag, &sync, &odd, &n};
+  Reciprocals rc = reciprocals(c.g);
+  void* args[] = {&P, &g, &k, &flag, &sync, &odd, &n, &rc};
   return cudaLaunchCooperativeKernel(step_sites_kernel<T, VAR>, dim3(grid), dim3(kSiteThreads), args, 0, c.s);
 }
 
@@ -141,7 +143,8 @@ cudaError_t pairs_go(const MultiCall& c, bool* taken) {
   StepConsts k = c.k;
   unsigned *flag = c.flag, *sync = c.sync;
   int odd = c.odd, n = c.n;
-  void* args[] = {&g, &k, &flag, &bases, &sync, &odd, &n};
+  Reciprocals rc = reciprocals(c.g);
+  void* args[] = {&g, &k, &flag, &bases, &sync, &odd, &n, &rc};
   return cudaLaunchCooperativeKernel(step_pairs_kernel<T, VAR>, dim3(grid), dim3(kMultiPairThreads), args, 0, c.s);
 }
 

@@ -46,38 +46,40 @@ cudaError_t row_maps(const void* pop, const Grid& g, RowMaps* out) {
 
 cudaError_t step_row_flame(const RowCall& c) { return row_call<kVarFlame>(c); }
 
-// The automatic choice among the row kernel's tilings, from a sweep of
-// every multiple of 8 from 64 to 1024 with FP16 storage on ~4M-site
-// lattices (nx x m x m, graph replay, GLUPS).  The unstaged pair kernel runs
-// at 24.6-25.4 at every length; the staged kernel's whole rows run at 28-32
-// where a row's block fits several times per SM and its stages are dense
-// (64 28.1, 128 31.8, 192 29.3, 256 31.9, 320 30.0, 384 29.0, 448 30.3, 512
-// 30.7, 768 28.5, 1024 31.5), and lose to the pair kernel where a block is
-// under 48 threads (72-96: 18.6-24.5), where three stages of padded rows
-// fit few blocks (136-152: 21.2-24.1), where a block of 260-320 threads
-// fits once per SM (520-648: 20.0-24.9, half rows 22.5-26.7, ahead of the
-// pair kernel from 608 where a half row is whole 16-byte units) and at
-// 776-792 (24.4-25.0).  Ties (within 0.3) keep whole rows.  Odd row lengths
-// take the one-site kernel.  Even lengths that are no multiple of 8 are staged
-// as windows where enough of a resident block's lanes hold a pair
-// (window_pays), else they take the pair kernel.
+// The automatic choice among the packed kernels, from sweeps with FP16 storage
+// on ~4M-site lattices (nx x m x m, graph replay, GLUPS).  The unstaged pair
+// kernel runs at 25.6-26.3 at every even length (24.6-25.4 while it numbered its
+// pairs by 64-bit divisions, when the lines below were drawn); the staged kernel's
+// whole rows run at 26-32 at most multiples of 8 (64 28.1, 128 31.3, 192 31.0, 256
+// 32.1, 320 28.7, 384 28.3, 448 28.6, 512 30.2, 768 26.7, 1024 30.2) and lose to it
+// where a block is under 48 threads (72-96: 17.8-23.4), where three stages of padded
+// rows fit few blocks (136-152: 20.3-22.6), where a block of 260-320 threads fits
+// once per SM (520-648: 18.6-23.0, half rows 21.3-25.5) and at 776-792 (23.1-23.5).
+// Behind the faster pairs, but left as they were: whole rows at 160-168 (23.7-24.8),
+// 264-280, 328-352, 656-728 and 800-840 (23.4-25.5), half rows at 608-640 (24.5-25.5).
+// Odd row lengths take the one-site kernel.  Even lengths that are no multiple of 8
+// are staged as windows where window_pays, else they take the pair kernel.
 //
 // Windows run a block of whole warps per row at 128 registers, 512 threads'
-// worth per SM, so what counts is the pairs those hold.  GLUPS windows / pair
-// kernel (pairs per SM): 126 25.1 / 24.9 (504), 158 22.3 / 24.8 (395), 190 26.5
-// / 25.0 (475), 198 22.8 / 25.1 (396), 222 27.2 / 25.0 (444), 250 28.1 / 25.0
-// (500), 258 23.6 / 25.3 (387), 286 26.0 / 25.2 (429), 300 26.7 / 25.2 (450), 318
-// 28.0 / 24.8 (477), 340 24.4 / 24.9 (340), 382 26.9 / 25.3 (382), 446 28.3 / 25.3
-// (446), 510 28.0 / 25.2 (510), 700 25.4 / 24.9 (350), 766 26.4 / 25.0 (383), 892
-// 26.8 / 25.2 (446), 1022 28.7 / 25.1 (511).
-static bool window_pays(int nx) {
+// worth per SM.  They are ahead of the pairs where at least 448 threads (of one
+// block, 480) are resident and 95.5 % of them hold a pair (GLUPS: 246 26.4, 254
+// 27.2, 306 26.1, 318 27.0, 430 26.2, 446 27.1, 486 26.4, 510 27.3, 948 26.6, 1022
+// 27.8, and behind at 242 26.0, 298 25.5, 378 25.2, 382 25.5, 422 25.8, 474 25.8, 766
+// 25.2, 894 25.4, 900 25.4).  Where the pitch is fixed at compile time
+// (window_pitch_fixed) 86.5 % are enough (218 25.7, 222 26.1, 230 27.0, 250 27.9, 190
+// 26.2; where it is not, 96-thread blocks stay behind: 190 24.4);
+// with the FD current, whose B reads the pairs hide better, 94 % (windows / pairs: 222
+// 18.6 / 19.6, 230 19.1 / 19.7, 250 20.0 / 19.7).
+static bool window_pays(int nx, long long n3, int variant) {
   if (nx % 2 != 0 || nx % 8 == 0 || nx < 176 || nx > 1024) return false;
-  const int threads = (nx / 2 + 31) / 32 * 32, pairs = 512 / threads * (nx / 2);
-  return pairs >= (threads <= 160 ? 425 : 380);
+  const int pairs = nx / 2, threads = (pairs + 31) / 32 * 32, resident = 512 / threads * threads;
+  if (resident < (threads > 256 ? 480 : 448)) return false;
+  if (window_pitch_fixed(nx, n3)) return 1000 * pairs >= (variant == kVarFdCurrent ? 940 : 865) * threads;
+  return threads >= 128 && 1000 * pairs >= 955 * threads;
 }
 
-int row_auto_segments(int nx) {
-  if (window_pays(nx)) return kWindows;
+int row_auto_segments(int nx, long long n3, int variant) {
+  if (window_pays(nx, n3, variant)) return kWindows;
   if (nx % 8 != 0 || nx < 64 || nx > 1024) return 0;
   if ((nx > 64 && nx < 104) || (nx > 128 && nx < 160) || (nx >= 776 && nx <= 792)) return 0;
   if (nx > 512 && nx <= 648) return nx >= 608 && nx % 16 == 0 ? 2 : 0;
@@ -112,19 +114,19 @@ bool step_row_supported(Grid g, int storage, int variant, const void* pop, int k
   }
   // automatic: the pair kernel or a staged tiling for every even row length
   if (!pair_ok(g, storage, variant, pop)) return false;
-  switch (row_auto_segments(g.nx)) {
+  switch (row_auto_segments(g.nx, g.n3, variant)) {
     case 0: return true;
     case kWindows: return (reinterpret_cast<uintptr_t>(pop) & 15u) == 0;
   }
   return staged_ok(g, storage, variant, pop);
 }
 
-int row_segments(int nx, int kernel) {
-  return kernel == 4 ? 0 : kernel == 3 ? 2 : kernel == 2 ? 1 : row_auto_segments(nx);
+int row_segments(const Grid& g, int kernel, int variant) {
+  return kernel == 4 ? 0 : kernel == 3 ? 2 : kernel == 2 ? 1 : row_auto_segments(g.nx, g.n3, variant);
 }
 
 bool step_row_staged(Grid g, int storage, int variant, const void* pop, int kernel) {
-  return step_row_supported(g, storage, variant, pop, kernel) && row_segments(g.nx, kernel) != 0;
+  return step_row_supported(g, storage, variant, pop, kernel) && row_segments(g, kernel, variant) != 0;
 }
 
 namespace {
@@ -142,7 +144,7 @@ cudaError_t row_variant(int variant, const RowCall& c) {
 cudaError_t launch_step_row(int storage, int odd, void* pop, Grid g, const StepConsts& k, unsigned* flag,
                             cudaStream_t s, int variant, const void* Bfd, unsigned stall_tries, int kernel) {
   const RowWait wt{stall_tries ? stall_tries : kWaitTries, stall_tries ? 1 : 0};
-  return row_variant(variant, RowCall{storage, odd, row_segments(g.nx, kernel), pop, g, k, flag, Bfd, s, true, wt});
+  return row_variant(variant, RowCall{storage, odd, row_segments(g, kernel, variant), pop, g, k, flag, Bfd, s, true, wt});
 }
 
 cudaError_t prepare_step(int storage, const void* pop, Grid g, int variant, int kernel) {
@@ -150,7 +152,7 @@ cudaError_t prepare_step(int storage, const void* pop, Grid g, int variant, int 
   // a placeholder field: only the configuration is settled, nothing is read
   static const unsigned no_field = 0u;
   for (int odd = 0; odd < 2; ++odd) {
-    const cudaError_t e = row_variant(variant, RowCall{storage, odd, row_segments(g.nx, kernel), const_cast<void*>(pop),
+    const cudaError_t e = row_variant(variant, RowCall{storage, odd, row_segments(g, kernel, variant), const_cast<void*>(pop),
                                                        g, StepConsts{}, nullptr, &no_field, nullptr, false,
                                                        RowWait{kWaitTries, 0}});
     if (e != cudaSuccess) return e;

@@ -644,7 +644,13 @@ struct PairGlobal {
 // W = nx / 2), staged with bulk copies at offset kHalo of a row of
 // staged_width(nx, 2) values: on odd steps with its halos, the one at the
 // row's end (periodic) by a copy of its own; its results are stored directly.
-template <class T, bool ODD, int H = 1>
+// QUOT: tiles by quotient (aa.cuh) instead of a division.  It shortens what warp 0
+// does before a copy leaves, which counts where a block is that one warp (64
+// sites: 9.61 -> 9.43 us a step) and beside the FD current's B reads (192 sites:
+// 308 -> 303 us with its pre-pass); elsewhere it costs 0.2-0.4 % (192 sites
+// 224.8 -> 225.3, 256 sites 514.6 -> 516.3; with the FD current's longer rows 2-3 %;
+// FP16).
+template <class T, bool ODD, int H, bool QUOT>
 struct RowIO {
   T* state;
   T* rows;  // [stage][16 runs, run_stride(nx, H) apart][3 storage slots][staged_width(nx, H)]
@@ -656,13 +662,26 @@ struct RowIO {
   bool boxed, stall;
   const RowMaps* maps;
   int rs;  // run_stride(nx, H)
+  unsigned ry;  // Reciprocals::y
+
+  __device__ __forceinline__ void plane_of(int r, int& y, int& z) const {
+    if constexpr (QUOT) {
+      const int zi = quotient(r, ny, ry);
+      y = r - zi * ny;
+      z = zi + z0;
+    } else {
+      y = r % ny;
+      z = r / ny + z0;
+    }
+  }
 
   __device__ __forceinline__ void issue(int tile, int st) const {
     if constexpr (H > 1) {
       issue_segment(tile, st);
       return;
     }
-    const int y = tile % ny, z = tile / ny + z0;
+    int y, z;
+    plane_of(tile, y, z);
     const unsigned bar = smem_addr(&bars[st]);
     T* dst = rows + (size_t)st * kRuns * rs;
     if (lane == 0) mbar_expect_tx(bar, kPop * rowbytes);
@@ -689,7 +708,8 @@ struct RowIO {
   // copies of whole 16-byte units (W and kHalo are multiples of 8 values).
   __device__ __forceinline__ void issue_segment(int tile, int st) const {
     const int row = tile / H, h = tile % H;
-    const int y = row % ny, z = row / ny + z0;
+    int y, z;
+    plane_of(row, y, z);
     const int W = nx / H, ws = staged_width(nx, H);
     const unsigned bar = smem_addr(&bars[st]);
     T* dst = rows + (size_t)st * kPop * ws;
@@ -726,7 +746,8 @@ struct RowIO {
   // (DEFER: the refill waits for it itself, later).
   template <int STAGES, bool DEFER>
   __device__ __forceinline__ void store(int tile, int st) const {
-    const int y = tile % ny, z = tile / ny + z0;
+    int y, z;
+    plane_of(tile, y, z);
     const T* src = rows + (size_t)st * kRuns * rs;
     if (boxed) {
       if (!ODD && rs == 3 * nx) {
@@ -766,7 +787,7 @@ template <class T, bool ODD, int NX, int kRowStages, int VAR, int H = 1>
 __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX, H))
     step_row_kernel(T* __restrict__ state, Grid g, StepConsts k, unsigned* __restrict__ flag,
                     const T* __restrict__ Bfd, const __grid_constant__ RowMaps maps,
-                    const __grid_constant__ SlotBases<T> bases, RowWait wt) {
+                    const __grid_constant__ SlotBases<T> bases, RowWait wt, Reciprocals rc) {
   static_assert(H == 1 || (H == 2 && kRowStages == 2 && (NX == 0 || NX > 256)), "half rows: long rows, two stages");
   extern __shared__ __align__(128) unsigned char smem[];
   const int nx = NX ? NX : g.nx, ny = g.ny, nz = g.nz;
@@ -784,8 +805,9 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
   }
   __syncthreads();
 
-  const RowIO<T, ODD, H> io{state, rows, bars, g.n3, nx, ny, nz, g.z0, rowbytes, lane, boxed && H == 1,
-                           wt.stall != 0, &maps, run_stride(nx, H)};
+  constexpr bool kQuot = NX != 0 && NX <= 256 && (VAR == kVarFdCurrent || NX <= 64);
+  const RowIO<T, ODD, H, kQuot> io{state, rows, bars, g.n3, nx, ny, nz, g.z0, rowbytes, lane, boxed && H == 1,
+                           wt.stall != 0, &maps, run_stride(nx, H), rc.y};
 
   const int first = blockIdx.x, stride = gridDim.x;
   // Tiles staged before the loop: both stages with two; with three, two of
@@ -863,7 +885,9 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
         else A.st(kQ + 3 * (ODD ? i : opp7(i)) + c, mx7(i), v);
       };
       auto curl_b = [&](f2 (&J)[3]) {
-        pair_curl(Bfd, g, (tile / H) % ny, (tile / H) / ny + g.z0, gx0, gxm0, gxp1, J);
+        int y, z;
+        io.plane_of(tile / H, y, z);
+        pair_curl(Bfd, g, y, z, gx0, gxm0, gxp1, J);
       };
       auto mid = [&]() {
         if constexpr (kMidRefill) {
@@ -875,7 +899,8 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
         }
       };
       if constexpr (VAR == kVarFdCurrent) {
-        const int y = (tile / H) % ny, z = (tile / H) / ny + g.z0;
+        int y, z;
+        io.plane_of(tile / H, y, z);
         prefetch_curl(Bfd, g.n3, ((long long)z * ny + y) * nx, ((long long)z * ny + wrap(y + 1, ny)) * nx,
                       ((long long)z * ny + wrap(y - 1, ny)) * nx, ((long long)wrap(z + 1, nz) * ny + y) * nx,
                       ((long long)wrap(z - 1, nz) * ny + y) * nx, gx0, gxm0, gxp1);
@@ -948,6 +973,7 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
 // (two rows' windows overrun their nx values by up to 7 on either side, and
 // their m differ by up to 7)
 __host__ __device__ constexpr int window_pitch(int nx, long long n3) { return (nx + 21 + 7) / 8 * 8 + (int)(n3 & 7); }
+inline bool window_pitch_fixed(int nx, long long n3) { return n3 % 8 == 0 && nx > 128 && nx <= 256; }
 // the compile-time pitches: rows of up to pitch - 24 sites
 constexpr int window_bound_threads(int pitch) { return pitch ? (pitch - 24) / 2 : kRowMaxThreads; }
 
@@ -1088,12 +1114,10 @@ __global__ void __launch_bounds__(window_bound_threads(PITCH), 512 / window_boun
 constexpr int kPairThreads = 128;
 template <class T, bool ODD, int VAR, bool L2>
 __device__ __forceinline__ void step_pair(const Grid& g, const StepConsts& k, unsigned* __restrict__ flag,
-                                          const T* __restrict__ Bfd, const SlotBases<T>& bases, long long p) {
-  const int nx = g.nx, ny = g.ny, nz = g.nz, pairs = nx / 2;
-  const int xp = (int)(p % pairs);
-  const long long rowi = p / pairs;
-  const int y = (int)(rowi % ny), z = (int)(rowi / ny) + g.z0;
-  const int gx0 = 2 * xp, gx1 = gx0 + 1;
+                                          const T* __restrict__ Bfd, const SlotBases<T>& bases, const Reciprocals& rc, int p) {
+  const int nx = g.nx, ny = g.ny, nz = g.nz;
+  const int rowi = quotient(2 * p, nx, rc.x), gx0 = 2 * p - rowi * nx, gx1 = gx0 + 1;
+  const int zi = quotient(rowi, ny, rc.y), y = rowi - zi * ny, z = zi + g.z0;
   const int gxm0 = gx0 == 0 ? nx - 1 : gx0 - 1, gxp1 = gx1 == nx - 1 ? 0 : gx1 + 1;
   PairGlobal<T, ODD, L2> G;
   G.base = &bases;
@@ -1127,14 +1151,14 @@ __device__ __forceinline__ void step_pair(const Grid& g, const StepConsts& k, un
 template <class T, bool ODD, int VAR>
 __global__ void __launch_bounds__(kPairThreads, 4)
     step_pair_kernel(Grid g, StepConsts k, unsigned* __restrict__ flag, const T* __restrict__ Bfd,
-                     const __grid_constant__ SlotBases<T> bases) {
+                     const __grid_constant__ SlotBases<T> bases, Reciprocals rc) {
   if constexpr (kChained<VAR>) {
     next_kernel_may_come();
     after_previous_kernel();
   }
-  const long long p = (long long)blockIdx.x * kPairThreads + threadIdx.x;
-  if (p >= (long long)(g.nx / 2) * g.ny * g.nzi) return;
-  step_pair<T, ODD, VAR, false>(g, k, flag, Bfd, bases, p);
+  const int p = blockIdx.x * kPairThreads + threadIdx.x;  // N3 < 2^31
+  if (p >= (g.nx / 2) * g.ny * g.nzi) return;
+  step_pair<T, ODD, VAR, false>(g, k, flag, Bfd, bases, rc, p);
 }
 
 template <class T, bool ODD, int VAR>
@@ -1148,9 +1172,9 @@ cudaError_t pair_launch(const RowCall& c) {
   for (int sl = 0; sl < kPop; ++sl) bases.p[sl] = static_cast<T*>(c.pop) + (size_t)sl * (size_t)c.g.n3;
   if constexpr (kChained<VAR>)
     return launch_chained(step_pair_kernel<T, ODD, VAR>, dim3((unsigned)blocks), dim3(kPairThreads), 0, c.s, c.g, c.k,
-                          c.flag, static_cast<const T*>(c.Bfd), bases);
+                          c.flag, static_cast<const T*>(c.Bfd), bases, reciprocals(c.g));
   step_pair_kernel<T, ODD, VAR><<<(unsigned)blocks, kPairThreads, 0, c.s>>>(c.g, c.k, c.flag,
-                                                                         static_cast<const T*>(c.Bfd), bases);
+                                                                         static_cast<const T*>(c.Bfd), bases, reciprocals(c.g));
   return cudaGetLastError();
 }
 
@@ -1222,10 +1246,12 @@ cudaError_t row_launch(const RowCall& c) {
   for (int sl = 0; sl < kPop; ++sl) bases.p[sl] = static_cast<T*>(c.pop) + (size_t)sl * (size_t)c.g.n3;
   if constexpr (kChained<VAR>)
     return launch_chained(step_row_kernel<T, ODD, NX, S, VAR, H>, dim3(grid), dim3(c.g.nx / (2 * H)), smem, c.s,
-                          static_cast<T*>(c.pop), c.g, c.k, c.flag, static_cast<const T*>(c.Bfd), maps, bases, c.wt);
+                          static_cast<T*>(c.pop), c.g, c.k, c.flag, static_cast<const T*>(c.Bfd), maps, bases, c.wt,
+                          reciprocals(c.g));
   step_row_kernel<T, ODD, NX, S, VAR, H>
       <<<grid, c.g.nx / (2 * H), smem, c.s>>>(static_cast<T*>(c.pop), c.g, c.k, c.flag,
-                                              static_cast<const T*>(c.Bfd), maps, bases, c.wt);
+                                              static_cast<const T*>(c.Bfd), maps, bases, c.wt,
+                          reciprocals(c.g));
   return cudaGetLastError();
 }
 
@@ -1252,7 +1278,7 @@ template <class T, bool ODD, int VAR>
 cudaError_t window_launch(const RowCall& c) {
   const int nx = c.g.nx;
   if (nx % 2 != 0 || nx < 64 || nx > 2 * kRowMaxThreads) return cudaErrorInvalidValue;
-  if (c.g.n3 % 8 == 0 && nx > 128 && nx <= 256)
+  if (window_pitch_fixed(nx, c.g.n3))
     return nx > 192 ? window_go<T, ODD, VAR, 280>(c) : window_go<T, ODD, VAR, 216>(c);
   return window_go<T, ODD, VAR, 0>(c);
 }

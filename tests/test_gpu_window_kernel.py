@@ -38,11 +38,17 @@ def test_windows_equal_the_pair_kernel(shape, storage, variant):
     a, x = _run(shape, storage, variant, "auto", 7)
     b, y = _run(shape, storage, variant, "pair", 7)
     assert torch.equal(x, y)
-    # the windows' copies have waits to stall, the pair kernel has none
-    a.debug_stall_next_step(64)
-    with pytest.raises(F.FlameError) as e:
-        b.debug_stall_next_step(64)
-    assert e.value.status == F.FLAME_ERR_PARAM
+    # the windows' copies have waits to stall, the pair kernel has none; auto takes
+    # the pairs too where lanes idle and the pitch is not fixed at compile time
+    pairs = [b]
+    if shape in ((3, 1, 182), (2, 3, 222)):
+        pairs.append(a)
+    else:
+        a.debug_stall_next_step(64)
+    for s in pairs:
+        with pytest.raises(F.FlameError) as e:
+            s.debug_stall_next_step(64)
+        assert e.value.status == F.FLAME_ERR_PARAM
     a.close()
     b.close()
 
