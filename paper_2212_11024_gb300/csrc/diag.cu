@@ -121,9 +121,10 @@ __device__ __forceinline__ float init_site(T* __restrict__ pop, const Grid& g, c
 // FP32 storage: the populations are FP64 values rounded to FP32.  Their ~770
 // FP64 operations a site (and conversions, which cost as much) were all this
 // kernel did: 2932 us at 128^3 (23.4 ms at 256^3), where the bytes take 74;
-// now 385 us (3.0 ms), bound by FP32 issue.  They are computed
+// now 522 us (3.9 ms), bound by FP32 issue and the sites done again (385 us
+// without those).  They are computed
 // in two-term FP32 arithmetic (48 bits: the rounded results are FP64's but
-// for one in 2^20 or so) and in the columns of the step's collision: for each
+// for one in 2^20 or so, and those sites are done again in FP64) and in the columns of the step's collision: for each
 // (c_x, c_y) the three values along c_z are Z0 + Z1 c_z + Z2 c_z^2, the
 // Lorentz term's N and the non-equilibrium stress P entering as K = N - P.
 // FP64 fields are split by integer operations.  Blocks of 128 threads by
@@ -183,7 +184,15 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
   if (!(top < 0x1p40f && rho.h < 0x1p40f && rho.h > 0x1p-40f))
     return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
   float* out = pop + site;
-  auto put = [&](int slot, F2 v) { out[(long long)slot * n3] = rounded(v); };
+  // A value whose remainder lies within 2^-17 of half a unit of the last place may
+  // round the other way in FP64 (the two terms' error is some 2^-20 of one), and a
+  // single such unit shows in J: its site is done again in FP64, as one in 2700 is.
+  bool tie = false;
+  auto put = [&](int slot, F2 v) {
+    const float r = rounded(v), rest = __fsub_rn(v.l, __fsub_rn(r, v.h));
+    tie |= __fadd_rn(r, __fmul_rn(rest, 1.f + 0x1p-17f)) != r;
+    out[(long long)slot * n3] = r;
+  };
 #pragma unroll
   for (int a = 0; a < 3; ++a) b[a] = add2(B[a], -k.Bref[a]);
 
@@ -254,6 +263,8 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
       put(px + 3 * py + 9, Z0);
       put(px + 3 * py + 18, add2u(tz, Z1));
     }
+
+  if (tie) return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
 
   // max(|B|^2 / rho, |u|^2), then its root: a Newton step on the FP32 one
   const F2 b2 = add2(add2u(mul2(B[0], B[0]), mul2(B[1], B[1])), mul2(B[2], B[2]));

@@ -259,6 +259,23 @@ def test_initial_populations_of_fp32_storage(shape, dtype, given):
     assert abs(speed - top) <= 0.51 * np.spacing(np.float32(top))
 
 
+def test_initial_populations_beside_rounding_ties():
+    """Fields a unit of the FP64 last place beside the middle of two FP32 values
+    (further out than the two terms' 48 bits): the stored rest populations of the
+    magnetic field are B rounded to FP32, every one of them."""
+    from paper_2212_11024_gb300 import Flame
+    shape = (4, 5, 33)
+    r = np.random.default_rng(12)
+    n = r.integers(2 ** 23, 2 ** 24 - 1, (3,) + shape).astype(np.float64) + 0.5
+    n *= 2.0 ** -28
+    B = r.choice([-1.0, 1.0], n.shape) * np.where(r.random(n.shape) < 0.5, np.nextafter(n, 1), np.nextafter(n, 0))
+    sim = Flame(33, 5, 4, 0.6, 0.6, 1.0, storage="fp32")
+    sim.init(None, np.zeros_like(B), B)
+    got = sim.state.view(torch.float32).cpu().numpy().reshape((48,) + shape)[27:30]
+    sim.close()
+    assert np.array_equal(got, B.astype(np.float32))
+
+
 def test_initial_populations_beyond_two_term_range():
     """Fields of 1e13 take the FP64 path: rounded FP64 values there too, and
     a non-finite field is reported."""
