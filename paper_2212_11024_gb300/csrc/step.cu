@@ -170,10 +170,15 @@ cudaError_t step_launch(int odd, const Slots<T>& P, Grid g, const StepConsts& k,
 }
 
 // Blocks and grid of the one-site kernels: flat blocks (true) where blocks of x
-// rows leave many lanes idle.
-bool step_shape(const Grid& g, dim3* b, dim3* gr) {
+// rows leave a tenth of the lanes idle, and with 16-bit storage wherever they
+// leave any, but for the BGK fluid, whose flat blocks spill (GLUPS FP16, ~4M sites,
+// row blocks / flat: 63 23.6 / 24.3, 159 22.8 / 24.4, 191 23.4 / 24.4, 255 23.7 / 24.2,
+// 287 20.0 / 24.3, 1023 23.9 / 24.5; electron MHD and the FD current alike; BGK
+// 191 23.4 / 22.4, 255 23.5 / 21.9).
+template <class T>
+bool step_shape(const Grid& g, int variant, dim3* b, dim3* gr) {
   const int padded = (g.nx + 31) / 32 * 32;
-  const bool flat = g.nx < padded && (double)g.nx / padded < 0.9;
+  const bool flat = g.nx < padded && ((sizeof(T) == 2 && variant != kVarBgkFluid) || (double)g.nx / padded < 0.9);
   *b = flat ? dim3(kStepThreads, 1, 1) : site_block(g, kStepThreads);
   *gr = flat ? dim3((unsigned)((g.n3i + kStepThreads - 1) / kStepThreads), 1, 1) : site_grid(g, *b);
   return flat;
@@ -182,7 +187,7 @@ bool step_shape(const Grid& g, dim3* b, dim3* gr) {
 template <class T>
 cudaError_t between_t(int odd, const void* from, void* to, Grid g, const StepConsts& k, unsigned* flag, cudaStream_t s) {
   dim3 b, gr;
-  const bool flat = step_shape(g, &b, &gr);
+  const bool flat = step_shape<T>(g, kVarFlame, &b, &gr);
   const Slots<T> P = make_slots<T>(from, g), O = make_slots<T>(to, g);
   auto go = [&](auto kern) { return launch_chained(kern, gr, b, 0, s, P, O, g, k, flag, reciprocals(g)); };
   if (flat) return odd ? go(step_between_kernel<T, true, true>) : go(step_between_kernel<T, false, true>);
@@ -193,7 +198,7 @@ template <class T>
 cudaError_t step_t(int odd, void* pop, Grid g, const StepConsts& k, unsigned* flag, int variant, void* Bfd,
                    cudaStream_t s) {
   dim3 b, gr;
-  const bool flat = step_shape(g, &b, &gr);
+  const bool flat = step_shape<T>(g, variant, &b, &gr);
   const Slots<T> P = make_slots<T>(pop, g);
   switch (variant) {
     case kVarFlame: return step_launch<T, kVarFlame>(odd, P, g, k, flag, nullptr, gr, b, flat, s);

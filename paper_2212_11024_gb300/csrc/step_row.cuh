@@ -965,10 +965,10 @@ __global__ void __launch_bounds__(row_bound_threads(NX, H), row_bound_blocks(NX,
 // compile time, and every warp issues its share of the copies; PITCH = 0
 // reads it from the grid, and warp 0 issues them (FP16, ~4M-site lattices,
 // GLUPS: 250 sites 28.1 against 26.7, 222 27.2 against 25.4; longer rows 28.0
-// by warp 0 against 27.3 shared out at 510).  The unstaged pair kernel runs
-// at 24.7-25.3 at all of these.  Tried at 250 sites and not kept: the results
-// in place and stored by 48 bulk copies and 32-bit stores of the rows' ends
-// (22.2), the windows by tensor-map boxes of [48][N3] (27.9).
+// by warp 0 against 27.3 shared out at 510).  The unstaged pair kernel
+// ran at 24.7-25.3 at all of these then, at 25.6-26.3 now.  Tried at 250 sites and
+// not kept: the results in place and stored by 48 bulk copies and 32-bit stores of
+// the rows' ends (22.2), the windows by tensor-map boxes of [48][N3] (27.9).
 //
 // (two rows' windows overrun their nx values by up to 7 on either side, and
 // their m differ by up to 7)
