@@ -121,16 +121,16 @@ __device__ __forceinline__ float init_site(T* __restrict__ pop, const Grid& g, c
 // FP32 storage: the populations are FP64 values rounded to FP32.  Their ~770
 // FP64 operations a site (and conversions, which cost as much) were all this
 // kernel did: 2932 us at 128^3 (23.4 ms at 256^3), where the bytes take 74;
-// now 522 us (3.9 ms), bound by FP32 issue and the sites done again (385 us
-// without those).  They are computed
-// in two-term FP32 arithmetic (48 bits: the rounded results are FP64's but
-// for one in 2^20 or so, and those sites are done again in FP64) and in the columns of the step's collision: for each
+// now 476 us at 128^3, bound by FP32 issue and the sites done again (385 us
+// without those).  They are computed in two-term FP32 arithmetic (48 bits: the
+// rounded results are FP64's but for one in 2^20 or so, and the sites of those
+// are done again in FP64) and in the columns of the step's collision: for each
 // (c_x, c_y) the three values along c_z are Z0 + Z1 c_z + Z2 c_z^2, the
 // Lorentz term's N and the non-equilibrium stress P entering as K = N - P.
 // FP64 fields are split by integer operations.  Blocks of 128 threads by
-// registers: 168 (three per SM) 551 us, 128 (four) 462, 96 (five) 411, 80
-// (six, some of the field values reloaded) 385.  Sites with values outside
-// [2^-40, 2^40] (density) or 2^40 (fields) take the FP64 path.
+// registers, before sites were done again: 168 (three per SM) 551 us, 128 (four)
+// 462, 96 (five) 411, 80 (six, some of the field values reloaded) 385.  Sites with
+// values outside [2^-40, 2^40] (density) or 2^40 (fields) take the FP64 path.
 struct InitConsts {
   F2 p;    // -1 / (3 omega), or 0 without the non-equilibrium parts
   F2 iwB;  // 1 / omega_B, or 0
@@ -184,13 +184,14 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
   if (!(top < 0x1p40f && rho.h < 0x1p40f && rho.h > 0x1p-40f))
     return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
   float* out = pop + site;
-  // A value whose remainder lies within 2^-17 of half a unit of the last place may
+  // A value whose remainder lies within 2^-18 of half a unit of the last place may
   // round the other way in FP64 (the two terms' error is some 2^-20 of one), and a
-  // single such unit shows in J: its site is done again in FP64, as one in 2700 is.
+  // single such unit shows in J: its site is done again in FP64, as one in 5500 is (476 us
+  // at 128^3; within 2^-17, 522 us with the same outputs).
   bool tie = false;
   auto put = [&](int slot, F2 v) {
     const float r = rounded(v), rest = __fsub_rn(v.l, __fsub_rn(r, v.h));
-    tie |= __fadd_rn(r, __fmul_rn(rest, 1.f + 0x1p-17f)) != r;
+    tie |= __fadd_rn(r, __fmul_rn(rest, 1.f + 0x1p-18f)) != r;
     out[(long long)slot * n3] = r;
   };
 #pragma unroll

@@ -14,12 +14,13 @@ namespace {
 // at most 80 registers per thread (3 resident blocks per SM); the block
 // shape and register budget were chosen by timing at 256^3.  Where nx is
 // not a multiple of 32 a block of x rows leaves lanes idle (33 sites: 64
-// threads); where that is 10 % or more of them the blocks cover consecutive
-// sites instead (flat; a separate instantiation, so the row blocks keep
-// their registers).  GLUPS on ~8M-site lattices, FP32 / FP16 row blocks ->
+// threads); where that is 10 % or more of them, and more often with 16-bit
+// storage (step_shape), the blocks cover consecutive sites instead (flat; a
+// separate instantiation, so the row blocks keep their registers).  GLUPS on ~8M-site lattices, FP32 / FP16 row blocks ->
 // flat: 33 12.2 -> 15.6 / 13.5 -> 22.4, 65 14.1 -> 15.4 / 16.8 -> 22.4, 100
-// 14.8 -> 15.6 / 20.1 -> 22.6; flat runs at ~15.7 FP32 at any length, row
-// blocks with little waste stay ahead (250: 16.3, 255: 16.4, 256: 17.3).
+// 14.8 -> 15.6 / 20.1 -> 22.6 (24.0-24.5 since the sites are numbered without
+// divisions); flat runs at ~15.7 FP32 at any length, row blocks with little
+// waste stay ahead (250: 16.3, 255: 16.4, 256: 17.3).
 constexpr int kStepThreads = 256;
 constexpr int kStepMinBlocks = 3;
 
