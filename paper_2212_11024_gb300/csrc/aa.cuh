@@ -22,6 +22,28 @@ __device__ __forceinline__ int quotient(int p, int d, unsigned r) {
   return p - q * d >= d ? q + 1 : q;
 }
 
+// A load past L1 of what another SM may have written since this thread last read
+// the place, in a kernel whose blocks wait for one another.  volatile and "memory":
+// the compiler neither takes an earlier load's value for this one nor moves it
+// across the wait (the built-in load of a 16-bit value promises neither).
+template <class T>
+__device__ __forceinline__ T load_l2(const T* p) {
+  if constexpr (sizeof(T) == 2) {
+    unsigned short v;
+    asm volatile("ld.global.cg.b16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return *reinterpret_cast<const T*>(&v);
+  } else if constexpr (sizeof(T) == 4) {
+    unsigned v;
+    asm volatile("ld.global.cg.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return *reinterpret_cast<const T*>(&v);
+  } else {
+    static_assert(sizeof(T) == 8, "16, 32 or 64 bits");
+    unsigned long long v;
+    asm volatile("ld.global.cg.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return *reinterpret_cast<const T*>(&v);
+  }
+}
+
 // Site-index offsets of the periodic neighbours.
 struct Nbr {
   int xm, xp, ym, yp, zm, zp;

@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(kSumThreads)
   }
   __syncthreads();
   if (!last) return;
-  double t = threadIdx.x < gridDim.x ? __ldcg(stage + threadIdx.x) : 0.0;
+  double t = threadIdx.x < gridDim.x ? load_l2(stage + threadIdx.x) : 0.0;
   t = sum_of_block(t);
   if (threadIdx.x == 0) {
     *out = t;

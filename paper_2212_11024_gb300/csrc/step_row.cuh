@@ -598,12 +598,12 @@ struct SlotBases {
 template <class T, bool ODD, bool L2 = false>
 struct PairGlobal {
   static __device__ __forceinline__ float one(const T* p) {
-    if constexpr (L2) return Codec<T>::dec(__ldcg(p));
+    if constexpr (L2) return Codec<T>::dec(load_l2(p));
     else return Codec<T>::dec(*p);
   }
   static __device__ __forceinline__ f2 two(const T* p) {
     if constexpr (L2) {
-      const unsigned w = __ldcg(reinterpret_cast<const unsigned*>(p));
+      const unsigned w = load_l2(reinterpret_cast<const unsigned*>(p));
       return Codec2<T>::dec(reinterpret_cast<const T*>(&w));
     } else {
       return Codec2<T>::dec(p);

@@ -39,7 +39,7 @@ namespace {
 // L2 reads the populations past L1, for a kernel that takes several steps.
 template <bool L2, class T>
 __device__ __forceinline__ T load_pop(const T* p) {
-  if constexpr (L2) return __ldcg(p);
+  if constexpr (L2) return load_l2(p);
   else return *p;
 }
 
