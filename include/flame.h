@@ -116,7 +116,12 @@ typedef struct {
                          half rows (nx > 256 a multiple of 16), 4: unstaged pairs (nx
                          even), where they apply, else the one-site kernel.  All compute the same step in FP32; results
                          agree to FP32 rounding before encoding (the row kernel's tilings
-                         agree bit for bit). */
+                         agree bit for bit).  With 0, 1 and 4 a flame_step of several steps
+                         of a lattice of at most as many sites (or site pairs, where single
+                         steps take pairs or staged rows) as threads are resident at once
+                         is one launch of the one-site or the unstaged pair body (not
+                         with FLAME_FD_CURRENT, in graphs or under capture); 2 and 3 keep
+                         to the staged rows they name. */
     int halo_z;       /* 0: a periodic nx x ny x nz lattice.  1: one z-slab of a larger
                          periodic lattice split along z (the one-direction domain split
                          of Sec. 4): the state holds the slab's nz planes between two
@@ -302,8 +307,9 @@ flame_status flame_reduce_sums(flame_ctx *ctx, double *h_sums);
  * site count. */
 int flame_reduce_combine(const flame_params *p, const double *h_sums, double *h_scalars);
 
-/* The step kernel flame_step launches for these parameters (with a state
- * allocated as flame_create requires): FLAME_KERNEL_SITE (one site per
+/* The step kernel flame_step launches for one step at these parameters (with a
+ * state allocated as flame_create requires; several steps of a small lattice in
+ * one launch: flame_params.kernel): FLAME_KERNEL_SITE (one site per
  * thread), FLAME_KERNEL_ROWS (x rows staged in shared memory, two sites per
  * thread), FLAME_KERNEL_HALF_ROWS (half rows staged) or FLAME_KERNEL_PAIRS
  * (site pairs of rows of any even length: unstaged, or, by the library's

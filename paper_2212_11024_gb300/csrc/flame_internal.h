@@ -68,7 +68,7 @@ cudaError_t launch_step_between(int storage, int odd, const void* from, void* to
 // pairs, where the packed kernels apply) are at most the threads resident at
 // once; the same populations as n launches of launch_step.  sync: two zeroed
 // words that the launch leaves zeroed.  *taken: whether the lattice is small
-// enough (n = 0 only asks); not for kVarFdCurrent.
+// enough (n = 0 only asks); not for kVarFdCurrent, and not where staged rows are forced.
 struct MultiCall {
   int storage, odd;
   void* pop;

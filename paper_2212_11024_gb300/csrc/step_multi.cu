@@ -10,7 +10,9 @@
 // flame_step(10), single launches -> one launch: FP32 16^3 6.15 -> 3.1, 32^3
 // 6.16 -> 3.7, 40^3 7.2 -> 5.3; FP16 32^3 6.16 -> 4.1, 48^3 8.2 -> 6.1, 52^3 9.2 ->
 // 7.5.  512 threads per SM bound the lattices that take this (77,824 sites or
-// pairs): with 768, FP32 48^3 ran at 8.5 against 8.2.
+// pairs): with 768, FP32 48^3 ran at 8.5 against 8.2.  Lattices of the automatic
+// choice take their pairs here whatever tiling single steps have (the same bits);
+// a forced tiling (flame_params.kernel 2 and 3) is kept, a launch per step.
 #include "step_row.cuh"
 #include "step_site.cuh"
 
@@ -171,6 +173,8 @@ cudaError_t launch_steps(const MultiCall& c, bool* taken) {
   *taken = false;
   if (c.variant == kVarFdCurrent) return cudaSuccess;  // its pre-pass is a step's second phase
   const bool pairs = step_row_supported(c.g, c.storage, c.variant, c.pop, c.kernel);
+  // the caller asked for staged rows, which have no several-step form
+  if (pairs && (c.kernel == 2 || c.kernel == 3)) return cudaSuccess;
   switch (c.storage) {
     case 1: return multi_variant<float>(c, pairs, taken);
     case 2: return multi_variant<__half>(c, pairs, taken);
