@@ -141,17 +141,17 @@ __device__ __forceinline__ F2 from_double(double x) {
 
 // h + l as FP64, |l| <= ulp(h) / 2, rounded to nearest: the 53-bit result is
 // assembled from h's bits and l as an integer in units of its last place, so
-// that no FP64 instruction is issued.  Values of h outside [2^-75, 2^127]
+// that no FP64 instruction is issued.  Values of h outside [2^-74, 2^127]
 // take FP64 instructions.
 __device__ __forceinline__ double to_double(F2 a) {
   const unsigned hb = __float_as_uint(a.h), mag = hb & 0x7fffffffu, e = mag >> 23;
   if (mag == 0u) return (double)a.l;
-  if (e < 52u || e > 253u) return (double)a.h + (double)a.l;
-  // l in units of 2^(exponent(h) - 52), signed like h
-  const float unit = __uint_as_float((306u - e) << 23);
-  int n = __float2int_rn(__uint_as_float(__float_as_uint(a.l) ^ (hb & 0x80000000u)) * unit);
-  // below a power of two the last place is half as large
-  if ((mag & 0x007fffffu) == 0u && n < 0) n *= 2;
+  if (e < 53u || e > 253u) return (double)a.h + (double)a.l;
+  // l, signed like h, in units of the last place 2^(exponent(h) - 52), which is
+  // half as large below a power of two
+  const unsigned lb = __float_as_uint(a.l) ^ (hb & 0x80000000u);
+  const bool below = (mag & 0x007fffffu) == 0u && (lb >> 31) != 0u;
+  const int n = __float2int_rn(__uint_as_float(lb) * __uint_as_float(((below ? 307u : 306u) - e) << 23));
   const long long bits = ((long long)mag << 29) + (896ll << 52) + n;
   return __longlong_as_double(bits | ((long long)(hb >> 31) << 63));
 }
