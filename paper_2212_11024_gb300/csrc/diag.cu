@@ -445,55 +445,32 @@ struct SiteMoments64 {
   __device__ __forceinline__ double B(const StepConsts&, int a) const { return B_[a]; }
 };
 
-// The sums of an expansion type: F3 for FP64 results, F2 (unnormalised, 48
-// bits) where the results are summed over sites.
-template <class E>
-struct Sums;
-template <>
-struct Sums<F3> {
-  template <class A, class B>
-  static __device__ __forceinline__ F3 add(A a, B b) {
-    return add3(a, b);
-  }
-};
-template <>
-struct Sums<F2> {
-  template <class B>
-  static __device__ __forceinline__ F2 add(F2 a, B b) {
-    return add2u(a, b);
-  }
-};
-
 // 216 sum_i w_i s_i and 216 sum_i w_i c_ia s_i from the populations in
 // velocity-cube order.
-template <class E>
-__device__ __forceinline__ void fluid_sums(const float (&s)[kQ], E& r216, E (&j216)[3]) {
-  using S = Sums<E>;
-  E M00[3], M10[3], M01[3];
+__device__ __forceinline__ void fluid_sums(const float (&s)[kQ], F3& r216, F3 (&j216)[3]) {
+  F3 M00[3], M10[3], M01[3];
 #pragma unroll
   for (int pz = 0; pz < 3; ++pz) {
-    E m0[3];
+    F3 m0[3];
     F2 m1[3];
 #pragma unroll
     for (int py = 0; py < 3; ++py) {
       const int q = 3 * (py + 3 * pz);
-      m0[py] = S::add(two_sum(s[q + 2], s[q]), 4.f * s[q + 1]);
+      m0[py] = add3(two_sum(s[q + 2], s[q]), 4.f * s[q + 1]);
       m1[py] = two_diff(s[q + 2], s[q]);
     }
-    M00[pz] = S::add(S::add(m0[2], m0[0]), scaled(4.f, m0[1]));
-    M01[pz] = S::add(m0[2], -m0[0]);
-    M10[pz] = S::add(S::add(m1[2], m1[0]), scaled(4.f, m1[1]));
+    M00[pz] = add3(add3(m0[2], m0[0]), scaled(4.f, m0[1]));
+    M01[pz] = add3(m0[2], -m0[0]);
+    M10[pz] = add3(add3(m1[2], m1[0]), scaled(4.f, m1[1]));
   }
-  r216 = S::add(S::add(M00[2], M00[0]), scaled(4.f, M00[1]));
-  j216[0] = S::add(S::add(M10[2], M10[0]), scaled(4.f, M10[1]));
-  j216[1] = S::add(S::add(M01[2], M01[0]), scaled(4.f, M01[1]));
-  j216[2] = S::add(M00[2], -M00[0]);
+  r216 = add3(add3(M00[2], M00[0]), scaled(4.f, M00[1]));
+  j216[0] = add3(add3(M10[2], M10[0]), scaled(4.f, M10[1]));
+  j216[1] = add3(add3(M01[2], M01[0]), scaled(4.f, M01[1]));
+  j216[2] = add3(M00[2], -M00[0]);
 }
 
 // 8 dB and 8 Lambda_ab of the magnetic populations.
-template <class E>
-__device__ __forceinline__ void magnetic_sums(const float (&sg)[3][kM], E (&sB)[3], F2 (&d)[3][3]) {
-  using S = Sums<E>;
+__device__ __forceinline__ void magnetic_sums(const float (&sg)[3][kM], F3 (&sB)[3], F2 (&d)[3][3]) {
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
     F2 f[3];
@@ -502,7 +479,7 @@ __device__ __forceinline__ void magnetic_sums(const float (&sg)[3][kM], E (&sB)[
       f[a] = two_sum(sg[b][2 * a + 1], sg[b][2 * a + 2]);
       d[a][b] = two_diff(sg[b][2 * a + 1], sg[b][2 * a + 2]);
     }
-    sB[b] = S::add(S::add(S::add(f[0], f[1]), f[2]), 2.f * sg[b][0]);
+    sB[b] = add3(add3(add3(f[0], f[1]), f[2]), 2.f * sg[b][0]);
   }
 }
 
@@ -544,6 +521,13 @@ __device__ __noinline__ void general_moments(const float* pop, int site, Nbr nb,
   }
 }
 
+// U of 216 rho u and 216 rho.
+__device__ __forceinline__ void velocity64(double rho216, const F3 (&j216)[3], double (&U)[3]) {
+  const double ir = reciprocal(rho216);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) U[a] = quotient(to_double(j216[a]), rho216, ir);
+}
+
 template <bool ODD, class O, bool FLUID, bool CUR>
 __global__ void __launch_bounds__(128, 8)
     moments64_kernel(const float* __restrict__ pop, Grid g, StepConsts k, Consts64 d, MomentsOut<O> out) {
@@ -580,10 +564,9 @@ __global__ void __launch_bounds__(128, 8)
 #pragma unroll
     for (int b = 0; b < 3; ++b) m.B_[b] = d.Bref[b] + to_double(scaled(0.125f, sB[b]));
     if constexpr (FLUID) {
-      const double r = to_double(r216), rho216 = d.rho0x216 + r, ir = reciprocal(rho216);
+      const double r = to_double(r216);
       m.rho_ = fma(r, 1.0 / 216.0, d.rho0);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) m.U[a] = quotient(to_double(j216[a]), rho216, ir);
+      velocity64(d.rho0x216 + r, j216, m.U);
     }
     if constexpr (CUR) {
       const double* B = m.B_;
@@ -682,15 +665,25 @@ cudaError_t probe_t(int odd, const void* pop, Grid g, const StepConsts& k, int n
 //   15 sum ((omega_B/C^2) Tr Lambda)^2, 16 non-finite sites.
 //
 // Every site's terms in FP64 (16 additions and as many conversions; for FP32
-// storage the moments too) bound this kernel by the FP64 pipe.  A thread's
-// sums are two-term FP32 expansions instead: TwoSum is exact, so a sum keeps
-// 48 bits and its error stays below that of the terms, which come from FP32
-// arithmetic (16-bit storage) or from two-term arithmetic (FP32 storage:
-// 2^-46 a site, which averages out over the sites of a sum).  A block that
-// meets a value too large for this, or a non-finite one, sums its sites
-// again in FP64 (reduce_general).  flame_reduce, us, FP64 sums -> expansions:
-// FP32 storage 128^3 1353 -> 158, 256^3 9767 -> 871 (3.2 GB of state, 475 at
-// the HBM rate); FP16 128^3 317 -> 96, 256^3 1435 -> 523 (1.6 GB, 238).
+// storage the moments too) bound this kernel by the FP64 pipe.  What is a sum
+// or product of FP32 values runs in three-term FP32 expansions instead (72
+// bits, more than FP64 holds, for 13 to 22 FP32 operations an addition): the
+// sums of 16-bit storage, whose terms come from FP32 arithmetic, and for FP32
+// storage the sums over the populations and, over the sites, of density,
+// momentum and field.  What is left in FP64 there, the quotients, squares and
+// the sums of those, takes 50 operations a site.  A block that meets a value
+// too large for this, or a non-finite one, sums its sites again in FP64
+// (reduce_general).
+//
+// A thread's sums become FP64 numbers in shared memory, and a warp sums each
+// quantity of the block from there: 13 FP64 additions a warp and quantity,
+// against 40 by shuffles in every warp.
+//
+// flame_reduce_static, us at 64^3, 128^3, 256^3: FP32 storage 73, 336, 2380 (all in
+// FP64 1353 at 128^3, 9767 at 256^3; the moments in two-term FP32 arithmetic took
+// 140 and 855, but held 48 bits), FP16 36, 83, 532 (317 and 1435 with FP64 sums; 41,
+// 82, 506 with two-term ones).  Blocks per SM, two / three: FP32 341 / 336 at 128^3
+// and 2466 / 2380, FP16, whose three spill, 83 / 91 and 532 / 514.
 
 // The FP64 sums of a thread's sites.
 template <class T, bool ODD>
@@ -730,203 +723,168 @@ __device__ __noinline__ void reduce_general(const T* pop, Grid g, StepConsts k, 
   }
 }
 
-// A thread's sums: those of the layout above that are sums, in its order
-// (15 after 13), of terms whose scale `Terms::scale` takes out again.
-constexpr int kRedSums = 15;
 constexpr float kRedLimit = 0x1p100f;  // largest term the expansions take
 
-// One site's terms added to acc; returns the largest magnitude among them
-// (NaN for a non-finite site).  uu_max: the running maximum of |u|^2.
+// A thread's sums of the quantities above over its sites, but for 14, the
+// maximum of |u|^2, and 16, the number of sites.  add: one site's terms; the
+// largest magnitude among them, or NaN for a non-finite site.  finish: the
+// block's quantity v from the block's sums r of value().
 template <class T>
 struct Terms {
-  // rho - rho0, (rho - rho0) u, B - Bref, ...: FP32 per site
-  static __device__ __forceinline__ double scale(int) { return 1.0; }
-  static __device__ __forceinline__ double momentum(const StepConsts& k, double drho_u, double u) {
-    return (double)k.rho0 * u + drho_u;
-  }
-  double uu_max = 0.0;
-  float uu_f = 0.f;
+  // of rho - rho0, (rho - rho0) u, B - Bref, ...: FP32 per site
+  F3 lin[7], u[3], uu, bb, ub, jj, vv;
+  float top;
+  int n;
   template <bool ODD>
   __device__ __forceinline__ float add(const T* __restrict__ pop, int site, const Nbr& nb, const Grid& g,
-                                       const StepConsts& k, F2 (&acc)[kRedSums], int*) {
+                                       const StepConsts& k, const Consts64&) {
     float sf[kQ], sg[3][kM];
     load_site<T, ODD>(pop, site, nb, g.n3, sf, sg);
     const SiteMoments<float> m = site_moments(sf, sg, k);
     const float* b = m.dB;
-    const float uu = m.U[0] * m.U[0] + m.U[1] * m.U[1] + m.U[2] * m.U[2];
-    const float bb = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-    const float jj = m.J[0] * m.J[0] + m.J[1] * m.J[1] + m.J[2] * m.J[2];
+    const float u2 = m.U[0] * m.U[0] + m.U[1] * m.U[1] + m.U[2] * m.U[2];
+    const float b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+    const float j2 = m.J[0] * m.J[0] + m.J[1] * m.J[1] + m.J[2] * m.J[2];
     const float dv = 4.f * k.omegaB * m.trlam;
-    acc[0] = add2(acc[0], m.drho);
+    lin[0] = add3(lin[0], m.drho);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      acc[1 + a] = add2(acc[1 + a], mul2(m.drho, m.U[a]));
-      acc[4 + a] = add2(acc[4 + a], b[a]);
-      acc[10 + a] = add2(acc[10 + a], m.U[a]);
+      lin[1 + a] = add3(lin[1 + a], mul2(m.drho, m.U[a]));
+      lin[4 + a] = add3(lin[4 + a], b[a]);
+      u[a] = add3(u[a], m.U[a]);
     }
-    acc[7] = add2(acc[7], uu);
-    acc[8] = add2(acc[8], bb);
-    acc[9] = add2(acc[9], m.U[0] * b[0] + m.U[1] * b[1] + m.U[2] * b[2]);
-    acc[13] = add2(acc[13], jj);
-    acc[14] = add2(acc[14], dv * dv);
-    uu_f = fmaxf(uu_f, uu);
-    return fabsf(m.drho) * (1.f + uu) + uu + bb + jj + dv * dv + fabsf(b[0]) + fabsf(b[1]) + fabsf(b[2]);
+    uu = add3(uu, u2);
+    bb = add3(bb, b2);
+    ub = add3(ub, m.U[0] * b[0] + m.U[1] * b[1] + m.U[2] * b[2]);
+    jj = add3(jj, j2);
+    vv = add3(vv, dv * dv);
+    top = fmaxf(top, u2);
+    ++n;
+    return fabsf(m.drho) * (1.f + u2) + u2 + b2 + j2 + dv * dv + fabsf(b[0]) + fabsf(b[1]) + fabsf(b[2]);
   }
-  __device__ __forceinline__ double max_speed2() const { return (double)uu_f; }
+  __device__ __forceinline__ double value(int v) const {
+    return v < 7 ? to_double(lin[v]) : v == 7 ? to_double(uu) : v == 8 ? to_double(bb) : v == 9 ? to_double(ub)
+         : v < 13 ? to_double(u[v - 10]) : v == 13 ? to_double(jj) : v == 14 ? (double)top
+         : v == 15 ? to_double(vv) : (double)n;
+  }
+  static __device__ __forceinline__ double finish(const double* r, int v, const StepConsts& k, const Consts64&) {
+    if (v == 0) return fma(r[16], (double)k.rho0, r[0]);
+    if (v < 4) return fma((double)k.rho0, r[9 + v], r[v]);
+    if (v < 7) return fma(r[16], (double)k.Bref[v - 4], r[v]);
+    return v == 14 ? sqrt(r[14]) : v == 16 ? 0.0 : r[v];
+  }
 };
 
-// FP32 storage: two-term arithmetic per site on 216 (rho - rho0), 216 rho u
-// and 8 (B - Bref); u, B - Bref, J and the divergence estimate are scaled by
-// 2^40 before they are squared, which keeps the products' second terms of
-// fields down to 1e-27 in FP32's range.
+// FP32 storage: the sums of 216 (rho - rho0), 216 rho u and 8 (B - Bref), which
+// are sums of populations, as expansions; the others in FP64, constant factors
+// left to finish.  The current's system J + s J x B = y keeps y's part along B and
+// divides the square of the other by 1 + s^2 |B|^2, so that |J|^2 (1 + s^2 |B|^2)
+// = |y|^2 + s^2 (y.B)^2: no need of J itself.  y = 2 gq (U x B - A / 2).
 template <>
 struct Terms<float> {
-  static __device__ __forceinline__ double scale(int v) {
-    return v < 4 ? 1.0 / 216.0 : v < 7 ? 0.125 : (v >= 10 && v < 13) ? 0x1p-40 : 0x1p-80;
-  }
-  static __device__ __forceinline__ double momentum(const StepConsts&, double j, double) { return j; }
-  double uu_max = 0.0;
+  F3 lin[7];
+  double u[3], uu, bb, ub, jj, vv;  // jj: |y / (2 gq)|^2 ..., vv: (8 Tr Lambda)^2
+  long long top;                    // the bits of max |u|^2, which order as the values do
+  int n;
   template <bool ODD>
   __device__ __forceinline__ float add(const float* __restrict__ pop, int site, const Nbr& nb, const Grid& g,
-                                       const StepConsts& k, F2 (&acc)[kRedSums], int* bound) {
-    constexpr float kS = 0x1p40f;
+                                       const StepConsts& k, const Consts64& d) {
     float s[kQ], sg[3][kM];
     load_cube<ODD>(pop, site, nb, g.n3, s);
     load_magnetic<ODD>(pop, site, nb, g.n3, sg);
-    F2 r216, j216[3], sB[3], d[3][3];
+    F3 r216, j216[3], sB[3], A8[3];
+    F2 lam8[3][3];
     fluid_sums(s, r216, j216);
-    magnetic_sums(sg, sB, d);
-    const F2 rho216 = add2(mul2(216.f, k.rho0), r216);
-    const float ir = 1.f / rho216.h;
-    acc[0] = add2(acc[0], r216);
-    F2 U[3], B[3], b[3], y[3];
+    double U[3], b[3], B[3], y[3];
+    velocity64(to_double(add3(r216, mul2(216.f, k.rho0))), j216, U);
+    magnetic_sums(sg, sB, lam8);
+    const F3 tr8 = add3(add3(lam8[0][0], lam8[1][1]), lam8[2][2]);
+    float big = fabsf(r216.h) + fabsf(r216.l) + fabsf(tr8.h) + fabsf(tr8.l);
+    lin[0] = add3(lin[0], r216);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      acc[1 + a] = add2(acc[1 + a], j216[a]);
-      acc[4 + a] = add2(acc[4 + a], sB[a]);
-      U[a] = div2(fast_two_sum(j216[a].h, j216[a].l), rho216, ir);
-      b[a] = scaled(0.125f, fast_two_sum(sB[a].h, sB[a].l));
-      B[a] = add2(b[a], k.Bref[a]);
+      A8[a] = add3(lam8[(a + 1) % 3][(a + 2) % 3], -lam8[(a + 2) % 3][(a + 1) % 3]);
+      big += fabsf(j216[a].h) + fabsf(j216[a].l) + fabsf(sB[a].h) + fabsf(sB[a].l) + fabsf(A8[a].h) + fabsf(A8[a].l);
+      lin[1 + a] = add3(lin[1 + a], j216[a]);
+      lin[4 + a] = add3(lin[4 + a], sB[a]);
+      const F3 db = scaled(0.125f, sB[a]);
+      b[a] = to_double(db);
+      B[a] = to_double(add3(db, k.Bref[a]));
     }
-    // y = gq (2 U x B - A), J = (y - s y x B + s^2 (y.B) B) / (1 + s^2 |B|^2)
-    const float gq = 4.f * k.omegaB;
-    const F2 sH = mul2(2.f * k.alphaH, gq), ss = mul2(sH, sH);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const int p = (a + 1) % 3, q = (a + 2) % 3;
-      const F2 uxb = add2u(mul2(U[p], B[q]), -mul2(U[q], B[p]));
-      y[a] = mul2(gq, add2(scaled(2.f, uxb), scaled(-0.125f, add2u(d[p][q], -d[q][p]))));
-    }
-    const F2 b2 = add2u(add2u(mul2(B[0], B[0]), mul2(B[1], B[1])), mul2(B[2], B[2]));
-    const F2 yb = add2u(add2u(mul2(y[0], B[0]), mul2(y[1], B[1])), mul2(y[2], B[2]));
-    const F2 den = add2(mul2(ss, b2), 1.f), t = mul2(ss, yb);
-    const float iden = 1.f / den.h;
-    F2 uu{0.f, 0.f}, bb{0.f, 0.f}, ub{0.f, 0.f}, jj{0.f, 0.f};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const int p = (a + 1) % 3, q = (a + 2) % 3;
-      const F2 yxb = add2u(mul2(y[p], B[q]), -mul2(y[q], B[p]));
-      const F2 num = add2(add2u(y[a], -mul2(sH, yxb)), mul2(t, B[a]));
-      const F2 Js = scaled(kS, div2(num, den, iden)), Us = scaled(kS, U[a]), bs = scaled(kS, b[a]);
-      acc[10 + a] = add2(acc[10 + a], Us);
-      uu = add2u(uu, mul2(Us, Us));
-      bb = add2u(bb, mul2(bs, bs));
-      ub = add2u(ub, mul2(Us, bs));
-      jj = add2u(jj, mul2(Js, Js));
+      y[a] = fma(U[p], B[q], fma(-U[q], B[p], to_double(scaled(-0.0625f, A8[a]))));
+      u[a] += U[a];
+      bb = fma(b[a], b[a], bb);
+      ub = fma(U[a], b[a], ub);
     }
-    const F2 dv = scaled(kS, mul2(0.5f * k.omegaB, add2(add2u(d[0][0], d[1][1]), d[2][2])));
-    const F2 vv = mul2(dv, dv);
-    acc[7] = add2(acc[7], uu);
-    acc[8] = add2(acc[8], bb);
-    acc[9] = add2(acc[9], ub);
-    acc[13] = add2(acc[13], jj);
-    acc[14] = add2(acc[14], vv);
-    // max |u|^2 in FP64, taken only where the two-term value comes near the
-    // block's largest so far (a shared lower bound)
-    const float near = uu.h * (1.f + 0x1p-20f);
-    if (near > __int_as_float(*(volatile int*)bound)) {
-      const double r = fma(216.0, (double)k.rho0, to_double(fast_two_sum(r216.h, r216.l))), q = 1.0 / r;
-      double u[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) u[a] = quotient(to_double(fast_two_sum(j216[a].h, j216[a].l)), r, q);
-      uu_max = fmax(uu_max, u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-      if (isfinite(uu.h)) atomicMax(bound, __float_as_int(uu.h * (1.f - 0x1p-20f)));
-    }
-    return fabsf(r216.h) + uu.h + bb.h + jj.h + vv.h + fabsf(sB[0].h) + fabsf(sB[1].h) + fabsf(sB[2].h) +
-           fabsf(j216[0].h) + fabsf(j216[1].h) + fabsf(j216[2].h) + fabsf(r216.l + sB[0].l + sB[1].l + sB[2].l);
+    const double u2 = dot64(U, U), yB = dot64(y, B), dv = to_double(tr8);
+    const double j2 = fma(d.ss * yB, yB, dot64(y, y));
+    uu += u2;
+    jj = fma(j2, reciprocal(fma(d.ss, dot64(B, B), 1.0)), jj);
+    vv = fma(dv, dv, vv);
+    const long long bits = __double_as_longlong(u2);
+    top = bits > top ? bits : top;
+    ++n;
+    // not finite: a density of zero
+    return finite64(u2) && finite64(j2) ? big : __uint_as_float(0x7fc00000u);
   }
-  __device__ __forceinline__ double max_speed2() const { return uu_max; }
+  static __device__ __forceinline__ double dot64(const double (&a)[3], const double (&b)[3]) {
+    return fma(a[2], b[2], fma(a[1], b[1], a[0] * b[0]));
+  }
+  static __device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+  __device__ __forceinline__ double value(int v) const {
+    return v < 7 ? to_double(lin[v]) : v == 7 ? uu : v == 8 ? bb : v == 9 ? ub : v < 13 ? u[v - 10] : v == 13 ? jj
+         : v == 14 ? __longlong_as_double(top) : v == 15 ? vv : (double)n;
+  }
+  static __device__ __forceinline__ double finish(const double* r, int v, const StepConsts& k, const Consts64& d) {
+    if (v == 0) return fma(r[16], (double)k.rho0, r[0] / 216.0);
+    if (v < 4) return r[v] / 216.0;
+    if (v < 7) return fma(r[16], (double)k.Bref[v - 4], 0.125 * r[v]);
+    if (v == 13) return d.gq2 * d.gq2 * r[13];
+    if (v == 15) return d.gq8 * d.gq8 * r[15];
+    return v == 14 ? sqrt(r[14]) : v == 16 ? 0.0 : r[v];
+  }
 };
 
 constexpr int kRedThreads = 256;
 template <class T, bool ODD>
-__global__ void __launch_bounds__(kRedThreads, sizeof(T) == 4 ? 2 : 3)
-    reduce_kernel(const T* __restrict__ pop, Grid g, StepConsts k, double* __restrict__ partials) {
-  __shared__ double sh[kRedThreads / 32][kRedVals];
-  __shared__ int bound;
-  if (threadIdx.x == 0) bound = 0;
-  __syncthreads();
-  F2 acc[kRedSums];
-#pragma unroll
-  for (int v = 0; v < kRedSums; ++v) acc[v] = F2{0.f, 0.f};
-  Terms<T> terms;
-  int n = 0;
+__global__ void __launch_bounds__(kRedThreads, sizeof(T) == 4 ? 3 : 2)
+    reduce_kernel(const T* __restrict__ pop, Grid g, StepConsts k, Consts64 d, double* __restrict__ partials) {
+  __shared__ double sh[kRedVals][kRedThreads], total[kRedVals];
+  Terms<T> terms{};
   bool fits = true;
   const int off = g.z0 * g.nx * g.ny;
   for (long long s = (long long)blockIdx.x * kRedThreads + threadIdx.x; s < g.n3i; s += (long long)gridDim.x * kRedThreads) {
     const int site = (int)s + off;
     const int row = site / g.nx, x = site - row * g.nx, z = row / g.ny, y = row - z * g.ny;
-    const float big = terms.template add<ODD>(pop, site, make_nbr(x, y, z, g), g, k, acc, &bound);
-    fits = fits && big < kRedLimit;
-    ++n;
+    fits = fits && terms.template add<ODD>(pop, site, make_nbr(x, y, z, g), g, k, d) < kRedLimit;
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (__syncthreads_or(!fits)) {
-    double a64[kRedVals];
-    reduce_general<T, ODD>(pop, g, k, a64);
-    for (int v = 0; v < kRedVals; ++v) {
-      double a = a64[v];
-      for (int o = 16; o > 0; o >>= 1) {
-        const double t = __shfl_down_sync(0xffffffffu, a, o);
-        a = (v == 14) ? fmax(a, t) : a + t;
-      }
-      if (lane == 0) sh[warp][v] = a;
-    }
+  const bool general = __syncthreads_or(!fits);
+  if (general) {
+    double a[kRedVals];
+    reduce_general<T, ODD>(pop, g, k, a);
+    for (int v = 0; v < kRedVals; ++v) sh[v][threadIdx.x] = a[v];
   } else {
-    const double sites = (double)__reduce_add_sync(0xffffffffu, n);
-    double sum[kRedSums];
 #pragma unroll
-    for (int v = 0; v < kRedSums; ++v) {
-      F2 a = acc[v];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        a = add2(a, F2{__shfl_down_sync(0xffffffffu, a.h, o), __shfl_down_sync(0xffffffffu, a.l, o)});
-      sum[v] = lane == 0 ? Terms<T>::scale(v) * ((double)a.h + (double)a.l) : 0.0;
-    }
-    double top = terms.max_speed2();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_down_sync(0xffffffffu, top, o));
-    if (lane == 0) {
-      sh[warp][0] = sites * (double)k.rho0 + sum[0];
-      for (int a = 0; a < 3; ++a) {
-        sh[warp][1 + a] = Terms<T>::momentum(k, sum[1 + a], sum[10 + a]);
-        sh[warp][4 + a] = sites * (double)k.Bref[a] + sum[4 + a];
-        sh[warp][10 + a] = sum[10 + a];
-      }
-      for (int v = 7; v < 10; ++v) sh[warp][v] = sum[v];
-      sh[warp][13] = sum[13];
-      sh[warp][14] = sqrt(top);
-      sh[warp][15] = sum[14];
-      sh[warp][16] = 0.0;
-    }
+    for (int v = 0; v < kRedVals; ++v) sh[v][threadIdx.x] = terms.value(v);
   }
   __syncthreads();
-  if (threadIdx.x < kRedVals) {
-    const int v = threadIdx.x;
-    double a = sh[0][v];
-    for (int w = 1; w < kRedThreads / 32; ++w) a = (v == 14) ? fmax(a, sh[w][v]) : a + sh[w][v];
-    partials[(long long)blockIdx.x * kRedVals + v] = a;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int v = warp; v < kRedVals; v += kRedThreads / 32) {
+    double a = sh[v][lane];
+    for (int i = lane + 32; i < kRedThreads; i += 32) a = v == 14 ? fmax(a, sh[v][i]) : a + sh[v][i];
+    for (int o = 16; o > 0; o >>= 1) {
+      const double t = __shfl_down_sync(0xffffffffu, a, o);
+      a = v == 14 ? fmax(a, t) : a + t;
+    }
+    if (lane == 0) total[v] = a;
   }
+  __syncthreads();
+  if (threadIdx.x < kRedVals)
+    partials[(long long)blockIdx.x * kRedVals + threadIdx.x] =
+        general ? total[threadIdx.x] : Terms<T>::finish(total, threadIdx.x, k, d);
 }
 
 __global__ void reduce_final_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
@@ -1017,9 +975,9 @@ template <class T>
 cudaError_t reduce_t(int odd, const void* pop, Grid g, const StepConsts& k, int nblocks, double* partials,
                      double* out, cudaStream_t s) {
   if (odd)
-    reduce_kernel<T, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const T*>(pop), g, k, partials);
+    reduce_kernel<T, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const T*>(pop), g, k, Consts64(k), partials);
   else
-    reduce_kernel<T, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const T*>(pop), g, k, partials);
+    reduce_kernel<T, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const T*>(pop), g, k, Consts64(k), partials);
   reduce_final_kernel<<<1, 32 * kRedVals, 0, s>>>(partials, nblocks, out);
   return cudaGetLastError();
 }
@@ -1075,16 +1033,16 @@ cudaError_t launch_reduce_partials(int storage, int odd, const void* pop, Grid g
   if (nblocks < 1) return cudaErrorInvalidValue;
   switch (storage) {
     case 1:
-      if (odd) reduce_kernel<float, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const float*>(pop), g, k, partials);
-      else reduce_kernel<float, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const float*>(pop), g, k, partials);
+      if (odd) reduce_kernel<float, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const float*>(pop), g, k, Consts64(k), partials);
+      else reduce_kernel<float, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const float*>(pop), g, k, Consts64(k), partials);
       break;
     case 2:
-      if (odd) reduce_kernel<__half, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __half*>(pop), g, k, partials);
-      else reduce_kernel<__half, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __half*>(pop), g, k, partials);
+      if (odd) reduce_kernel<__half, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __half*>(pop), g, k, Consts64(k), partials);
+      else reduce_kernel<__half, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __half*>(pop), g, k, Consts64(k), partials);
       break;
     case 3:
-      if (odd) reduce_kernel<__nv_bfloat16, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __nv_bfloat16*>(pop), g, k, partials);
-      else reduce_kernel<__nv_bfloat16, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __nv_bfloat16*>(pop), g, k, partials);
+      if (odd) reduce_kernel<__nv_bfloat16, true><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __nv_bfloat16*>(pop), g, k, Consts64(k), partials);
+      else reduce_kernel<__nv_bfloat16, false><<<nblocks, kRedThreads, 0, s>>>(static_cast<const __nv_bfloat16*>(pop), g, k, Consts64(k), partials);
       break;
     default:
       return cudaErrorInvalidValue;

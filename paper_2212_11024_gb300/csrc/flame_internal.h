@@ -162,10 +162,10 @@ constexpr int kRedVals = 17;
 // kRedBlocksMax * kRedVals doubles of scratch).
 constexpr int kRedBlocksMax = 1024;
 // The reduction's block count over n sites on nsm SMs, `most` at most: as
-// many blocks as are resident (two per SM for FP32 storage, three for
+// many blocks as are resident (three per SM for FP32 storage, two for
 // 16-bit), so that one wave takes all sites.
 inline int reduce_block_count(int storage, int nsm, long long n, int most) {
-  long long want = (long long)nsm * (storage == 1 ? 2 : 3);
+  long long want = (long long)nsm * (storage == 1 ? 3 : 2);
   const long long per = (n + 255) / 256;
   if (want > per) want = per;
   if (want > most) want = most;
