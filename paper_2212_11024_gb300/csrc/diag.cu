@@ -120,30 +120,56 @@ __device__ __forceinline__ float init_site(T* __restrict__ pop, const Grid& g, c
 
 // FP32 storage: the populations are FP64 values rounded to FP32.  Their ~770
 // FP64 operations a site (and conversions, which cost as much) were all this
-// kernel did: 2932 us at 128^3 (23.4 ms at 256^3), where the bytes take 74;
-// now 476 us at 128^3, bound by FP32 issue and the sites done again (385 us
-// without those).  They are computed in two-term FP32 arithmetic (48 bits: the
-// rounded results are FP64's but for one in 2^20 or so, and the sites of those
-// are done again in FP64) and in the columns of the step's collision: for each
-// (c_x, c_y) the three values along c_z are Z0 + Z1 c_z + Z2 c_z^2, the
-// Lorentz term's N and the non-equilibrium stress P entering as K = N - P.
-// FP64 fields are split by integer operations.  Blocks of 128 threads by
-// registers, before sites were done again: 168 (three per SM) 551 us, 128 (four)
-// 462, 96 (five) 411, 80 (six, some of the field values reloaded) 385.  Sites with
-// values outside [2^-40, 2^40] (density) or 2^40 (fields) take the FP64 path.
+// kernel did: 2932 us at 128^3 (23.4 ms at 256^3), where the bytes take 74.
+// They are computed in two-term FP32 arithmetic (48 bits) and in the columns of
+// the step's collision: for each (c_x, c_y) the three values along c_z are
+// Z0 + Z1 c_z + Z2 c_z^2, the Lorentz term's N and the non-equilibrium stress P
+// entering as K = N - P.  Differences of the fields and of the reference state
+// are taken in FP64, as FP64 would (22 operations a site: the fields' own 48 bits
+// would leave less of a small deviation), and split by integer operations.
+//
+// A value whose rounding the two terms cannot tell (put_rounded) is stored as
+// FP64 gives it: its site is done again there.  So are sites with values outside
+// [2^-40, 2^40] (density) or of 2^40 and more (fields).
+//
+// 128^3 453 us, 256^3 3.3 ms (FP32 fields 330 us and 2.2 ms), bound by FP32 issue
+// and the sites done again, one in 1000 to 2000: 321 us without them.  Five blocks
+// of 128 threads per SM instead of six, whose 80 registers reload some field
+// values: 5 % slower.
 struct InitConsts {
   F2 p;    // -1 / (3 omega), or 0 without the non-equilibrium parts
   F2 iwB;  // 1 / omega_B, or 0
 };
 
-__device__ __forceinline__ F2 field2(const double* f, long long i) { return from_double(f[i]); }
-__device__ __forceinline__ F2 field2(const float* f, long long i) { return {f[i], 0.f}; }
-__device__ __forceinline__ float rounded(F2 a) { return __fadd_rn(a.h, a.l); }
+__device__ __forceinline__ F2 field2(double f) { return from_double(f); }
+__device__ __forceinline__ F2 field2(float f) { return {f, 0.f}; }
+// f - g, rounded to FP64 or exactly
+__device__ __forceinline__ F2 diff2(double f, double g) { return from_double(f - g); }
+__device__ __forceinline__ F2 diff2(float f, float g) { return two_diff(f, g); }
+__device__ __forceinline__ float diff1(double f, double g) { return (float)(f - g); }
+__device__ __forceinline__ float diff1(float f, float g) { return __fsub_rn(f, g); }
 
 template <class F>
 __device__ __noinline__ float init_site_fp64(float* pop, Grid g, StepConsts k, int noneq, const F* rho_f, const F* u,
                                              const F* Bf, const F* gu, const F* gB, int x, int y, int z) {
   return init_site<float, double, F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+}
+
+// The error of a sum of two-term values whose terms' magnitudes add up to m: 2^-46
+// m, and what underflow takes of some tens of products; none where there is no
+// term.  Against 113-bit arithmetic (random fields of 1e-9 to 0.3 on mean fields of
+// 0 and 0.1, with and without given gradients, 24M values) the error is 2^-45 m at
+// most and so seldom above 2^-46 m that 3e-10 values a site round to another FP32
+// number than FP64's exact result would, where FP64 arithmetic itself rounds 1e-6
+// to 4e-6 a site the other way.
+__device__ __forceinline__ float error2(float m) { return fminf(__fmaf_rn(0x1p-46f, m, 0x1p-143f), m); }
+
+// Stores v, which is off by at most e, rounded to FP32; true where e leaves open
+// which of two values that is.
+__device__ __forceinline__ bool put_rounded(float* out, F2 v, float e) {
+  const float r = __fadd_rn(v.h, v.l), rest = __fsub_rn(v.l, __fsub_rn(r, v.h));
+  *out = r;
+  return __fadd_rn(r, __fadd_rn(rest, copysignf(e, rest))) != r;
 }
 
 template <class F>
@@ -157,16 +183,19 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
   const int fwd[3] = {nb.xp, nb.yp, nb.zp}, back[3] = {nb.xm, nb.ym, nb.zm};
   // d_a F_b
   auto grad = [&](const F* f, const F* gf, int a, int b) -> F2 {
-    if (gf) return field2(gf + (3 * a + b) * n3, site);
-    return scaled(0.5f, add2(field2(f + b * n3, site + fwd[a]), -field2(f + b * n3, site + back[a])));
+    if (gf) return field2(gf[(3 * a + b) * n3 + site]);
+    return scaled(0.5f, diff2(f[b * n3 + site + fwd[a]], f[b * n3 + site + back[a]]));
   };
-  const F2 rho = rho_f ? field2(rho_f, site) : F2{1.f, 0.f};
+  const F rho_v = rho_f ? rho_f[site] : (F)1;
+  const F2 rho = field2(rho_v), drho = diff2(rho_v, (F)k.rho0);
   F2 U[3], B[3], b[3], dB[9], S[6];
-  float top = 0.f;
+  float mS[6], top = 0.f;  // mS: the magnitudes of the terms of S
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    U[a] = field2(u + a * n3, site);
-    B[a] = field2(Bf + a * n3, site);
+    const F Bv = Bf[a * n3 + site];
+    U[a] = field2(u[a * n3 + site]);
+    B[a] = field2(Bv);
+    b[a] = diff2(Bv, (F)k.Bref[a]);
     top = fmaxf(top, fmaxf(fabsf(U[a].h), fabsf(B[a].h)));
     if (isnan(U[a].h) || isnan(B[a].h)) top = __uint_as_float(0x7f800000u);
   }
@@ -178,62 +207,65 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
   constexpr int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};  // xx yy zz xy xz yz
 #pragma unroll
   for (int i = 0; i < 6; ++i) {  // d_a u_b + d_b u_a
-    S[i] = i < 3 ? scaled(2.f, grad(u, gu, i, i)) : add2(grad(u, gu, ia[i], ib[i]), grad(u, gu, ib[i], ia[i]));
-    top = isnan(S[i].h) ? __uint_as_float(0x7f800000u) : fmaxf(top, fabsf(S[i].h));
+    const F2 s = grad(u, gu, ia[i], ib[i]), t = i < 3 ? s : grad(u, gu, ib[i], ia[i]);
+    S[i] = i < 3 ? scaled(2.f, s) : add2(s, t);
+    mS[i] = fabsf(s.h) + fabsf(t.h);
+    top = isnan(mS[i]) ? __uint_as_float(0x7f800000u) : fmaxf(top, mS[i]);
   }
   if (!(top < 0x1p40f && rho.h < 0x1p40f && rho.h > 0x1p-40f))
     return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
   float* out = pop + site;
-  // A value whose remainder lies within 2^-18 of half a unit of the last place may
-  // round the other way in FP64 (the two terms' error is some 2^-20 of one), and a
-  // single such unit shows in J: its site is done again in FP64, as one in 5500 is (476 us
-  // at 128^3; within 2^-17, 522 us with the same outputs).
-  bool tie = false;
-  auto put = [&](int slot, F2 v) {
-    const float r = rounded(v), rest = __fsub_rn(v.l, __fsub_rn(r, v.h));
-    tie |= __fadd_rn(r, __fmul_rn(rest, 1.f + 0x1p-18f)) != r;
-    out[(long long)slot * n3] = r;
-  };
-#pragma unroll
-  for (int a = 0; a < 3; ++a) b[a] = add2(B[a], -k.Bref[a]);
+  bool open = false;
+  auto put = [&](int slot, F2 v, float e) { open |= put_rounded(out + (long long)slot * n3, v, e); };
 
   // magnetic: b_b + sign (4 (V_a B_b - B_a V_b) - d_a B_b / omega_B), V = U - d_i curl B
   {
     F2 V[3];
+    float mV[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const int p = (a + 1) % 3, q = (a + 2) % 3;
       V[a] = add2(U[a], mul2(-k.alphaH, add2(dB[3 * p + q], -dB[3 * q + p])));
+      mV[a] = fmaf(k.alphaH, fabsf(dB[3 * p + q].h) + fabsf(dB[3 * q + p].h), fabsf(U[a].h));
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      put(kQ + c, b[c]);
+      const float mb = fabsf(b[c].h);
+      out[(long long)(kQ + c) * n3] = diff1(Bf[c * n3 + site], (F)k.Bref[c]);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const F2 ne = -mul2(ic.iwB, dB[3 * a + c]);
         const F2 t = a == c ? ne : add2u(scaled(4.f, add2(mul2(V[a], B[c]), -mul2(B[a], V[c]))), ne);
-        put(kQ + 3 * (2 * a + 1) + c, add2u(b[c], t));
-        put(kQ + 3 * (2 * a + 2) + c, add2u(b[c], -t));
+        const float m = fmaf(ic.iwB.h, fabsf(dB[3 * a + c].h), mb);
+        const float e = error2(a == c ? m : fmaf(4.f, fmaf(mV[a], fabsf(B[c].h), fabsf(B[a].h) * mV[c]), m));
+        put(kQ + 3 * (2 * a + 1) + c, add2u(b[c], t), e);
+        put(kQ + 3 * (2 * a + 2) + c, add2u(b[c], -t), e);
       }
     }
   }
 
-  // fluid
+  // fluid; mL: the magnitudes of all terms but those of the equilibrium's velocity part
   F2 K[6], miso{0.f, 0.f};
+  float mK[6], mI = 0.f;
   const F2 rp = mul2(rho, ic.p);
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     const int a = ia[i], c = ib[i];
     const F2 N = add2u(mul2(b[c], B[a]), mul2(k.Bref[c], b[a]));
     K[i] = add2(N, -mul2(rp, S[i]));
+    mK[i] = fmaf(fabsf(rp.h), mS[i], fmaf(fabsf(b[c].h), fabsf(B[a].h), fabsf(k.Bref[c]) * fabsf(b[a].h)));
   }
 #pragma unroll
-  for (int a = 0; a < 3; ++a) miso = add2u(miso, scaled(0.5f, mul2(b[a], add2(B[a], k.Bref[a]))));
-  const F2 drho = add2(rho, -k.rho0);
+  for (int a = 0; a < 3; ++a) {
+    miso = add2u(miso, scaled(0.5f, mul2(b[a], add2(B[a], k.Bref[a]))));
+    mI = fmaf(fabsf(b[a].h), fabsf(B[a].h) + fabsf(k.Bref[a]), mI);
+  }
   const F2 base0 = add2(drho, add2(mul2(1.5f, add2(add2u(K[0], K[1]), K[2])), mul2(-4.5f, miso)));
   const F2 LA = mul2(4.5f, add2(miso, -K[0])), LB = mul2(4.5f, add2(miso, -K[1])), LZ = mul2(4.5f, add2(miso, -K[2]));
   const F2 LC = mul2(9.f, K[3]), NX = mul2(-9.f, K[4]), NY = mul2(-9.f, K[5]);
+  const float mL = fmaf(9.f, mI + ((mK[3] + mK[4]) + mK[5]), fmaf(6.f, (mK[0] + mK[1]) + mK[2], fabsf(drho.h)));
   F2 ex[3], ey[3];
+  float mx[2], my[2];  // of ex, ey at c = 0 and +-1
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     F2* e = h ? ey : ex;
@@ -241,9 +273,20 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
     e[0] = add2(q, -u3);
     e[1] = mul2(-1.5f, uu);
     e[2] = add2(q, u3);
+    float* m = h ? my : mx;
+    m[0] = 1.5f * uu.h;
+    m[1] = q.h + fabsf(u3.h);
   }
   const F2 uzz = mul2(U[2], U[2]);
   const F2 e0z = mul2(-1.5f, uzz), e1z = mul2(3.f, U[2]), e2z = mul2(4.5f, uzz);
+  float eZ[2][2], e0[2][2];  // the errors at c_z = +-1 and 0 by |c_x|, |c_y|
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float mr = rho.h * fmaf(mx[i & 1], my[i >> 1], mx[i & 1] + my[i >> 1]), mg = mr + rho.h;
+    const float m0 = fmaf(mg, 1.5f * uzz.h, mr + mL);
+    e0[i >> 1][i & 1] = error2(m0);
+    eZ[i >> 1][i & 1] = error2(fmaf(mg, e2z.h + fabsf(e1z.h), m0));
+  }
 #pragma unroll
   for (int py = 0; py < 3; ++py)
 #pragma unroll
@@ -260,12 +303,13 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
       if (cx) Z1 = add2u(Z1, cx > 0 ? NX : -NX);
       if (cy) Z1 = add2u(Z1, cy > 0 ? NY : -NY);
       const F2 tz = add2u(Z0, add2u(mul2(gg, e2z), LZ));
-      put(px + 3 * py, add2u(tz, -Z1));
-      put(px + 3 * py + 9, Z0);
-      put(px + 3 * py + 18, add2u(tz, Z1));
+      const float ez = eZ[cy != 0][cx != 0];
+      put(px + 3 * py, add2u(tz, -Z1), ez);
+      put(px + 3 * py + 9, Z0, e0[cy != 0][cx != 0]);
+      put(px + 3 * py + 18, add2u(tz, Z1), ez);
     }
 
-  if (tie) return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+  if (open) return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
 
   // max(|B|^2 / rho, |u|^2), then its root: a Newton step on the FP32 one
   const F2 b2 = add2(add2u(mul2(B[0], B[0]), mul2(B[1], B[1])), mul2(B[2], B[2]));
