@@ -130,7 +130,7 @@ __device__ __forceinline__ float init_site(T* __restrict__ pop, const Grid& g, c
 //
 // A value whose rounding the two terms cannot tell (put_rounded) is stored as
 // FP64 gives it: its site is done again there.  So are sites with values outside
-// [2^-40, 2^40] (density) or of 2^40 and more (fields).
+// [2^-10, 2^10] (density) or of 2^40 and more (fields).
 //
 // 128^3 453 us, 256^3 3.3 ms (FP32 fields 330 us and 2.2 ms), bound by FP32 issue
 // and the sites done again, one in 1000 to 2000: 321 us without them.  Five blocks
@@ -199,6 +199,7 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
     top = fmaxf(top, fmaxf(fabsf(U[a].h), fabsf(B[a].h)));
     if (isnan(U[a].h) || isnan(B[a].h)) top = __uint_as_float(0x7f800000u);
   }
+  const float top_ub = top;
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     dB[i] = grad(Bf, gB, i / 3, i % 3);
@@ -212,7 +213,7 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
     mS[i] = fabsf(s.h) + fabsf(t.h);
     top = isnan(mS[i]) ? __uint_as_float(0x7f800000u) : fmaxf(top, mS[i]);
   }
-  if (!(top < 0x1p40f && rho.h < 0x1p40f && rho.h > 0x1p-40f))
+  if (!(top < 0x1p40f && rho.h < 0x1p10f && rho.h > 0x1p-10f))
     return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
   float* out = pop + site;
   bool open = false;
@@ -311,13 +312,20 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
 
   if (open) return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
 
-  // max(|B|^2 / rho, |u|^2), then its root: a Newton step on the FP32 one
+  // max(|B|^2 / rho, |u|^2), then its root: a Newton step on the FP32 one.  Small
+  // fields are scaled, so that their squares stay in range
+  const float sc = top_ub < 0x1p-50f ? 0x1p80f : 1.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    U[a] = scaled(sc, U[a]);
+    B[a] = scaled(sc, B[a]);
+  }
   const F2 b2 = add2(add2u(mul2(B[0], B[0]), mul2(B[1], B[1])), mul2(B[2], B[2]));
   const F2 u2 = add2(add2u(mul2(U[0], U[0]), mul2(U[1], U[1])), mul2(U[2], U[2]));
   const F2 va = div2(b2, rho, 1.f / rho.h);
   const F2 s2 = va.h > u2.h || (va.h == u2.h && va.l > u2.l) ? va : u2;
   const float r = sqrtf(s2.h);
-  return r > 0x1p-40f ? r + __fadd_rn(__fmaf_rn(-r, r, s2.h), s2.l) / (2.f * r) : r;
+  return (r > 0.f ? r + __fadd_rn(__fmaf_rn(-r, r, s2.h), s2.l) / (2.f * r) : r) / sc;
 }
 
 template <class T, class R, class F>

@@ -1,5 +1,6 @@
 """The initial populations of FP32 storage hold what FP64 holds of them where FP32
-pairs would not: small deviations from a mean field, values left by cancellation."""
+pairs would not: small deviations from a mean field, values left by cancellation;
+and the speed of fields whose squares FP32 lacks."""
 import numpy as np
 import pytest
 
@@ -94,3 +95,17 @@ def test_values_left_by_cancellation():
     tol = 0.5 * np.spacing(np.abs(ref).astype(np.float32)).astype(LD) + 3 * EPS * mag
     off = (np.abs(got - ref) / tol)[27:]
     assert (off <= 1).all(), (float(off.max()), int((off > 1).sum()))
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("amp", [1e-15, 1e-21, 1e-30, 1e-37])
+def test_speed_of_tiny_fields(amp, dtype):
+    """max(|u|, |B|) rounded to FP32 (half a unit of it, and two-term arithmetic)."""
+    r = np.random.default_rng(33)
+    shape = (3, 4, 33)
+    for ku, kB in ((1.0, 0.5), (0.5, 1.0)):
+        u = (ku * amp * r.standard_normal((3,) + shape)).astype(dtype)
+        B = (kB * amp * r.standard_normal((3,) + shape)).astype(dtype)
+        _, speed = _init(u, B, (0.0, 0.0, 0.0), 0.625, 1.5)
+        top = max(np.sqrt((f.astype(LD) ** 2).sum(0)).max() for f in (u, B))
+        assert abs(LD(speed) - top) <= 0.51 * np.spacing(np.float32(top))
