@@ -498,7 +498,9 @@ flame_status flame_reduce_static(flame_ctx *ctx, int nblocks, double *d_scalars)
  * listed at flame_params.kernel), FLAME_ERR_STATE (before flame_init). */
 flame_status flame_debug_stall_next_step(flame_ctx *ctx, unsigned tries);
 
-/* Release the context and its internal workspace (not the caller's state). */
+/* Release the context and its internal workspace (not the caller's state).
+ * FFT plans with a work area of at most 8 MB outlive it, for the next context of
+ * the same lattice on the device: at most 8 of them in the process. */
 void flame_destroy(flame_ctx *ctx);
 
 /* Human-readable text of a status code (static storage). */

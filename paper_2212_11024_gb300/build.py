@@ -18,7 +18,7 @@ LIB = os.path.join(BUILD, "libflame.so")
 SOURCES = ["step.cu", "step_multi.cu", "step_row.cu", "step_row_bgk.cu", "step_row_emhd.cu", "step_row_fd.cu", "diag.cu",
            "adjoint.cu", "api.cu", "reduce_static.cu", "spectral.cu", "plans.cu"]
 HEADERS = ["lattice.cuh", "aa.cuh", "expansion.cuh", "reduce_final.cuh", "pdl.cuh", "step_row.cuh", "step_site.cuh",
-           "flame_internal.h", "plans.h"]
+           "flame_internal.h", "idle_list.h", "plans.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -5,15 +5,19 @@
 // 5.6 on them.  A context takes its plans from a pool and gives them back when
 // it is destroyed; between the two they are its own, and the stream is set
 // before each use.  The pool is bounded: it keeps at most kMostPlans idle plans
-// without a work area of more than kMostWork bytes and destroys the oldest
-// beyond that.  A plan belongs to one driver context of one device (a device
-// that was reset gets a new one) and is given out in that context only.
+// without a work area of more than kMostWork bytes.  A plan belongs to one driver
+// context of one device (a device that was reset gets a new one): it is given out
+// in that context only, and destroyed only by a call in that context, beyond the
+// bound the oldest of the context's own, or the plan that comes where all those
+// kept are others' (IdleList).  Plans of a context that is gone went with it; what
+// is left of them in the list is a few words each.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cufft.h>
 
 #include <mutex>
 
+#include "idle_list.h"
 #include "plans.h"
 
 namespace flame {
@@ -45,9 +49,7 @@ bool context_id(unsigned long long* id) {
 
 struct Pool {
   std::mutex mu;
-  Key key[kMostPlans];
-  cufftHandle plan[kMostPlans];
-  int n = 0;
+  IdleList<Key, cufftHandle, kMostPlans> idle;
 };
 // never destroyed: contexts may be released during the process's exit, after
 // static objects are gone
@@ -65,20 +67,12 @@ cufftResult plan_take(const Grid& g, cufftType type, FftPlan* f) {
   f->pooled = cudaGetDevice(&f->device) == cudaSuccess && context_id(&f->ctx);
   cufftResult r = CUFFT_SUCCESS;
   if (f->pooled) {
-    const Key k = key_of(*f, g);
     Pool& p = pool();
     std::lock_guard<std::mutex> lock(p.mu);
-    for (int i = p.n - 1; i >= 0; --i)
-      if (p.key[i] == k) {
-        f->handle = p.plan[i];
-        f->live = true;
-        --p.n;
-        for (int j = i; j < p.n; ++j) {
-          p.key[j] = p.key[j + 1];
-          p.plan[j] = p.plan[j + 1];
-        }
-        return r;
-      }
+    if (p.idle.take(key_of(*f, g), &f->handle)) {
+      f->live = true;
+      return r;
+    }
   }
   r = cufftPlan3d(&f->handle, g.nz, g.ny, g.nx, type);
   f->live = r == CUFFT_SUCCESS;
@@ -98,18 +92,7 @@ void plan_give(const Grid& g, FftPlan* f) {
   bool drop = false;
   {
     std::lock_guard<std::mutex> lock(p.mu);
-    if (p.n == kMostPlans) {
-      // the oldest; one of a driver context that is gone went with it
-      drop = p.key[0].ctx == f->ctx;
-      old = p.plan[0];
-      --p.n;
-      for (int j = 0; j < p.n; ++j) {
-        p.key[j] = p.key[j + 1];
-        p.plan[j] = p.plan[j + 1];
-      }
-    }
-    p.key[p.n] = key_of(*f, g);
-    p.plan[p.n++] = f->handle;
+    drop = p.idle.give(key_of(*f, g), f->handle, &old);
   }
   if (drop) cufftDestroy(old);
 }
