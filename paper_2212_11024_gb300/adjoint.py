@@ -71,6 +71,9 @@ class _Run:
         other = torch.empty_like(lam)
         # dL/d(d_i) of every step, and of the initialisation in the last place
         ddi = torch.zeros(self.nsteps + 1, dtype=torch.float64, device=dev)
+        ubar = torch.empty((3,) + self.shape, dtype=torch.float64, device=dev)
+        Bbar = torch.empty((3,) + self.shape, dtype=torch.float64, device=dev)
+        sim._before()  # the sweep's kernels after what torch's stream has queued so far
         starts = sorted(self.ckpt.keys())
         for s0 in reversed(starts):
             s1 = min(s0 + self.k, self.nsteps)
@@ -88,8 +91,6 @@ class _Run:
                                               ctypes.c_void_p(ddi.data_ptr() + 8 * t)), "flame_step_adjoint")
                 lam, other = other, lam
             del seg
-        ubar = torch.empty((3,) + self.shape, dtype=torch.float64, device=dev)
-        Bbar = torch.empty((3,) + self.shape, dtype=torch.float64, device=dev)
         _check(lib.flame_init_adjoint(sim._ctx, ctypes.c_void_p(u0.data_ptr()), ctypes.c_void_p(B0.data_ptr()),
                                       ctypes.c_void_p(lam.data_ptr()), ctypes.c_void_p(ubar.data_ptr()),
                                       ctypes.c_void_p(Bbar.data_ptr()), ctypes.c_void_p(ddi.data_ptr() + 8 * self.nsteps)),
