@@ -451,6 +451,12 @@ flame_status flame_step(flame_ctx* c, int n) {
       bool taken = false;
       e = flame::launch_steps(multi_call(c, m), &taken);
       if (e == cudaSuccess && !taken) e = cudaErrorInvalidConfiguration;
+      // a stream with fewer SMs than the device: its blocks are not resident together
+      if (e == cudaErrorCooperativeLaunchTooLarge) {
+        (void)cudaGetLastError();
+        c->multi = multi = false;
+        continue;
+      }
     } else {
       e = flame::launch_step(c->p.storage, c->parity, c->state, c->g, c->k, c->d_flags, c->stream, c->p.variant,
                              c->d_bfield, c->p.kernel);
