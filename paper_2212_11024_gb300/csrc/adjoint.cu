@@ -75,6 +75,12 @@ __device__ __forceinline__ Line line(float am, float a0, float ap) {
 __device__ __forceinline__ float f0(float u, float uu, float a, float h, float e) { return fmaf(uu, e, fmaf(u, h, a)); }
 __device__ __forceinline__ float f1(float u2, float h, float e) { return fmaf(u2, e, h); }
 
+// The ticket of the sum that follows (sum_partials_kernel), cleared by the kernel
+// whose partials it adds: what the memory held before does not matter.
+__device__ __forceinline__ void clear_ticket(unsigned* ticket) {
+  if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x | threadIdx.y) == 0) *ticket = 0u;
+}
+
 // Per-warp partial sums (no block barrier at the end of the step kernel);
 // blocks are whole warps (site_block rounds x to 32).
 __device__ __forceinline__ void warp_sum_to(double v, double* out) {
@@ -449,9 +455,10 @@ __device__ __forceinline__ float adjoint_site(const StepConsts& k, const float (
 template <class T, bool ODD>
 __global__ void __launch_bounds__(kAdjThreads, (kAdjMinBlocks<T, ODD>))
     adjoint_step_kernel(Slots<T> P, Grid g, StepConsts k, const __grid_constant__ LamSlots L,
-                        double* __restrict__ partials) {
+                        double* __restrict__ partials, unsigned* __restrict__ ticket) {
   next_kernel_may_come();
   after_previous_kernel();
+  clear_ticket(ticket);
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z + g.z0;
@@ -569,7 +576,8 @@ __global__ void __launch_bounds__(128, 4)
                                           const double* __restrict__ Bf, const float* __restrict__ lam,
                                           double* __restrict__ ubl, double* __restrict__ Bbl,
                                           double* __restrict__ dub, double* __restrict__ dBb,
-                                          double* __restrict__ partials) {
+                                          double* __restrict__ partials, unsigned* __restrict__ ticket) {
+  clear_ticket(ticket);
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z + g.z0;
@@ -720,8 +728,8 @@ __global__ void init_adjoint_stencil_kernel(Grid g, const double* __restrict__ u
 }
 
 // Deterministic sum of n partials: up to kSumBlocks blocks sum fixed chunks into
-// stage[], and the last of them to finish adds the stage in a fixed order and
-// leaves the ticket at zero.  (Two kernels had taken 8 us a step.)
+// stage[], and the last of them to finish, by the ticket, adds the stage in a fixed
+// order.  (Two kernels had taken 8 us a step.)
 constexpr int kSumBlocks = 64;
 constexpr int kSumThreads = 256;
 __device__ __forceinline__ double sum_of_block(double a) {
@@ -755,19 +763,18 @@ __global__ void __launch_bounds__(kSumThreads)
   if (!last) return;
   double t = threadIdx.x < gridDim.x ? load_l2(stage + threadIdx.x) : 0.0;
   t = sum_of_block(t);
-  if (threadIdx.x == 0) {
-    *out = t;
-    *ticket = 0u;
-  }
+  if (threadIdx.x == 0) *out = t;
 }
-// Sum of n partials into *out; the buffer holds n partials, kSumBlocks doubles
-// and the ticket (zeroed when it was allocated).
+// The buffer holds cap partials, kSumBlocks doubles and the ticket.
+inline unsigned* ticket_of(double* partials, long long cap) {
+  return reinterpret_cast<unsigned*>(partials + cap + kSumBlocks);
+}
+// Sum of n partials into *out.
 inline cudaError_t sum_partials(double* partials, long long cap, long long n, double* out, cudaStream_t s) {
   const long long want = (n + 4 * kSumThreads - 1) / (4 * kSumThreads);
   double* stage = partials + cap;
   return launch_chained(sum_partials_kernel, dim3((unsigned)(want < kSumBlocks ? want : kSumBlocks)), dim3(kSumThreads), 0,
-                        s, static_cast<const double*>(partials), n, stage,
-                        reinterpret_cast<unsigned*>(stage + kSumBlocks), out);
+                        s, static_cast<const double*>(partials), n, stage, ticket_of(partials, cap), out);
 }
 
 // The partials of either adjoint: one per warp of the step kernel, one per
@@ -790,10 +797,11 @@ cudaError_t adjoint_t(int odd, const void* pop, Grid g, const StepConsts& k, con
     L.in[q] = lin + (size_t)q * (size_t)g.n3;
     L.out[q] = lout + (size_t)q * (size_t)g.n3;
   }
-  auto go = [&](auto kern) { return launch_chained(kern, gr, b, 0, s, P, g, k, L, partials); };
+  const long long cap = partials_cap(g);
+  auto go = [&](auto kern) { return launch_chained(kern, gr, b, 0, s, P, g, k, L, partials, ticket_of(partials, cap)); };
   const cudaError_t e = odd ? go(adjoint_step_kernel<T, true>) : go(adjoint_step_kernel<T, false>);
   if (e != cudaSuccess) return e;
-  return sum_partials(partials, partials_cap(g), nblk * ((b.x * b.y) >> 5), ddi, s);
+  return sum_partials(partials, cap, nblk * ((b.x * b.y) >> 5), ddi, s);
 }
 
 }  // namespace
@@ -819,9 +827,10 @@ cudaError_t launch_init_adjoint(Grid g, const StepConsts& k, const double* u, co
   double* Bbl = ws + 3 * n3;
   double* dub = ws + 6 * n3;
   double* dBb = ws + 15 * n3;
-  init_adjoint_local_kernel<<<gr, b, 0, s>>>(g, k, u, B, lam, ubl, Bbl, dub, dBb, partials);
+  const long long cap = partials_cap(g);
+  init_adjoint_local_kernel<<<gr, b, 0, s>>>(g, k, u, B, lam, ubl, Bbl, dub, dBb, partials, ticket_of(partials, cap));
   init_adjoint_stencil_kernel<<<gr, b, 0, s>>>(g, ubl, Bbl, dub, dBb, ubar, Bbar);
-  const cudaError_t e = sum_partials(partials, partials_cap(g), (long long)gr.x * gr.y * gr.z, ddi, s);
+  const cudaError_t e = sum_partials(partials, cap, (long long)gr.x * gr.y * gr.z, ddi, s);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -940,16 +940,13 @@ flame_status flame_step_between(flame_ctx* c, const void* d_from, void* d_to) {
   return FLAME_OK;
 }
 
-// The adjoints' partial sums and their ticket, zeroed (on the context's stream).
+// The adjoints' partial sums and their ticket.
 static cudaError_t adj_partials(flame_ctx* c) {
   if (c->d_adj_partials) return cudaSuccess;
-  const size_t bytes = sizeof(double) * (size_t)flame::adjoint_partials_needed(c->g);
-  cudaError_t e = cudaMalloc(&c->d_adj_partials, bytes);
-  if (e != cudaSuccess) {
-    c->d_adj_partials = nullptr;
-    return e;
-  }
-  return cudaMemsetAsync(c->d_adj_partials, 0, bytes, c->stream);
+  const cudaError_t e =
+      cudaMalloc(&c->d_adj_partials, sizeof(double) * (size_t)flame::adjoint_partials_needed(c->g));
+  if (e != cudaSuccess) c->d_adj_partials = nullptr;
+  return e;
 }
 
 flame_status flame_step_adjoint(flame_ctx* c, const void* d_state, int parity, const float* d_adj_in,

@@ -203,7 +203,7 @@ struct CtxView {
 // Adjoint kernels (adjoint.cu).  The step adjoint reads the forward state at
 // time t (AA parity `odd`), lambda_{t+1} and writes lambda_t (FP32, natural
 // slot order [48][N3]); both write partial d(loss)/d(d_i) into `partials`
-// (adjoint_partials_needed(g) doubles, zeroed once) and their sum into *ddi.
+// (adjoint_partials_needed(g) doubles) and their sum into *ddi.
 long long adjoint_partials_needed(Grid g);
 cudaError_t launch_step_adjoint(int storage, int odd, const void* pop, Grid g, const StepConsts& k, const float* lin,
                                 float* lout, double* partials, double* ddi, cudaStream_t s);
