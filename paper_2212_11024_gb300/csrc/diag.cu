@@ -2,6 +2,8 @@
 // hot path: initialisation from macroscopic fields, moments and
 // decoded populations (FP64), and the deterministic FP64 reduction of the
 // scalar diagnostics.
+#include <type_traits>
+
 #include "aa.cuh"
 #include "expansion.cuh"
 #include "reduce_final.cuh"
@@ -13,7 +15,7 @@ namespace {
 // Initialisation (once per run).  The arithmetic type R is FP32 for 16-bit
 // storage, whose encoding rounds to 2^-11 (FP16) or 2^-8 (BF16) relative, far
 // above FP32's 2^-24; the gradients too are taken in R.  FP32 storage takes
-// two-term FP32 arithmetic (init_site2), and FP64 where that does not reach.
+// two-term FP32 arithmetic, and FP64 where that does not reach (init_columns).
 
 // Periodic central difference of field f along axis a at (x, y, z), in the
 // per-site arithmetic type R (GB300's FP64 pipe is 1/64 of its FP32 rate, so
@@ -129,31 +131,64 @@ __device__ __forceinline__ float init_site(T* __restrict__ pop, const Grid& g, c
 // would leave less of a small deviation), and split by integer operations.
 //
 // A value whose rounding the two terms cannot tell (put_rounded) is stored as
-// FP64 gives it: its site is done again there.  So are sites with values outside
-// [2^-10, 2^10] (density) or of 2^40 and more (fields).
+// FP64 gives it: its site is done again there, in the same columns (with every
+// velocity's products written out that took ~770 operations, now ~330).  So are
+// sites with values outside [2^-10, 2^10] (density) or of 2^40 and more (fields).
 //
-// 128^3 453 us, 256^3 3.3 ms (FP32 fields 330 us and 2.2 ms), bound by FP32 issue
-// and the sites done again, one in 1000 to 2000: 321 us without them.  Five blocks
-// of 128 threads per SM instead of six, whose 80 registers reload some field
-// values: 5 % slower.
+// 128^3 417 us, 256^3 3.2 ms (FP32 fields 302 us and 2.1 ms), bound by FP32 issue
+// and the sites done again, one in 1000 to 2000 of random fields: 321 us without
+// them.  Where populations cancel at every site (a wave with u = b) all are: 1.4 ms
+// (1.6 ms).  Five blocks of 128 threads per SM instead of six, whose 80 registers
+// reload some field values: 5 % slower.
 struct InitConsts {
   F2 p;    // -1 / (3 omega), or 0 without the non-equilibrium parts
   F2 iwB;  // 1 / omega_B, or 0
+  double w3, iw3, wB, iwB64;  // 3 omega, omega_B and their reciprocals
 };
 
-__device__ __forceinline__ F2 field2(double f) { return from_double(f); }
-__device__ __forceinline__ F2 field2(float f) { return {f, 0.f}; }
-// f - g, rounded to FP64 or exactly
-__device__ __forceinline__ F2 diff2(double f, double g) { return from_double(f - g); }
-__device__ __forceinline__ F2 diff2(float f, float g) { return two_diff(f, g); }
-__device__ __forceinline__ float diff1(double f, double g) { return (float)(f - g); }
-__device__ __forceinline__ float diff1(float f, float g) { return __fsub_rn(f, g); }
-
-template <class F>
-__device__ __noinline__ float init_site_fp64(float* pop, Grid g, StepConsts k, int noneq, const F* rho_f, const F* u,
-                                             const F* Bf, const F* gu, const F* gB, int x, int y, int z) {
-  return init_site<float, double, F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+// a / b given r = 1 / b: the remainder of the first quotient corrects it.
+__device__ __forceinline__ double quotient(double a, double b, double r) {
+  const double q = a * r;
+  return fma(fma(-q, b, a), r, q);
 }
+
+// The two arithmetics of the columns below.
+struct TwoTerm {
+  using V = F2;
+  static __device__ __forceinline__ F2 field(double f) { return from_double(f); }
+  static __device__ __forceinline__ F2 field(float f) { return {f, 0.f}; }
+  // f - g, rounded to FP64 or exactly
+  static __device__ __forceinline__ F2 diff(double f, double g) { return from_double(f - g); }
+  static __device__ __forceinline__ F2 diff(float f, float g) { return two_diff(f, g); }
+  static __device__ __forceinline__ F2 add(F2 a, F2 b) { return add2(a, b); }
+  static __device__ __forceinline__ F2 add(F2 a, float b) { return add2(a, b); }
+  static __device__ __forceinline__ F2 addu(F2 a, F2 b) { return add2u(a, b); }
+  static __device__ __forceinline__ F2 mul(F2 a, F2 b) { return mul2(a, b); }
+  static __device__ __forceinline__ F2 mul(float a, F2 b) { return mul2(a, b); }
+  static __device__ __forceinline__ F2 twice(float c, F2 a) { return scaled(c, a); }  // c a power of two
+  static __device__ __forceinline__ float head(F2 a) { return a.h; }
+  // -rho / (3 omega), d / omega_B
+  static __device__ __forceinline__ F2 stress(const InitConsts& ic, int, F2 rho) { return mul2(rho, ic.p); }
+  static __device__ __forceinline__ F2 relaxed(const InitConsts& ic, int, F2 d) { return mul2(ic.iwB, d); }
+};
+struct Fp64 {
+  using V = double;
+  static __device__ __forceinline__ double field(double f) { return f; }
+  static __device__ __forceinline__ double field(float f) { return widened(f); }
+  static __device__ __forceinline__ double diff(double f, double g) { return f - g; }
+  static __device__ __forceinline__ double diff(float f, float g) { return widened(f) - widened(g); }
+  static __device__ __forceinline__ double add(double a, double b) { return a + b; }
+  static __device__ __forceinline__ double addu(double a, double b) { return a + b; }
+  static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+  static __device__ __forceinline__ double twice(double c, double a) { return c * a; }
+  static __device__ __forceinline__ float head(double) { return 0.f; }  // no magnitudes are kept
+  static __device__ __forceinline__ double stress(const InitConsts& ic, int noneq, double rho) {
+    return noneq ? -quotient(rho, ic.w3, ic.iw3) : 0.0;
+  }
+  static __device__ __forceinline__ double relaxed(const InitConsts& ic, int noneq, double d) {
+    return noneq ? quotient(d, ic.wB, ic.iwB64) : 0.0;
+  }
+};
 
 // The error of a sum of two-term values whose terms' magnitudes add up to m: 2^-46
 // m, and what underflow takes of some tens of products; none where there is no
@@ -164,6 +199,9 @@ __device__ __noinline__ float init_site_fp64(float* pop, Grid g, StepConsts k, i
 // to 4e-6 a site the other way.
 __device__ __forceinline__ float error2(float m) { return fminf(__fmaf_rn(0x1p-46f, m, 0x1p-143f), m); }
 
+__device__ __forceinline__ float diff1(double f, double g) { return (float)(f - g); }
+__device__ __forceinline__ float diff1(float f, float g) { return __fsub_rn(f, g); }
+
 // Stores v, which is off by at most e, rounded to FP32; true where e leaves open
 // which of two values that is.
 __device__ __forceinline__ bool put_rounded(float* out, F2 v, float e) {
@@ -172,149 +210,16 @@ __device__ __forceinline__ bool put_rounded(float* out, F2 v, float e) {
   return __fadd_rn(r, __fadd_rn(rest, copysignf(e, rest))) != r;
 }
 
-template <class F>
-__device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid& g, const StepConsts& k,
-                                            const InitConsts& ic, int noneq, const F* __restrict__ rho_f,
-                                            const F* __restrict__ u, const F* __restrict__ Bf,
-                                            const F* __restrict__ gu, const F* __restrict__ gB, int x, int y, int z) {
-  const long long n3 = g.n3;
-  const int site = (z * g.ny + y) * g.nx + x;
-  const Nbr nb = make_nbr(x, y, z, g);
-  const int fwd[3] = {nb.xp, nb.yp, nb.zp}, back[3] = {nb.xm, nb.ym, nb.zm};
-  // d_a F_b
-  auto grad = [&](const F* f, const F* gf, int a, int b) -> F2 {
-    if (gf) return field2(gf[(3 * a + b) * n3 + site]);
-    return scaled(0.5f, diff2(f[b * n3 + site + fwd[a]], f[b * n3 + site + back[a]]));
-  };
-  const F rho_v = rho_f ? rho_f[site] : (F)1;
-  const F2 rho = field2(rho_v), drho = diff2(rho_v, (F)k.rho0);
-  F2 U[3], B[3], b[3], dB[9], S[6];
-  float mS[6], top = 0.f;  // mS: the magnitudes of the terms of S
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const F Bv = Bf[a * n3 + site];
-    U[a] = field2(u[a * n3 + site]);
-    B[a] = field2(Bv);
-    b[a] = diff2(Bv, (F)k.Bref[a]);
-    top = fmaxf(top, fmaxf(fabsf(U[a].h), fabsf(B[a].h)));
-    if (isnan(U[a].h) || isnan(B[a].h)) top = __uint_as_float(0x7f800000u);
-  }
-  const float top_ub = top;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    dB[i] = grad(Bf, gB, i / 3, i % 3);
-    top = isnan(dB[i].h) ? __uint_as_float(0x7f800000u) : fmaxf(top, fabsf(dB[i].h));
-  }
-  constexpr int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};  // xx yy zz xy xz yz
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {  // d_a u_b + d_b u_a
-    const F2 s = grad(u, gu, ia[i], ib[i]), t = i < 3 ? s : grad(u, gu, ib[i], ia[i]);
-    S[i] = i < 3 ? scaled(2.f, s) : add2(s, t);
-    mS[i] = fabsf(s.h) + fabsf(t.h);
-    top = isnan(mS[i]) ? __uint_as_float(0x7f800000u) : fmaxf(top, mS[i]);
-  }
-  if (!(top < 0x1p40f && rho.h < 0x1p10f && rho.h > 0x1p-10f))
-    return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
-  float* out = pop + site;
-  bool open = false;
-  auto put = [&](int slot, F2 v, float e) { open |= put_rounded(out + (long long)slot * n3, v, e); };
+__device__ __forceinline__ bool put_rounded(float* out, double v, float) {
+  *out = (float)v;
+  return false;
+}
 
-  // magnetic: b_b + sign (4 (V_a B_b - B_a V_b) - d_a B_b / omega_B), V = U - d_i curl B
-  {
-    F2 V[3];
-    float mV[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const int p = (a + 1) % 3, q = (a + 2) % 3;
-      V[a] = add2(U[a], mul2(-k.alphaH, add2(dB[3 * p + q], -dB[3 * q + p])));
-      mV[a] = fmaf(k.alphaH, fabsf(dB[3 * p + q].h) + fabsf(dB[3 * q + p].h), fabsf(U[a].h));
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float mb = fabsf(b[c].h);
-      out[(long long)(kQ + c) * n3] = diff1(Bf[c * n3 + site], (F)k.Bref[c]);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const F2 ne = -mul2(ic.iwB, dB[3 * a + c]);
-        const F2 t = a == c ? ne : add2u(scaled(4.f, add2(mul2(V[a], B[c]), -mul2(B[a], V[c]))), ne);
-        const float m = fmaf(ic.iwB.h, fabsf(dB[3 * a + c].h), mb);
-        const float e = error2(a == c ? m : fmaf(4.f, fmaf(mV[a], fabsf(B[c].h), fabsf(B[a].h) * mV[c]), m));
-        put(kQ + 3 * (2 * a + 1) + c, add2u(b[c], t), e);
-        put(kQ + 3 * (2 * a + 2) + c, add2u(b[c], -t), e);
-      }
-    }
-  }
-
-  // fluid; mL: the magnitudes of all terms but those of the equilibrium's velocity part
-  F2 K[6], miso{0.f, 0.f};
-  float mK[6], mI = 0.f;
-  const F2 rp = mul2(rho, ic.p);
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const int a = ia[i], c = ib[i];
-    const F2 N = add2u(mul2(b[c], B[a]), mul2(k.Bref[c], b[a]));
-    K[i] = add2(N, -mul2(rp, S[i]));
-    mK[i] = fmaf(fabsf(rp.h), mS[i], fmaf(fabsf(b[c].h), fabsf(B[a].h), fabsf(k.Bref[c]) * fabsf(b[a].h)));
-  }
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    miso = add2u(miso, scaled(0.5f, mul2(b[a], add2(B[a], k.Bref[a]))));
-    mI = fmaf(fabsf(b[a].h), fabsf(B[a].h) + fabsf(k.Bref[a]), mI);
-  }
-  const F2 base0 = add2(drho, add2(mul2(1.5f, add2(add2u(K[0], K[1]), K[2])), mul2(-4.5f, miso)));
-  const F2 LA = mul2(4.5f, add2(miso, -K[0])), LB = mul2(4.5f, add2(miso, -K[1])), LZ = mul2(4.5f, add2(miso, -K[2]));
-  const F2 LC = mul2(9.f, K[3]), NX = mul2(-9.f, K[4]), NY = mul2(-9.f, K[5]);
-  const float mL = fmaf(9.f, mI + ((mK[3] + mK[4]) + mK[5]), fmaf(6.f, (mK[0] + mK[1]) + mK[2], fabsf(drho.h)));
-  F2 ex[3], ey[3];
-  float mx[2], my[2];  // of ex, ey at c = 0 and +-1
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    F2* e = h ? ey : ex;
-    const F2 uu = mul2(U[h], U[h]), u3 = mul2(3.f, U[h]), q = mul2(3.f, uu);
-    e[0] = add2(q, -u3);
-    e[1] = mul2(-1.5f, uu);
-    e[2] = add2(q, u3);
-    float* m = h ? my : mx;
-    m[0] = 1.5f * uu.h;
-    m[1] = q.h + fabsf(u3.h);
-  }
-  const F2 uzz = mul2(U[2], U[2]);
-  const F2 e0z = mul2(-1.5f, uzz), e1z = mul2(3.f, U[2]), e2z = mul2(4.5f, uzz);
-  float eZ[2][2], e0[2][2];  // the errors at c_z = +-1 and 0 by |c_x|, |c_y|
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float mr = rho.h * fmaf(mx[i & 1], my[i >> 1], mx[i & 1] + my[i >> 1]), mg = mr + rho.h;
-    const float m0 = fmaf(mg, 1.5f * uzz.h, mr + mL);
-    e0[i >> 1][i & 1] = error2(m0);
-    eZ[i >> 1][i & 1] = error2(fmaf(mg, e2z.h + fabsf(e1z.h), m0));
-  }
-#pragma unroll
-  for (int py = 0; py < 3; ++py)
-#pragma unroll
-    for (int px = 0; px < 3; ++px) {
-      const int cx = px - 1, cy = py - 1;
-      const F2 rexy = mul2(rho, add2(mul2(ex[px], ey[py]), add2(ex[px], ey[py])));
-      const F2 gg = add2(rexy, rho);
-      F2 L = base0;
-      if (cx) L = add2u(L, LA);
-      if (cy) L = add2u(L, LB);
-      if (cx * cy) L = add2u(L, cx * cy > 0 ? -LC : LC);
-      const F2 Z0 = add2u(add2u(mul2(gg, e0z), rexy), L);
-      F2 Z1 = mul2(gg, e1z);
-      if (cx) Z1 = add2u(Z1, cx > 0 ? NX : -NX);
-      if (cy) Z1 = add2u(Z1, cy > 0 ? NY : -NY);
-      const F2 tz = add2u(Z0, add2u(mul2(gg, e2z), LZ));
-      const float ez = eZ[cy != 0][cx != 0];
-      put(px + 3 * py, add2u(tz, -Z1), ez);
-      put(px + 3 * py + 9, Z0, e0[cy != 0][cx != 0]);
-      put(px + 3 * py + 18, add2u(tz, Z1), ez);
-    }
-
-  if (open) return init_site_fp64<F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
-
-  // max(|B|^2 / rho, |u|^2), then its root: a Newton step on the FP32 one.  Small
-  // fields are scaled, so that their squares stay in range
-  const float sc = top_ub < 0x1p-50f ? 0x1p80f : 1.f;
+// max(|B|^2 / rho, |u|^2), then its root: a Newton step on the FP32 one.  Small
+// fields (top: the largest component) are scaled, so that their squares stay in
+// range.
+__device__ __forceinline__ float speed2(F2 rho, F2 (&U)[3], F2 (&B)[3], float top) {
+  const float sc = top < 0x1p-50f ? 0x1p80f : 1.f;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     U[a] = scaled(sc, U[a]);
@@ -326,6 +231,167 @@ __device__ __forceinline__ float init_site2(float* __restrict__ pop, const Grid&
   const F2 s2 = va.h > u2.h || (va.h == u2.h && va.l > u2.l) ? va : u2;
   const float r = sqrtf(s2.h);
   return (r > 0.f ? r + __fadd_rn(__fmaf_rn(-r, r, s2.h), s2.l) / (2.f * r) : r) / sc;
+}
+
+template <class F>
+__device__ __noinline__ float init_site_fp64(float* pop, Grid g, StepConsts k, InitConsts ic, int noneq, const F* rho_f, const F* u,
+                                const F* Bf, const F* gu, const F* gB, int x, int y, int z);
+
+// One site's populations, in TwoTerm arithmetic where that does, else in FP64;
+// returns its speed max(|B| / sqrt(rho), |u|).
+template <class Ar, class F>
+__device__ __forceinline__ float init_columns(float* __restrict__ pop, const Grid& g, const StepConsts& k,
+                                              const InitConsts& ic, int noneq, const F* __restrict__ rho_f,
+                                              const F* __restrict__ u, const F* __restrict__ Bf,
+                                              const F* __restrict__ gu, const F* __restrict__ gB, int x, int y, int z) {
+  using V = typename Ar::V;
+  constexpr bool kTwo = std::is_same_v<Ar, TwoTerm>;
+  const long long n3 = g.n3;
+  const int site = (z * g.ny + y) * g.nx + x;
+  const Nbr nb = make_nbr(x, y, z, g);
+  const int fwd[3] = {nb.xp, nb.yp, nb.zp}, back[3] = {nb.xm, nb.ym, nb.zm};
+  // d_a F_b
+  auto grad = [&](const F* f, const F* gf, int a, int b) -> V {
+    if (gf) return Ar::field(gf[(3 * a + b) * n3 + site]);
+    return Ar::twice(0.5f, Ar::diff(f[b * n3 + site + fwd[a]], f[b * n3 + site + back[a]]));
+  };
+  const F rho_v = rho_f ? rho_f[site] : (F)1;
+  const V rho = Ar::field(rho_v), drho = Ar::diff(rho_v, (F)k.rho0);
+  V U[3], B[3], b[3], dB[9], S[6];
+  float mS[6], top = 0.f;  // mS: the magnitudes of the terms of S
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const F Bv = Bf[a * n3 + site];
+    U[a] = Ar::field(u[a * n3 + site]);
+    B[a] = Ar::field(Bv);
+    b[a] = Ar::diff(Bv, (F)k.Bref[a]);
+    top = fmaxf(top, fmaxf(fabsf(Ar::head(U[a])), fabsf(Ar::head(B[a]))));
+    if (isnan(Ar::head(U[a])) || isnan(Ar::head(B[a]))) top = __uint_as_float(0x7f800000u);
+  }
+  const float top_ub = top;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    dB[i] = grad(Bf, gB, i / 3, i % 3);
+    top = isnan(Ar::head(dB[i])) ? __uint_as_float(0x7f800000u) : fmaxf(top, fabsf(Ar::head(dB[i])));
+  }
+  constexpr int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};  // xx yy zz xy xz yz
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {  // d_a u_b + d_b u_a
+    const V s = grad(u, gu, ia[i], ib[i]), t = i < 3 ? s : grad(u, gu, ib[i], ia[i]);
+    S[i] = i < 3 ? Ar::twice(2.f, s) : Ar::add(s, t);
+    mS[i] = fabsf(Ar::head(s)) + fabsf(Ar::head(t));
+    top = isnan(mS[i]) ? __uint_as_float(0x7f800000u) : fmaxf(top, mS[i]);
+  }
+  if (kTwo && !(top < 0x1p40f && Ar::head(rho) < 0x1p10f && Ar::head(rho) > 0x1p-10f))
+    return init_site_fp64<F>(pop, g, k, ic, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+  float* out = pop + site;
+  bool open = false;
+  auto put = [&](int slot, V v, float e) { open |= put_rounded(out + (long long)slot * n3, v, e); };
+
+  // magnetic: b_b + sign (4 (W_a B_b - B_a W_b) - d_a B_b / omega_B), W = U - d_i curl B
+  {
+    V W[3];
+    float mW[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int p = (a + 1) % 3, q = (a + 2) % 3;
+      W[a] = Ar::add(U[a], Ar::mul(-k.alphaH, Ar::add(dB[3 * p + q], -dB[3 * q + p])));
+      mW[a] = fmaf(k.alphaH, fabsf(Ar::head(dB[3 * p + q])) + fabsf(Ar::head(dB[3 * q + p])), fabsf(Ar::head(U[a])));
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float mb = fabsf(Ar::head(b[c]));
+      out[(long long)(kQ + c) * n3] = diff1(Bf[c * n3 + site], (F)k.Bref[c]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const V ne = -Ar::relaxed(ic, noneq, dB[3 * a + c]);
+        const V t = a == c ? ne : Ar::addu(Ar::twice(4.f, Ar::add(Ar::mul(W[a], B[c]), -Ar::mul(B[a], W[c]))), ne);
+        const float m = fmaf(ic.iwB.h, fabsf(Ar::head(dB[3 * a + c])), mb);
+        const float e = error2(a == c ? m : fmaf(4.f, fmaf(mW[a], fabsf(Ar::head(B[c])), fabsf(Ar::head(B[a])) * mW[c]), m));
+        put(kQ + 3 * (2 * a + 1) + c, Ar::addu(b[c], t), e);
+        put(kQ + 3 * (2 * a + 2) + c, Ar::addu(b[c], -t), e);
+      }
+    }
+  }
+
+  // fluid; mL: the magnitudes of all terms but those of the equilibrium's velocity part
+  V K[6], miso{};
+  float mK[6], mI = 0.f;
+  const V rp = Ar::stress(ic, noneq, rho);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int a = ia[i], c = ib[i];
+    const V N = Ar::addu(Ar::mul(b[c], B[a]), Ar::mul(k.Bref[c], b[a]));
+    K[i] = kTwo || noneq ? Ar::add(N, -Ar::mul(rp, S[i])) : N;
+    mK[i] = fmaf(fabsf(Ar::head(rp)), mS[i], fmaf(fabsf(Ar::head(b[c])), fabsf(Ar::head(B[a])), fabsf(k.Bref[c]) * fabsf(Ar::head(b[a]))));
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    miso = Ar::addu(miso, Ar::twice(0.5f, Ar::mul(b[a], Ar::add(B[a], k.Bref[a]))));
+    mI = fmaf(fabsf(Ar::head(b[a])), fabsf(Ar::head(B[a])) + fabsf(k.Bref[a]), mI);
+  }
+  const V base0 = Ar::add(drho, Ar::add(Ar::mul(1.5f, Ar::add(Ar::addu(K[0], K[1]), K[2])), Ar::mul(-4.5f, miso)));
+  const V LA = Ar::mul(4.5f, Ar::add(miso, -K[0])), LB = Ar::mul(4.5f, Ar::add(miso, -K[1])), LZ = Ar::mul(4.5f, Ar::add(miso, -K[2]));
+  const V LC = Ar::mul(9.f, K[3]), NX = Ar::mul(-9.f, K[4]), NY = Ar::mul(-9.f, K[5]);
+  const float mL = fmaf(9.f, mI + ((mK[3] + mK[4]) + mK[5]), fmaf(6.f, (mK[0] + mK[1]) + mK[2], fabsf(Ar::head(drho))));
+  V ex[3], ey[3];
+  float mx[2], my[2];  // of ex, ey at c = 0 and +-1
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    V* e = h ? ey : ex;
+    const V uu = Ar::mul(U[h], U[h]), u3 = Ar::mul(3.f, U[h]), q = Ar::mul(3.f, uu);
+    e[0] = Ar::add(q, -u3);
+    e[1] = Ar::mul(-1.5f, uu);
+    e[2] = Ar::add(q, u3);
+    float* m = h ? my : mx;
+    m[0] = 1.5f * Ar::head(uu);
+    m[1] = Ar::head(q) + fabsf(Ar::head(u3));
+  }
+  const V uzz = Ar::mul(U[2], U[2]);
+  const V e0z = Ar::mul(-1.5f, uzz), e1z = Ar::mul(3.f, U[2]), e2z = Ar::mul(4.5f, uzz);
+  float eZ[2][2], e0[2][2];  // the errors at c_z = +-1 and 0 by |c_x|, |c_y|
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float mr = Ar::head(rho) * fmaf(mx[i & 1], my[i >> 1], mx[i & 1] + my[i >> 1]), mg = mr + Ar::head(rho);
+    const float m0 = fmaf(mg, 1.5f * Ar::head(uzz), mr + mL);
+    e0[i >> 1][i & 1] = error2(m0);
+    eZ[i >> 1][i & 1] = error2(fmaf(mg, Ar::head(e2z) + fabsf(Ar::head(e1z)), m0));
+  }
+#pragma unroll
+  for (int py = 0; py < 3; ++py)
+#pragma unroll
+    for (int px = 0; px < 3; ++px) {
+      const int cx = px - 1, cy = py - 1;
+      const V rexy = Ar::mul(rho, Ar::add(Ar::mul(ex[px], ey[py]), Ar::add(ex[px], ey[py])));
+      const V gg = Ar::add(rexy, rho);
+      V L = base0;
+      if (cx) L = Ar::addu(L, LA);
+      if (cy) L = Ar::addu(L, LB);
+      if (cx * cy) L = Ar::addu(L, cx * cy > 0 ? -LC : LC);
+      const V Z0 = Ar::addu(Ar::addu(Ar::mul(gg, e0z), rexy), L);
+      V Z1 = Ar::mul(gg, e1z);
+      if (cx) Z1 = Ar::addu(Z1, cx > 0 ? NX : -NX);
+      if (cy) Z1 = Ar::addu(Z1, cy > 0 ? NY : -NY);
+      const V tz = Ar::addu(Z0, Ar::addu(Ar::mul(gg, e2z), LZ));
+      const float ez = eZ[cy != 0][cx != 0];
+      put(px + 3 * py, Ar::addu(tz, -Z1), ez);
+      put(px + 3 * py + 9, Z0, e0[cy != 0][cx != 0]);
+      put(px + 3 * py + 18, Ar::addu(tz, Z1), ez);
+    }
+
+  if constexpr (kTwo) {
+    if (open) return init_site_fp64<F>(pop, g, k, ic, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+    return speed2(rho, U, B, top_ub);
+  } else {
+    const double va = sqrt((B[0] * B[0] + B[1] * B[1] + B[2] * B[2]) / rho);
+    return (float)fmax(va, sqrt(U[0] * U[0] + U[1] * U[1] + U[2] * U[2]));
+  }
+}
+
+template <class F>
+__device__ __noinline__ float init_site_fp64(float* pop, Grid g, StepConsts k, InitConsts ic, int noneq, const F* rho_f,
+                                             const F* u, const F* Bf, const F* gu, const F* gB, int x, int y, int z) {
+  return init_columns<Fp64, F>(pop, g, k, ic, noneq, rho_f, u, Bf, gu, gB, x, y, z);
 }
 
 template <class T, class R, class F>
@@ -340,7 +406,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 1)
   float sp = 0.f;
   if (in) {
     if constexpr (sizeof(T) == 4)
-      sp = init_site2<F>(pop, g, k, ic, noneq, rho_f, u, Bf, gu, gB, x, y, z);
+      sp = init_columns<TwoTerm, F>(pop, g, k, ic, noneq, rho_f, u, Bf, gu, gB, x, y, z);
     else
       sp = init_site<T, R, F>(pop, g, k, noneq, rho_f, u, Bf, gu, gB, x, y, z);
     if (!isfinite(sp)) sp = __uint_as_float(0x7f800000u);
@@ -550,12 +616,6 @@ __device__ __forceinline__ void load_magnetic(const float* __restrict__ pop, int
   for (int b = 0; b < 3; ++b)
 #pragma unroll
     for (int i = 0; i < kM; ++i) sg[b][i] = pop[src7<ODD>(b, i, site, nb, n3)];
-}
-
-// a / b given r = 1 / b: the remainder of the first quotient corrects it.
-__device__ __forceinline__ double quotient(double a, double b, double r) {
-  const double q = a * r;
-  return fma(fma(-q, b, a), r, q);
 }
 
 // A site whose sums overflow FP32 or are not finite.
@@ -981,7 +1041,11 @@ cudaError_t init_t(int storage, void* pop, Grid g, const StepConsts& k, int none
                    const F* B, const F* gu, const F* gB, unsigned* speed_bits, cudaStream_t s) {
   const dim3 b = site_block(g), gr = site_grid(g, b);
   const InitConsts ic{noneq ? split(-1.0 / (3.0 * (double)k.omega)) : F2{0.f, 0.f},
-                      noneq ? split(1.0 / (double)k.omegaB) : F2{0.f, 0.f}};
+                      noneq ? split(1.0 / (double)k.omegaB) : F2{0.f, 0.f},
+                      3.0 * (double)k.omega,
+                      1.0 / (3.0 * (double)k.omega),
+                      (double)k.omegaB,
+                      1.0 / (double)k.omegaB};
   switch (storage) {
     case 1:
       init_kernel<float, double, F><<<gr, b, 0, s>>>(static_cast<float*>(pop), g, k, ic, noneq, rho, u, B, gu, gB,
