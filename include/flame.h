@@ -104,7 +104,7 @@ typedef struct {
                          entry points support FLAME_SCHEME only                          */
     int kernel;       /* 0: automatic -- FP16/BF16 storage (any variant) with nx even
                          uses the row kernel (two sites per thread in packed FP32
-                         pairs), in the tiling timed fastest for the row length: x rows
+                         pairs), in a tiling chosen from timings by row length: x rows
                          staged in shared memory by TMA, a whole row per block tile
                          (most lengths that are multiples of 8 from 64 to 1024) or half a
                          row (608, 624, 640), or site pairs of rows of any even length

@@ -783,13 +783,13 @@ cudaError_t probe_t(int odd, const void* pop, Grid g, const StepConsts& k, int n
 // sums of 16-bit storage, whose terms come from FP32 arithmetic, and for FP32
 // storage the sums over the populations and, over the sites, of density,
 // momentum and field.  What is left in FP64 there, the quotients, squares and
-// the sums of those, takes 50 operations a site.  A block that meets a value
-// too large for this, or a non-finite one, sums its sites again in FP64
-// (reduce_general).
+// the sums of those, keeps the FP64 pipe busy 79 % of the time.  A block that
+// meets a value too large for this, or a non-finite one, sums its sites again
+// in FP64 (reduce_general).
 //
 // A thread's sums become FP64 numbers in shared memory, and a warp sums each
-// quantity of the block from there: 13 FP64 additions a warp and quantity,
-// against 40 by shuffles in every warp.
+// quantity of the block from there: 13 FP64 additions for a quantity, against 40
+// by shuffles in each of the block's warps.
 //
 // flame_reduce_static, us at 64^3, 128^3, 256^3: FP32 storage 73, 336, 2380 (all in
 // FP64 1353 at 128^3, 9767 at 256^3; the moments in two-term FP32 arithmetic took

@@ -16,11 +16,11 @@ namespace {
 // not a multiple of 32 a block of x rows leaves lanes idle (33 sites: 64
 // threads); where that is 10 % or more of them, and more often with 16-bit
 // storage (step_shape), the blocks cover consecutive sites instead (flat; a
-// separate instantiation, so the row blocks keep their registers).  GLUPS on ~8M-site lattices, FP32 / FP16 row blocks ->
-// flat: 33 12.2 -> 15.6 / 13.5 -> 22.4, 65 14.1 -> 15.4 / 16.8 -> 22.4, 100
-// 14.8 -> 15.6 / 20.1 -> 22.6 (24.0-24.5 since the sites are numbered without
-// divisions); flat runs at ~15.7 FP32 at any length, row blocks with little
-// waste stay ahead (250: 16.3, 255: 16.4, 256: 17.3).
+// separate instantiation, so the row blocks keep their registers).  GLUPS on
+// ~8M-site lattices, FP32 / FP16 row blocks -> flat: 33 12.2 -> 15.6 / 13.5 ->
+// 22.4, 65 14.1 -> 15.4 / 16.8 -> 22.4, 100 14.8 -> 15.6 / 20.1 -> 22.6 (24.0-24.5
+// since the sites are numbered without divisions); flat runs at ~15.7 FP32 at any
+// length, row blocks with little waste stay ahead (250: 16.3, 255: 16.4, 256: 17.3).
 constexpr int kStepThreads = 256;
 constexpr int kStepMinBlocks = 3;
 
@@ -174,8 +174,8 @@ cudaError_t step_launch(int odd, const Slots<T>& P, Grid g, const StepConsts& k,
 // rows leave a tenth of the lanes idle, and with 16-bit storage wherever they
 // leave any, but for the BGK fluid, whose flat blocks spill (GLUPS FP16, ~4M sites,
 // row blocks / flat: 63 23.6 / 24.3, 159 22.8 / 24.4, 191 23.4 / 24.4, 255 23.7 / 24.2,
-// 287 20.0 / 24.3, 1023 23.9 / 24.5; electron MHD and the FD current alike; BGK
-// 191 23.4 / 22.4, 255 23.5 / 21.9).
+// 287 20.0 / 24.3, 1023 23.9 / 24.5; electron MHD alike, the FD current but for 191,
+// 1 % behind; BGK 191 23.4 / 22.4, 255 23.5 / 21.9).
 template <class T>
 bool step_shape(const Grid& g, int variant, dim3* b, dim3* gr) {
   const int padded = (g.nx + 31) / 32 * 32;

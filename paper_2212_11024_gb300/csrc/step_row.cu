@@ -50,8 +50,8 @@ cudaError_t step_row_flame(const RowCall& c) { return row_call<kVarFlame>(c); }
 // on ~4M-site lattices (nx x m x m, graph replay, GLUPS).  The unstaged pair
 // kernel runs at 25.6-26.3 at every even length (24.6-25.4 while it numbered its
 // pairs by 64-bit divisions, when the lines below were drawn); the staged kernel's
-// whole rows run at 26-32 at most multiples of 8 (64 28.1, 128 31.3, 192 31.0, 256
-// 32.1, 320 28.7, 384 28.3, 448 28.6, 512 30.2, 768 26.7, 1024 30.2) and lose to it
+// whole rows run at 26-32 at most multiples of 8 (64 28.1, 128 31.3, 192 31.1, 256
+// 32.1, 320 28.7, 384 29.8, 448 28.6, 512 30.2, 768 26.7, 1024 30.2) and lose to it
 // where a block is under 48 threads (72-96: 17.8-23.4), where three stages of padded
 // rows fit few blocks (136-152: 20.3-22.6), where a block of 260-320 threads fits
 // once per SM (520-648: 18.6-23.0, half rows 21.3-25.5) and at 776-792 (23.1-23.5).
@@ -69,7 +69,10 @@ cudaError_t step_row_flame(const RowCall& c) { return row_call<kVarFlame>(c); }
 // (window_pitch_fixed) 86.5 % are enough (218 25.7, 222 26.1, 230 27.0, 250 27.9, 190
 // 26.2; where it is not, 96-thread blocks stay behind: 190 24.4);
 // with the FD current, whose B reads the pairs hide better, 94 % (windows / pairs: 222
-// 18.6 / 19.6, 230 19.1 / 19.7, 250 20.0 / 19.7).
+// 18.6 / 19.6, 230 19.1 / 19.7, 250 20.0 / 19.8; 182 19.3 / 19.7 FP16, 19.2 / 19.0
+// BF16).  At run-time pitches it has the line of the others: FP16 windows / pairs 246
+// 19.3 / 19.6, 250 19.5 / 19.7, 306 19.4 / 19.5, 430 19.5 / 19.6, 446 20.1 / 19.8, 1022
+// 20.1 / 19.7, BF16 ahead at all of them (246 19.2 / 19.0, 1022 19.9 / 19.0).
 static bool window_pays(int nx, long long n3, int variant) {
   if (nx % 2 != 0 || nx % 8 == 0 || nx < 176 || nx > 1024) return false;
   const int pairs = nx / 2, threads = (pairs + 31) / 32 * 32, resident = 512 / threads * threads;

@@ -1192,8 +1192,8 @@ size_t row_smem_bytes(int nx, size_t elem, int stages, int H = 1) {
 // to 199 sites, two with direct stores from 200 (~4M-site lattices, GLUPS
 // three / two stages: 136 21.2 / 20.7, 160 25.2 / 24.2, 200 23.9 / 26.5,
 // 224 26.5 / 28.8, 248 28.8 / 28.6).  Compile-time row lengths: 192 with two
-// stages 31.7 against 29.8 for the general one's three (finite-difference
-// current 23.1 / 22.0), 384 with direct stores 30.4 against 29.2.
+// stages 31.1 against 28.8 for the general one's three (finite-difference
+// current 22.3 / 20.9), 384 with direct stores 29.8 against 28.1 (19.7 / 19.4).
 constexpr int row_stages(int nx) { return nx > 128 && nx < 200 && nx != 192 ? 3 : 2; }
 
 // Grid of one persistent instantiation, cached per device (the shared-memory
