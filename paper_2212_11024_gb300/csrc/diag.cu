@@ -843,7 +843,8 @@ constexpr float kRedLimit = 0x1p100f;  // largest term the expansions take
 // block's quantity v from the block's sums r of value().
 template <class T>
 struct Terms {
-  // of rho - rho0, (rho - rho0) u, B - Bref, ...: FP32 per site
+  // of rho - rho0, 2^60 (rho - rho0) u (whose second term FP32 holds for all u),
+  // B - Bref, ...: FP32 per site
   F3 lin[7], u[3], uu, bb, ub, jj, vv;
   float top;
   int n;
@@ -857,11 +858,11 @@ struct Terms {
     const float u2 = m.U[0] * m.U[0] + m.U[1] * m.U[1] + m.U[2] * m.U[2];
     const float b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
     const float j2 = m.J[0] * m.J[0] + m.J[1] * m.J[1] + m.J[2] * m.J[2];
-    const float dv = 4.f * k.omegaB * m.trlam;
+    const float dv = 4.f * k.omegaB * m.trlam, r60 = 0x1p60f * m.drho;
     lin[0] = add3(lin[0], m.drho);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      lin[1 + a] = add3(lin[1 + a], mul2(m.drho, m.U[a]));
+      lin[1 + a] = add3(lin[1 + a], mul2(r60, m.U[a]));
       lin[4 + a] = add3(lin[4 + a], b[a]);
       u[a] = add3(u[a], m.U[a]);
     }
@@ -872,7 +873,7 @@ struct Terms {
     vv = add3(vv, dv * dv);
     top = fmaxf(top, u2);
     ++n;
-    return fabsf(m.drho) * (1.f + u2) + u2 + b2 + j2 + dv * dv + fabsf(b[0]) + fabsf(b[1]) + fabsf(b[2]);
+    return fabsf(r60) * (1.f + u2) + u2 + b2 + j2 + dv * dv + fabsf(b[0]) + fabsf(b[1]) + fabsf(b[2]);
   }
   __device__ __forceinline__ double value(int v) const {
     return v < 7 ? to_double(lin[v]) : v == 7 ? to_double(uu) : v == 8 ? to_double(bb) : v == 9 ? to_double(ub)
@@ -881,7 +882,7 @@ struct Terms {
   }
   static __device__ __forceinline__ double finish(const double* r, int v, const StepConsts& k, const Consts64&) {
     if (v == 0) return fma(r[16], (double)k.rho0, r[0]);
-    if (v < 4) return fma((double)k.rho0, r[9 + v], r[v]);
+    if (v < 4) return fma((double)k.rho0, r[9 + v], 0x1p-60 * r[v]);
     if (v < 7) return fma(r[16], (double)k.Bref[v - 4], r[v]);
     return v == 14 ? sqrt(r[14]) : v == 16 ? 0.0 : r[v];
   }

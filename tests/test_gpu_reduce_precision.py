@@ -49,3 +49,22 @@ def test_sums_of_one_block_over_many_sites(storage):
     for a in range(3):
         t = m["rho"] * m["u"][a]
         assert abs(got[1 + a] - nx * t.sum()) <= 10 * EPS * nx * np.abs(t).sum(), a
+
+
+def test_momentum_of_tiny_velocities():
+    """BF16 storage holds velocities down to FP32's smallest numbers beside ordinary
+    densities: their momentum, one site's, is rho u to three roundings."""
+    from paper_2212_11024_gb300 import Flame
+    rest = next(slot for slot, c, _, _ in _slots() if slot < 27 and not np.any(c))
+    sim = Flame(1, 1, 1, 0.625, 0.625, 1.5, storage="bf16")
+    g = torch.Generator().manual_seed(6)
+    for amp in (1e-20, 1e-30, 1e-36):
+        v = amp * torch.randn(48, generator=g)
+        v[rest] = 0.37
+        sim.set_state(v.to(torch.bfloat16).view(torch.uint8).cuda(), 0, 0)
+        got = sim.reduce_sums()
+        m = {k: x.cpu().numpy().astype(np.longdouble).reshape(-1) for k, x in sim.moments().items()}
+        for a in range(3):
+            t = m["rho"][0] * m["u"][a]
+            assert abs(got[1 + a] - t) <= 3 * EPS * abs(t), (amp, a)
+    sim.close()
